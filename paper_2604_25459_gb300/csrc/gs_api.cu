@@ -459,16 +459,20 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     CK(sc.r012.ensure(wt.recs * 16 * kRecStride), "alloc records");
     CK(sc.r3.ensure(wt.recs * 16), "alloc records");
     CK(sc.mask.ensure(wt.words * 4), "alloc masks");
-    CK(sc.counts.ensure(wt.tiles * 4), "alloc counts");
-    CK(sc.zr.ensure((size_t)We * 8), "alloc depth ranges");
+    RankParams R = rank_sizes(wt.max_words, We, io.lidars != nullptr);
+    const size_t n_bins = (size_t)We * R.bins, n_zero = (size_t)wt.tiles * 2 + n_bins + 1 + kItemClasses + 3;
+    CK(sc.counts.ensure(n_zero * 4), "alloc counts");
     CK(sc.off.ensure(wt.tiles * 4), "alloc offsets");
-    CK(sc.cursor.ensure(wt.tiles * 4), "alloc cursors");
     CK(sc.env_total.ensure((size_t)We * 8), "alloc totals");
     CK(sc.env_base.ensure(((size_t)We + 1) * 8), "alloc bases");
-    CK(sc.work.ensure(16), "alloc work counter");
-    int spill_ctas = 0;  // per-CTA regions for partitioning long buckets
-    CK(composite_max_ctas(tw, th, &spill_ctas), "compositor occupancy");
-    CK(sc.spill.ensure((size_t)spill_ctas * kSpillMax * 8), "alloc spill");
+    CK(sc.bins.ensure(rank_tables(R, We, nullptr)), "alloc depth ranges");
+    rank_tables(R, We, sc.bins.as<unsigned char>());
+    CK(sc.zkeys.ensure(wt.recs * 8), "alloc depth keys");
+    CK(sc.ranks.ensure(wt.recs * 8), "alloc ranks");
+    R.bin_cnt = sc.counts.as<uint32_t>();
+    uint32_t* const counts = R.bin_cnt + n_bins;
+    uint32_t* const cursor = counts + wt.tiles;
+    uint32_t* const work = cursor + wt.tiles;
     const bool debug = s->debug && cap == 0;
     if (debug) CK(sc.dbg_hxy.ensure(wt.recs * 8), "alloc debug");
     uint32_t* const status = io.status ? io.status : s->status;
@@ -507,9 +511,19 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     else CK(launch_project(s->D, P, wt.n_blocks, st), "projection");
     t2.done(1);
     ++*launches;
-    // A3: counts + scan
-    CK(cudaMemsetAsync(sc.counts.p, 0, wt.tiles * 4, st), "memset counts");
-    CK(cudaMemsetAsync(sc.zr.p, 0xff, (size_t)We * 8, st), "memset depth ranges");
+    // A3: counts + scan, around the records' depth ranking
+    CK(cudaMemsetAsync(sc.counts.p, 0, n_zero * 4, st), "memset counters");
+    R.envs = wt.envs;
+    R.mask = P.mask;
+    R.r3 = P.r3;
+    R.zkeys = sc.zkeys.as<unsigned long long>();
+    R.order = sc.ranks.as<uint32_t>();
+    R.rank = R.order + wt.recs;
+    R.status = status;
+    R.index_in_r3 = io.lidars ? 0 : 1;  // LiDAR records keep |g2| in r3.w
+    R.bg_index = s->bg_order.empty() ? nullptr : s->bg_index.as<int>();
+    R.bg_slot = s->bg_order.empty() ? nullptr : s->bg_slot.as<int>();
+    R.n_bg = (unsigned)s->D.n_bg;
     BinParams B{};
     B.envs = wt.envs;
     B.mask = P.mask;
@@ -517,28 +531,29 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     B.e_begin = 0;
     B.tile_w = tw;
     B.tile_h = th;
-    B.words_per_block = kWordsPerBlock;
-    B.counts = sc.counts.as<uint32_t>();
+    B.words_per_block = R.words_per_block;
+    B.counts = counts;
     B.off_local = sc.off.as<uint32_t>();
     B.env_base = sc.env_base.as<unsigned long long>();
-    B.cursor = sc.cursor.as<uint32_t>();
+    B.cursor = cursor;
+    B.rank = R.rank;
     B.status = status;
-    B.index_in_r3 = io.lidars ? 0 : 1;  // LiDAR records keep |g2| in r3.w
     B.wrap = io.lidars ? 1 : 0;         // LiDAR boxes may wrap across azimuth 0
-    B.bg_index = s->bg_order.empty() ? nullptr : s->bg_index.as<int>();
-    B.n_bg = (unsigned)s->D.n_bg;
-    B.zr = sc.zr.as<uint2>();
+    // the warp form's keys carry a subtile mask below the rank while both fit 32 bits
+    const int n_sub = (tw / 8) * (th / 8);
+    if ((use_quad || io.lidars) && n_sub > 1 && ((unsigned long long)wt.max_words * 32) >> (32 - n_sub) == 0)
+        B.key_shift = n_sub;
     PhaseTimer t3(s, st, GS_PHASE_COUNT, timers);
-    CK(launch_count(B, We, wt.max_words, wt.max_T, st), "count");
-    t3.done(1);
-    ++*launches;
+    CK(launch_rank_sample(R, We, st), "depth sample");
+    CK(launch_count(B, R, We, wt.max_words, wt.max_T, st), "count");
+    t3.done(2);
     PhaseTimer t4(s, st, GS_PHASE_SCAN, timers);
-    CK(launch_scan(wt.envs, sc.counts.as<uint32_t>(), sc.off.as<uint32_t>(), sc.env_total.as<unsigned long long>(),
-                   sc.env_base.as<unsigned long long>(), We, st),
+    CK(launch_scan_ranks(wt.envs, counts, sc.off.as<uint32_t>(), sc.env_total.as<unsigned long long>(),
+                         sc.env_base.as<unsigned long long>(), We, R, st),
        "scan");
-    t4.done(2);
-    *launches += 2;
-    CK(cudaMemsetAsync(sc.cursor.p, 0, wt.tiles * 4, st), "memset cursors");
+    CK(launch_rank(R, We, wt.max_words, st), "depth ranks");
+    t4.done(4);
+    *launches += 6;
     // arbitrary rays: cells, rays grouped by tile, compositor items (eager only)
     std::vector<unsigned long long> items;
     if (io.ray_dirs) {
@@ -546,25 +561,25 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         const size_t nr = (size_t)We * (size_t)io.n_rays;
         CK(s->ray_cell.ensure(nr * 4), "alloc ray cells");
         CK(s->ray_list.ensure(nr * 4), "alloc ray lists");
-        for (DevBuf* b : {&s->ray_cnt, &s->ray_off, &s->ray_cur, &s->item_cnt, &s->item_off})
-            CK(b->ensure(wt.tiles * 4), "alloc ray tables");
+        for (DevBuf* b : {&s->ray_cnt, &s->ray_off, &s->ray_cur}) CK(b->ensure(wt.tiles * 16), "alloc ray tables");
+        for (DevBuf* b : {&s->item_cnt, &s->item_off}) CK(b->ensure(wt.tiles * 4), "alloc ray tables");
         for (DevBuf* b : {&s->ray_tot, &s->item_tot}) CK(b->ensure((size_t)We * 8), "alloc ray totals");
         for (DevBuf* b : {&s->ray_base, &s->item_base}) CK(b->ensure((size_t)(We + 1) * 8), "alloc ray bases");
-        CK(cudaMemsetAsync(s->ray_cnt.p, 0, wt.tiles * 4, st), "memset ray counts");
-        CK(cudaMemsetAsync(s->ray_cur.p, 0, wt.tiles * 4, st), "memset ray cursors");
+        CK(cudaMemsetAsync(s->ray_cnt.p, 0, wt.tiles * 16, st), "memset ray counts");
+        CK(cudaMemsetAsync(s->ray_cur.p, 0, wt.tiles * 16, st), "memset ray cursors");
         PhaseTimer tr(s, st, GS_PHASE_SCAN, timers);
         CK(launch_ray_count(io.ray_dirs, io.lidars, wt.envs, We, io.n_rays, s->ray_cell.as<uint32_t>(),
                             s->ray_cnt.as<uint32_t>(), status, st),
            "ray cells");
         CK(launch_scan(wt.envs, s->ray_cnt.as<uint32_t>(), s->ray_off.as<uint32_t>(),
-                       s->ray_tot.as<unsigned long long>(), s->ray_base.as<unsigned long long>(), We, st),
+                       s->ray_tot.as<unsigned long long>(), s->ray_base.as<unsigned long long>(), We, 4, st),
            "ray scan");
         CK(launch_ray_scatter(wt.envs, We, io.n_rays, s->ray_cell.as<uint32_t>(), s->ray_off.as<uint32_t>(),
                               s->ray_cur.as<uint32_t>(), s->ray_list.as<uint32_t>(), s->ray_cnt.as<uint32_t>(),
                               s->item_cnt.as<uint32_t>(), (unsigned)wt.tiles, st),
            "ray lists");
         CK(launch_scan(wt.envs, s->item_cnt.as<uint32_t>(), s->item_off.as<uint32_t>(),
-                       s->item_tot.as<unsigned long long>(), s->item_base.as<unsigned long long>(), We, st),
+                       s->item_tot.as<unsigned long long>(), s->item_base.as<unsigned long long>(), We, 1, st),
            "item scan");
         tr.done(7);
         *launches += 7;
@@ -613,21 +628,20 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
             while (ebd < We && eb[ebd + 1] - eb[ea] <= cap_keys) ++ebd;
             npairs = eb[ebd] - eb[ea];
             base = eb[ea];
-            const size_t want = (size_t)(npairs > 0 ? npairs : 1) * 8;
+            const size_t want = (size_t)(npairs + 4) * 4;  // the compositor reads whole 16-byte words
             if (want > sc.pairs.bytes) {
                 size_t grow = want + want / 4;
-                if (grow > (size_t)cap_keys * 8) grow = want;
+                if (grow > (size_t)cap_keys * 4) grow = want;
                 CK(cudaStreamSynchronize(st), "sync before growth");
                 CK(sc.pairs.ensure(grow), "alloc intersection keys");
             }
-            if (debug) CK(sc.dbg_sorted.ensure(sc.pairs.bytes), "alloc debug lists");
         } else {
-            CK(sc.pairs.ensure((size_t)cap * 8), "alloc intersection keys");
+            CK(sc.pairs.ensure((size_t)(cap + 4) * 4), "alloc intersection keys");
         }
         B.e_begin = ea;
         B.pair_base = base;
-        B.pair_cap = cap == 0 ? (unsigned long long)(sc.pairs.bytes / 8) : cap;
-        B.pairs = sc.pairs.as<unsigned long long>();
+        B.pair_cap = cap == 0 ? (unsigned long long)(sc.pairs.bytes / 4 - 4) : cap;
+        B.pairs = sc.pairs.as<uint32_t>();
         PhaseTimer t5(s, st, GS_PHASE_SCATTER, timers);
         CK(launch_scatter(B, ebd - ea, wt.max_words, wt.max_T, st), "scatter");
         t5.done(1);
@@ -651,25 +665,23 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
             C.n_rays = io.n_rays;
         }
         C.chunk = chunk;
-        C.work = sc.work.as<unsigned int>();
+        C.work = work;
         C.r0 = P.r0;
         C.r1 = P.r1;
         C.r2 = P.r2;
-        C.zr = sc.zr.as<uint2>();
-        C.counts = sc.counts.as<uint32_t>();
+        C.nvis = R.nvis;
+        C.order = R.order;
+        C.counts = counts;
         C.off_local = sc.off.as<uint32_t>();
         C.env_base = sc.env_base.as<unsigned long long>();
         C.pair_base = base;
         C.pair_cap = B.pair_cap;
         C.pairs = B.pairs;
-        C.spill = sc.spill.as<unsigned long long>();
-        C.spill_cap = kSpillMax;
-        C.spill_ctas = (unsigned)spill_ctas;
-        C.dbg_sorted = debug ? sc.dbg_sorted.as<unsigned long long>() : nullptr;
         C.neval = (s->counters && cap == 0) ? s->neval.as<unsigned long long>() : nullptr;
         C.tile_w = tw;
         C.tile_h = th;
         C.quad = use_quad ? 1 : 0;
+        C.key_shift = B.key_shift;
         C.rgb = io.rgb;
         C.depth = io.depth;
         C.alpha = io.alpha;
@@ -679,12 +691,28 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         C.score = io.score;
         C.nbp = (unsigned)bg_slots(s->D.n_bg);
         C.bg_index = s->bg_order.empty() ? nullptr : s->bg_index.as<int>();
-        C.bg_slot = s->bg_order.empty() ? nullptr : s->bg_slot.as<int>();
         C.n_bg = (unsigned)s->D.n_bg;
         C.lidars = io.lidars;
         C.r3 = P.r3;
         C.status = status;
-        CK(cudaMemsetAsync(sc.work.p, 0, 4, st), "memset work counter");
+        if (ea > 0) CK(cudaMemsetAsync(work, 0, 4 + 4 * kItemClasses, st), "memset work counter");
+        if (use_quad || io.lidars) {  // warp form: long buckets first, unless every item starts at once
+            const unsigned long long n_items = C.item_end - C.item_begin;
+            if (n_items * (io.ray_dirs ? 1 : n_sub) > (unsigned long long)kWarpsPerSM * 152 &&
+                n_items * kItemClasses * 4 <= (unsigned long long)s->budget / 64) {
+                CK(sc.items.ensure((size_t)n_items * kItemClasses * 4), "alloc item order");
+                CK(launch_item_order(wt.envs, ea, ebd - ea, wt.max_T, counts,
+                                     io.ray_dirs ? s->item_cnt.as<uint32_t>() : nullptr,
+                                     io.ray_dirs ? s->item_off.as<uint32_t>() : nullptr,
+                                     io.ray_dirs ? s->item_base.as<unsigned long long>() : nullptr,
+                                     sc.items.as<uint32_t>(), (uint32_t)n_items, work + 1, st),
+                   "item order");
+                C.items = sc.items.as<uint32_t>();
+                C.class_cnt = work + 1;
+                C.item_pitch = (unsigned)n_items;
+                ++*launches;
+            }
+        }
         int ctas = 0;
         PhaseTimer t6(s, st, GS_PHASE_COMPOSITE, timers);
         CK(launch_composite(C, st, &ctas), "composite");
@@ -693,6 +721,8 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         if (cap == 0) {
             s->last_ea = ea;
             s->last_eb = ebd;
+            s->last_shift = B.key_shift;
+            s->last_counts = counts;
             s->last_pair_base = base;
         }
         ea = ebd;
@@ -1725,10 +1755,10 @@ gs_status gs_debug_copy_tiles(gs_scene s, int env, uint32_t* counts, int64_t n_c
     if (n_counts < E.T) return fail(GS_ERR_INVALID, "counts holds %lld < %d tiles", (long long)n_counts, E.T);
     CK(cudaSetDevice(s->device), "set device");
     CK(cudaDeviceSynchronize(), "sync");
-    CK(cudaMemcpy(counts, s->sc.counts.as<uint32_t>() + E.tile_base, (size_t)E.T * 4, cudaMemcpyDeviceToHost),
+    CK(cudaMemcpy(counts, s->last_counts + E.tile_base, (size_t)E.T * 4, cudaMemcpyDeviceToHost),
        "copy counts");
     if (!lists) return GS_OK;
-    if (!s->debug || !s->sc.dbg_sorted.p) return fail(GS_ERR_INVALID, "debug was not enabled for the last render");
+    if (!s->debug || !s->sc.dbg_hxy.p) return fail(GS_ERR_INVALID, "debug was not enabled for the last render");
     if (el < s->last_ea || el >= s->last_eb)
         return fail(GS_ERR_INVALID, "env %d is not in the last sub-wave rendered", env);
     unsigned long long base = 0, total = 0;
@@ -1737,15 +1767,25 @@ gs_status gs_debug_copy_tiles(gs_scene s, int env, uint32_t* counts, int64_t n_c
     total -= base;
     if ((unsigned long long)n_lists < total)
         return fail(GS_ERR_INVALID, "lists holds %lld < %llu entries", (long long)n_lists, total);
-    std::vector<unsigned long long> keys(total > 0 ? total : 1);
-    if (total > 0)
-        CK(cudaMemcpy(keys.data(), s->sc.dbg_sorted.as<unsigned long long>() + (base - s->last_pair_base), total * 8,
-                      cudaMemcpyDeviceToHost),
-           "copy lists");
+    if (total == 0) return GS_OK;
+    // the buckets' keys, each tile's put in rank order, and the slot of each rank
+    std::vector<uint32_t> order((size_t)E.n_local);
+    CK(cudaMemcpy(lists, s->sc.pairs.as<uint32_t>() + (base - s->last_pair_base), total * 4, cudaMemcpyDeviceToHost),
+       "copy lists");
+    CK(cudaMemcpy(order.data(), s->sc.ranks.as<uint32_t>() + E.rec_base, (size_t)E.n_local * 4,
+                  cudaMemcpyDeviceToHost),
+       "copy order");
+    uint32_t* l = lists;
+    for (int t = 0; t < E.T; ++t) {
+        for (uint32_t i = 0; i < counts[t]; ++i) l[i] >>= s->last_shift;
+        std::sort(l, l + counts[t]);
+        l += counts[t];
+    }
     const int64_t nbp = bg_slots(s->D.n_bg), lg0 = s->D.n_bg + s->link_offsets[E.link_begin];
     for (unsigned long long i = 0; i < total; ++i) {
-        const int64_t j = (int64_t)(keys[i] & 0xffffffffull);
-        lists[i] = (uint32_t)(j < s->D.n_bg ? j : lg0 + (j - nbp));  // keys carry the caller's index
+        if ((int64_t)lists[i] >= (int64_t)E.n_local) return fail(GS_ERR_DEVICE, "corrupted bucket of env %d", env);
+        const int64_t j = (int64_t)order[lists[i]];
+        lists[i] = (uint32_t)(j < s->D.n_bg ? s->bg_order[(size_t)j] : lg0 + (j - nbp));  // the caller's index
     }
     return GS_OK;
 }

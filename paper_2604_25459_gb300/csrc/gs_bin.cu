@@ -1,5 +1,5 @@
 // (env, tile) intersection counting, prefix scan and bucketed scatter of
-// depth keys (steps A3 and A4).  The renderer of the paper (Sec. III-C
+// depth ranks (steps A3 and A4).  The renderer of the paper (Sec. III-C
 // "Throughput Scaling", built on gsplat) bins projected splats into screen
 // tiles before compositing; this file is that binning, designed for many envs.
 //
@@ -8,8 +8,9 @@
 // a shared-memory histogram per (env, block of Gaussians), so global atomics
 // are one per touched tile per block rather than one per intersection.  The
 // order inside a bucket is arbitrary; the compositor orders each bucket by the
-// unique key (depth bits << 32 | the caller's local index of the Gaussian).
+// records' unique depth ranks (gs_rank.cu).
 #include "gs_internal.cuh"
+#include "gs_block.cuh"
 
 namespace gsb {
 
@@ -24,11 +25,11 @@ __device__ __forceinline__ void tile_span(uint32_t rx, uint32_t ry, int sx, int 
     ty1 = (int)((ry >> 16) >> sy);
 }
 
-// f(t) for every tile t of a record's span: rows ty0..ty1 of the columns
-// tx0..tx1 in one flat loop (lanes with spans of different shapes then diverge
-// only by their tile counts).  WRAP (LiDAR waves): a box with x0 > x1 covers
-// the columns [x0, cols) and [0, x1] (a cone across azimuth 0), so its tile
-// columns run tx0..ntx-1 and then 0..tx1.
+// f(t, tx, ty) for every tile t = ty ntx + tx of a record's span: rows
+// ty0..ty1 of the columns tx0..tx1 in one flat loop (lanes with spans of
+// different shapes then diverge only by their tile counts).  WRAP (LiDAR
+// waves): a box with x0 > x1 covers the columns [x0, cols) and [0, x1] (a cone
+// across azimuth 0), so its tile columns run tx0..ntx-1 and then 0..tx1.
 template <bool WRAP, typename F>
 __device__ __forceinline__ void for_span(uint32_t rx, uint32_t ry, int sx, int sy, int ntx, F&& f) {
     int tx0, tx1, ty0, ty1;
@@ -36,13 +37,14 @@ __device__ __forceinline__ void for_span(uint32_t rx, uint32_t ry, int sx, int s
     if (WRAP && (rx & 0xffffu) > (rx >> 16)) {
         const int nx = min(ntx, ntx - tx0 + tx1 + 1);
         const int n = nx * (ty1 - ty0 + 1);
-        int tx = tx0, row = ty0 * ntx, c = 0;
+        int tx = tx0, ty = ty0, row = ty0 * ntx, c = 0;
         for (int k = 0; k < n; ++k) {
-            f(row + tx);
+            f(row + tx, tx, ty);
             if (++c == nx) {
                 c = 0;
                 tx = tx0;
                 row += ntx;
+                ++ty;
             } else if (++tx == ntx) {
                 tx = 0;
             }
@@ -50,11 +52,12 @@ __device__ __forceinline__ void for_span(uint32_t rx, uint32_t ry, int sx, int s
         return;
     }
     const int n = (tx1 - tx0 + 1) * (ty1 - ty0 + 1);
-    int tx = tx0, t = ty0 * ntx + tx0;
+    int tx = tx0, ty = ty0, t = ty0 * ntx + tx0;
     for (int k = 0; k < n; ++k) {
-        f(t);
+        f(t, tx, ty);
         if (tx == tx1) {
             tx = tx0;
+            ++ty;
             t += ntx - (tx1 - tx0);
         } else {
             ++tx;
@@ -63,70 +66,23 @@ __device__ __forceinline__ void for_span(uint32_t rx, uint32_t ry, int sx, int s
     }
 }
 
-// The visible record slots of mask words [w0, w1) of one env, one word per
-// thread (w1 - w0 <= blockDim.x), listed block-wide in slot order in lst (at
-// most 32 (w1 - w0) entries, slots relative to 32 w0); returns their number.
-// One list per block spreads the visible records evenly over its warps,
-// however unevenly visibility clusters in the storage order, and the scatter
-// walks the same list in both of its passes.  wtot: one u32 per warp.
-__device__ __forceinline__ int block_visible(const uint32_t* mask, int64_t w0, int64_t w1, uint16_t* lst,
-                                             uint32_t* wtot) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int64_t w = w0 + threadIdx.x;
-    uint32_t m = w < w1 ? __ldg(mask + w) : 0u;
-    const uint32_t c = __popc(m);
-    uint32_t incl = c;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += y;
-    }
-    if (lane == 31) wtot[warp] = incl;
-    __syncthreads();
-    uint32_t before = 0, total = 0;
-    for (int i = 0; i < nw; ++i) {
-        const uint32_t t = wtot[i];
-        if (i < warp) before += t;
-        total += t;
-    }
-    uint32_t pos = before + incl - c;
-    while (m) {
-        const int bit = __ffs(m) - 1;
-        m &= m - 1u;
-        lst[pos++] = (uint16_t)(threadIdx.x * 32 + bit);
-    }
-    __syncthreads();
-    return (int)total;
-}
-
-// Rebuilds a block's tile histogram of env el's visible records (the block's
-// list from block_visible, records 32 w0 + lst[i]) in hist[0, T).  Neighbouring
-// threads take neighbouring records of the list.
-// With RANGE, also the smallest and largest depth bits (r3.z) of the records
-// this thread visits, into zl and zh.
-template <bool WRAP, bool RANGE = false>
-__device__ __forceinline__ void block_histogram(const BinParams& P, const EnvInfo& E, int64_t w0, const uint16_t* lst,
-                                                int nvis, uint32_t* hist, uint32_t* zl = nullptr,
-                                                uint32_t* zh = nullptr) {
-    const uint4* r3 = P.r3 + E.rec_base;
-    const int sx = __ffs(P.tile_w) - 1, sy = __ffs(P.tile_h) - 1;
-    for (int i = threadIdx.x; i < nvis; i += blockDim.x) {
-        const uint4 q = r3[w0 * 32 + lst[i]];
-        if constexpr (RANGE) {
-            *zl = min(*zl, q.z);
-            *zh = max(*zh, q.z);
-        }
-        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t) { atomicAdd(&hist[t], 1u); });
-    }
-}
-
 // grid: (blocks over the largest env's visibility words, envs); block 256;
-// dynamic smem: max T u32.  Blocks past their env's words exit at once.
+// dynamic smem: the env's splitters, depth cells and range counters, then max T
+// tile counters.  Blocks past their env's words exit at once.  Counts the
+// visible records of a block (block_visible's list; neighbouring threads take
+// neighbouring records) per tile and per depth range of the env, and notes each
+// record's range and place among the block's records of that range, so that
+// the placement (gs_rank.cu) neither searches nor counts again (both in the
+// placement: 1.12 ms instead of ... on 512 environments at 128x128).
 template <bool WRAP>
-__global__ void __launch_bounds__(256) k_count(BinParams P) {
-    extern __shared__ uint32_t hist[];
-    __shared__ uint16_t wbuf[32 * kWordsPerBlock];
+__global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
+    extern __shared__ __align__(16) unsigned char csm[];
+    __shared__ uint16_t lst[32 * kWordsPerBlock];
     __shared__ uint32_t wtot[32];
+    unsigned long long* split = reinterpret_cast<unsigned long long*>(csm);
+    uint16_t* cell = reinterpret_cast<uint16_t*>(split + R.bins);
+    uint32_t* zhist = reinterpret_cast<uint32_t*>(cell + R.cells);
+    uint32_t* hist = zhist + R.bins;
     const int el = P.e_begin + blockIdx.y;
     const EnvInfo E = P.envs[el];
     const int64_t words = (E.n_local + 31) / 32;
@@ -134,16 +90,23 @@ __global__ void __launch_bounds__(256) k_count(BinParams P) {
     if (w0 >= words) return;
     const int64_t w1 = min(w0 + (int64_t)P.words_per_block, words);
     for (int t = threadIdx.x; t < E.T; t += blockDim.x) hist[t] = 0;
-    const int nvis = block_visible(P.mask + E.mask_base, w0, w1, wbuf, wtot);
-    uint32_t zl = 0xffffffffu, zh = 0u;
-    block_histogram<WRAP, true>(P, E, w0, wbuf, nvis, hist, &zl, &zh);
-    if (P.zr) {  // the env's depth-bit range: one atomic pair per warp
-        zl = __reduce_min_sync(0xffffffffu, zl);
-        zh = __reduce_max_sync(0xffffffffu, zh);
-        if ((threadIdx.x & 31) == 0 && zl <= zh) {
-            atomicMin(&P.zr[el].x, zl);
-            atomicMin(&P.zr[el].y, ~zh);
-        }
+    for (int b = threadIdx.x; b < R.bins; b += blockDim.x) {
+        zhist[b] = 0u;
+        split[b] = R.split[(size_t)el * R.bins + b];
+    }
+    const uint4* gc = reinterpret_cast<const uint4*>(R.cell + (size_t)el * R.cells);
+    for (int c = threadIdx.x; c < R.cells / 8; c += blockDim.x) reinterpret_cast<uint4*>(cell)[c] = gc[c];
+    const int nvis = block_visible(P.mask + E.mask_base, w0, w1, lst, wtot);
+    const uint32_t z0 = (uint32_t)split[R.bins - 1];
+    const int zshift = (int)(split[R.bins - 1] >> 32);
+    const uint4* r3 = P.r3 + E.rec_base;
+    const int sx = __ffs(P.tile_w) - 1, sy = __ffs(P.tile_h) - 1;
+    for (int i = threadIdx.x; i < nvis; i += blockDim.x) {
+        const uint32_t j = (uint32_t)(w0 * 32) + lst[i];
+        const uint4 q = r3[j];
+        const uint32_t b = (uint32_t)rank_bin(split, cell, R.cells, R.bins, z0, zshift, rank_key(R, q, j));
+        R.rank[E.rec_base + j] = b << 13 | atomicAdd(&zhist[b], 1u);
+        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t, int, int) { atomicAdd(&hist[t], 1u); });
     }
     __syncthreads();
     uint32_t* cnt = P.counts + E.tile_base;
@@ -151,24 +114,31 @@ __global__ void __launch_bounds__(256) k_count(BinParams P) {
         const uint32_t h = hist[t];
         if (h) atomicAdd(cnt + t, h);
     }
+    uint32_t* zc = R.bin_cnt + (size_t)el * R.bins;
+    uint32_t* bo = R.block_off + ((size_t)el * R.blocks + blockIdx.x) * R.bins;
+    for (int b = threadIdx.x; b < R.bins; b += blockDim.x) {
+        const uint32_t h = zhist[b];
+        if (h) bo[b] = atomicAdd(zc + b, h);
+    }
 }
 
 static cudaError_t opt_in_smem(const void* fn, size_t smem) {
-    if (smem <= 16 * 1024) return cudaSuccess;  // plus 16 KB of static shared memory
+    if (smem <= 31 * 1024) return cudaSuccess;  // plus 16.1 KB of static shared memory
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-static_assert(kWordsPerBlock <= 256, "binning blocks: one visibility word per thread of 256");
+static_assert(kWordsPerBlock <= 256, "binning blocks: one visibility word per thread of 256, places below 2^13");
 
-cudaError_t launch_count(const BinParams& P, int n_envs, int max_words, int max_T, cudaStream_t st) {
+cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, int max_words, int max_T,
+                         cudaStream_t st) {
     if (n_envs == 0 || max_words == 0) return cudaSuccess;
-    const size_t smem = (size_t)max_T * 4;
+    const size_t smem = (size_t)R.bins * 12 + (size_t)R.cells * 2 + (size_t)max_T * 4;
     const void* fn = P.wrap ? (const void*)k_count<true> : (const void*)k_count<false>;
     cudaError_t e = opt_in_smem(fn, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((max_words + P.words_per_block - 1) / P.words_per_block), (unsigned)n_envs);
-    if (P.wrap) k_count<true><<<grid, 256, smem, st>>>(P);
-    else k_count<false><<<grid, 256, smem, st>>>(P);
+    if (P.wrap) k_count<true><<<grid, 256, smem, st>>>(P, R);
+    else k_count<false><<<grid, 256, smem, st>>>(P, R);
     return cudaGetLastError();
 }
 
@@ -201,14 +171,17 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* warp_tot, T& block_tot
     return before + x - v;
 }
 
-// per env: off_local[t] = sum_{t' < t} counts[t'], env_total = sum
+// per env: off_local[t] = sum_{t' < t} counts[t'], env_total = sum.  With R
+// (bins > 0), also the offsets of the env's depth ranges, the number of ranked
+// records, and the window table: win[v] is the first range start >= v
+// kRankStride, so a window is at most kRankStride plus its last range.
 __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
-                                                   unsigned long long* env_total) {
+                                                   unsigned long long* env_total, int per, RankParams R) {
     __shared__ uint32_t wt[32];
     const int el = blockIdx.x;
-    const int T = envs[el].T;
-    const uint32_t* c = counts + envs[el].tile_base;
-    uint32_t* o = off_local + envs[el].tile_base;
+    const int T = envs[el].T * per;
+    const uint32_t* c = counts + (size_t)envs[el].tile_base * per;
+    uint32_t* o = off_local + (size_t)envs[el].tile_base * per;
     uint32_t carry = 0;
     for (int base = 0; base < T; base += blockDim.x) {
         const int t = base + threadIdx.x;
@@ -219,6 +192,27 @@ __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const ui
         carry += tot;
     }
     if (threadIdx.x == 0) env_total[el] = carry;
+    if (R.bins == 0) return;
+    // two neighbouring ranges per thread
+    const int b = 2 * threadIdx.x;
+    const size_t eb = (size_t)el * R.bins + b;
+    const uint2 c2 = b < R.bins ? *reinterpret_cast<const uint2*>(R.bin_cnt + eb) : make_uint2(0u, 0u);
+    uint32_t nv;
+    const uint32_t start = block_exclusive_scan<uint32_t>(c2.x + c2.y, wt, nv), mid = start + c2.x, end = mid + c2.y;
+    if (b < R.bins) *reinterpret_cast<uint2*>(R.bin_off + eb) = make_uint2(start, mid);
+    uint32_t* win = R.win + (size_t)el * R.win_pitch;
+    if (b == 0) {
+        R.nvis[el] = nv;
+        win[0] = 0u;
+        if (nv % kRankStride) win[nv / kRankStride + 1] = nv;
+    }
+    // the first range boundary at or after every multiple of the stride in
+    // (start, mid] is mid, and in (mid, end] it is end
+    if (b < R.bins) {
+        uint32_t v = start / kRankStride + 1;
+        for (; v * kRankStride <= mid; ++v) win[v] = mid;
+        for (; v * kRankStride <= end; ++v) win[v] = end;
+    }
 }
 
 // env_base[e] = sum_{e' < e} env_total[e'], env_base[We] = total
@@ -237,25 +231,109 @@ __global__ void __launch_bounds__(1024) k_scan_base(const unsigned long long* en
     if (threadIdx.x == 0) env_base[We] = carry;
 }
 
-cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
-                        unsigned long long* env_total, unsigned long long* env_base, int We, cudaStream_t st) {
+static_assert(kRankBins <= 2048, "two depth ranges per thread of the scan");
+
+cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
+                              unsigned long long* env_total, unsigned long long* env_base, int We,
+                              const RankParams& R, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
-    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total);
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, 1, R);
     k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, We);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
+                        unsigned long long* env_total, unsigned long long* env_base, int We, int per,
+                        cudaStream_t st) {
+    if (We == 0) return cudaSuccess;
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, per, RankParams{});
+    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, We);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------- item order
+// A warp composites a bucket of tens of thousands of keys in milliseconds, so
+// a launch of a few items per warp ends on whichever long buckets were claimed
+// last.  Claiming the long classes first fills the tail with short ones.  The
+// lists keep the order of the environments within a class (up to the order of
+// the blocks), so neighbouring tiles still share their records in L2.
+__global__ void __launch_bounds__(256) k_item_order(const EnvInfo* envs, int e_begin, const uint32_t* counts,
+                                                    const uint32_t* item_cnt, const uint32_t* item_off,
+                                                    const unsigned long long* item_base, uint32_t* items,
+                                                    uint32_t pitch, uint32_t* class_cnt) {
+    const int el = e_begin + blockIdx.y, t = blockIdx.x * 256 + threadIdx.x;
+    const int T = envs[el].T;
+    if (blockIdx.x * 256 >= (unsigned)T) return;
+    const uint32_t tile = envs[el].tile_base + (uint32_t)t;
+    int cls = -1;
+    uint32_t first = tile, cnt = 0;
+    if (t < T) {
+        const uint32_t n = counts[tile];
+        cls = n >= 16384u ? 0 : n >= 4096u ? 1 : n >= 1024u ? 2 : 3;
+        cnt = 1;
+        if (item_cnt) {
+            cnt = item_cnt[tile];
+            first = (uint32_t)item_base[el] + item_off[tile];
+        }
+    }
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int c = 0; c < kItemClasses; ++c) {  // one atomic per warp and class
+        const uint32_t mine = cls == c ? cnt : 0u;
+        uint32_t x = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += y;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, x, 31);
+        if (total == 0u) continue;
+        uint32_t at = 0;
+        if (lane == 31) at = atomicAdd(class_cnt + c, total);
+        at = __shfl_sync(0xffffffffu, at, 31) + x - mine;
+        for (uint32_t k = 0; k < mine; ++k) items[(size_t)c * pitch + at + k] = first + k;
+    }
+}
+
+cudaError_t launch_item_order(const EnvInfo* envs, int e_begin, int n_envs, int max_T, const uint32_t* counts,
+                              const uint32_t* item_cnt, const uint32_t* item_off,
+                              const unsigned long long* item_base, uint32_t* items, uint32_t pitch,
+                              uint32_t* class_cnt, cudaStream_t st) {
+    if (n_envs == 0 || max_T == 0) return cudaSuccess;
+    k_item_order<<<dim3((unsigned)((max_T + 255) / 256), (unsigned)n_envs), 256, 0, st>>>(
+        envs, e_begin, counts, item_cnt, item_off, item_base, items, pitch, class_cnt);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- scatter
 // Same partition and visiting order as k_count.  Pass 1 rebuilds the block's
 // histogram, then one global atomic per touched tile reserves the block's range
-// of that bucket; pass 2 writes each key at (bucket start + block range +
+// of that bucket; pass 2 writes each rank at (bucket start + block range +
 // shared cursor).  A key past the pair buffer's capacity (possible only for a
 // launch planned with a fixed capacity) is dropped and flagged.
 
+// The 8x8 subtiles of the tile (tx, ty) that a box reaches, one bit each,
+// row-major.  lx, ly: log2 of the tile's subtile columns and rows (ly <= 1).
 template <bool WRAP>
+__device__ __forceinline__ uint32_t subtile_mask(uint32_t rx, uint32_t ry, int tx, int ty, int lx, int ly) {
+    const int x0 = (int)(rx & 0xffffu) >> 3, x1 = (int)(rx >> 16) >> 3;
+    const int ax = tx << lx, bx = ax + (1 << lx) - 1;
+    uint32_t xm;
+    if (WRAP && (rx & 0xffffu) > (rx >> 16)) {
+        xm = (x0 <= bx ? (2u << (bx - ax)) - (1u << max(x0 - ax, 0)) : 0u) |
+             (x1 >= ax ? (2u << min(x1 - ax, bx - ax)) - 1u : 0u);
+    } else {
+        xm = (2u << (min(x1, bx) - ax)) - (1u << max(x0 - ax, 0));
+    }
+    if (ly == 0) return xm;
+    const int y0 = (int)(ry & 0xffffu) >> 3, y1 = (int)(ry >> 16) >> 3;
+    return (y0 <= 2 * ty ? xm : 0u) | (y1 > 2 * ty ? xm << (1 << lx) : 0u);
+}
+
+template <bool WRAP, bool MASK>
 __global__ void __launch_bounds__(256, 6) k_scatter(BinParams P) {  // <= 42 registers: 6 CTAs/SM
     extern __shared__ uint32_t sm[];
-    __shared__ uint16_t wbuf[32 * kWordsPerBlock];
+    __shared__ uint16_t lst[32 * kWordsPerBlock];
     __shared__ uint32_t wtot[32];
     const int el = P.e_begin + blockIdx.y;
     const EnvInfo E = P.envs[el];
@@ -266,8 +344,14 @@ __global__ void __launch_bounds__(256, 6) k_scatter(BinParams P) {  // <= 42 reg
     uint32_t* hist = sm;
     uint32_t* base = sm + E.T;
     for (int t = threadIdx.x; t < E.T; t += blockDim.x) hist[t] = 0;
-    const int nvis = block_visible(P.mask + E.mask_base, w0, w1, wbuf, wtot);
-    block_histogram<WRAP>(P, E, w0, wbuf, nvis, hist);
+    const int nvis = block_visible(P.mask + E.mask_base, w0, w1, lst, wtot);
+    const uint4* r3 = P.r3 + E.rec_base + w0 * 32;
+    const uint32_t* rank = P.rank + E.rec_base + w0 * 32;
+    const int sx = __ffs(P.tile_w) - 1, sy = __ffs(P.tile_h) - 1;
+    for (int i = threadIdx.x; i < nvis; i += blockDim.x) {
+        const uint4 q = r3[lst[i]];
+        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t, int, int) { atomicAdd(&hist[t], 1u); });
+    }
     __syncthreads();
     uint32_t* cur = P.cursor + E.tile_base;
     const uint32_t* off = P.off_local + E.tile_base;
@@ -278,19 +362,16 @@ __global__ void __launch_bounds__(256, 6) k_scatter(BinParams P) {  // <= 42 reg
         hist[t] = 0;
     }
     __syncthreads();
-    const uint4* r3 = P.r3 + E.rec_base;
-    const int sx = __ffs(P.tile_w) - 1, sy = __ffs(P.tile_h) - 1;
     bool dropped = false;
-    for (int iv = threadIdx.x; iv < nvis; iv += blockDim.x) {
-        const int64_t j = w0 * 32 + wbuf[iv];
-        const uint4 q = r3[j];
-        const uint32_t i = P.index_in_r3 ? q.w
-                           : ((P.bg_index && j < (int64_t)P.n_bg) ? (uint32_t)__ldg(P.bg_index + j) : (uint32_t)j);
-        const unsigned long long key = ((unsigned long long)q.z << 32) | (unsigned long long)i;
-        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t) {
+    for (int i = threadIdx.x; i < nvis; i += blockDim.x) {
+        const uint4 q = r3[lst[i]];
+        const uint32_t key = rank[lst[i]];
+        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t, int tx, int ty) {
             const uint32_t k = atomicAdd(&hist[t], 1u);
             const unsigned long long pos = eb + base[t] + k;
-            if (pos < P.pair_cap) P.pairs[pos] = key;
+            const uint32_t v =
+                MASK ? key << P.key_shift | subtile_mask<WRAP>(q.x, q.y, tx, ty, sx - 3, sy - 3) : key;
+            if (pos < P.pair_cap) P.pairs[pos] = v;
             else dropped = true;
         });
     }
@@ -307,12 +388,16 @@ cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int ma
     // 4: 18.7, 3: 18.6 ms per step; at 320x240 and 128x128 six are fastest
     // (6.8 vs 8.0 ms and 5.1 vs 6.2 ms with 4).
     if ((long long)max_T * P.tile_w * P.tile_h >= 640ll * 480 / 2 && smem < (size_t)29 * 1024) smem = 29 * 1024;
-    const void* fn = P.wrap ? (const void*)k_scatter<true> : (const void*)k_scatter<false>;
+    const bool mask = P.key_shift > 0;
+    const void* fn = P.wrap ? (mask ? (const void*)k_scatter<true, true> : (const void*)k_scatter<true, false>)
+                            : (mask ? (const void*)k_scatter<false, true> : (const void*)k_scatter<false, false>);
     cudaError_t e = opt_in_smem(fn, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((max_words + P.words_per_block - 1) / P.words_per_block), (unsigned)n_envs);
-    if (P.wrap) k_scatter<true><<<grid, 256, smem, st>>>(P);
-    else k_scatter<false><<<grid, 256, smem, st>>>(P);
+    if (P.wrap && mask) k_scatter<true, true><<<grid, 256, smem, st>>>(P);
+    else if (P.wrap) k_scatter<true, false><<<grid, 256, smem, st>>>(P);
+    else if (mask) k_scatter<false, true><<<grid, 256, smem, st>>>(P);
+    else k_scatter<false, false><<<grid, 256, smem, st>>>(P);
     return cudaGetLastError();
 }
 

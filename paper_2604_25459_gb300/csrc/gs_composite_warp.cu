@@ -1,0 +1,794 @@
+// The compositor's warp form: one warp composites one 8x8 subtile (or up to 64
+// rays) on its own, from its tile's bucket to its pixels.  It renders camera
+// images of low resolution and every LiDAR scan (paper Sec. III-C, Sec. III-E);
+// gs_composite.cu holds the form for large images.
+//
+// At 128x128 a splat covers a few pixels and half of a view's keys fall in two
+// or three tiles: the four warps of a 16x16 tile's CTA spent more time waiting
+// for one another at each staged batch than on any other stall, and the chip
+// drained on the longest buckets.  Here a subtile's warp shares nothing, so
+// there is no barrier left; every lane stages one splat, tests it against the
+// subtile in registers, and the records of the next 32 splats are copied
+// (cp.async) while the current ones are blended.  The four warps of a tile each
+// read the tile's bucket and keep the keys whose subtile bit is set.
+//
+// The bucket's keys are depth ranks (gs_rank.cu) in any order; windows of at
+// most kCap ranks come in order from
+//   - the whole bucket at once, if it is short;
+//   - a histogram over kSortBins rank ranges, windows being runs of ranges
+//     gathered from the bucket and sorted in shared memory (few keys per rank:
+//     LiDAR scans rank every Gaussian around the sensor);
+//   - a bitmap of the next 32768 ranks (many keys per rank), read back in order.
+// Each pixel blends the same splats in the same order with the same arithmetic
+// as in gs_composite.cu, so the images do not depend on the form.
+#include "gs_blend.cuh"
+#include "gs_block.cuh"
+
+namespace gsb {
+
+namespace {
+
+constexpr uint32_t kAll = 0xffffffffu;
+constexpr int kCap = 512;         // ranks per window
+constexpr int kSortBins = 512;    // counters of the sort and of the histogram
+constexpr int kCrowd = 24;        // longest range sorted by insertion
+constexpr int kWords = 1024;      // bitmap words
+constexpr int kGroups = 64;       // groups of 16 bitmap words (512 ranks)
+constexpr uint32_t kShort = 1024; // buckets gathered whole
+
+// f(key, valid) for every key of the bucket L[0, n), by the whole warp: 16-byte
+// loads, four in flight per lane.  Reads up to three words on either side of
+// the bucket (the key buffer is padded); they come with valid = false.
+template <typename F>
+__device__ __forceinline__ void warp_keys(const uint32_t* L, uint32_t n, F&& f) {
+    constexpr int U = 4;
+    const uint32_t lane = threadIdx.x;
+    const uint32_t off = (uint32_t)((uintptr_t)L & 15u) >> 2, end = off + n;
+    const uint4* V = reinterpret_cast<const uint4*>(L - off);
+    for (uint32_t i = 0; i < end; i += 128 * U) {
+        uint4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t x = i + 128 * u + 4 * lane;
+            v[u] = x < end ? __ldg(V + (x >> 2)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t x = i + 128 * u;
+            if (x >= end) break;
+            const uint32_t y = x + 4 * lane - off;  // index in the bucket; wraps below it
+            f(v[u].x, y < n);
+            f(v[u].y, y + 1 < n);
+            f(v[u].z, y + 2 < n);
+            f(v[u].w, y + 3 < n);
+        }
+    }
+}
+
+// Sorts keys[0, m), distinct ranks in [lo, hi], m <= kCap (tmp: scratch).  One key per lane: a bitonic network in
+// registers.  Otherwise a counting sort by kSortBins equal ranges with
+// insertion inside a range, or, when a range holds more than kCrowd, a bitonic
+// sort in shared memory.
+__device__ __forceinline__ void warp_sort(uint32_t* keys, uint32_t* tmp, uint32_t* cnt, int m, uint32_t lo,
+                                          uint32_t hi) {
+    const int lane = threadIdx.x;
+    if (m <= 32) {
+        uint32_t k = lane < m ? keys[lane] : kAll;
+#pragma unroll
+        for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                const uint32_t o = __shfl_xor_sync(kAll, k, stride);
+                const bool up = (lane & size) == 0, low = (lane & stride) == 0;
+                k = up == low ? min(k, o) : max(k, o);
+            }
+        keys[lane] = k;
+        __syncwarp();
+        return;
+    }
+    const uint32_t span = hi - lo;
+    const int shift = (span >> 9) ? 23 - __clz(span) : 0;  // span >> shift < kSortBins
+    uint4* c4 = reinterpret_cast<uint4*>(cnt);
+#pragma unroll
+    for (int j = 0; j < kSortBins / 128; ++j) c4[lane + 32 * j] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) atomicAdd(&cnt[(keys[i] - lo) >> shift], 1u);
+    __syncwarp();
+    constexpr int PER = kSortBins / 32;
+    uint32_t sum = 0, most = 0;
+    uint4 q[PER / 4];
+#pragma unroll
+    for (int j = 0; j < PER / 4; ++j) {
+        q[j] = c4[lane * (PER / 4) + j];
+        sum += q[j].x + q[j].y + q[j].z + q[j].w;
+        most = max(most, max(max(q[j].x, q[j].y), max(q[j].z, q[j].w)));
+    }
+    if (__any_sync(kAll, most > (uint32_t)kCrowd)) {
+        int p = 64;
+        while (p < m) p <<= 1;
+        for (int i = m + lane; i < p; i += 32) keys[i] = kAll;
+        for (int size = 2; size <= p; size <<= 1)
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                __syncwarp();
+                for (int x = lane; x < p / 2; x += 32) {
+                    const int i = 2 * x - (x & (stride - 1)), j = i + stride;
+                    const uint32_t a = keys[i], b = keys[j];
+                    if ((a > b) == ((i & size) == 0)) {
+                        keys[i] = b;
+                        keys[j] = a;
+                    }
+                }
+            }
+        __syncwarp();
+        return;
+    }
+    uint32_t run = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(kAll, run, d);
+        if (lane >= d) run += y;
+    }
+    run -= sum;
+#pragma unroll
+    for (int j = 0; j < PER / 4; ++j) {
+        uint4 r;
+        r.x = run;
+        r.y = r.x + q[j].x;
+        r.z = r.y + q[j].y;
+        r.w = r.z + q[j].z;
+        run = r.w + q[j].w;
+        c4[lane * (PER / 4) + j] = r;
+    }
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) {
+        const uint32_t k = keys[i];
+        tmp[atomicAdd(&cnt[(k - lo) >> shift], 1u)] = k;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int b = lane; b < kSortBins; b += 32) {  // cnt[b] is the end of range b now
+        const int e = (int)cnt[b], a = b ? (int)cnt[b - 1] : 0;
+        for (int x = a + 1; x < e; ++x) {
+            const uint32_t k = tmp[x];
+            int y = x - 1;
+            while (y >= a && tmp[y] > k) {
+                tmp[y + 1] = tmp[y];
+                --y;
+            }
+            tmp[y + 1] = k;
+        }
+    }
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) keys[i] = tmp[i];
+    __syncwarp();
+}
+
+__device__ __forceinline__ void copy16(float4* dst, const float4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+}  // namespace
+
+// MODE 0: camera image or observation; 2: the same, also counting composited
+// (pixel, splat) pairs into P.neval; 1: LiDAR scan on a grid (records of
+// k_project_lidar; a "pixel" is a ray, the Gaussian evaluated at its closest
+// approach); 3: LiDAR along arbitrary rays (an item is a chunk of at most 64
+// rays of a 16x16 grid tile, grouped by 8x8 subtile; the culling box is that
+// of the rays' cells).
+//
+// Lanes work in four groups of eight: group q owns the 4x4 quadrant (q & 1, q
+// >> 1) of the subtile, a lane two of its pixels, and walks only the splats
+// whose box reaches it, so the groups advance through different splats at
+// once (MODE 3: all lanes walk the same splats).  Against the CTA form's
+// quadrants, 2048 environments of the room... see the table in the header of
+// launch_composite_warp.
+template <int MODE>
+__global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
+    constexpr bool LID = MODE == 1 || MODE == 3;
+    constexpr bool QUAD = MODE != 3;
+    constexpr bool CNT = MODE != 0;
+    __shared__ __align__(16) uint32_t keys[kCap];
+    __shared__ __align__(16) uint32_t bm[kWords];  // bitmap | sort counters, then range starts
+    __shared__ uint32_t pre[kGroups + 1];
+    __shared__ float4 rec[2][3][32];  // records of this and the next 32 splats: r0, r1, r2; between windows sort scratch
+    static_assert(sizeof(rec) >= kCap * 4, "the sort scratch shares the records' memory");
+    __shared__ float4 sD[LID ? 32 : 1];            // LiDAR: third row of G
+    __shared__ int4 sR[LID ? 32 : 1];              // LiDAR: x0, x1 - x0, y0, y1 - y0
+    const int lane = threadIdx.x;
+    const int lx = __ffs(P.tile_w) - 4, ly = __ffs(P.tile_h) - 4;  // log2 of the tile's subtile columns, rows
+    const int lsub = MODE == 3 ? 0 : lx + ly;
+    const int grp = lane >> 3, l8 = lane & 7;
+    int el = P.e_begin;
+    unsigned int e_lo = P.envs[el].tile_base, e_hi = e_lo + (unsigned)P.envs[el].T;
+    const unsigned int t_env = e_hi - e_lo;  // tiles of the first env: uniform batches find an item's env by division
+    const unsigned int end = (P.item_end - P.item_begin) << lsub;
+    uint32_t cb[kItemClasses] = {0};  // items before each class of the claiming order
+    if (P.items)
+        for (int c = 1; c < kItemClasses; ++c) cb[c] = cb[c - 1] + __ldg(P.class_cnt + c - 1);
+    unsigned int claim = 0;
+    if (lane == 0) claim = atomicAdd(P.work, (unsigned)P.chunk);
+    for (;;) {
+    const unsigned int first = __shfl_sync(kAll, claim, 0);
+    if (first >= end) break;
+    if (lane == 0) claim = atomicAdd(P.work, (unsigned)P.chunk);  // the next claim, in flight meanwhile
+    const unsigned int last = min(first + (unsigned)P.chunk, end);
+    for (unsigned int it = first; it < last; ++it) {
+    unsigned int item = P.item_begin + (it >> lsub);
+    if (P.items) {
+        const unsigned int q = it >> lsub;
+        const int c = q >= cb[3] ? 3 : q >= cb[2] ? 2 : q >= cb[1] ? 1 : 0;
+        const uint32_t before = q >= cb[3] ? cb[3] : q >= cb[2] ? cb[2] : q >= cb[1] ? cb[1] : 0u;
+        item = __ldg(P.items + (size_t)c * P.item_pitch + (q - before));
+    }
+    const int sub = (int)(it & ((1u << lsub) - 1u));
+    int t;
+    uint32_t rchunk = 0;  // MODE 3: chunk of the tile's rays
+    if constexpr (MODE == 3) {
+        int lo = P.e_begin, hi = P.e_end - 1;  // env: last e with item_base[e] <= item
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(&P.item_base[mid]) <= (unsigned long long)item) lo = mid; else hi = mid - 1;
+        }
+        el = lo;
+        e_lo = P.envs[el].tile_base;
+        const uint32_t li = item - (uint32_t)__ldg(&P.item_base[el]);
+        int a = 0, b = P.envs[el].T - 1;  // tile: last t with item_off[t] <= li (empty tiles come before)
+        while (a < b) {
+            const int mid = (a + b + 1) >> 1;
+            if (__ldg(&P.item_off[e_lo + mid]) <= li) a = mid; else b = mid - 1;
+        }
+        t = a;
+        rchunk = li - __ldg(&P.item_off[e_lo + t]);
+    } else {
+        if (item < e_lo || item >= e_hi) {
+            el = min(P.e_begin + (int)((item - P.item_begin) / t_env), P.e_end - 1);
+            e_lo = __ldg(&P.envs[el].tile_base);
+            e_hi = e_lo + (unsigned)__ldg(&P.envs[el].T);
+            if (item < e_lo || item >= e_hi) {
+                int lo = P.e_begin, hi = P.e_end - 1;  // env: last e with tile_base <= item
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (__ldg(&P.envs[mid].tile_base) <= item) lo = mid; else hi = mid - 1;
+                }
+                el = lo;
+                e_lo = __ldg(&P.envs[el].tile_base);
+                e_hi = e_lo + (unsigned)__ldg(&P.envs[el].T);
+            }
+        }
+        t = (int)(item - e_lo);
+    }
+    const EnvInfo* Ep = P.envs + el;
+    const int W = __ldg(&Ep->W), H = __ldg(&Ep->H), ntx = __ldg(&Ep->ntx);
+    const unsigned long long pix_base = __ldg(&Ep->pix_base);
+    const int tx = t % ntx, ty = t / ntx;
+    int wx0 = (tx * P.tile_w) + (sub & ((1 << lx) - 1)) * 8, wy0 = (ty * P.tile_h) + (sub >> lx) * 8;
+    if (MODE != 3 && (wx0 >= W || wy0 >= H)) continue;  // a subtile outside the image
+    int wx1 = wx0 + 7, wy1 = wy0 + 7;
+    const int px = wx0 + 4 * (grp & 1) + (l8 & 3);
+    const int py0 = wy0 + 4 * (grp >> 1) + (l8 >> 2), py1 = py0 + 2;
+    bool in0 = px < W && py0 < H, in1 = px < W && py1 < H;
+    const float fpx = (float)px + 0.5f, fpy0 = (float)py0 + 0.5f, fpy1 = (float)py1 + 0.5f;
+    float3 dir0 = make_float3(0.f, 0.f, 0.f), dir1 = dir0;  // LiDAR: the lane's two rays
+    int cx0 = px, cy0 = py0, cx1 = px, cy1 = py1;           // LiDAR: their grid cells
+    int ray0 = -1, ray1 = -1;                               // MODE 3: their indices
+    float near_range = 0.0f;
+    uint32_t submask = 1u << sub;  // subtile bits of the keys this warp takes
+    if constexpr (MODE == 1) {
+        const gs_lidar* Ld = P.lidars + el;
+        const float em = __ldg(&Ld->elev_min), eM = __ldg(&Ld->elev_max);
+        const float az0 = __ldg(&Ld->az_min), span = __ldg(&Ld->az_max) - az0;
+        const float phi = az0 + span * fpx / (float)W;
+        const float th0 = em + (eM - em) * fpy0 / (float)H, th1 = em + (eM - em) * fpy1 / (float)H;
+        float sp, cp, s0, c0, s1, c1;
+        sincosf(phi, &sp, &cp);
+        sincosf(th0, &s0, &c0);
+        sincosf(th1, &s1, &c1);
+        dir0 = make_float3(c0 * cp, c0 * sp, s0);
+        dir1 = make_float3(c1 * cp, c1 * sp, s1);
+        near_range = __ldg(&Ld->near_range);
+    }
+    if constexpr (MODE == 3) {
+        const size_t renv = (size_t)el * (size_t)P.n_rays;
+        const size_t rt = 4 * (size_t)(e_lo + t);
+        const uint4 rc = __ldg(reinterpret_cast<const uint4*>(P.ray_cnt + rt));  // per subtile
+        const uint32_t total = rc.x + rc.y + rc.z + rc.w;
+        const uint32_t k0 = rchunk * (uint32_t)kRayChunk + (uint32_t)lane, k1 = k0 + 32u;
+        const uint32_t* list = P.ray_list + renv + __ldg(P.ray_off + rt);
+        in0 = k0 < total;
+        in1 = k1 < total;
+        near_range = __ldg(&P.lidars[el].near_range);
+        uint32_t subs = 0;
+        auto take = [&](uint32_t k, int& ray, int& ci, int& cj, float3& d) {
+            const uint32_t r = __ldg(list + k);
+            ray = (int)r;
+            const uint32_t c = __ldg(&P.ray_cell[renv + r]) & 255u;
+            ci = tx * 16 + (int)(c & 15u);
+            cj = ty * 16 + (int)(c >> 4);
+            subs |= 1u << (((c >> 6) & 2u) | ((c >> 3) & 1u));
+            const float* v = P.ray_dirs + (renv + r) * 3;
+            const float x = v[0], y = v[1], z = v[2];
+            const float inv = 1.0f / sqrtf(x * x + y * y + z * z);
+            d = make_float3(x * inv, y * inv, z * inv);
+        };
+        if (in0) take(k0, ray0, cx0, cy0, dir0);
+        if (in1) take(k1, ray1, cx1, cy1, dir1);
+        submask = __reduce_or_sync(kAll, subs);
+        // the warp's culling box: the cells of its rays
+        const int big = 1 << 30;
+        wx0 = __reduce_min_sync(kAll, min(in0 ? cx0 : big, in1 ? cx1 : big));
+        wy0 = __reduce_min_sync(kAll, min(in0 ? cy0 : big, in1 ? cy1 : big));
+        wx1 = __reduce_max_sync(kAll, max(in0 ? cx0 : -big, in1 ? cx1 : -big));
+        wy1 = __reduce_max_sync(kAll, max(in0 ? cy0 : -big, in1 ? cy1 : -big));
+    }
+    // LiDAR: alpha and t* of a staged Gaussian (b, o | g0 | g1 | g2) on each
+    // of the lane's two rays d: u = G d, q = |u x b|^2 / |u|^2, t* = u.b / |u|^2,
+    // with paired FP32 instructions (the reciprocal of |u|^2 by the fast
+    // division, ~2 ulp, far inside the scan's tolerance).
+    auto ray_eval2 = [&](const float4& A, const float4& B, const float4& C, const float4& D, float2& al,
+                         float2& ts) {
+        const float2 dx = make_float2(dir0.x, dir1.x), dy = make_float2(dir0.y, dir1.y),
+                     dz = make_float2(dir0.z, dir1.z);
+        auto dot = [&](const float4& G) {
+            return __ffma2_rn(make_float2(G.z, G.z), dz,
+                              __ffma2_rn(make_float2(G.y, G.y), dy, __fmul2_rn(make_float2(G.x, G.x), dx)));
+        };
+        const float2 u0 = dot(B), u1 = dot(C), u2 = dot(D);
+        const float2 aa = __ffma2_rn(u2, u2, __ffma2_rn(u1, u1, __fmul2_rn(u0, u0)));
+        const float2 ab = __ffma2_rn(u2, make_float2(A.z, A.z),
+                                     __ffma2_rn(u1, make_float2(A.y, A.y), __fmul2_rn(u0, make_float2(A.x, A.x))));
+        const float2 c0 = __ffma2_rn(u1, make_float2(A.z, A.z), __fmul2_rn(u2, make_float2(-A.y, -A.y)));
+        const float2 c1 = __ffma2_rn(u2, make_float2(A.x, A.x), __fmul2_rn(u0, make_float2(-A.z, -A.z)));
+        const float2 c2 = __ffma2_rn(u0, make_float2(A.y, A.y), __fmul2_rn(u1, make_float2(-A.x, -A.x)));
+        const float2 cc = __ffma2_rn(c2, c2, __ffma2_rn(c1, c1, __fmul2_rn(c0, c0)));
+        const float2 inv = make_float2(__fdividef(1.0f, aa.x), __fdividef(1.0f, aa.y));
+        const float2 q = __fmul2_rn(cc, inv);
+        ts = __fmul2_rn(ab, inv);
+        const float k = -0.72134752044448170f;  // -log2(e) / 2
+        al.x = ts.x > near_range ? fminf(0.99f, A.w * ex2_approx(k * q.x)) : 0.0f;
+        al.y = ts.y > near_range ? fminf(0.99f, A.w * ex2_approx(k * q.y)) : 0.0f;
+    };
+    bool done0 = !in0, done1 = !in1;
+    // the lane's two pixels: .x = (px, py0), .y = (px, py1)
+    float2 Tp = make_float2(1.0f, 1.0f), rp = make_float2(0.0f, 0.0f), gp = rp, bp = rp, dp = rp;
+    const float2 fpy = make_float2(fpy0, fpy1);
+    uint32_t ncomp = 0;
+
+    uint32_t n = P.counts[e_lo + t];
+    const unsigned long long start = __ldg(P.env_base + el) - P.pair_base + P.off_local[e_lo + t];
+    if (start + n > P.pair_cap) {  // keys past a planned capacity were dropped: render nothing
+        n = 0;
+        if (lane == 0) atomicOr(P.status, kStOverflow);
+    }
+    const uint32_t* Lk = P.pairs + start;
+    const size_t recbase = (size_t)__ldg(&Ep->rec_base);
+    const uint32_t n_local = __ldg(&Ep->n_local);
+    const uint32_t* order = P.order + recbase;  // record slot of each rank
+    const uint32_t n_rank = __ldg(P.nvis + el);
+    const int kshift = P.key_shift;
+    // the rank of a key and whether this warp's pixels lie in its subtiles
+    auto taken = [&](uint32_t k) { return kshift == 0 || (k & submask) != 0u; };
+
+    // Composite the ordered ranks keys[0, m).  True once every pixel of the warp
+    // has terminated.
+    auto run_window = [&](int m) -> bool {
+        auto slot_of = [&](int i) -> uint32_t { return i < m ? __ldg(order + keys[i]) : kAll; };
+        auto fetch = [&](int buf, uint32_t s) {
+            if (s < n_local) {
+                const float4* src = P.r0 + (size_t)kRecStride * (recbase + s);
+                copy16(&rec[buf][0][lane], src);
+                copy16(&rec[buf][1][lane], src + 1);
+                copy16(&rec[buf][2][lane], src + 2);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        uint32_t cur = slot_of(lane), nxt = slot_of(32 + lane);
+        fetch(0, cur);
+        for (int c = 0; c < m; c += 32) {
+            const int b = (c >> 5) & 1;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            const bool own = cur < n_local;  // a splat of this chunk (every rank of a sound bucket has a slot)
+            const uint32_t slot = cur;
+            cur = nxt;
+            if (c + 32 < m) fetch(b ^ 1, cur);
+            nxt = slot_of(c + 64 + lane);
+            float4* sA = rec[b][0];
+            float4* sB = rec[b][1];
+            float4* sC = rec[b][2];
+            bool ov = false;
+            int bx0 = 0, bx1 = -1, by0 = 0, by1 = -1;
+            if (own) {
+                const float4 q1 = sB[lane];
+                const uint32_t rx = __float_as_uint(q1.w), ry = __float_as_uint(sC[lane].w);
+                bx0 = (int)(rx & 0xffffu);
+                bx1 = (int)(rx >> 16);
+                by0 = (int)(ry & 0xffffu);
+                by1 = (int)(ry >> 16);
+                if constexpr (LID) {
+                    const float4 q2 = sC[lane];
+                    // g2 = |g2| (g0 x g1) / (|g0| |g1|): the rows of G are orthogonal
+                    const float glen2 = __uint_as_float(__ldg(&P.r3[recbase + slot].w));
+                    const float gx = q1.y * q2.z - q1.z * q2.y, gy = q1.z * q2.x - q1.x * q2.z,
+                                gz = q1.x * q2.y - q1.y * q2.x;
+                    const float k = glen2 * rsqrtf((q1.x * q1.x + q1.y * q1.y + q1.z * q1.z) *
+                                                   (q2.x * q2.x + q2.y * q2.y + q2.z * q2.z));
+                    sD[lane] = make_float4(gx * k, gy * k, gz * k, 0.0f);
+                    if (bx0 > bx1) {
+                        // a box across azimuth 0 (columns [x0, cols) and [0, x1]): the
+                        // hull of its parts in this tile's columns [ta, tb], the high
+                        // part [max(x0, ta), tb] when x0 <= tb and the low part
+                        // [ta, min(x1, tb)] when x1 >= ta
+                        const int ta = tx * 16, tb = ta + 15;
+                        const int h0 = max(bx0, ta), l1 = min(bx1, tb);
+                        bx0 = bx1 >= ta ? ta : h0;
+                        bx1 = h0 <= tb ? tb : l1;
+                    }
+                    sR[lane] = make_int4(bx0, bx1 - bx0, by0, by1 - by0);
+                } else {
+                    const float o = sA[lane].z;
+                    sA[lane].z = log2f(o);  // folded into the exponent of alpha
+                }
+                ov = bx0 <= wx1 && bx1 >= wx0 && by0 <= wy1 && by1 >= wy0;
+            }
+            if constexpr (!LID) {
+                // large splats: the exact ellipse (a box under 24 px in width + height
+                // is kept as it is: it overstates the ellipse least)
+                const bool big = ov && bx1 - bx0 + by1 - by0 >= 24;
+                if (__any_sync(kAll, big)) {
+                    if (big) {
+                        const float4 A = sA[lane];
+                        float4 B = sB[lane];
+                        B.w = A.z + 7.9943534f;  // log2(255 o): alpha >= 1/255 iff q <= w
+                        ov = reaches_rect(A, B, (float)wx0 + 0.5f, (float)wy0 + 0.5f);
+                    }
+                }
+            }
+            uint32_t m32;
+            if constexpr (QUAD) {  // per quadrant: the splats whose box reaches it
+                const bool c0 = ov && bx0 <= wx0 + 3, c1 = ov && bx1 >= wx0 + 4;
+                const bool r0 = by0 <= wy0 + 3, r1 = by1 >= wy0 + 4;
+                const uint32_t ma = __ballot_sync(kAll, c0 && r0), mb = __ballot_sync(kAll, c1 && r0);
+                const uint32_t mc = __ballot_sync(kAll, c0 && r1), md = __ballot_sync(kAll, c1 && r1);
+                const uint32_t dm = __ballot_sync(kAll, done0 && done1);
+                m32 = grp == 0 ? ma : (grp == 1 ? mb : (grp == 2 ? mc : md));
+                if (((dm >> (8 * grp)) & 0xffu) == 0xffu) m32 = 0u;
+            } else {
+                m32 = __ballot_sync(kAll, ov);
+            }
+            __syncwarp();  // the lanes' staged values
+            // two splats per step: their four alpha evaluations are independent;
+            // the blends then run in depth order
+            while (QUAD ? __any_sync(kAll, m32 != 0u) : m32 != 0u) {
+                const bool one = !QUAD || m32 != 0u;
+                const int j1 = one ? __ffs(m32) - 1 : 0;
+                m32 &= m32 - 1u;
+                const bool two = m32 != 0u;
+                const int j2 = two ? __ffs(m32) - 1 : j1;
+                if (two) m32 &= m32 - 1u;
+                // Camera pixels need no box test (a pixel outside a splat's support box
+                // has q > q* (1 + 2e-4): its alpha falls below 1/255); LiDAR rays have
+                // one (their grid box is a looser cone bound and a ray evaluation costs
+                // more).
+                bool h10 = one && !done0, h11 = one && !done1, h20 = two && !done0, h21 = two && !done1;
+                if constexpr (LID) {
+                    const int4 R1 = sR[j1];
+                    const int4 R2 = sR[j2];
+                    auto inb = [](const int4& R, int x, int y) {
+                        return (unsigned)(x - R.x) <= (unsigned)R.y && (unsigned)(y - R.z) <= (unsigned)R.w;
+                    };
+                    h10 = h10 && inb(R1, cx0, cy0);
+                    h11 = h11 && inb(R1, cx1, cy1);
+                    h20 = h20 && inb(R2, cx0, cy0);
+                    h21 = h21 && inb(R2, cx1, cy1);
+                    // Grid scans evaluate every lane's rays (no divergent branch, so the
+                    // vote below sees every lane); along arbitrary rays the per-ray boxes
+                    // cull so much that the branch pays.
+                    if (MODE == 1 || h10 || h11 || h20 || h21) {
+                        float2 al1, ts1, al2, ts2;
+                        ray_eval2(sA[j1], sB[j1], sC[j1], sD[j1], al1, ts1);
+                        ray_eval2(sA[j2], sB[j2], sC[j2], sD[j2], al2, ts2);
+                        bool voted = false;  // both splats blended by the vote path
+                        if constexpr (MODE == 1) {
+                            // as in the camera form: both splats with selects unless a ray stops
+                            const bool u10 = h10 && al1.x >= (1.0f / 255.0f), u11 = h11 && al1.y >= (1.0f / 255.0f);
+                            const float2 am1 = make_float2(u10 ? al1.x : 0.0f, u11 ? al1.y : 0.0f);
+                            const float2 x1 = __fmul2_rn(am1, Tp);
+                            const float2 Tn1 = __fadd2_rn(Tp, make_float2(-x1.x, -x1.y));
+                            const bool v20 = h20 && al2.x >= (1.0f / 255.0f), v21 = h21 && al2.y >= (1.0f / 255.0f);
+                            const float2 am2 = make_float2(v20 ? al2.x : 0.0f, v21 ? al2.y : 0.0f);
+                            const float2 x2 = __fmul2_rn(am2, Tn1);
+                            const float2 Tn2 = __fadd2_rn(Tn1, make_float2(-x2.x, -x2.y));
+                            const bool stop = Tn2.x < 1e-4f || Tn2.y < 1e-4f;  // Tn2 <= Tn1
+                            if (!__any_sync(kAll, stop)) {
+                                ncomp += (uint32_t)u10 + (uint32_t)u11 + (uint32_t)v20 + (uint32_t)v21;
+                                dp = __ffma2_rn(x1, ts1, dp);
+                                dp = __ffma2_rn(x2, ts2, dp);
+                                Tp = Tn2;
+                                voted = true;
+                            }
+                        }
+                        if (!voted) {
+                            const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (h10 && al1.x >= (1.0f / 255.0f)) {
+                                ++ncomp;
+                                blend(al1.x, none, ts1.x, Tp.x, rp.x, gp.x, bp.x, dp.x, done0);
+                            }
+                            if (h11 && al1.y >= (1.0f / 255.0f)) {
+                                ++ncomp;
+                                blend(al1.y, none, ts1.y, Tp.y, rp.y, gp.y, bp.y, dp.y, done1);
+                            }
+                            if (h20 && !done0 && al2.x >= (1.0f / 255.0f)) {
+                                ++ncomp;
+                                blend(al2.x, none, ts2.x, Tp.x, rp.x, gp.x, bp.x, dp.x, done0);
+                            }
+                            if (h21 && !done1 && al2.y >= (1.0f / 255.0f)) {
+                                ++ncomp;
+                                blend(al2.y, none, ts2.y, Tp.y, rp.y, gp.y, bp.y, dp.y, done1);
+                            }
+                        }
+                    }
+                } else {
+                    // the arithmetic and the vote of the CTA form (gs_composite.cu)
+                    const float4 A1 = sA[j1], B1 = sB[j1];
+                    const float4 A2 = sA[j2], B2 = sB[j2];
+                    const float2 a1 = splat_alpha2<true>(A1, B1, fpx, fpy);
+                    const float2 a2 = splat_alpha2<true>(A2, B2, fpx, fpy);
+                    const bool u10 = h10 && a1.x >= (1.0f / 255.0f);
+                    const bool u11 = h11 && a1.y >= (1.0f / 255.0f);
+                    const float2 am1 = make_float2(u10 ? a1.x : 0.0f, u11 ? a1.y : 0.0f);
+                    const float2 x1 = __fmul2_rn(am1, Tp);
+                    const float2 Tn1 = __fadd2_rn(Tp, make_float2(-x1.x, -x1.y));
+                    const bool v20 = h20 && a2.x >= (1.0f / 255.0f);
+                    const bool v21 = h21 && a2.y >= (1.0f / 255.0f);
+                    const float2 am2 = make_float2(v20 ? a2.x : 0.0f, v21 ? a2.y : 0.0f);
+                    const float2 x2 = __fmul2_rn(am2, Tn1);
+                    const float2 Tn2 = __fadd2_rn(Tn1, make_float2(-x2.x, -x2.y));
+                    const bool stop = Tn2.x < 1e-4f || Tn2.y < 1e-4f;
+                    if (!__any_sync(kAll, stop)) {
+                        if constexpr (CNT) ncomp += (uint32_t)u10 + (uint32_t)u11 + (uint32_t)v20 + (uint32_t)v21;
+                        const float4 C1 = sC[j1], C2 = sC[j2];
+                        rp = __ffma2_rn(x1, make_float2(C1.x, C1.x), rp);
+                        gp = __ffma2_rn(x1, make_float2(C1.y, C1.y), gp);
+                        bp = __ffma2_rn(x1, make_float2(C1.z, C1.z), bp);
+                        dp = __ffma2_rn(x1, make_float2(A1.w, A1.w), dp);
+                        rp = __ffma2_rn(x2, make_float2(C2.x, C2.x), rp);
+                        gp = __ffma2_rn(x2, make_float2(C2.y, C2.y), gp);
+                        bp = __ffma2_rn(x2, make_float2(C2.z, C2.z), bp);
+                        dp = __ffma2_rn(x2, make_float2(A2.w, A2.w), dp);
+                        Tp = Tn2;
+                    } else {
+                        if constexpr (CNT) ncomp += (uint32_t)u10 + (uint32_t)u11;
+                        blend2(a1, u10, u11, sC[j1], A1.w, Tp, rp, gp, bp, dp, done0, done1);
+                        const bool u20 = h20 && !done0 && a2.x >= (1.0f / 255.0f);
+                        const bool u21 = h21 && !done1 && a2.y >= (1.0f / 255.0f);
+                        if constexpr (CNT) ncomp += (uint32_t)u20 + (uint32_t)u21;
+                        blend2(a2, u20, u21, sC[j2], A2.w, Tp, rp, gp, bp, dp, done0, done1);
+                    }
+                }
+            }
+            if (__all_sync(kAll, done0 && done1)) {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncwarp();
+                return true;
+            }
+        }
+        return false;
+    };
+
+    // Appends the taken ranks in [lo, hi) of the bucket to keys (the first
+    // kCap of them) and returns how many there are; wl, wh: their bounds.
+    uint32_t wl = 0, wh = 0;
+    auto gather = [&](uint32_t lo, uint32_t width) -> uint32_t {
+        uint32_t have = 0, a = kAll, z = 0u;
+        const uint32_t below = (1u << lane) - 1u;
+        warp_keys(Lk, n, [&](uint32_t k, bool valid) {
+            const uint32_t r = k >> kshift;
+            const bool in = valid && taken(k) && r - lo < width;
+            const uint32_t b = __ballot_sync(kAll, in);
+            if (in) {
+                const uint32_t at = have + (uint32_t)__popc(b & below);
+                if (at < (uint32_t)kCap) keys[at] = r;
+                a = min(a, r);
+                z = max(z, r);
+            }
+            have += (uint32_t)__popc(b);
+        });
+        wl = __reduce_min_sync(kAll, a);
+        wh = __reduce_max_sync(kAll, z);
+        __syncwarp();
+        return have;
+    };
+
+    // how the windows come: the bucket at once, runs of histogram ranges, or bitmaps
+    enum { kWhole, kRuns, kBitmap } how = kBitmap;
+    uint32_t whole = 0;
+    int hs = 0;            // histogram: log2 of the ranks per range
+    uint32_t htotal = 0;
+    int g0 = 0;            // next range or group
+    uint32_t r0 = 0;       // next ranks of the bitmap
+    bool loaded = false;   // a bitmap is set up
+    if (n <= kShort) {
+        whole = n ? gather(0u, kAll) : 0u;
+        if (whole <= (uint32_t)kCap) how = kWhole;
+    }
+    if (how == kBitmap) {
+        const uint32_t est = kshift ? n / 2 : n;
+        if (est / kCap + 2 < n_rank / (kWords * 32) + 1) {
+            while (((n_rank - 1u) >> hs) >= (uint32_t)kSortBins) ++hs;
+            for (int i = lane; i < kSortBins; i += 32) bm[i] = 0u;
+            __syncwarp();
+            warp_keys(Lk, n, [&](uint32_t k, bool valid) {
+                const uint32_t r = k >> kshift;
+                if (valid && taken(k) && r < n_rank) atomicAdd(&bm[r >> hs], 1u);
+            });
+            __syncwarp();
+            constexpr int PER = kSortBins / 32;
+            uint32_t c[PER], sum = 0, most = 0;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                c[j] = bm[lane * PER + j];
+                sum += c[j];
+                most = max(most, c[j]);
+            }
+            uint32_t run = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(kAll, run, d);
+                if (lane >= d) run += y;
+            }
+            htotal = __shfl_sync(kAll, run, 31);
+            run -= sum;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                bm[kSortBins + lane * PER + j] = run;
+                run += c[j];
+            }
+            __syncwarp();
+            if (!__any_sync(kAll, most > (uint32_t)kCap)) how = kRuns;
+        }
+    }
+    for (;;) {
+        int wn = 0;
+        if (how == kWhole) {
+            wn = (int)whole;
+            whole = 0;
+            if (wn == 0) break;
+        } else if (how == kRuns) {
+            if (g0 >= kSortBins) break;
+            const uint32_t* start_of = bm + kSortBins;
+            auto begin = [&](int g) { return g < kSortBins ? start_of[g] : htotal; };
+            const uint32_t base = begin(g0);
+            if (base >= htotal) break;
+            int lo = g0 + 1, hi = kSortBins;  // last g1 with begin(g1) - base <= kCap
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (begin(mid) - base <= (uint32_t)kCap) lo = mid; else hi = mid - 1;
+            }
+            wn = (int)(begin(lo) - base);
+            const uint32_t a = (uint32_t)g0 << hs;
+            g0 = lo;
+            if (wn == 0) continue;
+            gather(a, ((uint32_t)lo << hs) - a);
+        } else {
+            if (loaded && g0 >= kGroups) {
+                loaded = false;
+                r0 += (uint32_t)(kWords * 32);
+            }
+            if (!loaded) {
+                if (r0 >= n_rank || n == 0) break;
+                for (int i = lane; i < kWords / 4; i += 32)
+                    reinterpret_cast<uint4*>(bm)[i] = make_uint4(0u, 0u, 0u, 0u);
+                __syncwarp();
+                warp_keys(Lk, n, [&](uint32_t k, bool valid) {
+                    const uint32_t d = (k >> kshift) - r0;
+                    if (valid && taken(k) && d < (uint32_t)(kWords * 32)) atomicOr(&bm[d >> 5], 1u << (d & 31u));
+                });
+                __syncwarp();
+                // ranks set before each group: a lane counts two groups
+                uint32_t c[2] = {0u, 0u};
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {  // rotated: neighbouring lanes hit different banks
+                    c[0] += __popc(bm[(2 * lane) * 16 + ((i + lane) & 15)]);
+                    c[1] += __popc(bm[(2 * lane + 1) * 16 + ((i + lane) & 15)]);
+                }
+                uint32_t run = c[0] + c[1];
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(kAll, run, d);
+                    if (lane >= d) run += y;
+                }
+                if (lane == 31) pre[kGroups] = run;
+                pre[2 * lane] = run - c[0] - c[1];
+                pre[2 * lane + 1] = run - c[1];
+                __syncwarp();
+                loaded = true;
+                g0 = 0;
+            }
+            const uint32_t base = pre[g0];
+            const uint32_t fit = base + (uint32_t)kCap;
+            // groups whose end is within kCap of the window's start (ends ascend)
+            const int g1 = __popc(__ballot_sync(kAll, pre[2 * lane + 1] <= fit)) +
+                           __popc(__ballot_sync(kAll, pre[2 * lane + 2] <= fit));
+            wn = (int)(pre[g1] - base);
+            if (wn > 0) {
+                // a half-warp reads a group's words back in order
+                for (int gb = g0; gb < g1; gb += 2) {
+                    const int g = gb + (lane >> 4);
+                    uint32_t w = g < g1 ? bm[g * 16 + (lane & 15)] : 0u;
+                    const uint32_t pc = __popc(w);
+                    uint32_t x = pc;
+#pragma unroll
+                    for (int d = 1; d < 16; d <<= 1) {
+                        const uint32_t y = __shfl_up_sync(kAll, x, d, 16);
+                        if ((lane & 15) >= d) x += y;
+                    }
+                    if (w) {
+                        uint32_t at = pre[g] - base + x - pc;
+                        const uint32_t r = r0 + (uint32_t)(g * 16 + (lane & 15)) * 32u;
+                        while (w) {
+                            keys[at++] = r + (uint32_t)(__ffs(w) - 1);
+                            w &= w - 1u;
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+            g0 = g1;
+            if (wn == 0) continue;
+        }
+        if (how != kBitmap) warp_sort(keys, reinterpret_cast<uint32_t*>(&rec[0][0][0]), bm, wn, wl, wh);
+        if (run_window(wn)) break;
+        __syncwarp();
+    }
+
+    if (CNT && P.neval) {
+        const uint32_t c = __reduce_add_sync(kAll, ncomp);
+        if (lane == 0 && c) atomicAdd(P.neval, (unsigned long long)c);
+    }
+    if constexpr (LID) {  // range and hit per ray, at the ray's index or grid cell
+        const size_t o0 = pix_base + (MODE == 3 ? (size_t)ray0 : (size_t)py0 * W + px);
+        const size_t o1 = pix_base + (MODE == 3 ? (size_t)ray1 : (size_t)py1 * W + px);
+        if (in0) {
+            const float a = 1.0f - Tp.x;
+            P.depth[o0] = a > 0.0f ? dp.x / a : 0.0f;
+            if (P.alpha) P.alpha[o0] = a;
+        }
+        if (in1) {
+            const float a = 1.0f - Tp.y;
+            P.depth[o1] = a > 0.0f ? dp.y / a : 0.0f;
+            if (P.alpha) P.alpha[o1] = a;
+        }
+    } else {
+        const PixelStore store(P, el);
+        if (in0) store.put(P, pix_base + (size_t)py0 * W + px, Tp.x, rp.x, gp.x, bp.x, dp.x);
+        if (in1) store.put(P, pix_base + (size_t)py1 * W + px, Tp.y, rp.y, gp.y, bp.y, dp.y);
+    }
+    __syncwarp();
+    }  // items of the claim
+    }  // claims
+}
+
+template <int MODE>
+static cudaError_t launch_warps(const CompParams& P, cudaStream_t st, int* ctas) {
+    static PerDevice resident;
+    int full = 0;
+    const cudaError_t e = resident.ctas((const void*)k_composite_warp<MODE>, 32, &full);
+    if (e != cudaSuccess) return e;
+    const int subs = MODE == 3 ? 1 : (P.tile_w / 8) * (P.tile_h / 8);
+    const unsigned long long items = (unsigned long long)(P.item_end - P.item_begin) * subs;
+    if (items > 0xffffffffull) return cudaErrorInvalidValue;
+    const unsigned long long claims = (items + P.chunk - 1) / P.chunk;
+    *ctas = (int)std::min((unsigned long long)full, claims);
+    k_composite_warp<MODE><<<*ctas, 32, 0, st>>>(P);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_composite_warp(const CompParams& P, cudaStream_t st, int* ctas) {
+    if (P.ray_list) return launch_warps<3>(P, st, ctas);
+    if (P.lidars) return launch_warps<1>(P, st, ctas);
+    if (P.neval) return launch_warps<2>(P, st, ctas);
+    return launch_warps<0>(P, st, ctas);
+}
+
+}  // namespace gsb

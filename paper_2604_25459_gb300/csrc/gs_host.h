@@ -54,10 +54,15 @@ struct DevBuf {
 
 // Device scratch of a render: one set per scene (eager calls) and one per plan.
 struct Scratch {
-    DevBuf envs, blocks, cams, xf, r012, r3, mask, counts, off, cursor, env_total, env_base, pairs, dbg_hxy,
-        dbg_sorted, work, spill, zr;  // r012: records' r0, r1, r2 interleaved (kRecStride); zr: depth ranges
-    DevBuf* all[18] = {&envs,   &blocks,    &cams,     &xf,    &r012,   &r3,         &mask, &counts, &off,
-                       &cursor, &env_total, &env_base, &pairs, &dbg_hxy, &dbg_sorted, &work, &spill, &zr};
+    // r012: records' r0, r1, r2 interleaved (kRecStride); counts: every counter
+    // that a wave starts from zero (tile counts and cursors, depth-range counts
+    // and cursors, the compositor's work counter); bins: splitters, offsets and
+    // windows of the depth ranges and the ranked records per env; ranks: order,
+    // then rank, per record slot
+    DevBuf envs, blocks, cams, xf, r012, r3, mask, counts, off, env_total, env_base, bins, zkeys, ranks, pairs,
+        dbg_hxy, items;
+    DevBuf* all[17] = {&envs, &blocks,    &cams,     &xf,   &r012,  &r3,    &mask,  &counts,    &off,
+                       &env_total, &env_base, &bins, &zkeys, &ranks, &pairs, &dbg_hxy, &items};
     void release() {
         for (DevBuf* b : all) b->release();
     }
@@ -93,7 +98,8 @@ struct gs_scene_s {
     cudaEvent_t ev_copied[2] = {nullptr, nullptr};
     // host tables of the last wave (debug hooks)
     std::vector<gsb::EnvInfo> last_envs;
-    int last_e0 = -1, last_We = 0, last_ea = 0, last_eb = 0;
+    int last_e0 = -1, last_We = 0, last_ea = 0, last_eb = 0, last_shift = 0;
+    const uint32_t* last_counts = nullptr;  // device: tile counts of the last wave
     unsigned long long last_pair_base = 0;
     gs_stats stats{};
     // profiling (per-phase CUDA events on the render stream) and counters

@@ -20,14 +20,16 @@
 //       r0, r1, r2 lie side by side at float4 index kRecStride s of one array
 //       (the compositor gathers all three: two 32-byte sectors instead of
 //       three half-used ones), its fourth word r3 at index s of another (the
-//       binning reads only r3, coalesced across a warp).  Keys are (depth bits << 32 |
-//       i) with i the caller's local index (background: its index before the
-//       Morton reordering; links: j), so equal depths order by global index;
-//       the compositor maps i back to the record slot j.
+//       binning reads only r3, coalesced across a warp).
+//     rank[rec_base + j], order[rec_base + r]  the env's visible records in depth
+//       order: sorted by (depth bits << 32 | i) with i the caller's local index
+//       (background: its index before the Morton reordering; links: j), so equal
+//       depths order by global index; rank[j] is record j's place and order[r]
+//       the slot of place r.  nvis[el] records are ranked.
 //     xf[envs[el].xf_base + f]  frame f = 0 background, f = 1 + (l - link_begin)
 //     counts/off_local/cursor[envs[el].tile_base + t]  per (env, tile)
 //     env_base[el]              exclusive scan of per-env intersection totals
-//     pairs[...]                u64 keys bucketed by (env, tile)
+//     pairs[...]                u32 ranks bucketed by (env, tile)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -148,6 +150,37 @@ struct ProjParams {
                                // anywhere in a cell, not only at its centre)
 };
 
+// Depth ranking of a wave's visible records (gs_rank.cu): per env a sample
+// sort into `bins` key ranges, then windows of ranges sorted in shared memory.
+struct RankParams {
+    const EnvInfo* envs;
+    const uint32_t* mask;
+    const uint4* r3;
+    int bins;                     // key ranges per env: a power of two, <= kRankBins
+    int cells;                    // depth cells of the range lookup: a power of two
+    int win_pitch;                // window table entries per env
+    int words_per_block;          // of the count and of the placement (the same blocks)
+    int blocks;                   // binning blocks per env
+    unsigned long long* split;    // [We][bins]: splitters 0 .. bins-2, then the lookup's first depth and shift
+    uint16_t* cell;               // [We][cells]: first range of each depth cell
+    uint32_t* bin_cnt;            // [We][bins], zeroed
+    uint32_t* bin_off;            // [We][bins]
+    uint32_t* block_off;          // [We][blocks][bins]: keys of the range in earlier blocks
+    uint32_t* win;                // [We][win_pitch]: window v holds positions [win[v], win[v+1])
+    uint32_t* nvis;               // [We]
+    unsigned long long* zkeys;    // [recs]: an env's keys from rec_base, grouped by range
+    uint32_t* order;              // [recs]
+    uint32_t* rank;               // [recs]; until the sort: range << 13 | place among the block's keys of it
+    uint32_t* status;
+    // the caller's local index of a record: camera records hold it in r3.w
+    // (index_in_r3), LiDAR records map through bg_index (nullable: caller's
+    // index of the background Gaussian in storage slot j < n_bg)
+    int index_in_r3;
+    const int* bg_index;
+    const int* bg_slot;           // nullable: storage slot of the caller's background Gaussian i
+    unsigned int n_bg;
+};
+
 struct BinParams {
     const EnvInfo* envs;
     const uint32_t* mask;
@@ -161,20 +194,11 @@ struct BinParams {
     unsigned long long pair_base;   // env_base[e_begin], subtracted from absolute offsets
     unsigned long long pair_cap;    // keys the pair buffer holds
     uint32_t* cursor;
-    unsigned long long* pairs;
+    uint32_t* pairs;
+    const uint32_t* rank;
     uint32_t* status;
-    // Keys carry the caller's local index of the Gaussian, so equal depths
-    // order by it: camera records hold it in r3.w (index_in_r3), LiDAR
-    // records are mapped through bg_index (nullable: caller's index of the
-    // background Gaussian in storage slot j < n_bg)
-    int index_in_r3;
-    const int* bg_index;
-    unsigned int n_bg;
     int wrap;  // LiDAR: a box with x0 > x1 covers columns [x0, cols) and [0, x1]
-    // nullable, per env of the wave: (smallest depth bits, ~largest depth bits)
-    // of the env's visible records, taken by the count pass with atomicMin on
-    // both words (set to all ones before it)
-    uint2* zr;
+    int key_shift;           // see CompParams
 };
 
 struct CompParams {
@@ -183,26 +207,29 @@ struct CompParams {
     unsigned int item_begin, item_end;  // (env, tile) items: envs[e_begin].tile_base .. envs[e_end].tile_base
     int chunk;                       // items claimed per atomic
     unsigned int* work;              // work counter (zeroed before the launch)
+    // nullable (warp form): the items in claiming order, kItemClasses lists of
+    // class_cnt[c] items each, list c from items + c * item_pitch
+    const uint32_t* items;
+    const uint32_t* class_cnt;
+    unsigned int item_pitch;
     const float4* r0;
     const float4* r1;
     const float4* r2;
-    // nullable, per env of the wave: the depth-bit range of its keys (see
-    // BinParams::zr); long buckets are partitioned over it instead of over
-    // their own key range, which saves a pass over their keys
-    const uint2* zr;
+    const uint32_t* nvis;            // per env of the wave: ranked records
+    const uint32_t* order;           // record slot of rank r at rec_base + r
     const uint32_t* counts;
     const uint32_t* off_local;
     const unsigned long long* env_base;
     unsigned long long pair_base;
     unsigned long long pair_cap;
-    const unsigned long long* pairs;
-    unsigned long long* spill;       // nullable: spill_cap keys per CTA for partitioning long buckets
-    unsigned int spill_cap;          // kCompCap <= spill_cap <= kSpillMax
-    unsigned int spill_ctas;         // regions in spill: the launch uses at most this many CTAs
-    unsigned long long* dbg_sorted;  // nullable: receives the full depth-ordered lists
+    const uint32_t* pairs;
     unsigned long long* neval;       // nullable: composited (pixel, Gaussian) pair counter
     int tile_w, tile_h;
-    int quad;       // 16x16 or 8x8 camera tiles: per-quadrant splat lists (k_composite's QUAD form)
+    int quad;       // camera images: the warp form (k_composite_warp)
+    // The warp form's keys carry, below the rank, one bit per 8x8 subtile of
+    // the tile that the record's box reaches (row-major): key = rank <<
+    // key_shift | mask.  key_shift = 0: no mask (plain ranks).
+    int key_shift;
     float* rgb;     // images at envs[e].pix_base (x3 for rgb); unused when rgb8 is set
     float* depth;   // unused when depth16 is set
     float* alpha;   // nullable
@@ -211,19 +238,18 @@ struct CompParams {
     const gs_appearance* appear;  // nullable: per env (wave-local index) for rgb8
     float* score;         // nullable: contribution pass (no images): score[g] += sum of alpha T
     unsigned int nbp;     // background slots (slot j < nbp is the background Gaussian stored at j)
-    const int* bg_index;  // nullable: caller's index of the background Gaussian in slot j (contribution pass)
-    const int* bg_slot;   // nullable: keys carry the caller's background index i < n_bg; its record slot is bg_slot[i]
+    const int* bg_index;  // nullable: caller's index of the background Gaussian in slot j (contribution pass, debug)
     unsigned int n_bg;
     const gs_lidar* lidars;  // nullable: LiDAR scan (range in depth, hit in alpha), per env of the wave
     const uint4* r3;         // LiDAR scan: records' fourth word (|g2|)
     uint32_t* status;
-    // Arbitrary rays (set with lidars): items are (env, tile, chunk of <= 256
+    // Arbitrary rays (set with lidars): items are (env, tile, chunk of <= 64
     // rays); outputs are indexed by ray, at envs[e].pix_base + ray.
     const float* ray_dirs;         // [wave env][n_rays][3], sensor frame
     const uint32_t* ray_cell;      // [wave env][n_rays]: tile << 8 | cell in tile (row-major 16x16)
-    const uint32_t* ray_list;      // [wave env][n_rays]: ray indices grouped by tile
-    const uint32_t* ray_cnt;       // per (env, tile) at tile_base: rays in the tile
-    const uint32_t* ray_off;       // per (env, tile): first entry of the tile in the env's ray_list
+    const uint32_t* ray_list;      // [wave env][n_rays]: ray indices grouped by tile, then 8x8 subtile
+    const uint32_t* ray_cnt;       // per (env, tile, subtile) at 4 tile_base: rays in the subtile
+    const uint32_t* ray_off;       // per (env, tile, subtile): its first entry in the env's ray_list
     const uint32_t* item_off;      // per (env, tile): first item of the tile within its env
     const unsigned long long* item_base;  // per wave env (+1): first item of the env
     int n_rays;
@@ -249,32 +275,88 @@ cudaError_t launch_project_lidar(const ProjParams& P, int n_blocks, cudaStream_t
 // (env, tile); then the rays grouped by tile and the compositor's items
 // (chunks of at most kRayChunk rays per tile).  ray_cnt and ray_cur are zeroed
 // by the caller.
-constexpr int kRayChunk = 256;
+constexpr int kRayChunk = 64;
 cudaError_t launch_ray_count(const float* dirs, const gs_lidar* lidars, const EnvInfo* envs, int We, int n_rays,
                              uint32_t* cell, uint32_t* cnt, uint32_t* status, cudaStream_t st);
 cudaError_t launch_ray_scatter(const EnvInfo* envs, int We, int n_rays, const uint32_t* cell, const uint32_t* off,
                                uint32_t* cur, uint32_t* list, const uint32_t* cnt, uint32_t* item_cnt,
                                unsigned int tiles, cudaStream_t st);
-// grid.x covers the largest env's mask words; max_T sizes the shared histogram
-cudaError_t launch_count(const BinParams& P, int n_envs, int max_words, int max_T, cudaStream_t st);
+// grid.x covers the largest env's mask words; max_T sizes the shared histogram.
+// The count also histograms the records over the env's depth ranges (R).
+cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, int max_words, int max_T,
+                         cudaStream_t st);
+// per: counters per tile (counts and off_local hold per T from per tile_base).
 cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
-                        unsigned long long* env_total, unsigned long long* env_base, int We, cudaStream_t st);
+                        unsigned long long* env_total, unsigned long long* env_base, int We, int per,
+                        cudaStream_t st);
+// As launch_scan, with the scans of the depth ranges and their window tables.
+cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
+                              unsigned long long* env_total, unsigned long long* env_base, int We,
+                              const RankParams& R, cudaStream_t st);
 cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int max_T, cudaStream_t st);
-// grid = persistent CTAs; returns the grid size used through *ctas
+// Lists a launch's items by the length of their buckets, longest class first
+// (CompParams::items); class_cnt is zeroed by the caller.  Rays: item_cnt and
+// item_off per (env, tile) and item_base per env give a tile's items.
+constexpr int kItemClasses = 4;  // buckets of >= 16384, >= 4096, >= 1024 and fewer keys
+cudaError_t launch_item_order(const EnvInfo* envs, int e_begin, int n_envs, int max_T, const uint32_t* counts,
+                              const uint32_t* item_cnt, const uint32_t* item_off,
+                              const unsigned long long* item_base, uint32_t* items, uint32_t pitch,
+                              uint32_t* class_cnt, cudaStream_t st);
+// Depth ranking: splitters before the count, ranks after the scan.
+cudaError_t launch_rank_sample(const RankParams& R, int n_envs, cudaStream_t st);
+cudaError_t launch_rank(const RankParams& R, int n_envs, int max_words, cudaStream_t st);
+// grid = persistent CTAs; returns the grid size used through *ctas.  The warp
+// form (launch_composite_warp) renders LiDAR scans and, with P.quad, images.
 cudaError_t launch_composite(const CompParams& P, cudaStream_t st, int* ctas);
-// Most CTAs a compositing launch of this tile shape uses on the current
-// device (resident CTAs per SM x SMs): the number of spill regions to provide.
-cudaError_t composite_max_ctas(int tile_w, int tile_h, int* ctas);
+cudaError_t launch_composite_warp(const CompParams& P, cudaStream_t st, int* ctas);
+// Resident warps of the warp form (the items that run at once).
+constexpr int kWarpsPerSM = 20;
 
-constexpr int kWordsPerBlock = 256;  // binning block: 8 warps x 32 visibility words (8192 slots)
-
-// Depth-ordered window held in shared memory by the compositor.  Smaller
-// windows sort less in tiles that terminate early, larger ones re-scan long
-// buckets less often; 768 measured best on the 2048 x 640x480 workload
-// (1024: +2 %, 512: +4 %, 2048: +19 % compositing time).
+constexpr int kWordsPerBlock = 256;  // binning block: at most one visibility word per thread of 256 (8192 slots)
+constexpr int kRankBins = 2048;      // depth ranges per env, at most
+constexpr int kRankStride = 768;     // ranks per window of the depth sort
+// Depth ranges of an env of n record slots: one per 512 slots for cameras
+// (which see a quarter of a room), one per 256 for LiDARs (which see all of it).
+inline int rank_bins(long long n, bool lidar) {
+    const int most = lidar ? kRankBins : kRankBins / 2;
+    int b = 32;
+    while (b < most && (long long)b * (lidar ? 256 : 512) < n) b *= 2;
+    return b;
+}
+// Sizes the ranking of We envs of at most max_words visibility words.  Binning
+// blocks: as few words as still give every SM a few blocks, but no fewer slots
+// than two per range (a block keeps an offset per range).
+inline RankParams rank_sizes(long long max_words, int We, bool lidar) {
+    RankParams R{};
+    R.bins = rank_bins(max_words * 32, lidar);
+    R.cells = R.bins < 1024 ? 4 * R.bins : 4096;
+    R.win_pitch = (int)(max_words * 32 / kRankStride) + 2;
+    int w = kWordsPerBlock;
+    while (w > 16 && w > R.bins / 16 && (max_words + w - 1) / w * We < 4 * 152) w /= 2;
+    R.words_per_block = w;
+    R.blocks = (int)((max_words + w - 1) / w);
+    return R;
+}
+// Bytes of the ranking's per-env tables (everything but bin_cnt, zkeys, order
+// and rank) for We envs, and their layout from a 16-byte aligned base.
+inline size_t rank_tables(RankParams& R, int We, unsigned char* base) {
+    const size_t nb = (size_t)We * R.bins;
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        unsigned char* p = base + o;
+        o = (o + bytes + 15) & ~size_t(15);
+        return p;
+    };
+    R.split = reinterpret_cast<unsigned long long*>(take(nb * 8));
+    R.cell = reinterpret_cast<uint16_t*>(take((size_t)We * R.cells * 2));
+    R.bin_off = reinterpret_cast<uint32_t*>(take(nb * 4));
+    R.block_off = reinterpret_cast<uint32_t*>(take(nb * R.blocks * 4));
+    R.win = reinterpret_cast<uint32_t*>(take((size_t)We * R.win_pitch * 4));
+    R.nvis = reinterpret_cast<uint32_t*>(take((size_t)We * 4));
+    return o;
+}
+// Depth-ordered window held in shared memory by the compositor.
 constexpr int kCompCap = 768;
-constexpr int kBins = 2048;         // key ranges of the long-bucket partition
-constexpr int kSpillMax = 32768;    // keys per CTA in the spill region, at most
 // Plain renders use the compositor's quadrant form (QUAD) on 16x16 or 8x8 tiles when
 // no image of the wave has more pixels than this (measured crossover on the
 // room workload: faster at 320x240 and below, slower at 640x480).

@@ -50,6 +50,9 @@ __device__ __forceinline__ bool grid_range(float a, float b, float origin, float
     return true;
 }
 
+// 8x8 subtile (row-major in the 16x16 tile) of a ray's cell word.
+__device__ __forceinline__ uint32_t ray_sub(uint32_t cell) { return ((cell >> 6) & 2u) | ((cell >> 3) & 1u); }
+
 }  // namespace
 
 __global__ void __launch_bounds__(256) k_project_lidar(ProjParams P) {
@@ -251,10 +254,10 @@ __global__ void __launch_bounds__(256) k_ray_count(const float* __restrict__ dir
     }
     const int t = (j >> 4) * E.ntx + (i >> 4);
     cell[k] = ((uint32_t)t << 8) | ((uint32_t)(j & 15) << 4) | (uint32_t)(i & 15);
-    atomicAdd(cnt + E.tile_base + t, 1u);
+    atomicAdd(cnt + 4 * (size_t)(E.tile_base + t) + ray_sub(cell[k]), 1u);
 }
 
-// Rays grouped by tile: list[el][off[tile] + rank] = r.
+// Rays grouped by tile and 8x8 subtile: list[el][off[tile, sub] + rank] = r.
 __global__ void __launch_bounds__(256) k_ray_scatter(const EnvInfo* envs, int n_rays, const uint32_t* cell,
                                                      const uint32_t* off, uint32_t* cur, uint32_t* list) {
     const int el = blockIdx.y;
@@ -264,8 +267,8 @@ __global__ void __launch_bounds__(256) k_ray_scatter(const EnvInfo* envs, int n_
     const uint32_t c = cell[k];
     if (c == 0xffffffffu) return;
     const unsigned int tb = envs[el].tile_base;
-    const uint32_t t = c >> 8;
-    const uint32_t pos = off[tb + t] + atomicAdd(cur + tb + t, 1u);
+    const size_t t = 4 * (size_t)(tb + (c >> 8)) + ray_sub(c);
+    const uint32_t pos = off[t] + atomicAdd(cur + t, 1u);
     list[(size_t)el * n_rays + pos] = (uint32_t)r;
 }
 
@@ -274,7 +277,8 @@ __global__ void __launch_bounds__(256) k_ray_items(const EnvInfo* envs, int We, 
                                                    uint32_t* item_cnt) {
     const unsigned int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= envs[We].tile_base) return;
-    item_cnt[i] = (cnt[i] + (uint32_t)kRayChunk - 1u) / (uint32_t)kRayChunk;
+    const uint4 c = reinterpret_cast<const uint4*>(cnt)[i];  // the tile's four subtiles
+    item_cnt[i] = (c.x + c.y + c.z + c.w + (uint32_t)kRayChunk - 1u) / (uint32_t)kRayChunk;
 }
 
 cudaError_t launch_ray_count(const float* dirs, const gs_lidar* lidars, const EnvInfo* envs, int We, int n_rays,

@@ -215,12 +215,45 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         P.dbg_hxy = nullptr;
         P.bg_index = v.bg_index;
         NA_CK(launch_project(v.D, P, nb, st), "projection");
+        // The part of the array behind the fixed tables: its first half holds the
+        // intersection ranks (and, before they exist, the depth keys), its second
+        // half the depth ranking.  A wave is accepted when 8 bytes per
+        // intersection fit the whole part (ranks take 4), and its size leaves a
+        // quarter of the array: 4 MiB per half, against at most 3.1 MiB of depth
+        // keys or of order and rank (8 B for each of at most 24 MiB / 64 B record
+        // slots) and 0.6 MiB of depth ranges with the largest binning blocks.
+        const size_t half = up256((kNoAllocBytes - y.pairs) / 2);
+        RankParams R = rank_sizes(max_words, Wn, false);
+        const size_t n_bins = (size_t)Wn * R.bins;
+        while (R.words_per_block < kWordsPerBlock &&
+               sen.rec_base * 8 + n_bins * 4 + 1024 + rank_tables(R, Wn, nullptr) > half) {
+            R.words_per_block *= 2;  // fewer per-block tables
+            R.blocks = (max_words + R.words_per_block - 1) / R.words_per_block;
+        }
+        R.envs = d_envs;
+        R.mask = P.mask;
+        R.r3 = P.r3;
+        unsigned char* tab = base + y.pairs + half;
+        R.order = reinterpret_cast<uint32_t*>(tab);
+        R.rank = R.order + sen.rec_base;
+        R.bin_cnt = R.rank + sen.rec_base;
+        tab += up256(sen.rec_base * 8 + n_bins * 4);
+        tab += rank_tables(R, Wn, tab);
+        R.zkeys = reinterpret_cast<unsigned long long*>(base + y.pairs);
+        R.status = v.status;
+        R.index_in_r3 = 1;
+        R.bg_index = v.bg_index;
+        R.bg_slot = v.bg_slot;
+        R.n_bg = (unsigned)v.D.n_bg;
+        if (tab > base + kNoAllocBytes || sen.rec_base * 8 > half)  // never (see above)
+            return report(GS_ERR_UNSUPPORTED, "no-allocation scratch too small for the depth ranking");
         uint32_t* counts = reinterpret_cast<uint32_t*>(base + y.counts);
         uint32_t* off = reinterpret_cast<uint32_t*>(base + y.off);
         uint32_t* cursor = reinterpret_cast<uint32_t*>(base + y.cursor);
         auto* env_total = reinterpret_cast<unsigned long long*>(base + y.env_total);
         auto* env_base = reinterpret_cast<unsigned long long*>(base + y.env_base);
         NA_CK(cudaMemsetAsync(counts, 0, (size_t)sen.tile_base * 4, st), "clear counts");
+        NA_CK(cudaMemsetAsync(R.bin_cnt, 0, n_bins * 4, st), "clear depth-range counts");
         BinParams B{};
         B.envs = d_envs;
         B.mask = P.mask;
@@ -228,17 +261,17 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.e_begin = 0;
         B.tile_w = tw;
         B.tile_h = th;
-        B.index_in_r3 = 1;
-        B.bg_index = v.bg_index;
-        B.n_bg = (unsigned)v.D.n_bg;
-        B.words_per_block = kWordsPerBlock;
+        B.words_per_block = R.words_per_block;
+        B.rank = R.rank;
         B.counts = counts;
         B.off_local = off;
         B.env_base = env_base;
         B.cursor = cursor;
         B.status = v.status;
-        NA_CK(launch_count(B, Wn, max_words, max_T, st), "count");
-        NA_CK(launch_scan(d_envs, counts, off, env_total, env_base, Wn, st), "scan");
+        NA_CK(launch_rank_sample(R, Wn, st), "depth sample");
+        NA_CK(launch_count(B, R, Wn, max_words, max_T, st), "count");
+        NA_CK(launch_scan_ranks(d_envs, counts, off, env_total, env_base, Wn, R, st), "scan");
+        NA_CK(launch_rank(R, Wn, max_words, st), "depth ranks");
         unsigned long long eb[kMaxWave + 1];
         NA_CK(cudaMemcpyAsync(eb, env_base, sizeof(unsigned long long) * (Wn + 1), cudaMemcpyDeviceToHost, st),
               "read totals");
@@ -252,7 +285,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         NA_CK(cudaMemsetAsync(cursor, 0, (size_t)sen.tile_base * 4, st), "clear cursors");
         B.pair_base = 0;
         B.pair_cap = (kNoAllocBytes - y.pairs) / 8;
-        B.pairs = reinterpret_cast<unsigned long long*>(base + y.pairs);
+        B.pairs = reinterpret_cast<uint32_t*>(base + y.pairs);
         NA_CK(launch_scatter(B, Wn, max_words, max_T, st), "scatter");
         CompParams C{};
         C.envs = d_envs;
@@ -261,19 +294,19 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         C.item_begin = 0;
         C.item_end = sen.tile_base;
         C.chunk = 1;
-        C.bg_slot = v.bg_slot;
         C.n_bg = (unsigned)v.D.n_bg;
         C.work = reinterpret_cast<unsigned int*>(base + y.work);
         C.r0 = P.r0;
         C.r1 = P.r1;
         C.r2 = P.r2;
+        C.nvis = R.nvis;
+        C.order = R.order;
         C.counts = counts;
         C.off_local = off;
         C.env_base = env_base;
         C.pair_base = 0;
         C.pair_cap = B.pair_cap;
         C.pairs = B.pairs;
-        C.dbg_sorted = nullptr;
         C.neval = nullptr;
         C.tile_w = tw;
         C.tile_h = th;

@@ -283,21 +283,20 @@ __device__ __forceinline__ void sh_basis(float x, float y, float z, float* Y) {
 // Colour max(0, sum_k Y_k sh_k + 0.5) per channel for Gaussian g.  The
 // coefficients are consumed plane by plane as they arrive (flattened value f
 // = 3k + channel), so only the basis and three sums stay live; each channel
-// accumulates in ascending k.
-template <int D, int DT>
-__device__ __forceinline__ void sh_colour(const void* base, int64_t n, int64_t g, float x, float y, float z,
-                                          float& r, float& gr, float& b) {
+// accumulates in ascending k.  plane(p) gives 16-byte plane p.
+template <int D, int DT, typename F>
+__device__ __forceinline__ void sh_colour(F&& plane, float x, float y, float z, float& r, float& gr, float& b) {
     constexpr int NV = 3 * (D + 1) * (D + 1);
     float Y[16];
     sh_basis<D>(x, y, z, Y);
     float acc[3] = {0.0f, 0.0f, 0.0f};
     if constexpr (DT == GS_F32) {
         constexpr int NP = (NV + 3) / 4;
-        const float4* P = static_cast<const float4*>(base);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            const float4 v = __ldg(P + (size_t)p * n + g);
-            const float w[4] = {v.x, v.y, v.z, v.w};
+            const uint4 v = plane(p);
+            const float w[4] = {__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z),
+                                __uint_as_float(v.w)};
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 const int f = 4 * p + h;
@@ -306,10 +305,9 @@ __device__ __forceinline__ void sh_colour(const void* base, int64_t n, int64_t g
         }
     } else {
         constexpr int NP = (NV + 7) / 8;
-        const uint4* P = static_cast<const uint4*>(base);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            const uint4 v = __ldg(P + (size_t)p * n + g);
+            const uint4 v = plane(p);
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int h = 0; h < 8; ++h) {
@@ -345,11 +343,17 @@ __device__ __forceinline__ bool pixel_range(float c, float h, int n, int& lo, in
     return true;
 }
 
-constexpr int kProjStageEnvs = 256;  // envs per shared-memory chunk of a projection block
+constexpr int kProjStageEnvs = 64;  // envs per shared-memory chunk of a projection block
 
 template <int D, int DT>
 __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
     constexpr int NV = 3 * (D + 1) * (D + 1);
+    constexpr int NP = DT == GS_F32 ? (NV + 3) / 4 : (NV + 7) / 8;
+    // Each thread keeps its Gaussian's SH planes here from the first env that
+    // sees it: a block projects its 256 Gaussians for a group of envs, and
+    // re-reading 192 bytes per visible pair through L1 and L2 is what bounded
+    // the kernel.
+    extern __shared__ uint4 s_sh[];  // [NP][256]
     const ProjBlock blk = P.blocks[blockIdx.x];
     const int t = threadIdx.x;
     const bool act = t < blk.n;
@@ -384,6 +388,8 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
     __shared__ unsigned long long s_rb[kProjStageEnvs];  // record base
     __shared__ float4 s_rec[8][3 * 32];                  // per warp: the records of an env, before their store
     const bool frame0 = blk.frame0 != 0;
+    const bool once = blk.e1 - blk.e0 == 1;
+    bool have_sh = false;
     for (int c0 = blk.e0; c0 < blk.e1; c0 += kProjStageEnvs) {
     const int c1 = min(c0 + kProjStageEnvs, blk.e1);
     __syncthreads();  // the previous chunk's entries are no longer read
@@ -466,8 +472,6 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
                     const float hy = sqrtf(qstar * cC) * 1.0001f;
                     int i0, i1, j0, j1;
                     if (ok && pixel_range(u, hx, W, i0, i1) && pixel_range(v, hy, H, j0, j1)) {
-                        // SH coefficients are re-read per visible env (L1/L2 hits) and
-                        // streamed into the colour sums
                         const float4 O = __ldg(&Xp->o);
                         float dx = a0.x - O.x, dy = a0.y - O.y, dz = a0.z - O.z;
                         const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
@@ -475,7 +479,18 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
                         dy *= inv;
                         dz *= inv;
                         float r, gg, b;
-                        sh_colour<D, DT>(P.sh, P.n_gauss, g, dx, dy, dz, r, gg, b);
+                        const uint4* gsh = static_cast<const uint4*>(P.sh) + g;
+                        if (once) {
+                            sh_colour<D, DT>([&](int p) { return __ldg(gsh + (size_t)p * P.n_gauss); }, dx, dy, dz,
+                                             r, gg, b);
+                        } else {
+                            if (!have_sh) {
+#pragma unroll
+                                for (int p = 0; p < NP; ++p) s_sh[p * 256 + t] = __ldg(gsh + (size_t)p * P.n_gauss);
+                                have_sh = true;
+                            }
+                            sh_colour<D, DT>([&](int p) { return s_sh[p * 256 + t]; }, dx, dy, dz, r, gg, b);
+                        }
                         const uint32_t rx = (uint32_t)i0 | ((uint32_t)i1 << 16);
                         const uint32_t ry = (uint32_t)j0 | ((uint32_t)j1 << 16);
                         const size_t ri = (size_t)s_rb[ei] + local;
@@ -505,24 +520,33 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
     }  // env chunks
 }
 
+template <int D, int DT>
+static cudaError_t launch_project_dt(const ProjParams& P, int n_blocks, cudaStream_t st) {
+    const int smem = sh_planes_for(D, (gs_dtype)DT) * 256 * 16;
+    const cudaError_t e =
+        cudaFuncSetAttribute((const void*)k_project<D, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_project<D, DT><<<n_blocks, 256, smem, st>>>(P);
+    return cudaGetLastError();
+}
+
 template <int D>
-static void launch_project_d(const DevGaussians& Dg, const ProjParams& P, int n_blocks, cudaStream_t st) {
+static cudaError_t launch_project_d(const DevGaussians& Dg, const ProjParams& P, int n_blocks, cudaStream_t st) {
     switch (Dg.dtype) {
-        case GS_F32: k_project<D, GS_F32><<<n_blocks, 256, 0, st>>>(P); break;
-        case GS_BF16: k_project<D, GS_BF16><<<n_blocks, 256, 0, st>>>(P); break;
-        default: k_project<D, GS_F16><<<n_blocks, 256, 0, st>>>(P); break;
+        case GS_F32: return launch_project_dt<D, GS_F32>(P, n_blocks, st);
+        case GS_BF16: return launch_project_dt<D, GS_BF16>(P, n_blocks, st);
+        default: return launch_project_dt<D, GS_F16>(P, n_blocks, st);
     }
 }
 
 cudaError_t launch_project(const DevGaussians& Dg, const ProjParams& P, int n_blocks, cudaStream_t st) {
     if (n_blocks == 0) return cudaSuccess;
     switch (Dg.sh_degree) {
-        case 0: launch_project_d<0>(Dg, P, n_blocks, st); break;
-        case 1: launch_project_d<1>(Dg, P, n_blocks, st); break;
-        case 2: launch_project_d<2>(Dg, P, n_blocks, st); break;
-        default: launch_project_d<3>(Dg, P, n_blocks, st); break;
+        case 0: return launch_project_d<0>(Dg, P, n_blocks, st);
+        case 1: return launch_project_d<1>(Dg, P, n_blocks, st);
+        case 2: return launch_project_d<2>(Dg, P, n_blocks, st);
+        default: return launch_project_d<3>(Dg, P, n_blocks, st);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace gsb
