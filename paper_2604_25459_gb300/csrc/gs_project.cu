@@ -192,6 +192,29 @@ cudaError_t launch_link_table(const float* poses, const gs_camera* cams, const E
 
 // ------------------------------------------------------------------ A2: projection
 
+// The projection's sums of products are pinned to one order of fused and
+// rounded products (the first product of a pair is fused, the second rounded),
+// so that a record's bits do not depend on how the code around them compiles:
+// images hang on their records through thresholds (the alpha floor, the stop
+// rule, the depth order).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+// a b + c d
+template <typename T>
+__device__ __forceinline__ T dot2(T a, T b, T c, T d) { return fma_rn(a, b, mul_rn(c, d)); }
+// a . b
+template <typename T>
+__device__ __forceinline__ T dot3(T ax, T ay, T az, T bx, T by, T bz) {
+    return fma_rn(az, bz, dot2(ax, bx, ay, by));
+}
+// one row of a rigid transform at p
+template <typename T>
+__device__ __forceinline__ T row_at(const float4& r, const float4& p) {
+    return dot3<T>(r.x, r.y, r.z, p.x, p.y, p.z) + (T)r.w;
+}
+
 // 2D covariance of one Gaussian before the 0.3 px^2 low-pass, in factored
 // form: M = J W F (2x3) with W the rotation part of X, J the EWA Jacobian at
 // the guard-band-clamped centre and F the Gaussian's covariance factor, so
@@ -202,31 +225,29 @@ template <typename T>
 __device__ __forceinline__ void ewa_factor(const LinkXf& X, const float4& a0, const float4& a1, const float4& a2,
                                            const float4& a3, float fx, float fy, float limxn, float limxp,
                                            float limyn, float limyp, T& A, T& B, T& C, T& K) {
-    const T mx = (T)X.r0.x * a0.x + (T)X.r0.y * a0.y + (T)X.r0.z * a0.z + (T)X.r0.w;
-    const T my = (T)X.r1.x * a0.x + (T)X.r1.y * a0.y + (T)X.r1.z * a0.z + (T)X.r1.w;
-    const T mz = (T)X.r2.x * a0.x + (T)X.r2.y * a0.y + (T)X.r2.z * a0.z + (T)X.r2.w;
+    const T mx = row_at<T>(X.r0, a0), my = row_at<T>(X.r1, a0), mz = row_at<T>(X.r2, a0);
     const T iz = T(1) / mz;
-    T tx = mx * iz, ty = my * iz;
+    T tx = mul_rn(mx, iz), ty = mul_rn(my, iz);
     tx = tx < -(T)limxn ? -(T)limxn : (tx > (T)limxp ? (T)limxp : tx);
     ty = ty < -(T)limyn ? -(T)limyn : (ty > (T)limyp ? (T)limyp : ty);
-    const T j00 = (T)fx * iz, j02 = -(T)fx * tx * iz;
-    const T j11 = (T)fy * iz, j12 = -(T)fy * ty * iz;
-    const T w0x = j00 * X.r0.x + j02 * X.r2.x, w0y = j00 * X.r0.y + j02 * X.r2.y, w0z = j00 * X.r0.z + j02 * X.r2.z;
-    const T w1x = j11 * X.r1.x + j12 * X.r2.x, w1y = j11 * X.r1.y + j12 * X.r2.y, w1z = j11 * X.r1.z + j12 * X.r2.z;
+    const T j00 = mul_rn((T)fx, iz), j02 = mul_rn(mul_rn(-(T)fx, tx), iz);
+    const T j11 = mul_rn((T)fy, iz), j12 = mul_rn(mul_rn(-(T)fy, ty), iz);
+    const T w0x = dot2<T>(j00, X.r0.x, j02, X.r2.x), w0y = dot2<T>(j00, X.r0.y, j02, X.r2.y),
+            w0z = dot2<T>(j00, X.r0.z, j02, X.r2.z);
+    const T w1x = dot2<T>(j11, X.r1.x, j12, X.r2.x), w1y = dot2<T>(j11, X.r1.y, j12, X.r2.y),
+            w1z = dot2<T>(j11, X.r1.z, j12, X.r2.z);
     // F row-major: (F00 F01 F02 | F10 F11 F12 | F20 F21 F22)
-    const T f00 = a1.x, f01 = a1.y, f02 = a1.z, f10 = a1.w, f11 = a2.x, f12 = a2.y, f20 = a2.z, f21 = a2.w,
-            f22 = a3.x;
-    const T m0x = w0x * f00 + w0y * f10 + w0z * f20;
-    const T m0y = w0x * f01 + w0y * f11 + w0z * f21;
-    const T m0z = w0x * f02 + w0y * f12 + w0z * f22;
-    const T m1x = w1x * f00 + w1y * f10 + w1z * f20;
-    const T m1y = w1x * f01 + w1y * f11 + w1z * f21;
-    const T m1z = w1x * f02 + w1y * f12 + w1z * f22;
-    A = m0x * m0x + m0y * m0y + m0z * m0z;
-    B = m0x * m1x + m0y * m1y + m0z * m1z;
-    C = m1x * m1x + m1y * m1y + m1z * m1z;
-    const T kx = m0y * m1z - m0z * m1y, ky = m0z * m1x - m0x * m1z, kz = m0x * m1y - m0y * m1x;
-    K = kx * kx + ky * ky + kz * kz;
+    const T m0x = dot3<T>(w0x, w0y, w0z, a1.x, a1.w, a2.z);
+    const T m0y = dot3<T>(w0x, w0y, w0z, a1.y, a2.x, a2.w);
+    const T m0z = dot3<T>(w0x, w0y, w0z, a1.z, a2.y, a3.x);
+    const T m1x = dot3<T>(w1x, w1y, w1z, a1.x, a1.w, a2.z);
+    const T m1y = dot3<T>(w1x, w1y, w1z, a1.y, a2.x, a2.w);
+    const T m1z = dot3<T>(w1x, w1y, w1z, a1.z, a2.y, a3.x);
+    A = dot3<T>(m0x, m0y, m0z, m0x, m0y, m0z);
+    B = dot3<T>(m0x, m0y, m0z, m1x, m1y, m1z);
+    C = dot3<T>(m1x, m1y, m1z, m1x, m1y, m1z);
+    const T kx = dot2<T>(m0y, m1z, -m0z, m1y), ky = dot2<T>(m0z, m1x, -m0x, m1z), kz = dot2<T>(m0x, m1y, -m0y, m1x);
+    K = dot3<T>(kx, ky, kz, kx, ky, kz);
 }
 
 // Near-degenerate 2D covariance (a thin Gaussian seen edge-on): the factor,
@@ -262,20 +283,29 @@ __device__ __forceinline__ void sh_basis(float x, float y, float z, float* Y) {
         Y[3] = -0.4886025119029199f * x;
     }
     if constexpr (D >= 2) {
-        const float xx = x * x, yy = y * y, zz = z * z;
+        // products that sums below must not fuse (see mul_rn)
+        const float xx = mul_rn(x, x), yy = mul_rn(y, y), zz = mul_rn(z, z);
         Y[4] = 1.0925484305920792f * x * y;
         Y[5] = -1.0925484305920792f * y * z;
-        Y[6] = 0.31539156525252005f * (2.0f * zz - xx - yy);
+        // degree 2 has always summed these two with the squares fused, degree 3
+        // with the squares rounded; both keep their bits
+        if constexpr (D == 2) {
+            Y[6] = 0.31539156525252005f * fma_rn(-y, y, fma_rn(-x, x, 2.0f * zz));
+            Y[8] = 0.5462742152960396f * fma_rn(x, x, -yy);
+        } else {
+            Y[6] = 0.31539156525252005f * (fma_rn(2.0f, zz, -xx) - yy);
+            Y[8] = 0.5462742152960396f * (xx - yy);
+        }
         Y[7] = -1.0925484305920792f * x * z;
-        Y[8] = 0.5462742152960396f * (xx - yy);
         if constexpr (D >= 3) {
-            Y[9] = -0.5900435899266435f * y * (3.0f * xx - yy);
+            const float q = fma_rn(4.0f, zz, -xx) - yy;
+            Y[9] = -0.5900435899266435f * y * fma_rn(3.0f, xx, -yy);
             Y[10] = 2.890611442640554f * x * y * z;
-            Y[11] = -0.4570457994644658f * y * (4.0f * zz - xx - yy);
-            Y[12] = 0.3731763325901154f * z * (2.0f * zz - 3.0f * xx - 3.0f * yy);
-            Y[13] = -0.4570457994644658f * x * (4.0f * zz - xx - yy);
+            Y[11] = -0.4570457994644658f * y * q;
+            Y[12] = 0.3731763325901154f * z * fma_rn(-3.0f, yy, fma_rn(-3.0f, xx, 2.0f * zz));
+            Y[13] = -0.4570457994644658f * x * q;
             Y[14] = 1.445305721320277f * z * (xx - yy);
-            Y[15] = -0.5900435899266435f * x * (xx - 3.0f * yy);
+            Y[15] = -0.5900435899266435f * x * fma_rn(-3.0f, yy, xx);
         }
     }
 }
@@ -300,7 +330,7 @@ __device__ __forceinline__ void sh_colour(F&& plane, float x, float y, float z, 
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 const int f = 4 * p + h;
-                if (f < NV) acc[f % 3] += Y[f / 3] * w[h];
+                if (f < NV) acc[f % 3] = fma_rn(Y[f / 3], w[h], acc[f % 3]);
             }
         }
     } else {
@@ -319,7 +349,7 @@ __device__ __forceinline__ void sh_colour(F&& plane, float x, float y, float z, 
                         val = __uint_as_float((uint32_t)bits << 16);
                     else
                         val = __half2float(__ushort_as_half(bits));
-                    acc[f % 3] += Y[f / 3] * val;
+                    acc[f % 3] = fma_rn(Y[f / 3], val, acc[f % 3]);
                 }
             }
         }
@@ -376,18 +406,19 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
     // through the storage order, link slots are their own
     const uint32_t key_index = (blk.frame0 && P.bg_index && act) ? (uint32_t)__ldg(P.bg_index + local) : local;
     // Every block stages, per env of a chunk, the camera, guard-band limits
-    // and table offsets in shared memory; background blocks (one link frame
-    // for every thread) also stage the frame's z row.  The many culled (env,
-    // Gaussian) pairs then wait on shared loads instead of chains of table
-    // loads, and the visible ones read their camera from shared memory.
-    __shared__ float4 s_r2[kProjStageEnvs];     // background blocks: frame 0's z row
+    // and table offsets in shared memory, and the link transform where one
+    // frame holds for every thread (all background blocks, all but a few link
+    // blocks).  A pair then waits on shared loads alone instead of on a chain
+    // of table loads that miss the L1.
+    __shared__ float4 s_xf[4][kProjStageEnvs];  // one frame: rows of the transform, camera centre
     __shared__ float4 s_cam[kProjStageEnvs];    // fx, fy, cx, cy
     __shared__ float4 s_lim[kProjStageEnvs];    // guard-band limits
     __shared__ int4 s_misc[kProjStageEnvs];     // W, H, xf_base, near plane (bits)
     __shared__ unsigned long long s_mb[kProjStageEnvs];  // visibility-word base
     __shared__ unsigned long long s_rb[kProjStageEnvs];  // record base
     __shared__ float4 s_rec[8][3 * 32];                  // per warp: the records of an env, before their store
-    const bool frame0 = blk.frame0 != 0;
+    const int li0 = __float_as_int(__ldg(P.p3 + blk.g_first).w) - blk.lb;  // the first thread's frame
+    const bool frame1 = __syncthreads_and(!act || li == li0) != 0;
     const bool once = blk.e1 - blk.e0 == 1;
     bool have_sh = false;
     for (int c0 = blk.e0; c0 < blk.e1; c0 += kProjStageEnvs) {
@@ -397,7 +428,13 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
         const EnvInfo* Ei = P.envs + c0 + i;
         const gs_camera* ci = P.cams + c0 + i;
         const int xb = __ldg(&Ei->xf_base);
-        if (frame0) s_r2[i] = __ldg(&P.xf[xb].r2);
+        if (frame1) {
+            const LinkXf* X = P.xf + xb + li0;
+            s_xf[0][i] = __ldg(&X->r0);
+            s_xf[1][i] = __ldg(&X->r1);
+            s_xf[2][i] = __ldg(&X->r2);
+            s_xf[3][i] = __ldg(&X->o);
+        }
         s_cam[i] = make_float4(__ldg(&ci->fx), __ldg(&ci->fy), __ldg(&ci->cx), __ldg(&ci->cy));
         s_lim[i] = make_float4(__ldg(&Ei->lim[0]), __ldg(&Ei->lim[1]), __ldg(&Ei->lim[2]), __ldg(&Ei->lim[3]));
         s_misc[i] = make_int4(__ldg(&ci->width), __ldg(&ci->height), xb, __float_as_int(__ldg(&ci->near_plane)));
@@ -415,21 +452,20 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
             // so only the z row of the transform and the near plane are read here
             LinkXf X;
             const float near = __int_as_float(misc.w);
-            X.r2 = frame0 ? s_r2[ei] : __ldg(&Xp->r2);
-            const float mz = X.r2.x * a0.x + X.r2.y * a0.y + X.r2.z * a0.z + X.r2.w;
+            X.r2 = frame1 ? s_xf[2][ei] : __ldg(&Xp->r2);
+            const float mz = row_at<float>(X.r2, a0);
             if (mz > near) {
-                X.r0 = __ldg(&Xp->r0);
-                X.r1 = __ldg(&Xp->r1);
-                const float mx = X.r0.x * a0.x + X.r0.y * a0.y + X.r0.z * a0.z + X.r0.w;
-                const float my = X.r1.x * a0.x + X.r1.y * a0.y + X.r1.z * a0.z + X.r1.w;
+                X.r0 = frame1 ? s_xf[0][ei] : __ldg(&Xp->r0);
+                X.r1 = frame1 ? s_xf[1][ei] : __ldg(&Xp->r1);
+                const float mx = row_at<float>(X.r0, a0), my = row_at<float>(X.r1, a0);
                 const float4 cam = s_cam[ei], lim = s_lim[ei];
                 const float fx = cam.x, fy = cam.y, cx = cam.z, cy = cam.w;
                 const int W = misc.x, H = misc.y;
                 const float limxn = lim.x, limxp = lim.y;  // per env, from the tables
                 const float limyn = lim.z, limyp = lim.w;
                 const float iz = 1.0f / mz;
-                const float u = fx * mx * iz + cx;
-                const float v = fy * my * iz + cy;
+                const float u = fma_rn(mul_rn(fx, mx), iz, cx);
+                const float v = fma_rn(mul_rn(fy, my), iz, cy);
                 // Conservative cull: the support half extent is at most
                 // sqrt(q* (|J_row|^2 tr(Sigma) + 0.3)) with |J_row|^2 <= (f/z)^2 (1 + lim^2).
                 // The test is on squares: a centre at distance d outside [0.5, W - 0.5]
@@ -455,7 +491,7 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
                     if (K >= 0x1p-10f * A * C) {
                         cA = A + 0.3f;
                         cC = C + 0.3f;
-                        const float det = K + 0.3f * (A + C) + 0.09f;
+                        const float det = fma_rn(0.3f, A + C, K) + 0.09f;
                         // reciprocal square roots (MUFU, <= 2 ulp): the support box below
                         // keeps its IEEE square roots and a 1e-4 margin over this ellipse
                         const float rc = rsqrtf(cC), rd = rsqrtf(det);
@@ -463,8 +499,19 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
                         l01 = -kS * B * rc * rd;
                         l11 = kS * rc;
                     } else {
-                        conic_factor_fp64(X, a0, a1, a2, a3, fx, fy, limxn, limxp, limyn, limyp, l00, l01, l11, cA,
-                                          cC);
+                        // copies: the callee takes addresses, and values whose address
+                        // is taken here would live in local memory for every pair
+                        // (200 bytes of stores per record, three times its own size)
+                        const LinkXf X64 = X;
+                        const float4 b0 = a0, b1 = a1, b2 = a2, b3 = a3;
+                        float o[5];
+                        conic_factor_fp64(X64, b0, b1, b2, b3, fx, fy, limxn, limxp, limyn, limyp, o[0], o[1], o[2],
+                                          o[3], o[4]);
+                        l00 = o[0];
+                        l01 = o[1];
+                        l11 = o[2];
+                        cA = o[3];
+                        cC = o[4];
                         if (P.nfp64) atomicAdd(P.nfp64, 1ull);
                     }
                     const bool ok = true;
@@ -472,9 +519,9 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
                     const float hy = sqrtf(qstar * cC) * 1.0001f;
                     int i0, i1, j0, j1;
                     if (ok && pixel_range(u, hx, W, i0, i1) && pixel_range(v, hy, H, j0, j1)) {
-                        const float4 O = __ldg(&Xp->o);
+                        const float4 O = frame1 ? s_xf[3][ei] : __ldg(&Xp->o);
                         float dx = a0.x - O.x, dy = a0.y - O.y, dz = a0.z - O.z;
-                        const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
+                        const float inv = rsqrtf(dot3<float>(dx, dy, dz, dx, dy, dz));
                         dx *= inv;
                         dy *= inv;
                         dz *= inv;
