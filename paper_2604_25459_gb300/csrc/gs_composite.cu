@@ -388,100 +388,109 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
         }
     };
 
-    // A depth-ordered window of wn ranks in src (keys or tmp), `before` ranks of
-    // the bucket preceding it: swap in the record slots and composite it.
-    uint32_t before = 0;
-    auto emit_window = [&](const uint32_t* src, uint32_t wn) {
-        for (uint32_t i = tid; i < wn; i += NT) keys[i] = __ldg(order + src[i]);
+    // The next window: its wn ranks in depth order in src (keys or tmp).
+    uint32_t before = 0;          // ranks of the bucket in earlier windows
+    bool whole = n <= (uint32_t)CAP;  // the bucket is one window, sorted at once
+    bool loaded = false;          // a bitmap of the ranks [r0, r0 + 32 BMW) is set up
+    uint32_t r0 = 0;
+    int g0 = 0;                   // its next group
+    while (before < n && !finished) {
+        const uint32_t* src = keys;
+        uint32_t wn = 0;
+        if (whole) {
+            uint32_t lo = 0xffffffffu, hi = 0u;
+            for (uint32_t i = tid; i < n; i += NT) {
+                const uint32_t k = Lk[i];
+                keys[i] = k;
+                lo = min(lo, k);
+                hi = max(hi, k);
+            }
+            block_minmax_u32<NT>(lo, hi, red);
+            whole = rank_sort<NT, SB>(keys, tmp, bm, red, (int)n, lo, hi, c32_dirty);
+            if (!whole) continue;  // crowded ranks: through bitmaps
+            wn = n;
+            src = tmp;
+        } else {
+            if (loaded && g0 >= NG) {
+                loaded = false;
+                r0 += (uint32_t)(BMW * 32);
+                __syncthreads();  // bm is rewritten for the next ranks
+            }
+            if (!loaded) {
+                if (r0 >= n_rank) {  // ranks beyond the env's: a corrupted bucket
+                    if (tid == 0) atomicOr(P.status, kStOverflow);
+                    break;
+                }
+                c32_dirty = true;
+                for (int i = tid; i < BMW / 4; i += NT) reinterpret_cast<uint4*>(bm)[i] = make_uint4(0u, 0u, 0u, 0u);
+                __syncthreads();
+                for_ranks<NT>(Lk, n, [&](uint32_t k) {
+                    const uint32_t d = k - r0;
+                    if (d < (uint32_t)(BMW * 32)) atomicOr(&bm[d >> 5], 1u << (d & 31u));
+                });
+                __syncthreads();
+                // ranks set before each group: thread t counts groups GPT t ..
+                constexpr int GPT = NG / NT;
+                uint32_t c[GPT], sum = 0;
+#pragma unroll
+                for (int j = 0; j < GPT; ++j) {
+                    const int g = tid * GPT + j;
+                    c[j] = 0;
+#pragma unroll
+                    for (int i = 0; i < kGroupWords; ++i)  // rotated: neighbouring threads hit different banks
+                        c[j] += __popc(bm[g * kGroupWords + ((i + tid) & (kGroupWords - 1))]);
+                    sum += c[j];
+                }
+                uint32_t run = block_excl_scan_u32<NT>(sum, red);
+#pragma unroll
+                for (int j = 0; j < GPT; ++j) {
+                    pre[tid * GPT + j] = run;
+                    run += c[j];
+                }
+                if (tid == NT - 1) pre[NG] = run;
+                __syncthreads();
+                loaded = true;
+                g0 = 0;
+            }
+            // a run of whole groups of at most CAP ranks
+            const uint32_t base = pre[g0];
+            int lo = g0 + 1, hi = NG;  // last g1 with pre[g1] - base <= CAP
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (pre[mid] - base <= (uint32_t)CAP) lo = mid; else hi = mid - 1;
+            }
+            const int g1 = lo;
+            wn = pre[g1] - base;
+            if (wn > 0) {
+                // a half-warp reads a group's words back in order
+                for (int gb = g0 + 2 * warp; gb < g1; gb += NT / 16) {
+                    const int g = gb + (lane >> 4);
+                    uint32_t w = g < g1 ? bm[g * kGroupWords + (lane & 15)] : 0u;
+                    const uint32_t pc = __popc(w);
+                    uint32_t x = pc;
+#pragma unroll
+                    for (int d = 1; d < 16; d <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xffffffffu, x, d, 16);
+                        if ((lane & 15) >= d) x += y;
+                    }
+                    if (w) {
+                        uint32_t at = pre[g] - base + x - pc;
+                        const uint32_t r = r0 + (uint32_t)(g * kGroupWords + (lane & 15)) * 32u;
+                        while (w) {
+                            keys[at++] = r + (uint32_t)(__ffs(w) - 1);
+                            w &= w - 1u;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+            g0 = g1;
+            if (wn == 0) continue;
+        }
+        for (uint32_t i = tid; i < wn; i += NT) keys[i] = __ldg(order + src[i]);  // record slots
         __syncthreads();
         run_window(wn);
         before += wn;
-    };
-
-    bool ordered = n == 0;
-    if (n > 0 && n <= (uint32_t)CAP) {  // one window
-        uint32_t lo = 0xffffffffu, hi = 0u;
-        for (uint32_t i = tid; i < n; i += NT) {
-            const uint32_t k = Lk[i];
-            keys[i] = k;
-            lo = min(lo, k);
-            hi = max(hi, k);
-        }
-        block_minmax_u32<NT>(lo, hi, red);
-        if (rank_sort<NT, SB>(keys, tmp, bm, red, (int)n, lo, hi, c32_dirty)) {
-            ordered = true;
-            emit_window(tmp, n);
-        }
-    }
-    if (!ordered) {  // bitmaps of NG * 512 ranks at a time
-        c32_dirty = true;
-        for (uint32_t r0 = 0; r0 < n_rank && before < n && !finished; r0 += (uint32_t)(BMW * 32)) {
-            for (int i = tid; i < BMW / 4; i += NT) reinterpret_cast<uint4*>(bm)[i] = make_uint4(0u, 0u, 0u, 0u);
-            __syncthreads();
-            for_ranks<NT>(Lk, n, [&](uint32_t k) {
-                const uint32_t d = k - r0;
-                if (d < (uint32_t)(BMW * 32)) atomicOr(&bm[d >> 5], 1u << (d & 31u));
-            });
-            __syncthreads();
-            // ranks set before each group: thread t counts groups GPT t ..
-            constexpr int GPT = NG / NT;
-            uint32_t c[GPT], sum = 0;
-#pragma unroll
-            for (int j = 0; j < GPT; ++j) {
-                const int g = tid * GPT + j;
-                c[j] = 0;
-#pragma unroll
-                for (int i = 0; i < kGroupWords; ++i)  // rotated: neighbouring threads hit different banks
-                    c[j] += __popc(bm[g * kGroupWords + ((i + tid) & (kGroupWords - 1))]);
-                sum += c[j];
-            }
-            uint32_t run = block_excl_scan_u32<NT>(sum, red);
-#pragma unroll
-            for (int j = 0; j < GPT; ++j) {
-                pre[tid * GPT + j] = run;
-                run += c[j];
-            }
-            if (tid == NT - 1) pre[NG] = run;
-            __syncthreads();
-            // windows: runs of whole groups of at most CAP ranks
-            for (int g0 = 0; g0 < NG && !finished;) {
-                const uint32_t base = pre[g0];
-                int lo = g0 + 1, hi = NG;  // last g1 with pre[g1] - base <= CAP
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (pre[mid] - base <= (uint32_t)CAP) lo = mid; else hi = mid - 1;
-                }
-                const int g1 = lo;
-                const uint32_t wn = pre[g1] - base;
-                if (wn > 0) {
-                    // a half-warp reads a group's words back in order
-                    for (int gb = g0 + 2 * warp; gb < g1; gb += NT / 16) {
-                        const int g = gb + (lane >> 4);
-                        uint32_t w = g < g1 ? bm[g * kGroupWords + (lane & 15)] : 0u;
-                        const uint32_t pc = __popc(w);
-                        uint32_t x = pc;
-#pragma unroll
-                        for (int d = 1; d < 16; d <<= 1) {
-                            const uint32_t y = __shfl_up_sync(0xffffffffu, x, d, 16);
-                            if ((lane & 15) >= d) x += y;
-                        }
-                        if (w) {
-                            uint32_t at = pre[g] - base + x - pc;
-                            const uint32_t r = r0 + (uint32_t)(g * kGroupWords + (lane & 15)) * 32u;
-                            while (w) {
-                                keys[at++] = r + (uint32_t)(__ffs(w) - 1);
-                                w &= w - 1u;
-                            }
-                        }
-                    }
-                    __syncthreads();
-                    emit_window(keys, wn);
-                }
-                g0 = g1;
-            }
-            __syncthreads();  // bm is rewritten for the next ranks
-        }
-        if (before < n && !finished && tid == 0) atomicOr(P.status, kStOverflow);  // a corrupted bucket
     }
 
     if (CNT && P.neval) {

@@ -13,7 +13,7 @@
 // read the tile's bucket and keep the keys whose subtile bit is set.
 //
 // The bucket's keys are depth ranks (gs_rank.cu) in any order; windows of at
-// most kCap ranks come in order from
+// most CAP ranks come in order from
 //   - the whole bucket at once, if it is short;
 //   - a histogram over kSortBins rank ranges, windows being runs of ranges
 //     gathered from the bucket and sorted in shared memory (few keys per rank:
@@ -29,11 +29,10 @@ namespace gsb {
 namespace {
 
 constexpr uint32_t kAll = 0xffffffffu;
-constexpr int kCap = 512;         // ranks per window
+constexpr int kWarps = 4;         // warps per CTA (independent; one CTA per warp would cost 1 KB of shared memory each)
 constexpr int kSortBins = 512;    // counters of the sort and of the histogram
-constexpr int kCrowd = 24;        // longest range sorted by insertion
+constexpr int kCrowd = 32;        // longest range sorted by counting
 constexpr int kWords = 1024;      // bitmap words
-constexpr int kGroups = 64;       // groups of 16 bitmap words (512 ranks)
 constexpr uint32_t kShort = 1024; // buckets gathered whole
 
 // f(key, valid) for every key of the bucket L[0, n), by the whole warp: 16-byte
@@ -42,7 +41,7 @@ constexpr uint32_t kShort = 1024; // buckets gathered whole
 template <typename F>
 __device__ __forceinline__ void warp_keys(const uint32_t* L, uint32_t n, F&& f) {
     constexpr int U = 4;
-    const uint32_t lane = threadIdx.x;
+    const uint32_t lane = threadIdx.x & 31u;
     const uint32_t off = (uint32_t)((uintptr_t)L & 15u) >> 2, end = off + n;
     const uint4* V = reinterpret_cast<const uint4*>(L - off);
     for (uint32_t i = 0; i < end; i += 128 * U) {
@@ -51,6 +50,16 @@ __device__ __forceinline__ void warp_keys(const uint32_t* L, uint32_t n, F&& f) 
         for (int u = 0; u < U; ++u) {
             const uint32_t x = i + 128 * u + 4 * lane;
             v[u] = x < end ? __ldg(V + (x >> 2)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (i >= off && i + 128 * U <= end) {  // no word outside the bucket
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                f(v[u].x, true);
+                f(v[u].y, true);
+                f(v[u].z, true);
+                f(v[u].w, true);
+            }
+            continue;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -65,13 +74,13 @@ __device__ __forceinline__ void warp_keys(const uint32_t* L, uint32_t n, F&& f) 
     }
 }
 
-// Sorts keys[0, m), distinct ranks in [lo, hi], m <= kCap (tmp: scratch).  One key per lane: a bitonic network in
-// registers.  Otherwise a counting sort by kSortBins equal ranges with
-// insertion inside a range, or, when a range holds more than kCrowd, a bitonic
+// Sorts keys[0, m), distinct ranks in [lo, hi], m <= 512 (tmp: scratch).  One key per lane: a bitonic network in
+// registers.  Otherwise a counting sort by kSortBins equal ranges,
+// a rank's place in its range being the number of smaller ones, or, when a range holds more than kCrowd, a bitonic
 // sort in shared memory.
 __device__ __forceinline__ void warp_sort(uint32_t* keys, uint32_t* tmp, uint32_t* cnt, int m, uint32_t lo,
                                           uint32_t hi) {
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31;
     if (m <= 32) {
         uint32_t k = lane < m ? keys[lane] : kAll;
 #pragma unroll
@@ -145,21 +154,16 @@ __device__ __forceinline__ void warp_sort(uint32_t* keys, uint32_t* tmp, uint32_
         tmp[atomicAdd(&cnt[(k - lo) >> shift], 1u)] = k;
     }
     __syncwarp();
-#pragma unroll 1
-    for (int b = lane; b < kSortBins; b += 32) {  // cnt[b] is the end of range b now
-        const int e = (int)cnt[b], a = b ? (int)cnt[b - 1] : 0;
-        for (int x = a + 1; x < e; ++x) {
-            const uint32_t k = tmp[x];
-            int y = x - 1;
-            while (y >= a && tmp[y] > k) {
-                tmp[y + 1] = tmp[y];
-                --y;
-            }
-            tmp[y + 1] = k;
-        }
+    // cnt[b] is the end of range b now; a rank's place in its range is the
+    // number of smaller ranks there
+    for (int i = lane; i < m; i += 32) {
+        const uint32_t k = tmp[i];
+        const int b = (int)((k - lo) >> shift);
+        const uint32_t e = cnt[b];
+        uint32_t place = b ? cnt[b - 1] : 0u;
+        for (uint32_t x = place; x < e; ++x) place += tmp[x] < k ? 1u : 0u;
+        keys[place] = k;
     }
-    __syncwarp();
-    for (int i = lane; i < m; i += 32) keys[i] = tmp[i];
     __syncwarp();
 }
 
@@ -184,18 +188,31 @@ __device__ __forceinline__ void copy16(float4* dst, const float4* src) {
 // quadrants, 2048 environments of the room... see the table in the header of
 // launch_composite_warp.
 template <int MODE>
-__global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
+__global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k_composite_warp(CompParams P) {
     constexpr bool LID = MODE == 1 || MODE == 3;
     constexpr bool QUAD = MODE != 3;
     constexpr bool CNT = MODE != 0;
-    __shared__ __align__(16) uint32_t keys[kCap];
-    __shared__ __align__(16) uint32_t bm[kWords];  // bitmap | sort counters, then range starts
-    __shared__ uint32_t pre[kGroups + 1];
-    __shared__ float4 rec[2][3][32];  // records of this and the next 32 splats: r0, r1, r2; between windows sort scratch
-    static_assert(sizeof(rec) >= kCap * 4, "the sort scratch shares the records' memory");
-    __shared__ float4 sD[LID ? 32 : 1];            // LiDAR: third row of G
-    __shared__ int4 sR[LID ? 32 : 1];              // LiDAR: x0, x1 - x0, y0, y1 - y0
-    const int lane = threadIdx.x;
+    constexpr int CAP = LID ? 512 : 256;   // ranks per window, and per group of bitmap words
+    constexpr int GW = CAP / 32;           // words per group
+    constexpr int NG = kWords / GW;        // groups
+    struct Smem {                          // a warp's own
+        uint32_t keys[CAP];                // the window's ranks
+        uint32_t bm[kWords];               // bitmap | sort counters, then range starts
+        float4 rec[2][3][32];              // records of this and the next 32 splats: r0, r1, r2; between windows sort scratch
+        float4 sD[LID ? 32 : 1];           // LiDAR: third row of G
+        int4 sR[LID ? 32 : 1];             // LiDAR: x0, x1 - x0, y0, y1 - y0
+        uint32_t pre[NG + 1];              // ranks set before each group of the bitmap
+    };
+    static_assert(sizeof(Smem::rec) >= CAP * 4, "the sort scratch shares the records' memory");
+    __shared__ __align__(16) Smem smem[kWarps];
+    Smem& sm = smem[threadIdx.x >> 5];
+    uint32_t* const keys = sm.keys;
+    uint32_t* const bm = sm.bm;
+    uint32_t* const pre = sm.pre;
+    auto& rec = sm.rec;
+    auto& sD = sm.sD;
+    auto& sR = sm.sR;
+    const int lane = threadIdx.x & 31;
     const int lx = __ffs(P.tile_w) - 4, ly = __ffs(P.tile_h) - 4;  // log2 of the tile's subtile columns, rows
     const int lsub = MODE == 3 ? 0 : lx + ly;
     const int grp = lane >> 3, l8 = lane & 7;
@@ -367,7 +384,8 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
     const uint32_t n_rank = __ldg(P.nvis + el);
     const int kshift = P.key_shift;
     // the rank of a key and whether this warp's pixels lie in its subtiles
-    auto taken = [&](uint32_t k) { return kshift == 0 || (k & submask) != 0u; };
+    const uint32_t any_sub = kshift == 0 ? 1u : 0u;
+    auto taken = [&](uint32_t k) { return ((k & submask) | any_sub) != 0u; };
 
     // Composite the ordered ranks keys[0, m).  True once every pixel of the warp
     // has terminated.
@@ -577,7 +595,7 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
     };
 
     // Appends the taken ranks in [lo, hi) of the bucket to keys (the first
-    // kCap of them) and returns how many there are; wl, wh: their bounds.
+    // CAP of them) and returns how many there are; wl, wh: their bounds.
     uint32_t wl = 0, wh = 0;
     auto gather = [&](uint32_t lo, uint32_t width) -> uint32_t {
         uint32_t have = 0, a = kAll, z = 0u;
@@ -588,7 +606,7 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
             const uint32_t b = __ballot_sync(kAll, in);
             if (in) {
                 const uint32_t at = have + (uint32_t)__popc(b & below);
-                if (at < (uint32_t)kCap) keys[at] = r;
+                if (at < (uint32_t)CAP) keys[at] = r;
                 a = min(a, r);
                 z = max(z, r);
             }
@@ -610,11 +628,11 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
     bool loaded = false;   // a bitmap is set up
     if (n <= kShort) {
         whole = n ? gather(0u, kAll) : 0u;
-        if (whole <= (uint32_t)kCap) how = kWhole;
+        if (whole <= (uint32_t)CAP) how = kWhole;
     }
     if (how == kBitmap) {
         const uint32_t est = kshift ? n / 2 : n;
-        if (est / kCap + 2 < n_rank / (kWords * 32) + 1) {
+        if (est / CAP + 2 < n_rank / (kWords * 32) + 1) {
             while (((n_rank - 1u) >> hs) >= (uint32_t)kSortBins) ++hs;
             for (int i = lane; i < kSortBins; i += 32) bm[i] = 0u;
             __syncwarp();
@@ -645,7 +663,7 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
                 run += c[j];
             }
             __syncwarp();
-            if (!__any_sync(kAll, most > (uint32_t)kCap)) how = kRuns;
+            if (!__any_sync(kAll, most > (uint32_t)CAP)) how = kRuns;
         }
     }
     for (;;) {
@@ -660,10 +678,10 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
             auto begin = [&](int g) { return g < kSortBins ? start_of[g] : htotal; };
             const uint32_t base = begin(g0);
             if (base >= htotal) break;
-            int lo = g0 + 1, hi = kSortBins;  // last g1 with begin(g1) - base <= kCap
+            int lo = g0 + 1, hi = kSortBins;  // last g1 with begin(g1) - base <= CAP
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
-                if (begin(mid) - base <= (uint32_t)kCap) lo = mid; else hi = mid - 1;
+                if (begin(mid) - base <= (uint32_t)CAP) lo = mid; else hi = mid - 1;
             }
             wn = (int)(begin(lo) - base);
             const uint32_t a = (uint32_t)g0 << hs;
@@ -671,7 +689,7 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
             if (wn == 0) continue;
             gather(a, ((uint32_t)lo << hs) - a);
         } else {
-            if (loaded && g0 >= kGroups) {
+            if (loaded && g0 >= NG) {
                 loaded = false;
                 r0 += (uint32_t)(kWords * 32);
             }
@@ -680,52 +698,63 @@ __global__ void __launch_bounds__(32, 20) k_composite_warp(CompParams P) {
                 for (int i = lane; i < kWords / 4; i += 32)
                     reinterpret_cast<uint4*>(bm)[i] = make_uint4(0u, 0u, 0u, 0u);
                 __syncwarp();
+                const uint32_t k0 = r0 << kshift, span = (uint32_t)(kWords * 32) << kshift;
                 warp_keys(Lk, n, [&](uint32_t k, bool valid) {
-                    const uint32_t d = (k >> kshift) - r0;
-                    if (valid && taken(k) && d < (uint32_t)(kWords * 32)) atomicOr(&bm[d >> 5], 1u << (d & 31u));
+                    const uint32_t d = k - k0;
+                    if (valid && d < span && taken(k)) atomicOr(&bm[d >> (5 + kshift)], 1u << ((d >> kshift) & 31u));
                 });
                 __syncwarp();
-                // ranks set before each group: a lane counts two groups
-                uint32_t c[2] = {0u, 0u};
+                // ranks set before each group: a lane counts GPL groups
+                constexpr int GPL = NG / 32;
+                uint32_t c[GPL], run = 0;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {  // rotated: neighbouring lanes hit different banks
-                    c[0] += __popc(bm[(2 * lane) * 16 + ((i + lane) & 15)]);
-                    c[1] += __popc(bm[(2 * lane + 1) * 16 + ((i + lane) & 15)]);
+                for (int k = 0; k < GPL; ++k) {
+                    c[k] = 0u;
+#pragma unroll
+                    for (int i = 0; i < GW; ++i)  // rotated: neighbouring lanes hit different banks
+                        c[k] += __popc(bm[(GPL * lane + k) * GW + ((i + lane) & (GW - 1))]);
+                    run += c[k];
                 }
-                uint32_t run = c[0] + c[1];
+                const uint32_t mine = run;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
                     const uint32_t y = __shfl_up_sync(kAll, run, d);
                     if (lane >= d) run += y;
                 }
-                if (lane == 31) pre[kGroups] = run;
-                pre[2 * lane] = run - c[0] - c[1];
-                pre[2 * lane + 1] = run - c[1];
+                if (lane == 31) pre[NG] = run;
+                run -= mine;
+#pragma unroll
+                for (int k = 0; k < GPL; ++k) {
+                    pre[GPL * lane + k] = run;
+                    run += c[k];
+                }
                 __syncwarp();
                 loaded = true;
                 g0 = 0;
             }
             const uint32_t base = pre[g0];
-            const uint32_t fit = base + (uint32_t)kCap;
-            // groups whose end is within kCap of the window's start (ends ascend)
-            const int g1 = __popc(__ballot_sync(kAll, pre[2 * lane + 1] <= fit)) +
-                           __popc(__ballot_sync(kAll, pre[2 * lane + 2] <= fit));
+            const uint32_t fit = base + (uint32_t)CAP;
+            // groups whose end is within CAP of the window's start (ends ascend)
+            int g1 = 0;
+#pragma unroll
+            for (int k = 0; k < NG / 32; ++k) g1 += __popc(__ballot_sync(kAll, pre[32 * k + lane + 1] <= fit));
             wn = (int)(pre[g1] - base);
             if (wn > 0) {
-                // a half-warp reads a group's words back in order
-                for (int gb = g0; gb < g1; gb += 2) {
-                    const int g = gb + (lane >> 4);
-                    uint32_t w = g < g1 ? bm[g * 16 + (lane & 15)] : 0u;
+                // GW lanes read a group's words back in order
+                const int word = lane & (GW - 1);
+                for (int gb = g0; gb < g1; gb += 32 / GW) {
+                    const int g = gb + lane / GW;
+                    uint32_t w = g < g1 ? bm[g * GW + word] : 0u;
                     const uint32_t pc = __popc(w);
                     uint32_t x = pc;
 #pragma unroll
-                    for (int d = 1; d < 16; d <<= 1) {
-                        const uint32_t y = __shfl_up_sync(kAll, x, d, 16);
-                        if ((lane & 15) >= d) x += y;
+                    for (int d = 1; d < GW; d <<= 1) {
+                        const uint32_t y = __shfl_up_sync(kAll, x, d, GW);
+                        if (word >= d) x += y;
                     }
                     if (w) {
                         uint32_t at = pre[g] - base + x - pc;
-                        const uint32_t r = r0 + (uint32_t)(g * 16 + (lane & 15)) * 32u;
+                        const uint32_t r = r0 + (uint32_t)(g * GW + word) * 32u;
                         while (w) {
                             keys[at++] = r + (uint32_t)(__ffs(w) - 1);
                             w &= w - 1u;
@@ -773,14 +802,16 @@ template <int MODE>
 static cudaError_t launch_warps(const CompParams& P, cudaStream_t st, int* ctas) {
     static PerDevice resident;
     int full = 0;
-    const cudaError_t e = resident.ctas((const void*)k_composite_warp<MODE>, 32, &full);
+    const cudaError_t e = resident.ctas((const void*)k_composite_warp<MODE>, 32 * kWarps, &full);
     if (e != cudaSuccess) return e;
     const int subs = MODE == 3 ? 1 : (P.tile_w / 8) * (P.tile_h / 8);
     const unsigned long long items = (unsigned long long)(P.item_end - P.item_begin) * subs;
     if (items > 0xffffffffull) return cudaErrorInvalidValue;
     const unsigned long long claims = (items + P.chunk - 1) / P.chunk;
-    *ctas = (int)std::min((unsigned long long)full, claims);
-    k_composite_warp<MODE><<<*ctas, 32, 0, st>>>(P);
+    // few claims: fewer warps per CTA, so that they spread over the SMs
+    const int warps = (int)std::min((claims + full - 1) / full, (unsigned long long)kWarps);
+    *ctas = (int)std::min((unsigned long long)full, (claims + warps - 1) / warps);
+    k_composite_warp<MODE><<<*ctas, 32 * warps, 0, st>>>(P);
     return cudaGetLastError();
 }
 

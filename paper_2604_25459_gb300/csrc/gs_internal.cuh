@@ -309,7 +309,7 @@ cudaError_t launch_rank(const RankParams& R, int n_envs, int max_words, cudaStre
 // form (launch_composite_warp) renders LiDAR scans and, with P.quad, images.
 cudaError_t launch_composite(const CompParams& P, cudaStream_t st, int* ctas);
 cudaError_t launch_composite_warp(const CompParams& P, cudaStream_t st, int* ctas);
-// Resident warps of the warp form (the items that run at once).
+// About the resident warps of the warp form per SM (the items that run at once).
 constexpr int kWarpsPerSM = 20;
 
 constexpr int kWordsPerBlock = 256;  // binning block: at most one visibility word per thread of 256 (8192 slots)

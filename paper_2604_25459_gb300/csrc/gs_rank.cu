@@ -24,7 +24,7 @@ constexpr int kSampleLooks = 8;     // slots looked at per thread of k_rank_samp
 constexpr int kSortThreads = 256;
 constexpr int kSortCap = 2048;      // keys of a window sorted in shared memory
 constexpr int kSubBins = 1024;      // depth ranges of a window's counting sort
-constexpr int kInsert = 24;         // longest range sorted by insertion
+constexpr int kInsert = 32;         // longest range sorted by counting
 
 // Ascending bitonic sort of a[0, m), m a power of two, by the whole block.
 __device__ __forceinline__ void bitonic_sort(unsigned long long* a, int m) {
@@ -164,26 +164,41 @@ __global__ void __launch_bounds__(256) k_rank_place(RankParams P) {
     const uint32_t* bo = P.block_off + ((size_t)el * P.blocks + blockIdx.x) * P.bins;
     for (int b = threadIdx.x; b < P.bins; b += 256) first[b] = P.bin_off[(size_t)el * P.bins + b] + bo[b];
     __syncthreads();
-    for (uint32_t w = w0 + (threadIdx.x >> 5); w < w1; w += 8) {
-        const uint32_t m = __ldg(P.mask + E.mask_base + w);
-        if (!((m >> lane) & 1u)) continue;
-        const uint32_t j = w * 32 + lane;
-        const uint32_t at = P.rank[E.rec_base + j];
-        P.zkeys[E.rec_base + first[at >> 13] + (at & 0x1fffu)] = rank_key(P, P.r3[E.rec_base + j], j);
+    constexpr int U = 4;  // words in flight per warp
+    for (uint32_t w = w0 + (threadIdx.x >> 5); w < w1; w += 8 * U) {
+        uint32_t at[U];
+        uint4 q[U];
+        bool vis[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            vis[u] = w + 8 * u < w1 && ((__ldg(P.mask + E.mask_base + w + 8 * u) >> lane) & 1u);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const size_t j = E.rec_base + (w + 8 * u) * 32 + lane;
+            if (vis[u]) {
+                at[u] = P.rank[j];
+                q[u] = P.r3[j];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (vis[u])
+                P.zkeys[E.rec_base + first[at[u] >> 13] + (at[u] & 0x1fffu)] =
+                    rank_key(P, q[u], (w + 8 * u) * 32 + lane);
     }
 }
 
 // Sorts an env's windows of whole ranges (positions [win[v], win[v+1])) and
 // writes order and rank.  A window of at most kSortCap keys is sorted in
-// shared memory: a counting sort by kSubBins ranges of its depth bits with
-// insertion inside a range, or a bitonic sort of the whole keys when a range
+// shared memory: a counting sort by kSubBins ranges of its depth bits, a key's
+// place in its range being the number of smaller keys in it, or a bitonic sort of the whole keys when a range
 // holds more than kInsert.  A larger window (a sample that missed a crowd) is
 // cut into pieces of at most kSortCap keys by radix selection over its keys.
-__global__ void __launch_bounds__(kSortThreads) k_rank_sort(RankParams P) {
+__global__ void __launch_bounds__(kSortThreads, 4) k_rank_sort(RankParams P) {
     constexpr int NT = kSortThreads;
     constexpr int PT = kSortCap / NT;  // keys per thread
     __shared__ unsigned long long tmp[kSortCap];
-    __shared__ uint32_t cnt[kSubBins];
+    __shared__ uint32_t cnt[kSubBins + 1];
     __shared__ uint32_t red[64];
     __shared__ unsigned long long sel_lo, sel_hi;
     __shared__ uint32_t sel_n;
@@ -199,6 +214,14 @@ __global__ void __launch_bounds__(kSortThreads) k_rank_sort(RankParams P) {
     // sort src[0, m) (global keys, or tmp itself) and give the keys the places
     // first, first + 1, ...
     auto sort_out = [&](const unsigned long long* src, int m, uint32_t first) {
+        auto put = [&](uint32_t place, unsigned long long key) {
+            const uint32_t g = (uint32_t)key;
+            const uint32_t slot = (P.bg_slot && g < P.n_bg) ? (uint32_t)__ldg(P.bg_slot + g) : g;
+            if (slot < E.n_local) {  // always, for keys that the placement wrote
+                order[place] = slot;
+                rank[slot] = place;
+            }
+        };
         unsigned long long k[PT];
         uint32_t zl = 0xffffffffu, zh = 0u;
 #pragma unroll
@@ -216,11 +239,13 @@ __global__ void __launch_bounds__(kSortThreads) k_rank_sort(RankParams P) {
         const int shift = (span >> 10) ? 22 - __clz(span) : 0;  // span >> shift < kSubBins
         uint32_t at[PT];  // range << 16 | place in it
 #pragma unroll
-        for (int u = 0; u < PT; ++u)
+        for (int u = 0; u < PT; ++u) {
+            if (u * NT >= m) break;  // uniform
             if (tid + u * NT < m) {
                 const uint32_t b = ((uint32_t)(k[u] >> 32) - zl) >> shift;
                 at[u] = b << 16 | atomicAdd(&cnt[b], 1u);
             }
+        }
         __syncthreads();
         constexpr int PER = kSubBins / NT;
         uint32_t loc[PER], sum = 0;
@@ -238,38 +263,32 @@ __global__ void __launch_bounds__(kSortThreads) k_rank_sort(RankParams P) {
             for (int u = 0; u < PT; ++u)
                 if (tid + u * NT < p) tmp[tid + u * NT] = k[u];
             bitonic_sort(tmp, p);
-        } else {
-            uint32_t run = block_excl_scan_u32<NT>(sum, red);
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                cnt[tid * PER + j] = run;
-                run += loc[j];
-            }
+            for (int i = tid; i < m; i += NT) put(first + (uint32_t)i, tmp[i]);
             __syncthreads();
-#pragma unroll
-            for (int u = 0; u < PT; ++u)
-                if (tid + u * NT < m) tmp[cnt[at[u] >> 16] + (at[u] & 0xffffu)] = k[u];
-            __syncthreads();
-            for (int b = tid; b < kSubBins; b += NT) {
-                const int a = (int)cnt[b], e = b + 1 < kSubBins ? (int)cnt[b + 1] : m;
-                for (int x = a + 1; x < e; ++x) {
-                    const unsigned long long q = tmp[x];
-                    int y = x - 1;
-                    while (y >= a && tmp[y] > q) {
-                        tmp[y + 1] = tmp[y];
-                        --y;
-                    }
-                    tmp[y + 1] = q;
-                }
-            }
-            __syncthreads();
+            return;
         }
-        for (int i = tid; i < m; i += NT) {
-            const uint32_t g = (uint32_t)tmp[i];
-            const uint32_t slot = (P.bg_slot && g < P.n_bg) ? (uint32_t)__ldg(P.bg_slot + g) : g;
-            if (slot < E.n_local) {  // always, for keys that the placement wrote
-                order[first + i] = slot;
-                rank[slot] = first + (uint32_t)i;
+        uint32_t run = block_excl_scan_u32<NT>(sum, red);
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            cnt[tid * PER + j] = run;
+            run += loc[j];
+        }
+        if (tid == NT - 1) cnt[kSubBins] = run;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < PT; ++u) {
+            if (u * NT >= m) break;
+            if (tid + u * NT < m) tmp[cnt[at[u] >> 16] + (at[u] & 0xffffu)] = k[u];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < PT; ++u) {
+            if (u * NT >= m) break;
+            if (tid + u * NT < m) {
+                const uint32_t b = at[u] >> 16, s = cnt[b], e = cnt[b + 1];
+                uint32_t place = s;
+                for (uint32_t x = s; x < e; ++x) place += tmp[x] < k[u] ? 1u : 0u;
+                put(first + place, k[u]);
             }
         }
         __syncthreads();
