@@ -60,7 +60,7 @@ struct gs_plan_s {
     struct Wave {
         int e0, e1;
         DevBuf envs, blocks, cams;
-        int n_blocks = 0, xf_items = 0, max_words = 0, max_T = 0;
+        int n_blocks = 0, xf_items = 0, max_words = 0, max_T = 0, max_hist = 0;
         unsigned long long recs = 0, words = 0, tiles = 0;
         unsigned long long cap = 0;  // intersection-key capacity
     };
@@ -404,11 +404,12 @@ gs_status upload_tables(gs_scene s, const std::vector<EnvSpec>& specs, int e0, i
     int nb2 = 0;
     build_wave_tables(s->D, s->link_offsets.data(), sp, We, tw, th, pix_rebase, s->h_envs.data(), s->h_blocks.data(),
                       &nb2, nb);
-    int max_words = 0, max_T = 0;
+    int max_words = 0, max_T = 0, max_hist = 0;
     for (int e = 0; e < We; ++e) {
         s->h_cams[e] = *sp[e].cam;
         max_words = std::max(max_words, (int)((s->h_envs[e].n_local + 31) / 32));
         max_T = std::max(max_T, s->h_envs[e].T);
+        max_hist = std::max(max_hist, (s->h_envs[e].ntx + 1) * (s->h_envs[e].T / s->h_envs[e].ntx + 1));
     }
     CK(d_envs.ensure(sizeof(EnvInfo) * ((size_t)We + 1)), "alloc env table");
     CK(d_blocks.ensure(sizeof(ProjBlock) * (size_t)std::max(nb, 1)), "alloc block table");
@@ -432,7 +433,7 @@ gs_status upload_tables(gs_scene s, const std::vector<EnvSpec>& specs, int e0, i
     }
     const EnvInfo& sen = s->h_envs[We];
     *wt = WaveTables{d_envs.as<EnvInfo>(), d_blocks.as<ProjBlock>(), d_cams.as<gs_camera>(), We, nb, sen.xf_base,
-                     max_words, max_T, sen.rec_base, sen.mask_base, sen.tile_base, s->h_envs.data()};
+                     max_words, max_T, max_hist, sen.rec_base, sen.mask_base, sen.tile_base, s->h_envs.data()};
     return GS_OK;
 }
 
@@ -531,7 +532,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     B.e_begin = 0;
     B.tile_w = tw;
     B.tile_h = th;
-    B.words_per_block = R.words_per_block;
+    B.words_per_block = scatter_words(wt.max_words, We, wt.max_T);
     B.counts = counts;
     B.off_local = sc.off.as<uint32_t>();
     B.env_base = sc.env_base.as<unsigned long long>();
@@ -545,7 +546,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         B.key_shift = n_sub;
     PhaseTimer t3(s, st, GS_PHASE_COUNT, timers);
     CK(launch_rank_sample(R, We, st), "depth sample");
-    CK(launch_count(B, R, We, wt.max_words, wt.max_T, st), "count");
+    CK(launch_count(B, R, We, wt.max_T, wt.max_hist, st), "count");
     t3.done(2);
     PhaseTimer t4(s, st, GS_PHASE_SCAN, timers);
     CK(launch_scan_ranks(wt.envs, counts, sc.off.as<uint32_t>(), sc.env_total.as<unsigned long long>(),
@@ -643,7 +644,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         B.pair_cap = cap == 0 ? (unsigned long long)(sc.pairs.bytes / 4 - 4) : cap;
         B.pairs = sc.pairs.as<uint32_t>();
         PhaseTimer t5(s, st, GS_PHASE_SCATTER, timers);
-        CK(launch_scatter(B, ebd - ea, wt.max_words, wt.max_T, st), "scatter");
+        CK(launch_scatter(B, ebd - ea, wt.max_words, wt.max_T, wt.max_hist, st), "scatter");
         t5.done(1);
         ++*launches;
         CompParams C{};
@@ -1003,6 +1004,7 @@ gs_status plan_tables(gs_plan p, const std::vector<EnvSpec>& specs) {
         w.xf_items = wt.xf_items;
         w.max_words = wt.max_words;
         w.max_T = wt.max_T;
+        w.max_hist = wt.max_hist;
         w.recs = wt.recs;
         w.words = wt.words;
         w.tiles = wt.tiles;
@@ -1014,7 +1016,7 @@ gs_status plan_tables(gs_plan p, const std::vector<EnvSpec>& specs) {
 WaveTables plan_wave_tables(gs_plan p, size_t i, std::vector<EnvInfo>& host) {
     auto& w = p->waves[i];
     return WaveTables{w.envs.as<EnvInfo>(), w.blocks.as<ProjBlock>(), w.cams.as<gs_camera>(), w.e1 - w.e0,
-                      w.n_blocks, w.xf_items, w.max_words, w.max_T, w.recs, w.words, w.tiles, host.data()};
+                      w.n_blocks, w.xf_items, w.max_words, w.max_T, w.max_hist, w.recs, w.words, w.tiles, host.data()};
 }
 
 // Eager pass over all waves (host syncs); records each wave's key total.

@@ -66,15 +66,67 @@ __device__ __forceinline__ void for_span(uint32_t rx, uint32_t ry, int sx, int s
     }
 }
 
+// A block's tile histogram of the boxes on a grid of ntx x nty tiles, in hist
+// with a row pitch of ntx + 1.  DIFF: each box adds to the corners of a 2D
+// difference array (ntx + 1) x (nty + 1), which block_sum2d then sums, so a box
+// costs four atomics whatever its span: at 640x480 spans average 11 tiles and
+// reach all 1200, and one lane walking a long span held its whole block up.
+// On small grids (spans of one or two tiles) the walk is cheaper.
+template <bool WRAP, bool DIFF>
+__device__ __forceinline__ void add_box(uint32_t rx, uint32_t ry, int sx, int sy, int ntx, uint32_t* hist) {
+    if constexpr (!DIFF) {
+        for_span<WRAP>(rx, ry, sx, sy, ntx, [&](int, int tx, int ty) { atomicAdd(&hist[ty * (ntx + 1) + tx], 1u); });
+    } else {
+        static_assert(!WRAP, "wrapped boxes walk their spans");
+        int tx0, tx1, ty0, ty1;
+        tile_span(rx, ry, sx, sy, tx0, tx1, ty0, ty1);
+        uint32_t* top = hist + ty0 * (ntx + 1);
+        uint32_t* end = hist + (ty1 + 1) * (ntx + 1);
+        atomicAdd(top + tx0, 1u);
+        atomicAdd(top + tx1 + 1, ~0u);
+        atomicAdd(end + tx0, ~0u);
+        atomicAdd(end + tx1 + 1, 1u);
+    }
+}
+
+// Sums a difference array along rows, then columns (block-wide).
+__device__ __forceinline__ void block_sum2d(uint32_t* hist, int ntx, int nty) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __syncthreads();
+    for (int y = warp; y < nty; y += nw) {  // a warp per row
+        uint32_t* row = hist + y * (ntx + 1);
+        uint32_t carry = 0;
+        for (int x0 = 0; x0 < ntx; x0 += 32) {
+            uint32_t v = x0 + lane < ntx ? row[x0 + lane] : 0u;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, v, d);
+                if (lane >= d) v += o;
+            }
+            v += carry;
+            if (x0 + lane < ntx) row[x0 + lane] = v;
+            carry = __shfl_sync(0xffffffffu, v, 31);
+        }
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < ntx; x += blockDim.x) {
+        uint32_t run = 0;
+        for (int y = 0; y < nty; ++y) hist[y * (ntx + 1) + x] = run += hist[y * (ntx + 1) + x];
+    }
+    __syncthreads();
+}
+
+// Words of a block's tile histogram.
+__host__ __device__ __forceinline__ int hist_words(int ntx, int nty) { return (ntx + 1) * (nty + 1); }
+
 // grid: (blocks over the largest env's visibility words, envs); block 256;
-// dynamic smem: the env's splitters, depth cells and range counters, then max T
-// tile counters.  Blocks past their env's words exit at once.  Counts the
-// visible records of a block (block_visible's list; neighbouring threads take
-// neighbouring records) per tile and per depth range of the env, and notes each
-// record's range and place among the block's records of that range, so that
-// the placement (gs_rank.cu) neither searches nor counts again (both in the
-// placement: 1.12 ms instead of ... on 512 environments at 128x128).
-template <bool WRAP>
+// dynamic smem: the env's splitters, depth cells and range counters, then the
+// largest tile histogram.  Blocks past their env's words exit at once.  Counts
+// the visible records of a block (block_visible's list; neighbouring threads
+// take neighbouring records) per tile and per depth range of the env, and notes
+// each record's range and place among the block's records of that range, so
+// that the placement (gs_rank.cu) neither searches nor counts again.
+template <bool WRAP, bool DIFF>
 __global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
     extern __shared__ __align__(16) unsigned char csm[];
     __shared__ uint16_t lst[32 * kWordsPerBlock];
@@ -86,10 +138,11 @@ __global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
     const int el = P.e_begin + blockIdx.y;
     const EnvInfo E = P.envs[el];
     const int64_t words = (E.n_local + 31) / 32;
-    const int64_t w0 = (int64_t)blockIdx.x * P.words_per_block;
+    const int64_t w0 = (int64_t)blockIdx.x * R.words_per_block;
     if (w0 >= words) return;
-    const int64_t w1 = min(w0 + (int64_t)P.words_per_block, words);
-    for (int t = threadIdx.x; t < E.T; t += blockDim.x) hist[t] = 0;
+    const int64_t w1 = min(w0 + (int64_t)R.words_per_block, words);
+    const int ntx = E.ntx, nty = E.T / ntx;
+    for (int t = threadIdx.x; t < hist_words(ntx, nty); t += blockDim.x) hist[t] = 0;
     for (int b = threadIdx.x; b < R.bins; b += blockDim.x) {
         zhist[b] = 0u;
         split[b] = R.split[(size_t)el * R.bins + b];
@@ -106,12 +159,13 @@ __global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
         const uint4 q = r3[j];
         const uint32_t b = (uint32_t)rank_bin(split, cell, R.cells, R.bins, z0, zshift, rank_key(R, q, j));
         R.rank[E.rec_base + j] = b << 13 | atomicAdd(&zhist[b], 1u);
-        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t, int, int) { atomicAdd(&hist[t], 1u); });
+        add_box<WRAP, DIFF>(q.x, q.y, sx, sy, ntx, hist);
     }
-    __syncthreads();
+    if constexpr (DIFF) block_sum2d(hist, ntx, nty);
+    else __syncthreads();
     uint32_t* cnt = P.counts + E.tile_base;
     for (int t = threadIdx.x; t < E.T; t += blockDim.x) {
-        const uint32_t h = hist[t];
+        const uint32_t h = hist[t + t / ntx];
         if (h) atomicAdd(cnt + t, h);
     }
     uint32_t* zc = R.bin_cnt + (size_t)el * R.bins;
@@ -123,23 +177,25 @@ __global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
 }
 
 static cudaError_t opt_in_smem(const void* fn, size_t smem) {
-    if (smem <= 31 * 1024) return cudaSuccess;  // plus 16.1 KB of static shared memory
+    if (smem <= 30 * 1024) return cudaSuccess;  // plus at most 17.2 KB of static shared memory
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 static_assert(kWordsPerBlock <= 256, "binning blocks: one visibility word per thread of 256, places below 2^13");
 
-cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, int max_words, int max_T,
+cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, int max_T, int max_hist,
                          cudaStream_t st) {
-    if (n_envs == 0 || max_words == 0) return cudaSuccess;
-    const size_t smem = (size_t)R.bins * 12 + (size_t)R.cells * 2 + (size_t)max_T * 4;
-    const void* fn = P.wrap ? (const void*)k_count<true> : (const void*)k_count<false>;
-    cudaError_t e = opt_in_smem(fn, smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((max_words + P.words_per_block - 1) / P.words_per_block), (unsigned)n_envs);
-    if (P.wrap) k_count<true><<<grid, 256, smem, st>>>(P, R);
-    else k_count<false><<<grid, 256, smem, st>>>(P, R);
-    return cudaGetLastError();
+    if (n_envs == 0 || R.blocks == 0) return cudaSuccess;
+    const bool diff = !P.wrap && max_T >= kDiffTiles;
+    const size_t smem = (size_t)R.bins * 12 + (size_t)R.cells * 2 + (size_t)max_hist * 4;
+    auto launch = [&](auto fn) -> cudaError_t {
+        const cudaError_t e = opt_in_smem((const void*)fn, smem);
+        if (e != cudaSuccess) return e;
+        fn<<<dim3((unsigned)R.blocks, (unsigned)n_envs), 256, smem, st>>>(P, R);
+        return cudaGetLastError();
+    };
+    if (P.wrap) return launch(k_count<true, false>);
+    return diff ? launch(k_count<false, true>) : launch(k_count<false, false>);
 }
 
 // ---------------------------------------------------------------- scan
@@ -330,75 +386,103 @@ __device__ __forceinline__ uint32_t subtile_mask(uint32_t rx, uint32_t ry, int t
     return (y0 <= 2 * ty ? xm : 0u) | (y1 > 2 * ty ? xm << (1 << lx) : 0u);
 }
 
-template <bool WRAP, bool MASK>
+constexpr int kLongSpan = 64;   // tiles: longer spans are walked by a warp
+constexpr int kLongList = 512;  // of them listed at a time
+
+template <bool WRAP, bool MASK, bool DIFF>
 __global__ void __launch_bounds__(256, 6) k_scatter(BinParams P) {  // <= 42 registers: 6 CTAs/SM
-    extern __shared__ uint32_t sm[];
+    extern __shared__ uint32_t cur[];  // the block's histogram, then its next position per tile
     __shared__ uint16_t lst[32 * kWordsPerBlock];
+    __shared__ uint16_t far[DIFF ? kLongList : 1];
     __shared__ uint32_t wtot[32];
+    __shared__ uint32_t n_far;
     const int el = P.e_begin + blockIdx.y;
     const EnvInfo E = P.envs[el];
     const int64_t words = (E.n_local + 31) / 32;
     const int64_t w0 = (int64_t)blockIdx.x * P.words_per_block;
     if (w0 >= words) return;
     const int64_t w1 = min(w0 + (int64_t)P.words_per_block, words);
-    uint32_t* hist = sm;
-    uint32_t* base = sm + E.T;
-    for (int t = threadIdx.x; t < E.T; t += blockDim.x) hist[t] = 0;
+    const int ntx = E.ntx, nty = E.T / ntx;
+    for (int t = threadIdx.x; t < hist_words(ntx, nty); t += blockDim.x) cur[t] = 0;
+    if (threadIdx.x == 0) n_far = 0u;
     const int nvis = block_visible(P.mask + E.mask_base, w0, w1, lst, wtot);
     const uint4* r3 = P.r3 + E.rec_base + w0 * 32;
     const uint32_t* rank = P.rank + E.rec_base + w0 * 32;
     const int sx = __ffs(P.tile_w) - 1, sy = __ffs(P.tile_h) - 1;
     for (int i = threadIdx.x; i < nvis; i += blockDim.x) {
         const uint4 q = r3[lst[i]];
-        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t, int, int) { atomicAdd(&hist[t], 1u); });
+        add_box<WRAP, DIFF>(q.x, q.y, sx, sy, ntx, cur);
     }
-    __syncthreads();
-    uint32_t* cur = P.cursor + E.tile_base;
+    if constexpr (DIFF) block_sum2d(cur, ntx, nty);
+    else __syncthreads();
     const uint32_t* off = P.off_local + E.tile_base;
-    const unsigned long long eb = P.env_base[el] - P.pair_base;
     for (int t = threadIdx.x; t < E.T; t += blockDim.x) {
-        const uint32_t h = hist[t];
-        if (h) base[t] = off[t] + atomicAdd(cur + t, h);
-        hist[t] = 0;
+        uint32_t& c = cur[t + t / ntx];
+        if (c) c = off[t] + atomicAdd(P.cursor + E.tile_base + t, c);
     }
     __syncthreads();
+    const unsigned long long eb = P.env_base[el] - P.pair_base;
     bool dropped = false;
-    for (int i = threadIdx.x; i < nvis; i += blockDim.x) {
-        const uint4 q = r3[lst[i]];
-        const uint32_t key = rank[lst[i]];
-        for_span<WRAP>(q.x, q.y, sx, sy, E.ntx, [&](int t, int tx, int ty) {
-            const uint32_t k = atomicAdd(&hist[t], 1u);
-            const unsigned long long pos = eb + base[t] + k;
-            const uint32_t v =
-                MASK ? key << P.key_shift | subtile_mask<WRAP>(q.x, q.y, tx, ty, sx - 3, sy - 3) : key;
-            if (pos < P.pair_cap) P.pairs[pos] = v;
-            else dropped = true;
-        });
+    auto put = [&](const uint4& q, uint32_t key, int tx, int ty) {
+        const unsigned long long pos = eb + atomicAdd(&cur[ty * (ntx + 1) + tx], 1u);
+        const uint32_t v = MASK ? key << P.key_shift | subtile_mask<WRAP>(q.x, q.y, tx, ty, sx - 3, sy - 3) : key;
+        if (pos < P.pair_cap) P.pairs[pos] = v;
+        else dropped = true;
+    };
+    // uniform trip count: the block drains its list of long spans together
+    for (int i0 = 0; i0 < nvis; i0 += blockDim.x) {
+        const int i = i0 + threadIdx.x;
+        if (i < nvis) {
+            const uint4 q = r3[lst[i]];
+            bool walk = true;
+            if constexpr (DIFF) {
+                int tx0, tx1, ty0, ty1;
+                tile_span(q.x, q.y, sx, sy, tx0, tx1, ty0, ty1);
+                if ((tx1 - tx0 + 1) * (ty1 - ty0 + 1) > kLongSpan) {
+                    far[atomicAdd(&n_far, 1u)] = (uint16_t)i;  // at most blockDim.x more per round
+                    walk = false;
+                }
+            }
+            if (walk) {
+                const uint32_t key = rank[lst[i]];
+                for_span<WRAP>(q.x, q.y, sx, sy, ntx, [&](int, int tx, int ty) { put(q, key, tx, ty); });
+            }
+        }
+        if constexpr (DIFF) {
+            __syncthreads();
+            const uint32_t nf = n_far;
+            if (nf + blockDim.x > (uint32_t)kLongList || (i0 + (int)blockDim.x >= nvis && nf)) {
+                for (uint32_t k = threadIdx.x >> 5; k < nf; k += blockDim.x >> 5) {
+                    const uint4 q = r3[lst[far[k]]];
+                    const uint32_t key = rank[lst[far[k]]];
+                    int tx0, tx1, ty0, ty1;
+                    tile_span(q.x, q.y, sx, sy, tx0, tx1, ty0, ty1);
+                    const int nx = tx1 - tx0 + 1, n = nx * (ty1 - ty0 + 1);
+                    for (int t = threadIdx.x & 31; t < n; t += 32) put(q, key, tx0 + t % nx, ty0 + t / nx);
+                }
+                __syncthreads();
+                if (threadIdx.x == 0) n_far = 0u;
+                __syncthreads();
+            }
+        }
     }
     if (__syncthreads_or(dropped) && threadIdx.x == 0) atomicOr(P.status, kStOverflow);
 }
 
-cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int max_T, cudaStream_t st) {
+cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int max_T, int max_hist, cudaStream_t st) {
     if (n_envs == 0 || max_words == 0) return cudaSuccess;
-    size_t smem = (size_t)max_T * 8;
-    // Large images (at least half a 640x480 frame per env): at most 4 CTAs per
-    // SM, by padding the shared memory (29 KB dynamic + 16 KB static + the
-    // per-CTA reserve: 5 no longer fit).  Measured on the 2048-env room
-    // workload at 640x480: 6 CTAs/SM (what 40 registers allow) 20.7 ms, 5: 19.9,
-    // 4: 18.7, 3: 18.6 ms per step; at 320x240 and 128x128 six are fastest
-    // (6.8 vs 8.0 ms and 5.1 vs 6.2 ms with 4).
-    if ((long long)max_T * P.tile_w * P.tile_h >= 640ll * 480 / 2 && smem < (size_t)29 * 1024) smem = 29 * 1024;
-    const bool mask = P.key_shift > 0;
-    const void* fn = P.wrap ? (mask ? (const void*)k_scatter<true, true> : (const void*)k_scatter<true, false>)
-                            : (mask ? (const void*)k_scatter<false, true> : (const void*)k_scatter<false, false>);
-    cudaError_t e = opt_in_smem(fn, smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((max_words + P.words_per_block - 1) / P.words_per_block), (unsigned)n_envs);
-    if (P.wrap && mask) k_scatter<true, true><<<grid, 256, smem, st>>>(P);
-    else if (P.wrap) k_scatter<true, false><<<grid, 256, smem, st>>>(P);
-    else if (mask) k_scatter<false, true><<<grid, 256, smem, st>>>(P);
-    else k_scatter<false, false><<<grid, 256, smem, st>>>(P);
-    return cudaGetLastError();
+    const bool diff = !P.wrap && max_T >= kDiffTiles, mask = P.key_shift > 0;
+    const size_t smem = (size_t)max_hist * 4;
+    auto launch = [&](auto fn) -> cudaError_t {
+        const cudaError_t e = opt_in_smem((const void*)fn, smem);
+        if (e != cudaSuccess) return e;
+        fn<<<dim3((unsigned)((max_words + P.words_per_block - 1) / P.words_per_block), (unsigned)n_envs), 256, smem,
+             st>>>(P);
+        return cudaGetLastError();
+    };
+    if (P.wrap) return mask ? launch(k_scatter<true, true, false>) : launch(k_scatter<true, false, false>);
+    if (diff) return mask ? launch(k_scatter<false, true, true>) : launch(k_scatter<false, false, true>);
+    return mask ? launch(k_scatter<false, true, false>) : launch(k_scatter<false, false, false>);
 }
 
 }  // namespace gsb

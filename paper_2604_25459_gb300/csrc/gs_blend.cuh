@@ -12,6 +12,12 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
+// A 16-byte copy from global to shared memory that the thread waits for later.
+__device__ __forceinline__ void copy16(float4* dst, const float4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
 // One pixel's blend step for a splat whose alpha is `al` (already >= 1/255);
 // returns the weight w = alpha T added (0 when the step stops instead):
 // T' = T (1 - alpha), evaluated as T - w; stop (splat not added) when

@@ -28,7 +28,7 @@
 
 namespace gsb {
 
-constexpr int kInsertMax = 32;   // longest of them sorted by insertion
+constexpr int kInsertMax = 32;   // longest rank range sorted by counting
 constexpr int kGroupWords = 16;  // bitmap words per group (512 ranks)
 
 // f(L[i]) for every i in [0, len), spread over the block: 16-byte loads of the
@@ -59,15 +59,15 @@ __device__ __forceinline__ void for_ranks(const uint32_t* L, uint32_t len, F&& f
     if (tid < len - done) f(L[done + tid]);
 }
 
-// Sorts keys[0, n), distinct ranks in [lo, hi], into tmp and returns true: a
-// counting sort by kSortBins equal ranges, then an insertion sort of each
-// range.  Returns false, with keys untouched, when a range holds more than
+// Sorts keys[0, n), distinct ranks in [lo, hi] (tmp: scratch), and returns
+// true: a counting sort by SB equal ranges, a rank's place in its range being
+// the number of smaller ranks there.  Returns false, with keys untouched, when a range holds more than
 // kInsertMax ranks.  c32 (kSortBins words) holds zeros on entry unless `dirty`
 // is set (it is cleared here then); a successful sort leaves it zeroed again
 // (each thread clears its own ranges after the last barrier; the next reader
 // comes after the caller's next barriers).  red: 32 words.
 template <int NT, int SB>
-__device__ bool rank_sort(const uint32_t* keys, uint32_t* tmp, uint32_t* c32, uint32_t* red, int n, uint32_t lo,
+__device__ bool rank_sort(uint32_t* keys, uint32_t* tmp, uint32_t* c32, uint32_t* red, int n, uint32_t lo,
                           uint32_t hi, bool& dirty) {
     constexpr int PER = SB / NT;
     static_assert(SB % NT == 0, "ranges per thread");
@@ -127,23 +127,12 @@ __device__ bool rank_sort(const uint32_t* keys, uint32_t* tmp, uint32_t* c32, ui
         tmp[atomicAdd(&c32[(k - lo) >> shift], 1u)] = k;
     }
     __syncthreads();
-    // range b is now [c32[b-1], c32[b]) (c32 holds each range's end); the
-    // ranges are interleaved over the threads, so a cluster of crowded
-    // neighbouring ranges spreads over many threads instead of the few that
-    // hold them in the blocked layout
-#pragma unroll 1
-    for (int b = tid; b < SB; b += NT) {
-        const int e = (int)c32[b];
-        const int a = b ? (int)c32[b - 1] : 0;
-        for (int x = a + 1; x < e; ++x) {
-            const uint32_t k = tmp[x];
-            int y = x - 1;
-            while (y >= a && tmp[y] > k) {
-                tmp[y + 1] = tmp[y];
-                --y;
-            }
-            tmp[y + 1] = k;
-        }
+    for (int i = tid; i < n; i += NT) {  // c32[b] is the end of range b now
+        const uint32_t k = tmp[i];
+        const uint32_t b = (k - lo) >> shift, e = c32[b];
+        uint32_t place = b ? c32[b - 1] : 0u;
+        for (uint32_t x = place; x < e; ++x) place += tmp[x] < k ? 1u : 0u;
+        keys[place] = k;
     }
     __syncthreads();
 #pragma unroll
@@ -174,13 +163,14 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
     constexpr int NB = NT;  // splats staged per batch (one per thread)
     constexpr int CAP = NT == 32 ? 512 : kCompCap;
     constexpr int SB = NT == 32 ? 512 : 1024;      // rank ranges of the short-bucket sort
-    constexpr int NG = NT == 64 ? 64 : NT;         // bitmap groups
+    constexpr int NG = NT > 128 ? 128 : NT;        // bitmap groups
     constexpr int BMW = NG * kGroupWords;          // bitmap words (32 ranks each)
     constexpr int UB = CAP * 4 > NB * 64 ? CAP * 4 : NB * 64;
     constexpr int NW = NT / 32;
     static_assert(BMW >= SB, "the short-bucket counters share the bitmap's memory");
     static_assert(CAP >= kGroupWords * 32, "a group's ranks fit a window");
-    __shared__ uint32_t keys[CAP];                      // the window: ranks, then record slots
+    __shared__ uint32_t keys[CAP];                      // the window's ranks
+    __shared__ float4 raw[3][NB];                       // records of the next batch, in flight
     __shared__ __align__(16) unsigned char ubuf[UB];    // sort scratch | staged records
     __shared__ __align__(16) uint32_t bm[BMW];          // bitmap | counters of the short-bucket sort
     __shared__ uint32_t pre[NG + 1];                    // ranks set before each group of the bitmap
@@ -250,18 +240,31 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
         return g_link0 + (long long)(j - P.nbp);
     };
     bool finished = false;
-    // Composite the window keys[0, wn) (record slots in depth order).  Sets
+    // Composite the window keys[0, wn) (ranks in depth order).  Sets
     // `finished` once every pixel of the tile has terminated.
     auto run_window = [&](uint32_t wn) {
+        // The records of a batch are copied (cp.async) while the batch before it
+        // is blended; a thread stages the splat it copied itself, so the copies
+        // need no barrier of their own.
+        auto slot_of = [&](uint32_t i) -> uint32_t { return i < wn ? __ldg(order + keys[i]) : 0xffffffffu; };
+        auto fetch = [&](uint32_t g) {
+            if (g < n_local) {
+                const float4* src = P.r0 + (size_t)kRecStride * (recbase + g);
+                copy16(&raw[0][tid], src);
+                copy16(&raw[1][tid], src + 1);
+                copy16(&raw[2][tid], src + 2);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        uint32_t g = slot_of(tid), g_next = slot_of(NB + tid);
+        fetch(g);
         for (uint32_t b = 0; b < wn; b += NB) {
             const int cnt_b = (int)min((uint32_t)NB, wn - b);
-            for (int s = tid; s < cnt_b; s += NT) {
-                const uint32_t g = keys[b + s];
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            if (tid < cnt_b) {
+                const int s = tid;
                 if (g < n_local) {
-                    const size_t ri = recbase + g;
-                    const float4 q0 = P.r0[kRecStride * ri];
-                    const float4 q1 = P.r1[kRecStride * ri];
-                    const float4 q2 = P.r2[kRecStride * ri];
+                    const float4 q0 = raw[0][tid], q1 = raw[1][tid], q2 = raw[2][tid];
                     const uint32_t rx = __float_as_uint(q1.w), ry = __float_as_uint(q2.w);
                     sA[s] = make_float4(q0.x, q0.y, log2f(q0.z), q0.w);
                     // alpha >= 1/255 iff q <= w (w only feeds the subtile cull, whose
@@ -279,6 +282,11 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                     sR[s] = make_int4(1 << 20, -1, 1 << 20, -1);
                     atomicOr(P.status, kStOverflow);
                 }
+            }
+            g = g_next;
+            if (b + NB < wn) {
+                fetch(g);
+                g_next = slot_of(b + 2 * NB + tid);
             }
             __syncthreads();
             if (!__all_sync(0xffffffffu, done0 && done1)) {
@@ -383,19 +391,19 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
             const bool all = __syncthreads_and(done0 && done1) != 0;
             if (all) {
                 finished = true;
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
                 break;
             }
         }
     };
 
-    // The next window: its wn ranks in depth order in src (keys or tmp).
+    // The next window: its wn ranks in depth order in keys.
     uint32_t before = 0;          // ranks of the bucket in earlier windows
     bool whole = n <= (uint32_t)CAP;  // the bucket is one window, sorted at once
     bool loaded = false;          // a bitmap of the ranks [r0, r0 + 32 BMW) is set up
     uint32_t r0 = 0;
     int g0 = 0;                   // its next group
     while (before < n && !finished) {
-        const uint32_t* src = keys;
         uint32_t wn = 0;
         if (whole) {
             uint32_t lo = 0xffffffffu, hi = 0u;
@@ -409,7 +417,6 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
             whole = rank_sort<NT, SB>(keys, tmp, bm, red, (int)n, lo, hi, c32_dirty);
             if (!whole) continue;  // crowded ranks: through bitmaps
             wn = n;
-            src = tmp;
         } else {
             if (loaded && g0 >= NG) {
                 loaded = false;
@@ -430,12 +437,13 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                 });
                 __syncthreads();
                 // ranks set before each group: thread t counts groups GPT t ..
-                constexpr int GPT = NG / NT;
+                constexpr int GPT = NG < NT ? 1 : NG / NT;
                 uint32_t c[GPT], sum = 0;
 #pragma unroll
                 for (int j = 0; j < GPT; ++j) {
                     const int g = tid * GPT + j;
                     c[j] = 0;
+                    if (g >= NG) continue;
 #pragma unroll
                     for (int i = 0; i < kGroupWords; ++i)  // rotated: neighbouring threads hit different banks
                         c[j] += __popc(bm[g * kGroupWords + ((i + tid) & (kGroupWords - 1))]);
@@ -444,10 +452,10 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                 uint32_t run = block_excl_scan_u32<NT>(sum, red);
 #pragma unroll
                 for (int j = 0; j < GPT; ++j) {
-                    pre[tid * GPT + j] = run;
+                    if (tid * GPT + j <= NG) pre[tid * GPT + j] = run;
                     run += c[j];
                 }
-                if (tid == NT - 1) pre[NG] = run;
+                if (NG >= NT && tid == NT - 1) pre[NG] = run;
                 __syncthreads();
                 loaded = true;
                 g0 = 0;
@@ -487,8 +495,6 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
             g0 = g1;
             if (wn == 0) continue;
         }
-        for (uint32_t i = tid; i < wn; i += NT) keys[i] = __ldg(order + src[i]);  // record slots
-        __syncthreads();
         run_window(wn);
         before += wn;
     }

@@ -167,11 +167,6 @@ __device__ __forceinline__ void warp_sort(uint32_t* keys, uint32_t* tmp, uint32_
     __syncwarp();
 }
 
-__device__ __forceinline__ void copy16(float4* dst, const float4* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
 }  // namespace
 
 // MODE 0: camera image or observation; 2: the same, also counting composited

@@ -155,7 +155,7 @@ struct WaveTables {       // device copies of one wave's tables
     const EnvInfo* envs;
     const ProjBlock* blocks;
     const gs_camera* cams;
-    int We, n_blocks, xf_items, max_words, max_T;
+    int We, n_blocks, xf_items, max_words, max_T, max_hist;
     unsigned long long recs, words, tiles;
     const EnvInfo* host_envs;  // We + 1 host entries
 };

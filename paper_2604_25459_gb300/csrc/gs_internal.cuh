@@ -187,7 +187,7 @@ struct BinParams {
     const uint4* r3;
     int e_begin;             // first env (wave-local) handled by this launch
     int tile_w, tile_h;
-    int words_per_block;
+    int words_per_block;     // of the scatter (the count shares the ranking's blocks)
     uint32_t* counts;
     const uint32_t* off_local;
     const unsigned long long* env_base;
@@ -281,9 +281,10 @@ cudaError_t launch_ray_count(const float* dirs, const gs_lidar* lidars, const En
 cudaError_t launch_ray_scatter(const EnvInfo* envs, int We, int n_rays, const uint32_t* cell, const uint32_t* off,
                                uint32_t* cur, uint32_t* list, const uint32_t* cnt, uint32_t* item_cnt,
                                unsigned int tiles, cudaStream_t st);
-// grid.x covers the largest env's mask words; max_T sizes the shared histogram.
-// The count also histograms the records over the env's depth ranges (R).
-cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, int max_words, int max_T,
+// max_T, max_hist: tiles and padded tile histogram ((ntx + 1) (nty + 1)) of the
+// largest env.  The count also histograms the records over the env's depth
+// ranges (R).
+cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, int max_T, int max_hist,
                          cudaStream_t st);
 // per: counters per tile (counts and off_local hold per T from per tile_base).
 cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
@@ -293,7 +294,7 @@ cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* o
 cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                               unsigned long long* env_total, unsigned long long* env_base, int We,
                               const RankParams& R, cudaStream_t st);
-cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int max_T, cudaStream_t st);
+cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int max_T, int max_hist, cudaStream_t st);
 // Lists a launch's items by the length of their buckets, longest class first
 // (CompParams::items); class_cnt is zeroed by the caller.  Rays: item_cnt and
 // item_off per (env, tile) and item_base per env give a tile's items.
@@ -336,6 +337,21 @@ inline RankParams rank_sizes(long long max_words, int We, bool lidar) {
     R.words_per_block = w;
     R.blocks = (int)((max_words + w - 1) / w);
     return R;
+}
+// Tile grids of at least this many tiles are counted by difference arrays
+// (average spans at 128x128, 64 tiles, are 2.1 tiles; at 320x240, 300: 4.5; at
+// 640x480: 11).
+constexpr int kDiffTiles = 256;
+// Visibility words per scatter block: many blocks per SM, as one block may hold
+// a link that fills the image (at 640x480, 32 envs: 30 us per env with 256
+// words, 13 with 32), and on large grids 64, whose writes stay in reach of the
+// L2 (256 envs: 8.5 us per env with 256, 7.15 with 64, 8.6 with 32); on small
+// grids the per-block tables weigh more (512 envs at 128x128: 2.3 us with 256,
+// 2.7 with 64).
+inline int scatter_words(long long max_words, int n_envs, int max_T) {
+    int w = max_T >= kDiffTiles ? 64 : kWordsPerBlock;
+    while (w > 16 && (max_words + w - 1) / w * n_envs < 62 * 152) w /= 2;
+    return w;
 }
 // Bytes of the ranking's per-env tables (everything but bin_cnt, zkeys, order
 // and rank) for We envs, and their layout from a 16-byte aligned base.

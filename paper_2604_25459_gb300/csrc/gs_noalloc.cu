@@ -261,7 +261,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.e_begin = 0;
         B.tile_w = tw;
         B.tile_h = th;
-        B.words_per_block = R.words_per_block;
+        B.words_per_block = scatter_words(max_words, Wn, max_T);
         B.rank = R.rank;
         B.counts = counts;
         B.off_local = off;
@@ -269,7 +269,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.cursor = cursor;
         B.status = v.status;
         NA_CK(launch_rank_sample(R, Wn, st), "depth sample");
-        NA_CK(launch_count(B, R, Wn, max_words, max_T, st), "count");
+        NA_CK(launch_count(B, R, Wn, max_T, (ntx + 1) * (nty + 1), st), "count");
         NA_CK(launch_scan_ranks(d_envs, counts, off, env_total, env_base, Wn, R, st), "scan");
         NA_CK(launch_rank(R, Wn, max_words, st), "depth ranks");
         unsigned long long eb[kMaxWave + 1];
@@ -286,7 +286,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.pair_base = 0;
         B.pair_cap = (kNoAllocBytes - y.pairs) / 8;
         B.pairs = reinterpret_cast<uint32_t*>(base + y.pairs);
-        NA_CK(launch_scatter(B, Wn, max_words, max_T, st), "scatter");
+        NA_CK(launch_scatter(B, Wn, max_words, max_T, (ntx + 1) * (nty + 1), st), "scatter");
         CompParams C{};
         C.envs = d_envs;
         C.e_begin = 0;
