@@ -300,88 +300,97 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                     bool ov = j < cnt_b && R.x <= wx1 && R.x + R.y >= wx0 && R.z <= wy1 && R.z + R.w >= wy0;
                     const bool rr = reaches_rect(sA[jj], sB[jj], (float)wx0 + 0.5f, (float)wy0 + 0.5f);
                     ov = ov && (R.y + R.w < 24 || rr);
-                    uint32_t m = __ballot_sync(0xffffffffu, ov);
-                    float2 score_pair = make_float2(0.0f, 0.0f);  // contribution pass only
+                    const uint32_t m = __ballot_sync(0xffffffffu, ov);
                     // Splats of opacity <= 0.98 never reach the 0.99 cap of alpha (o 2^-q
                     // with q >= 0), so a chunk without brighter splats walks a copy of the
                     // loop without the cap.
                     const bool clamp_chunk =  // staged log2(o) > log2(0.98)
                         __any_sync(0xffffffffu, j < cnt_b && sA[j].z > -0.029146346f);
-                    auto walk = [&](auto clamp_tag) {
-                    constexpr bool CL = decltype(clamp_tag)::value;
-                    // two splats per iteration: their four alpha evaluations are
-                    // independent; the blends then run in depth order
-                    while (m != 0u) {
-                        const int k1 = __ffs(m) - 1;
-                        m &= m - 1u;
-                        const bool two = m != 0u;
-                        const int k2 = two ? __ffs(m) - 1 : k1;
-                        if (two) m &= m - 1u;
-                        const int j1 = c + k1, j2 = c + k2;
-                        // No per-pixel box test: a pixel outside a splat's support box has
-                        // q > q* (1 + 2e-4), so its alpha falls below 1/255 and the alpha
-                        // test alone rejects it.
-                        const bool h10 = !done0, h11 = !done1, h20 = two && !done0, h21 = two && !done1;
-                        {
-                            const float4 A1 = sA[j1], B1 = sB[j1];
-                            const float4 A2 = sA[j2], B2 = sB[j2];
-                            const float2 a1 = splat_alpha2<CL>(A1, B1, fpx, fpy);
-                            const float2 a2 = splat_alpha2<CL>(A2, B2, fpx, fpy);
-                            const bool u10 = h10 && a1.x >= (1.0f / 255.0f);
-                            const bool u11 = h11 && a1.y >= (1.0f / 255.0f);
-                            float w1 = 0.0f, w2 = 0.0f;
-                            // Both splats' blends with plain selects while no pixel of the
-                            // warp stops at either (the common case); else one splat at a
-                            // time with the stop rule.  Either way the arithmetic is that
-                            // of blend2, so the images do not depend on the path taken.
-                            // Every lane of the warp reaches the vote: the camera path has
-                            // no divergent branch around it (branches here measured slower
-                            // than evaluating every lane's pixels).
-                            const float2 am1 = make_float2(u10 ? a1.x : 0.0f, u11 ? a1.y : 0.0f);
-                            const float2 x1 = __fmul2_rn(am1, Tp);
-                            const float2 Tn1 = __fadd2_rn(Tp, make_float2(-x1.x, -x1.y));
-                            const bool v20 = h20 && a2.x >= (1.0f / 255.0f);
-                            const bool v21 = h21 && a2.y >= (1.0f / 255.0f);
+                    // One step blends two splats (TWO): their four alpha evaluations are
+                    // independent, the blends run in depth order; an odd last splat has a
+                    // step of its own.  No per-pixel box test: a pixel outside a splat's
+                    // support box has q > q* (1 + 2e-4), so its alpha falls below 1/255
+                    // and the alpha test alone rejects it.
+                    auto step = [&](auto clamp_tag, auto two_tag, int j1, int j2) {
+                        constexpr bool CL = decltype(clamp_tag)::value, TWO = decltype(two_tag)::value;
+                        const float4 A1 = sA[j1], B1 = sB[j1];
+                        const float4 A2 = sA[j2], B2 = sB[j2];
+                        const float2 a1 = splat_alpha2<CL>(A1, B1, fpx, fpy);
+                        float2 a2 = make_float2(0.0f, 0.0f);
+                        if constexpr (TWO) a2 = splat_alpha2<CL>(A2, B2, fpx, fpy);
+                        const bool u10 = !done0 && a1.x >= (1.0f / 255.0f);
+                        const bool u11 = !done1 && a1.y >= (1.0f / 255.0f);
+                        float w1 = 0.0f, w2 = 0.0f;
+                        // The blends with plain selects while no pixel of the warp stops at
+                        // either splat (the common case); else one splat at a time with the
+                        // stop rule.  Either way the arithmetic is that of blend2, so the
+                        // images do not depend on the path taken.  Every lane of the warp
+                        // reaches the vote: the camera path has no divergent branch around
+                        // it (branches here measured slower than evaluating every lane's
+                        // pixels).
+                        const float2 am1 = make_float2(u10 ? a1.x : 0.0f, u11 ? a1.y : 0.0f);
+                        const float2 x1 = __fmul2_rn(am1, Tp);
+                        const float2 Tn1 = __fadd2_rn(Tp, make_float2(-x1.x, -x1.y));
+                        float2 x2 = make_float2(0.0f, 0.0f), Tn2 = Tn1;
+                        bool v20 = false, v21 = false;
+                        if constexpr (TWO) {
+                            v20 = !done0 && a2.x >= (1.0f / 255.0f);
+                            v21 = !done1 && a2.y >= (1.0f / 255.0f);
                             const float2 am2 = make_float2(v20 ? a2.x : 0.0f, v21 ? a2.y : 0.0f);
-                            const float2 x2 = __fmul2_rn(am2, Tn1);
-                            const float2 Tn2 = __fadd2_rn(Tn1, make_float2(-x2.x, -x2.y));
-                            // Tn2 = Tn1 - am2 Tn1 <= Tn1 (am2 >= 0, rounding is monotone),
-                            // so a pixel that stops at either splat has Tn2 < 1e-4
-                            const bool stop = Tn2.x < 1e-4f || Tn2.y < 1e-4f;
-                            if (!__any_sync(0xffffffffu, stop)) {
-                                if constexpr (CNT) ncomp += (uint32_t)u10 + (uint32_t)u11 + (uint32_t)v20 + (uint32_t)v21;
-                                const float4 C1 = sC[j1], C2 = sC[j2];
-                                rp = __ffma2_rn(x1, make_float2(C1.x, C1.x), rp);
-                                gp = __ffma2_rn(x1, make_float2(C1.y, C1.y), gp);
-                                bp = __ffma2_rn(x1, make_float2(C1.z, C1.z), bp);
-                                dp = __ffma2_rn(x1, make_float2(A1.w, A1.w), dp);
+                            x2 = __fmul2_rn(am2, Tn1);
+                            Tn2 = __fadd2_rn(Tn1, make_float2(-x2.x, -x2.y));
+                        }
+                        // Tn2 = Tn1 - am2 Tn1 <= Tn1 (am2 >= 0, rounding is monotone),
+                        // so a pixel that stops at either splat has Tn2 < 1e-4
+                        const bool stop = Tn2.x < 1e-4f || Tn2.y < 1e-4f;
+                        if (!__any_sync(0xffffffffu, stop)) {
+                            if constexpr (CNT) ncomp += (uint32_t)u10 + (uint32_t)u11 + (uint32_t)v20 + (uint32_t)v21;
+                            const float4 C1 = sC[j1];
+                            rp = __ffma2_rn(x1, make_float2(C1.x, C1.x), rp);
+                            gp = __ffma2_rn(x1, make_float2(C1.y, C1.y), gp);
+                            bp = __ffma2_rn(x1, make_float2(C1.z, C1.z), bp);
+                            dp = __ffma2_rn(x1, make_float2(A1.w, A1.w), dp);
+                            if constexpr (TWO) {
+                                const float4 C2 = sC[j2];
                                 rp = __ffma2_rn(x2, make_float2(C2.x, C2.x), rp);
                                 gp = __ffma2_rn(x2, make_float2(C2.y, C2.y), gp);
                                 bp = __ffma2_rn(x2, make_float2(C2.z, C2.z), bp);
                                 dp = __ffma2_rn(x2, make_float2(A2.w, A2.w), dp);
-                                Tp = Tn2;
-                                w1 = x1.x + x1.y;
-                                w2 = x2.x + x2.y;
-                            } else {
-                                if constexpr (CNT) ncomp += (uint32_t)u10 + (uint32_t)u11;
-                                w1 = blend2(a1, u10, u11, sC[j1], A1.w, Tp, rp, gp, bp, dp, done0, done1);
-                                const bool u20 = h20 && !done0 && a2.x >= (1.0f / 255.0f);
-                                const bool u21 = h21 && !done1 && a2.y >= (1.0f / 255.0f);
+                            }
+                            Tp = Tn2;
+                            w1 = x1.x + x1.y;
+                            w2 = x2.x + x2.y;
+                        } else {
+                            if constexpr (CNT) ncomp += (uint32_t)u10 + (uint32_t)u11;
+                            w1 = blend2(a1, u10, u11, sC[j1], A1.w, Tp, rp, gp, bp, dp, done0, done1);
+                            if constexpr (TWO) {
+                                const bool u20 = !done0 && a2.x >= (1.0f / 255.0f);
+                                const bool u21 = !done1 && a2.y >= (1.0f / 255.0f);
                                 if constexpr (CNT) ncomp += (uint32_t)u20 + (uint32_t)u21;
                                 w2 = blend2(a2, u20, u21, sC[j2], A2.w, Tp, rp, gp, bp, dp, done0, done1);
                             }
-                            if constexpr (SC) score_pair = make_float2(w1, w2);
                         }
-                        if constexpr (SC) {  // warp-uniform: every lane reaches this point
-                            // the lanes add their weights
-                            const float s1 = warp_sum(score_pair.x), s2 = warp_sum(score_pair.y);
-                            score_pair = make_float2(0.0f, 0.0f);
+                        if constexpr (SC) {  // warp-uniform: the lanes add their weights
+                            const float s1 = warp_sum(w1), s2 = TWO ? warp_sum(w2) : 0.0f;
                             if (lane == 0) {
                                 if (s1 > 0.0f) atomicAdd(P.score + score_index(sG[j1]), s1);
-                                if (two && s2 > 0.0f) atomicAdd(P.score + score_index(sG[j2]), s2);
+                                if (TWO && s2 > 0.0f) atomicAdd(P.score + score_index(sG[j2]), s2);
                             }
                         }
-                    }
+                    };
+                    auto walk = [&](auto clamp_tag) {
+                        uint32_t r = __brev(m);  // the first splat is the leading bit
+                        while (r & (r - 1u)) {
+                            const int k1 = __clz(r);
+                            r ^= 0x80000000u >> k1;
+                            const int k2 = __clz(r);
+                            r ^= 0x80000000u >> k2;
+                            step(clamp_tag, std::true_type{}, c + k1, c + k2);
+                        }
+                        if (r) {
+                            const int k1 = __clz(r);
+                            step(clamp_tag, std::false_type{}, c + k1, c + k1);
+                        }
                     };
                     if (clamp_chunk) walk(std::true_type{});
                     else walk(std::false_type{});
