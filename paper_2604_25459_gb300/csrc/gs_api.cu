@@ -562,18 +562,18 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         const size_t nr = (size_t)We * (size_t)io.n_rays;
         CK(s->ray_cell.ensure(nr * 4), "alloc ray cells");
         CK(s->ray_list.ensure(nr * 4), "alloc ray lists");
-        for (DevBuf* b : {&s->ray_cnt, &s->ray_off, &s->ray_cur}) CK(b->ensure(wt.tiles * 16), "alloc ray tables");
+        for (DevBuf* b : {&s->ray_cnt, &s->ray_off, &s->ray_cur}) CK(b->ensure(wt.tiles * 4 * kRayGroups), "alloc ray tables");
         for (DevBuf* b : {&s->item_cnt, &s->item_off}) CK(b->ensure(wt.tiles * 4), "alloc ray tables");
         for (DevBuf* b : {&s->ray_tot, &s->item_tot}) CK(b->ensure((size_t)We * 8), "alloc ray totals");
         for (DevBuf* b : {&s->ray_base, &s->item_base}) CK(b->ensure((size_t)(We + 1) * 8), "alloc ray bases");
-        CK(cudaMemsetAsync(s->ray_cnt.p, 0, wt.tiles * 16, st), "memset ray counts");
-        CK(cudaMemsetAsync(s->ray_cur.p, 0, wt.tiles * 16, st), "memset ray cursors");
+        CK(cudaMemsetAsync(s->ray_cnt.p, 0, wt.tiles * 4 * kRayGroups, st), "memset ray counts");
+        CK(cudaMemsetAsync(s->ray_cur.p, 0, wt.tiles * 4 * kRayGroups, st), "memset ray cursors");
         PhaseTimer tr(s, st, GS_PHASE_SCAN, timers);
         CK(launch_ray_count(io.ray_dirs, io.lidars, wt.envs, We, io.n_rays, s->ray_cell.as<uint32_t>(),
                             s->ray_cnt.as<uint32_t>(), status, st),
            "ray cells");
         CK(launch_scan(wt.envs, s->ray_cnt.as<uint32_t>(), s->ray_off.as<uint32_t>(),
-                       s->ray_tot.as<unsigned long long>(), s->ray_base.as<unsigned long long>(), We, 4, st),
+                       s->ray_tot.as<unsigned long long>(), s->ray_base.as<unsigned long long>(), We, kRayGroups, st),
            "ray scan");
         CK(launch_ray_scatter(wt.envs, We, io.n_rays, s->ray_cell.as<uint32_t>(), s->ray_off.as<uint32_t>(),
                               s->ray_cur.as<uint32_t>(), s->ray_list.as<uint32_t>(), s->ray_cnt.as<uint32_t>(),
@@ -696,11 +696,10 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         C.lidars = io.lidars;
         C.r3 = P.r3;
         C.status = status;
-        if (ea > 0) CK(cudaMemsetAsync(work, 0, 4 + 4 * kItemClasses, st), "memset work counter");
-        if (use_quad || io.lidars) {  // warp form: long buckets first, unless every item starts at once
+        if (ea > 0) CK(cudaMemsetAsync(work, 0, 8 + 4 * kItemClasses, st), "memset work counter");
+        if (use_quad || io.lidars) {  // warp form: long buckets first
             const unsigned long long n_items = C.item_end - C.item_begin;
-            if (n_items * (io.ray_dirs ? 1 : n_sub) > (unsigned long long)kWarpsPerSM * 152 &&
-                n_items * kItemClasses * 4 <= (unsigned long long)s->budget / 64) {
+            if (n_items * kItemClasses * 4 <= (unsigned long long)s->budget / 64) {
                 CK(sc.items.ensure((size_t)n_items * kItemClasses * 4), "alloc item order");
                 CK(launch_item_order(wt.envs, ea, ebd - ea, wt.max_T, counts,
                                      io.ray_dirs ? s->item_cnt.as<uint32_t>() : nullptr,
@@ -711,6 +710,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
                 C.items = sc.items.as<uint32_t>();
                 C.class_cnt = work + 1;
                 C.item_pitch = (unsigned)n_items;
+                C.team_work = work + 1 + kItemClasses;
                 ++*launches;
             }
         }

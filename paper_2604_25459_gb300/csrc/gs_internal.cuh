@@ -212,6 +212,8 @@ struct CompParams {
     const uint32_t* items;
     const uint32_t* class_cnt;
     unsigned int item_pitch;
+    unsigned int* team_work;  // nullable: the teams' work counter (zeroed before the launch)
+    int team_classes;         // set by the launch: the first classes go to teams of four warps
     const float4* r0;
     const float4* r1;
     const float4* r2;
@@ -247,9 +249,9 @@ struct CompParams {
     // rays); outputs are indexed by ray, at envs[e].pix_base + ray.
     const float* ray_dirs;         // [wave env][n_rays][3], sensor frame
     const uint32_t* ray_cell;      // [wave env][n_rays]: tile << 8 | cell in tile (row-major 16x16)
-    const uint32_t* ray_list;      // [wave env][n_rays]: ray indices grouped by tile, then 8x8 subtile
-    const uint32_t* ray_cnt;       // per (env, tile, subtile) at 4 tile_base: rays in the subtile
-    const uint32_t* ray_off;       // per (env, tile, subtile): its first entry in the env's ray_list
+    const uint32_t* ray_list;      // [wave env][n_rays]: ray indices grouped by tile, then 4x4 quadrant
+    const uint32_t* ray_cnt;       // per (env, tile, quadrant) at kRayGroups tile_base: its rays
+    const uint32_t* ray_off;       // per (env, tile, quadrant): its first entry in the env's ray_list
     const uint32_t* item_off;      // per (env, tile): first item of the tile within its env
     const unsigned long long* item_base;  // per wave env (+1): first item of the env
     int n_rays;
@@ -276,6 +278,7 @@ cudaError_t launch_project_lidar(const ProjParams& P, int n_blocks, cudaStream_t
 // (chunks of at most kRayChunk rays per tile).  ray_cnt and ray_cur are zeroed
 // by the caller.
 constexpr int kRayChunk = 64;
+constexpr int kRayGroups = 16;  // 4x4 quadrants per tile, by which a tile's rays are grouped
 cudaError_t launch_ray_count(const float* dirs, const gs_lidar* lidars, const EnvInfo* envs, int We, int n_rays,
                              uint32_t* cell, uint32_t* cnt, uint32_t* status, cudaStream_t st);
 cudaError_t launch_ray_scatter(const EnvInfo* envs, int We, int n_rays, const uint32_t* cell, const uint32_t* off,
@@ -310,8 +313,6 @@ cudaError_t launch_rank(const RankParams& R, int n_envs, int max_words, cudaStre
 // form (launch_composite_warp) renders LiDAR scans and, with P.quad, images.
 cudaError_t launch_composite(const CompParams& P, cudaStream_t st, int* ctas);
 cudaError_t launch_composite_warp(const CompParams& P, cudaStream_t st, int* ctas);
-// About the resident warps of the warp form per SM (the items that run at once).
-constexpr int kWarpsPerSM = 20;
 
 constexpr int kWordsPerBlock = 256;  // binning block: at most one visibility word per thread of 256 (8192 slots)
 constexpr int kRankBins = 2048;      // depth ranges per env, at most

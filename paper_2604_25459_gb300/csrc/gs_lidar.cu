@@ -50,8 +50,13 @@ __device__ __forceinline__ bool grid_range(float a, float b, float origin, float
     return true;
 }
 
-// 8x8 subtile (row-major in the 16x16 tile) of a ray's cell word.
-__device__ __forceinline__ uint32_t ray_sub(uint32_t cell) { return ((cell >> 6) & 2u) | ((cell >> 3) & 1u); }
+// 4x4 quadrant of a ray's cell word in its 16x16 tile: subtile-major (8x8
+// subtiles row-major, then the quadrants of the subtile), so that 64
+// consecutive rays of a tile's list lie in few subtiles and 16 in few quadrants.
+__device__ __forceinline__ uint32_t ray_quad(uint32_t cell) {
+    const uint32_t i = cell & 15u, j = (cell >> 4) & 15u;
+    return (j >> 3 << 3) | (i >> 3 << 2) | ((j >> 2 & 1u) << 1) | (i >> 2 & 1u);
+}
 
 }  // namespace
 
@@ -254,10 +259,10 @@ __global__ void __launch_bounds__(256) k_ray_count(const float* __restrict__ dir
     }
     const int t = (j >> 4) * E.ntx + (i >> 4);
     cell[k] = ((uint32_t)t << 8) | ((uint32_t)(j & 15) << 4) | (uint32_t)(i & 15);
-    atomicAdd(cnt + 4 * (size_t)(E.tile_base + t) + ray_sub(cell[k]), 1u);
+    atomicAdd(cnt + kRayGroups * (size_t)(E.tile_base + t) + ray_quad(cell[k]), 1u);
 }
 
-// Rays grouped by tile and 8x8 subtile: list[el][off[tile, sub] + rank] = r.
+// Rays grouped by tile and quadrant: list[el][off[tile, quadrant] + rank] = r.
 __global__ void __launch_bounds__(256) k_ray_scatter(const EnvInfo* envs, int n_rays, const uint32_t* cell,
                                                      const uint32_t* off, uint32_t* cur, uint32_t* list) {
     const int el = blockIdx.y;
@@ -267,7 +272,7 @@ __global__ void __launch_bounds__(256) k_ray_scatter(const EnvInfo* envs, int n_
     const uint32_t c = cell[k];
     if (c == 0xffffffffu) return;
     const unsigned int tb = envs[el].tile_base;
-    const size_t t = 4 * (size_t)(tb + (c >> 8)) + ray_sub(c);
+    const size_t t = kRayGroups * (size_t)(tb + (c >> 8)) + ray_quad(c);
     const uint32_t pos = off[t] + atomicAdd(cur + t, 1u);
     list[(size_t)el * n_rays + pos] = (uint32_t)r;
 }
@@ -277,8 +282,13 @@ __global__ void __launch_bounds__(256) k_ray_items(const EnvInfo* envs, int We, 
                                                    uint32_t* item_cnt) {
     const unsigned int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= envs[We].tile_base) return;
-    const uint4 c = reinterpret_cast<const uint4*>(cnt)[i];  // the tile's four subtiles
-    item_cnt[i] = (c.x + c.y + c.z + c.w + (uint32_t)kRayChunk - 1u) / (uint32_t)kRayChunk;
+    uint32_t n = 0;
+#pragma unroll
+    for (int k = 0; k < kRayGroups / 4; ++k) {
+        const uint4 c = reinterpret_cast<const uint4*>(cnt)[(kRayGroups / 4) * (size_t)i + k];
+        n += c.x + c.y + c.z + c.w;
+    }
+    item_cnt[i] = (n + (uint32_t)kRayChunk - 1u) / (uint32_t)kRayChunk;
 }
 
 cudaError_t launch_ray_count(const float* dirs, const gs_lidar* lidars, const EnvInfo* envs, int We, int n_rays,
