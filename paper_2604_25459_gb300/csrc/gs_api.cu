@@ -446,15 +446,10 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
                    unsigned long long* total_out, int quad) {
     const int We = wt.We;
     bool use_quad = false;
-    if (((tw == 16 && th == 16) || (tw == 8 && th == 8)) && !io.lidars && !io.score) {
-        if (quad < 0) {
-            long long most = 0;
-            for (int e = 0; e < We; ++e)
-                most = std::max(most, (long long)wt.host_envs[e].W * wt.host_envs[e].H);
-            use_quad = most <= kQuadMaxPixels;
-        } else {
-            use_quad = quad != 0;
-        }
+    if (!io.lidars && !io.score) {
+        long long most = 0;
+        for (int e = 0; e < We; ++e) most = std::max(most, (long long)wt.host_envs[e].W * wt.host_envs[e].H);
+        use_quad = warp_form(tw, th, quad < 0 ? most : 0) && quad != 0;
     }
     CK(sc.xf.ensure(sizeof(LinkXf) * (size_t)std::max(wt.xf_items, 1)), "alloc link table");
     CK(sc.r012.ensure(wt.recs * 16 * kRecStride), "alloc records");
@@ -540,10 +535,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     B.rank = R.rank;
     B.status = status;
     B.wrap = io.lidars ? 1 : 0;         // LiDAR boxes may wrap across azimuth 0
-    // the warp form's keys carry a subtile mask below the rank while both fit 32 bits
-    const int n_sub = (tw / 8) * (th / 8);
-    if ((use_quad || io.lidars) && n_sub > 1 && ((unsigned long long)wt.max_words * 32) >> (32 - n_sub) == 0)
-        B.key_shift = n_sub;
+    if (use_quad || io.lidars) B.key_shift = subtile_bits(tw, th, (unsigned long long)wt.max_words * 32);
     PhaseTimer t3(s, st, GS_PHASE_COUNT, timers);
     CK(launch_rank_sample(R, We, st), "depth sample");
     CK(launch_count(B, R, We, wt.max_T, wt.max_hist, st), "count");

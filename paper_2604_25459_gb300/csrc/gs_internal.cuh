@@ -374,10 +374,21 @@ inline size_t rank_tables(RankParams& R, int We, unsigned char* base) {
 }
 // Depth-ordered window held in shared memory by the compositor.
 constexpr int kCompCap = 768;
-// Plain renders use the compositor's quadrant form (QUAD) on 16x16 or 8x8 tiles when
-// no image of the wave has more pixels than this (measured crossover on the
-// room workload: faster at 320x240 and below, slower at 640x480).
-constexpr int kQuadMaxPixels = 320 * 240;
+// Plain renders use the warp form of the compositor on 16x16 or 8x8 tiles when
+// no image of the wave has more pixels than this.  Scatter + compositing, CTA
+// form / warp form (us, the room): 400x300: 1 env 215 / 148, 4 586 / 307, 16
+// 837 / 776, 64 2290 / 2152; 480x360: 160 / 174, 419 / 352, 835 / 833, 2617 /
+// 2658; 640x480: 155 / 200, 379 / 475, 1007 / 1097, 3399 / 3859.
+constexpr int kQuadMaxPixels = 140000;
+inline bool warp_form(int tile_w, int tile_h, long long most_pixels) {
+    return ((tile_w == 16 && tile_h == 16) || (tile_w == 8 && tile_h == 8)) && most_pixels <= kQuadMaxPixels;
+}
+// Bits of the subtile mask below the ranks of the warp form's keys: one per 8x8
+// subtile while they and the ranks of n_slots records fit 32 bits, else none.
+inline int subtile_bits(int tile_w, int tile_h, unsigned long long n_slots) {
+    const int n = (tile_w / 8) * (tile_h / 8);
+    return n > 1 && (n_slots >> (32 - n)) == 0 ? n : 0;
+}
 
 // Read-only view of a scene's device data for entry points outside gs_api.cu.
 struct SceneView {

@@ -86,7 +86,7 @@ Layout layout(int We, int nb, int xf_items, unsigned long long recs, unsigned lo
     y.cursor = o;    o = up256(o + tiles * 4);
     y.env_total = o; o = up256(o + (size_t)We * 8);
     y.env_base = o;  o = up256(o + ((size_t)We + 1) * 8);
-    y.work = o;      o = up256(o + 16);
+    y.work = o;      o = up256(o + 32);
     y.pairs = o;
     return y;
 }
@@ -263,6 +263,8 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.tile_h = th;
         B.words_per_block = scatter_words(max_words, Wn, max_T);
         B.rank = R.rank;
+        const bool warp = warp_form(tw, th, (long long)px);
+        if (warp) B.key_shift = subtile_bits(tw, th, (unsigned long long)max_words * 32);
         B.counts = counts;
         B.off_local = off;
         B.env_base = env_base;
@@ -310,11 +312,25 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         C.neval = nullptr;
         C.tile_w = tw;
         C.tile_h = th;
+        C.quad = warp ? 1 : 0;
+        C.key_shift = B.key_shift;
         C.rgb = rgb + (size_t)e0 * px * 3;
         C.depth = depth + (size_t)e0 * px;
         C.alpha = alpha ? alpha + (size_t)e0 * px : nullptr;
         C.status = v.status;
-        NA_CK(cudaMemsetAsync(C.work, 0, 4, st), "clear work counter");
+        // the work counters, and behind the ranking's tables the warp form's item
+        // order, where it fits
+        C.team_work = C.work + 1;
+        NA_CK(cudaMemsetAsync(C.work, 0, 8 + 4 * kItemClasses, st), "clear work counters");
+        uint32_t* const items = reinterpret_cast<uint32_t*>(base + up256((size_t)(tab - base)));
+        if (warp && up256((size_t)(tab - base)) + (size_t)sen.tile_base * kItemClasses * 4 <= kNoAllocBytes) {
+            NA_CK(launch_item_order(d_envs, 0, Wn, max_T, counts, nullptr, nullptr, nullptr, items, sen.tile_base,
+                                    C.work + 2, st),
+                  "item order");
+            C.items = items;
+            C.class_cnt = C.work + 2;
+            C.item_pitch = sen.tile_base;
+        }
         int ctas = 0;
         NA_CK(launch_composite(C, st, &ctas), "composite");
     }
