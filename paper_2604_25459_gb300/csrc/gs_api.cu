@@ -55,7 +55,7 @@ struct gs_plan_s {
     std::vector<gs_camera> cams;
     int flags = 0;
     int tile_w = 16, tile_h = 16, chunk = 1;
-    int quad = 0;  // compositor's quadrant form (16x16 tiles), chosen by the autotuner
+    int quad = 0;  // the compositor's warp form: 0 no env, 1 every env, -1 by resolution (chosen by the autotuner)
     Scratch sc;
     struct Wave {
         int e0, e1;
@@ -445,18 +445,24 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
                    unsigned long long cap, cudaStream_t st, bool timers, int64_t* launches,
                    unsigned long long* total_out, int quad) {
     const int We = wt.We;
-    bool use_quad = false;
-    if (!io.lidars && !io.score) {
-        long long most = 0;
-        for (int e = 0; e < We; ++e) most = std::max(most, (long long)wt.host_envs[e].W * wt.host_envs[e].H);
-        use_quad = warp_form(tw, th, quad < 0 ? most : 0) && quad != 0;
+    // Envs [0, n_warp) go to the compositor's warp form, the others to the CTA
+    // form: all of them by the largest image, or, in a batch of mixed
+    // resolutions in ascending order, each by its own.
+    int n_warp = io.lidars ? We : 0;
+    if (!io.lidars && !io.score && quad != 0) {
+        auto small = [&](int e) {
+            return warp_form(tw, th, quad < 0 ? (long long)wt.host_envs[e].W * wt.host_envs[e].H : 0);
+        };
+        while (n_warp < We && small(n_warp)) ++n_warp;
+        for (int e = n_warp; e < We; ++e)
+            if (small(e)) n_warp = 0;  // unordered: by the largest image
     }
     CK(sc.xf.ensure(sizeof(LinkXf) * (size_t)std::max(wt.xf_items, 1)), "alloc link table");
     CK(sc.r012.ensure(wt.recs * 16 * kRecStride), "alloc records");
     CK(sc.r3.ensure(wt.recs * 16), "alloc records");
     CK(sc.mask.ensure(wt.words * 4), "alloc masks");
     RankParams R = rank_sizes(wt.max_words, We, io.lidars != nullptr);
-    const size_t n_bins = (size_t)We * R.bins, n_zero = (size_t)wt.tiles * 2 + n_bins + 1 + kItemClasses + 3;
+    const size_t n_bins = (size_t)We * R.bins, n_zero = (size_t)wt.tiles * 2 + n_bins + kWorkWords;
     CK(sc.counts.ensure(n_zero * 4), "alloc counts");
     CK(sc.off.ensure(wt.tiles * 4), "alloc offsets");
     CK(sc.env_total.ensure((size_t)We * 8), "alloc totals");
@@ -535,7 +541,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     B.rank = R.rank;
     B.status = status;
     B.wrap = io.lidars ? 1 : 0;         // LiDAR boxes may wrap across azimuth 0
-    if (use_quad || io.lidars) B.key_shift = subtile_bits(tw, th, (unsigned long long)wt.max_words * 32);
+    if (n_warp > 0) B.key_shift = subtile_bits(tw, th, (unsigned long long)wt.max_words * 32);
     PhaseTimer t3(s, st, GS_PHASE_COUNT, timers);
     CK(launch_rank_sample(R, We, st), "depth sample");
     CK(launch_count(B, R, We, wt.max_T, wt.max_hist, st), "count");
@@ -673,7 +679,6 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         C.neval = (s->counters && cap == 0) ? s->neval.as<unsigned long long>() : nullptr;
         C.tile_w = tw;
         C.tile_h = th;
-        C.quad = use_quad ? 1 : 0;
         C.key_shift = B.key_shift;
         C.rgb = io.rgb;
         C.depth = io.depth;
@@ -688,29 +693,43 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         C.lidars = io.lidars;
         C.r3 = P.r3;
         C.status = status;
-        if (ea > 0) CK(cudaMemsetAsync(work, 0, 8 + 4 * kItemClasses, st), "memset work counter");
-        if (use_quad || io.lidars) {  // warp form: long buckets first
-            const unsigned long long n_items = C.item_end - C.item_begin;
+        // work counters: the warp form's, its classes' and its teams', the CTA form's
+        if (ea > 0) CK(cudaMemsetAsync(work, 0, 4 * kWorkWords, st), "memset work counters");
+        const int es = std::min(std::max(n_warp, ea), ebd);  // warp form: [ea, es)
+        PhaseTimer t6(s, st, GS_PHASE_COMPOSITE, timers);
+        int kernels = 0, ctas = 0;
+        if (es > ea) {
+            CompParams Q = C;
+            Q.quad = 1;
+            if (!io.ray_dirs) Q.item_end = wt.host_envs[es].tile_base;
+            Q.e_end = es;
+            const unsigned long long n_items = Q.item_end - Q.item_begin;  // long buckets first
             if (n_items * kItemClasses * 4 <= (unsigned long long)s->budget / 64) {
                 CK(sc.items.ensure((size_t)n_items * kItemClasses * 4), "alloc item order");
-                CK(launch_item_order(wt.envs, ea, ebd - ea, wt.max_T, counts,
+                CK(launch_item_order(wt.envs, ea, es - ea, wt.max_T, counts,
                                      io.ray_dirs ? s->item_cnt.as<uint32_t>() : nullptr,
                                      io.ray_dirs ? s->item_off.as<uint32_t>() : nullptr,
                                      io.ray_dirs ? s->item_base.as<unsigned long long>() : nullptr,
                                      sc.items.as<uint32_t>(), (uint32_t)n_items, work + 1, st),
                    "item order");
-                C.items = sc.items.as<uint32_t>();
-                C.class_cnt = work + 1;
-                C.item_pitch = (unsigned)n_items;
-                C.team_work = work + 1 + kItemClasses;
-                ++*launches;
+                Q.items = sc.items.as<uint32_t>();
+                Q.class_cnt = work + 1;
+                Q.item_pitch = (unsigned)n_items;
+                Q.team_work = work + 1 + kItemClasses;
+                ++kernels;
             }
+            CK(launch_composite(Q, st, &ctas), "composite");
+            ++kernels;
         }
-        int ctas = 0;
-        PhaseTimer t6(s, st, GS_PHASE_COMPOSITE, timers);
-        CK(launch_composite(C, st, &ctas), "composite");
-        t6.done(1);
-        ++*launches;
+        if (es < ebd) {
+            C.e_begin = es;
+            C.item_begin = wt.host_envs[es].tile_base;
+            C.work = work + 2 + kItemClasses;
+            CK(launch_composite(C, st, &ctas), "composite");
+            ++kernels;
+        }
+        t6.done(kernels);
+        *launches += kernels;
         if (cap == 0) {
             s->last_ea = ea;
             s->last_eb = ebd;
@@ -1352,6 +1371,14 @@ gs_status gs_render_batch_v(gs_scene s, int n_envs, const gs_env* envs, const fl
     if (any_links && !link_poses) return fail(GS_ERR_INVALID, "null link_poses");
     std::vector<EnvSpec> specs;
     ST(specs_from_envs(s, n_envs, envs, &specs));
+    ST(check_specs(s, specs, s->tile_w, s->tile_h));
+    // Low resolutions first (see gs_plan_create): their images then take the
+    // compositor's warp form.  Outputs are placed by pixel_offset, so the order
+    // is not visible; debug renders keep the caller's, by which the copies index.
+    if (!s->debug)
+        std::stable_sort(specs.begin(), specs.end(), [](const EnvSpec& a, const EnvSpec& b) {
+            return (int64_t)a.cam->width * a.cam->height < (int64_t)b.cam->width * b.cam->height;
+        });
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     CK(cudaSetDevice(s->device), "set device");
     if (s->D.n == 0) {
@@ -1448,14 +1475,19 @@ gs_status gs_plan_launch(gs_plan p, const float* link_poses, float* rgb, float* 
         };
         std::vector<Cand> cands;
         if (p->flags & GS_PLAN_AUTOTUNE) {
+            // On square tiles also the warp form: for every env or, in a batch whose
+            // largest images are beyond its range, for the envs within it.
+            const gs_camera &first = p->envs.front().cam, &most = p->envs.back().cam;
+            const bool mixed = warp_form(16, 16, (long long)first.width * first.height) &&
+                               !warp_form(16, 16, (long long)most.width * most.height);
             const int shapes[5][2] = {{16, 16}, {32, 8}, {16, 8}, {8, 8}, {32, 16}};
             for (auto& sh : shapes)
                 for (int ch : {1, 4}) {
                     cands.push_back({sh[0], sh[1], ch, 0});
-                    if (sh[0] == sh[1]) cands.push_back({sh[0], sh[1], ch, 1});  // quadrant form: 16x16, 8x8
+                    if (sh[0] == sh[1]) cands.push_back({sh[0], sh[1], ch, mixed ? -1 : 1});
                 }
         } else {
-            cands.push_back({p->tile_w, p->tile_h, 1, 0});
+            cands.push_back({p->tile_w, p->tile_h, 1, -1});
         }
         cudaEvent_t a, b;
         CK(cudaEventCreate(&a), "event");
@@ -1540,7 +1572,7 @@ gs_status gs_plan_get_info(gs_plan p, gs_plan_info* out) {
     i.tile_w = p->tile_w;
     i.tile_h = p->tile_h;
     i.chunk = p->chunk;
-    i.quad = p->quad;
+    i.quad = p->quad != 0;
     i.waves = (int)p->waves.size();
     i.graph = p->exec != nullptr;
     i.tuned_candidates = p->tuned_candidates;

@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
         if (whole) {
             uint32_t lo = 0xffffffffu, hi = 0u;
             for (uint32_t i = tid; i < n; i += NT) {
-                const uint32_t k = Lk[i];
+                const uint32_t k = Lk[i] >> P.key_shift;
                 keys[i] = k;
                 lo = min(lo, k);
                 hi = max(hi, k);
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                 for (int i = tid; i < BMW / 4; i += NT) reinterpret_cast<uint4*>(bm)[i] = make_uint4(0u, 0u, 0u, 0u);
                 __syncthreads();
                 for_ranks<NT>(Lk, n, [&](uint32_t k) {
-                    const uint32_t d = k - r0;
+                    const uint32_t d = (k >> P.key_shift) - r0;
                     if (d < (uint32_t)(BMW * 32)) atomicOr(&bm[d >> 5], 1u << (d & 31u));
                 });
                 __syncthreads();

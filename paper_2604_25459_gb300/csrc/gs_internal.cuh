@@ -228,9 +228,9 @@ struct CompParams {
     unsigned long long* neval;       // nullable: composited (pixel, Gaussian) pair counter
     int tile_w, tile_h;
     int quad;       // camera images: the warp form (k_composite_warp)
-    // The warp form's keys carry, below the rank, one bit per 8x8 subtile of
-    // the tile that the record's box reaches (row-major): key = rank <<
-    // key_shift | mask.  key_shift = 0: no mask (plain ranks).
+    // Keys of waves with envs in the warp form carry, below the rank, one bit
+    // per 8x8 subtile of the tile that the record's box reaches (row-major): key
+    // = rank << key_shift | mask.  key_shift = 0: no mask (plain ranks).
     int key_shift;
     float* rgb;     // images at envs[e].pix_base (x3 for rgb); unused when rgb8 is set
     float* depth;   // unused when depth16 is set
@@ -301,6 +301,7 @@ cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int ma
 // Lists a launch's items by the length of their buckets, longest class first
 // (CompParams::items); class_cnt is zeroed by the caller.  Rays: item_cnt and
 // item_off per (env, tile) and item_base per env give a tile's items.
+constexpr int kWorkWords = 8;    // work counters of a launch (see run_wave)
 constexpr int kItemClasses = 4;  // buckets of >= 16384, >= 4096, >= 1024 and fewer keys
 cudaError_t launch_item_order(const EnvInfo* envs, int e_begin, int n_envs, int max_T, const uint32_t* counts,
                               const uint32_t* item_cnt, const uint32_t* item_off,
