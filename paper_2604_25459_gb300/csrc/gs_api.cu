@@ -1475,8 +1475,9 @@ gs_status gs_plan_launch(gs_plan p, const float* link_poses, float* rgb, float* 
         };
         std::vector<Cand> cands;
         if (p->flags & GS_PLAN_AUTOTUNE) {
-            // On square tiles also the warp form: for every env or, in a batch whose
-            // largest images are beyond its range, for the envs within it.
+            // On square tiles also the warp form: for every env and, in a batch whose
+            // largest images are beyond its range, for the envs within it (claim
+            // size 1, as both forms claim best).
             const gs_camera &first = p->envs.front().cam, &most = p->envs.back().cam;
             const bool mixed = warp_form(16, 16, (long long)first.width * first.height) &&
                                !warp_form(16, 16, (long long)most.width * most.height);
@@ -1484,7 +1485,7 @@ gs_status gs_plan_launch(gs_plan p, const float* link_poses, float* rgb, float* 
             for (auto& sh : shapes)
                 for (int ch : {1, 4}) {
                     cands.push_back({sh[0], sh[1], ch, 0});
-                    if (sh[0] == sh[1]) cands.push_back({sh[0], sh[1], ch, mixed ? -1 : 1});
+                    if (sh[0] == sh[1]) cands.push_back({sh[0], sh[1], ch, mixed && ch == 1 ? -1 : 1});
                 }
         } else {
             cands.push_back({p->tile_w, p->tile_h, 1, -1});
