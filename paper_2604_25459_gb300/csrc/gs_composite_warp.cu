@@ -226,19 +226,16 @@ struct Lane {
     float near_range;
 };
 
-// Pixels of quadrant q (q & 1, q >> 1) of the subtile at (wx0, wy0): lane l8 of
-// eight takes column l8 & 3 and rows l8 >> 2 and two below.
-template <int MODE>
-__device__ __forceinline__ void lane_pixels(const CompParams& P, int el, int W, int H, int wx0, int wy0, int q,
-                                            int l8, Lane& L) {
-    const int px = wx0 + 4 * (q & 1) + (l8 & 3), py = wy0 + 4 * (q >> 1) + (l8 >> 2);
+// Pixels (px, py) and (px, py + DY).
+template <int MODE, int DY>
+__device__ __forceinline__ void lane_pixels(const CompParams& P, int el, int W, int H, int px, int py, Lane& L) {
     L.in0 = px < W && py < H;
-    L.in1 = px < W && py + 2 < H;
+    L.in1 = px < W && py + DY < H;
     L.fpx = (float)px + 0.5f;
-    L.fpy = make_float2((float)py + 0.5f, (float)(py + 2) + 0.5f);
+    L.fpy = make_float2((float)py + 0.5f, (float)(py + DY) + 0.5f);
     L.cx0 = L.cx1 = px;
     L.cy0 = py;
-    L.cy1 = py + 2;
+    L.cy1 = py + DY;
     if constexpr (MODE == 1) {
         const gs_lidar* Ld = P.lidars + el;
         const float em = __ldg(&Ld->elev_min), eM = __ldg(&Ld->elev_max);
@@ -420,7 +417,7 @@ __device__ __forceinline__ void team_item(const CompParams& P, TeamSmem<MODE == 
         wx1 = __reduce_max_sync(kAll, max(L.in0 ? L.cx0 : -big, L.in1 ? L.cx1 : -big));
         wy1 = __reduce_max_sync(kAll, max(L.in0 ? L.cy0 : -big, L.in1 ? L.cy1 : -big));
     } else {
-        lane_pixels<MODE>(P, w.el, W, H, sx0, sy0, warp, l8, L);
+        lane_pixels<MODE, 2>(P, w.el, W, H, wx0 + (l8 & 3), wy0 + (l8 >> 2), L);
     }
     bool done0 = !L.in0, done1 = !L.in1;
     float2 Tp = make_float2(1.0f, 1.0f), acc = make_float2(0.0f, 0.0f);  // acc: channel grp (LiDAR: the range)
@@ -678,7 +675,8 @@ __device__ __forceinline__ void team_item(const CompParams& P, TeamSmem<MODE == 
 template <int MODE>
 __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k_composite_warp(CompParams P) {
     constexpr bool LID = MODE == 1 || MODE == 3;
-    constexpr bool QUAD = MODE != 3;
+    constexpr bool GROUPS = MODE != 3;
+    constexpr int GW_ = 2, GH = LID ? 2 : 4, GL = GW_ * GH / 2;  // a group's pixels and lanes
     constexpr bool CNT = MODE != 0;
     constexpr int CAP = LID ? 512 : 256;   // ranks per window, and per group of bitmap words
     constexpr int GW = CAP / 32;           // words per group
@@ -704,7 +702,7 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
     const int lane = threadIdx.x & 31;
     const int lx = __ffs(P.tile_w) - 4, ly = __ffs(P.tile_h) - 4;  // log2 of the tile's subtile columns, rows
     const int lsub = MODE == 3 ? 0 : lx + ly;
-    const int grp = lane >> 3, l8 = lane & 7;
+    const int grp = lane / GL, lg = lane % GL;
     Where w;
     w.el = P.e_begin;
     w.e_lo = __ldg(&P.envs[w.el].tile_base);
@@ -766,7 +764,8 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
         wx1 = __reduce_max_sync(kAll, max(L.in0 ? L.cx0 : -big, L.in1 ? L.cx1 : -big));
         wy1 = __reduce_max_sync(kAll, max(L.in0 ? L.cy0 : -big, L.in1 ? L.cy1 : -big));
     } else {
-        lane_pixels<MODE>(P, w.el, W, H, wx0, wy0, grp, l8, L);
+        const int gx0 = wx0 + GW_ * (grp % (8 / GW_)), gy0 = wy0 + GH * (grp / (8 / GW_));
+        lane_pixels<MODE, GH / 2>(P, w.el, W, H, gx0 + lg % GW_, gy0 + lg / GW_, L);
     }
     bool done0 = !L.in0, done1 = !L.in1;
     // the lane's two pixels: .x = (px, py0), .y = (px, py1)
@@ -838,22 +837,29 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
                 }
             }
             uint32_t m32;
-            if constexpr (QUAD) {  // per quadrant: the splats whose box reaches it
-                const bool c0 = ov && bx0 <= wx0 + 3, c1 = ov && bx1 >= wx0 + 4;
-                const bool r0 = by0 <= wy0 + 3, r1 = by1 >= wy0 + 4;
-                const uint32_t ma = __ballot_sync(kAll, c0 && r0), mb = __ballot_sync(kAll, c1 && r0);
-                const uint32_t mc = __ballot_sync(kAll, c0 && r1), md = __ballot_sync(kAll, c1 && r1);
+            if constexpr (GROUPS) {  // per group: the splats whose box reaches it
+                bool cx[8 / GW_], cy[8 / GH];
+#pragma unroll
+                for (int i = 0; i < 8 / GW_; ++i)
+                    cx[i] = ov && bx0 <= wx0 + GW_ * i + GW_ - 1 && bx1 >= wx0 + GW_ * i;
+#pragma unroll
+                for (int i = 0; i < 8 / GH; ++i) cy[i] = by0 <= wy0 + GH * i + GH - 1 && by1 >= wy0 + GH * i;
+                m32 = 0u;
+#pragma unroll
+                for (int g = 0; g < 32 / GL; ++g) {
+                    const uint32_t b = __ballot_sync(kAll, cx[g % (8 / GW_)] && cy[g / (8 / GW_)]);
+                    if (grp == g) m32 = b;
+                }
                 const uint32_t dm = __ballot_sync(kAll, done0 && done1);
-                m32 = grp == 0 ? ma : (grp == 1 ? mb : (grp == 2 ? mc : md));
-                if (((dm >> (8 * grp)) & 0xffu) == 0xffu) m32 = 0u;
+                if ((~dm >> (GL * grp) & ((1u << GL) - 1u)) == 0u) m32 = 0u;
             } else {
                 m32 = __ballot_sync(kAll, ov);
             }
             __syncwarp();  // the lanes' staged values
             // two splats per step: their four alpha evaluations are independent;
             // the blends then run in depth order
-            while (QUAD ? __any_sync(kAll, m32 != 0u) : m32 != 0u) {
-                const bool one = !QUAD || m32 != 0u;
+            while (GROUPS ? __any_sync(kAll, m32 != 0u) : m32 != 0u) {
+                const bool one = !GROUPS || m32 != 0u;
                 const int j1 = one ? __ffs(m32) - 1 : 0;
                 m32 &= m32 - 1u;
                 const bool two = m32 != 0u;
