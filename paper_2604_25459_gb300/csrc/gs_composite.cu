@@ -160,30 +160,23 @@ __device__ __forceinline__ float warp_sum(float v) {
 template <int TW, int TH, bool SC = false, bool CNT = SC>
 __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 256 ? 8 : (TW * TH >= 128 ? 12 : 24)))) k_composite(CompParams P) {
     constexpr int NT = TW * TH / 2;
-    constexpr int NB = NT;  // splats staged per batch (one per thread)
     constexpr int CAP = NT == 32 ? 512 : kCompCap;
     constexpr int SB = NT == 32 ? 512 : 1024;      // rank ranges of the short-bucket sort
     constexpr int NG = NT > 128 ? 128 : NT;        // bitmap groups
     constexpr int BMW = NG * kGroupWords;          // bitmap words (32 ranks each)
-    constexpr int UB = CAP * 4 > NB * 64 ? CAP * 4 : NB * 64;
     constexpr int NW = NT / 32;
     static_assert(BMW >= SB, "the short-bucket counters share the bitmap's memory");
     static_assert(CAP >= kGroupWords * 32, "a group's ranks fit a window");
     __shared__ uint32_t keys[CAP];                      // the window's ranks
-    __shared__ float4 raw[3][NB];                       // records of the next batch, in flight
-    __shared__ __align__(16) unsigned char ubuf[UB];    // sort scratch | staged records
+    __shared__ float4 recs[NW][2][3][32];               // a warp's records of this and the next 32 splats | sort scratch
     __shared__ __align__(16) uint32_t bm[BMW];          // bitmap | counters of the short-bucket sort
     __shared__ uint32_t pre[NG + 1];                    // ranks set before each group of the bitmap
     __shared__ uint32_t red[32];
-    uint32_t* tmp = reinterpret_cast<uint32_t*>(ubuf);
-    float4* sA = reinterpret_cast<float4*>(ubuf);  // u, v, o, z
-    float4* sB = sA + NB;                          // scaled conic factor l00, l01, l11
-    float4* sC = sB + NB;                          // r, g, b
-    int4* sR = reinterpret_cast<int4*>(sC + NB);   // x0, x1 - x0, y0, y1 - y0
-    __shared__ uint32_t sG[SC ? NB : 1];  // contribution pass: slot of each staged splat
-
+    static_assert(sizeof(recs) >= CAP * 4, "the sort scratch shares the records' memory");
+    uint32_t* tmp = reinterpret_cast<uint32_t*>(recs);
     __shared__ unsigned int s_item;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto& rec = recs[warp];
     bool c32_dirty = true;  // the short-bucket sort's counters (bm) need clearing before use
     int el = P.e_begin;  // env of the current item, cached across items (uniform in the CTA)
     unsigned int e_lo = P.envs[el].tile_base, e_hi = e_lo + (unsigned)P.envs[el].T;
@@ -241,71 +234,63 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
     };
     bool finished = false;
     // Composite the window keys[0, wn) (ranks in depth order).  Sets
-    // `finished` once every pixel of the tile has terminated.
+    // `finished` once every pixel of the tile has terminated.  Each warp walks
+    // the window on its own: a lane copies (cp.async) the record of one of the
+    // next 32 splats while the current 32 are blended.
     auto run_window = [&](uint32_t wn) {
-        // The records of a batch are copied (cp.async) while the batch before it
-        // is blended; a thread stages the splat it copied itself, so the copies
-        // need no barrier of their own.
         auto slot_of = [&](uint32_t i) -> uint32_t { return i < wn ? __ldg(order + keys[i]) : 0xffffffffu; };
-        auto fetch = [&](uint32_t g) {
+        auto fetch = [&](int buf, uint32_t g) {
             if (g < n_local) {
                 const float4* src = P.r0 + (size_t)kRecStride * (recbase + g);
-                copy16(&raw[0][tid], src);
-                copy16(&raw[1][tid], src + 1);
-                copy16(&raw[2][tid], src + 2);
+                copy16(&rec[buf][0][lane], src);
+                copy16(&rec[buf][1][lane], src + 1);
+                copy16(&rec[buf][2][lane], src + 2);
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        uint32_t g = slot_of(tid), g_next = slot_of(NB + tid);
-        fetch(g);
-        for (uint32_t b = 0; b < wn; b += NB) {
-            const int cnt_b = (int)min((uint32_t)NB, wn - b);
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            if (tid < cnt_b) {
-                const int s = tid;
-                if (g < n_local) {
-                    const float4 q0 = raw[0][tid], q1 = raw[1][tid], q2 = raw[2][tid];
-                    const uint32_t rx = __float_as_uint(q1.w), ry = __float_as_uint(q2.w);
-                    sA[s] = make_float4(q0.x, q0.y, log2f(q0.z), q0.w);
-                    // alpha >= 1/255 iff q <= w (w only feeds the subtile cull, whose
-                    // 1e-3 margin dwarfs the error of the fast logarithm)
-                    sB[s] = make_float4(q1.x, q1.y, q1.z, __log2f(255.0f * q0.z));
-                    sC[s] = q2;
-                    const int bx0 = (int)(rx & 0xffffu), by0 = (int)(ry & 0xffffu);
-                    sR[s] = make_int4(bx0, (int)(rx >> 16) - bx0, by0, (int)(ry >> 16) - by0);
-                    if constexpr (SC) sG[s] = g;
-                } else {  // never happens for a well-formed bucket; stage an empty range
-                    sA[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    sB[s] = sA[s];
-                    sC[s] = sA[s];
-                    sA[s].z = -126.0f;  // log2 of a vanishing opacity
-                    sR[s] = make_int4(1 << 20, -1, 1 << 20, -1);
-                    atomicOr(P.status, kStOverflow);
-                }
-            }
-            g = g_next;
-            if (b + NB < wn) {
-                fetch(g);
-                g_next = slot_of(b + 2 * NB + tid);
-            }
-            __syncthreads();
-            if (!__all_sync(0xffffffffu, done0 && done1)) {
-                for (int c = 0; c < cnt_b; c += 32) {
-                    const int j = c + lane;
-                    // box, then the exact ellipse for large splats (a box under 24 px in
-                    // width + height is kept as it is: it overstates the ellipse least),
-                    // evaluated by every lane
-                    const int jj = j < cnt_b ? j : c;
-                    const int4 R = sR[jj];
-                    bool ov = j < cnt_b && R.x <= wx1 && R.x + R.y >= wx0 && R.z <= wy1 && R.z + R.w >= wy0;
-                    const bool rr = reaches_rect(sA[jj], sB[jj], (float)wx0 + 0.5f, (float)wy0 + 0.5f);
-                    ov = ov && (R.y + R.w < 24 || rr);
+        if (!__all_sync(0xffffffffu, done0 && done1)) {
+            uint32_t g = slot_of(lane), g_next = slot_of(32 + lane);
+            fetch(0, g);
+            for (uint32_t c = 0; c < wn; c += 32) {
+                const int buf = (int)(c >> 5) & 1;
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncwarp();  // the other buffer is free
+                const uint32_t slot = g;
+                g = g_next;
+                if (c + 32 < wn) fetch(buf ^ 1, g);
+                g_next = slot_of(c + 64 + lane);
+                float4* sA = rec[buf][0];  // u, v, log2 o, z
+                float4* sB = rec[buf][1];  // scaled conic factor l00, l01, l11
+                float4* sC = rec[buf][2];  // r, g, b
+                {
+                    // The lane's splat against the subtile: its box, then the exact
+                    // ellipse for large splats (a box under 24 px in width + height is
+                    // kept as it is: it overstates the ellipse least).
+                    bool ov = false, bright = false;
+                    if (slot < n_local) {
+                        float4 A = sA[lane], B = sB[lane];
+                        const uint32_t rx = __float_as_uint(B.w), ry = __float_as_uint(sC[lane].w);
+                        const int bx0 = (int)(rx & 0xffffu), bx1 = (int)(rx >> 16);
+                        const int by0 = (int)(ry & 0xffffu), by1 = (int)(ry >> 16);
+                        ov = bx0 <= wx1 && bx1 >= wx0 && by0 <= wy1 && by1 >= wy0;
+                        A.z = log2f(A.z);  // folded into the exponent of alpha
+                        sA[lane].z = A.z;
+                        bright = ov && A.z > -0.029146346f;  // log2(0.98)
+                        if (ov && bx1 - bx0 + by1 - by0 >= 24) {
+                            // alpha >= 1/255 iff q <= w = log2(255 o); the cull's 1e-3
+                            // margin dwarfs the rounding of the constant
+                            B.w = A.z + 7.9943534f;
+                            ov = reaches_rect(A, B, (float)wx0 + 0.5f, (float)wy0 + 0.5f);
+                        }
+                    } else if (c + lane < wn) {  // never happens for a well-formed bucket
+                        atomicOr(P.status, kStOverflow);
+                    }
                     const uint32_t m = __ballot_sync(0xffffffffu, ov);
                     // Splats of opacity <= 0.98 never reach the 0.99 cap of alpha (o 2^-q
                     // with q >= 0), so a chunk without brighter splats walks a copy of the
                     // loop without the cap.
-                    const bool clamp_chunk =  // staged log2(o) > log2(0.98)
-                        __any_sync(0xffffffffu, j < cnt_b && sA[j].z > -0.029146346f);
+                    const bool clamp_chunk = __any_sync(0xffffffffu, bright);
+                    __syncwarp();  // the staged log2(o)
                     // One step blends two splats (TWO): their four alpha evaluations are
                     // independent, the blends run in depth order; an odd last splat has a
                     // step of its own.  No per-pixel box test: a pixel outside a splat's
@@ -372,9 +357,11 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                         }
                         if constexpr (SC) {  // warp-uniform: the lanes add their weights
                             const float s1 = warp_sum(w1), s2 = TWO ? warp_sum(w2) : 0.0f;
+                            const uint32_t g1 = __shfl_sync(0xffffffffu, slot, j1);
+                            const uint32_t g2 = __shfl_sync(0xffffffffu, slot, j2);
                             if (lane == 0) {
-                                if (s1 > 0.0f) atomicAdd(P.score + score_index(sG[j1]), s1);
-                                if (TWO && s2 > 0.0f) atomicAdd(P.score + score_index(sG[j2]), s2);
+                                if (s1 > 0.0f) atomicAdd(P.score + score_index(g1), s1);
+                                if (TWO && s2 > 0.0f) atomicAdd(P.score + score_index(g2), s2);
                             }
                         }
                     };
@@ -385,25 +372,21 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                             r ^= 0x80000000u >> k1;
                             const int k2 = __clz(r);
                             r ^= 0x80000000u >> k2;
-                            step(clamp_tag, std::true_type{}, c + k1, c + k2);
+                            step(clamp_tag, std::true_type{}, k1, k2);
                         }
                         if (r) {
                             const int k1 = __clz(r);
-                            step(clamp_tag, std::false_type{}, c + k1, c + k1);
+                            step(clamp_tag, std::false_type{}, k1, k1);
                         }
                     };
                     if (clamp_chunk) walk(std::true_type{});
                     else walk(std::false_type{});
-                    if (__all_sync(0xffffffffu, done0 && done1)) break;
                 }
+                if (__all_sync(0xffffffffu, done0 && done1)) break;
             }
-            const bool all = __syncthreads_and(done0 && done1) != 0;
-            if (all) {
-                finished = true;
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-                break;
-            }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
+        finished = __syncthreads_and(done0 && done1) != 0;
     };
 
     // The next window: its wn ranks in depth order in keys.
