@@ -14,11 +14,17 @@
 // a bit per rank in a bitmap of the next kGroups x 512 ranks and reading the
 // bits back in order: ranks are unique, so the bitmap is the sorted list, at
 // one shared-memory OR per key.  A window's ranks are mapped to record
-// slots, and composited in batches whose records are staged in shared memory;
-// warps test 32 splats at a time against their subtile with one ballot (box,
-// then the exact ellipse for large splats) and walk the overlapping ones two
-// at a time, every lane evaluating both at its pixels with no branch inside a
-// step.  Besides the image form the kernel has an observation
+// slots; each warp then walks the window on its own, 32 splats at a time:
+// a lane stages one of them (its record copied while the 32 before are
+// blended) and tests it against the warp's subtile (box, then the exact
+// ellipse for large splats), and the overlapping ones are blended two at a
+// time, every lane evaluating both at its pixels with no branch inside a step.
+// Warps of a tile meet at window ends only: batches of 128 splats staged by the
+// whole CTA loaded each record once instead of four times, but a warp with few
+// splats of a batch waited for the others (its top stall; 66 % of the issue
+// slots used, now 72 %): 256 views of 640x480 11.0 -> 10.7 ms.  What bounds
+// it is instruction issue: 72 steps of 2 splats x 64 pixels per subtile, 75
+// instructions each.  Besides the image form the kernel has an observation
 // form (8-bit colour after per-env appearance, half depth), a contribution
 // form (per-Gaussian blending weights, for pruning) and a LiDAR form (rays of
 // an (azimuth, beam) grid, Gaussians evaluated in ray space).

@@ -666,17 +666,23 @@ __device__ __forceinline__ void team_item(const CompParams& P, TeamSmem<MODE == 
 // rays of a 16x16 grid tile, grouped by 8x8 subtile; the culling box is that
 // of the rays' cells).
 //
-// Lanes work in four groups of eight: group q owns the 4x4 quadrant (q & 1, q
-// >> 1) of the subtile, a lane two of its pixels, and walks only the splats
-// whose box reaches it, so the groups advance through different splats at
-// once (MODE 3: all lanes walk the same splats; groups with boxes of their own
-// were slower on 128 envs, 8.1 instead of 7.5 ms, as the per-ray boxes cull
-// whole steps).
+// Lanes work in groups, a lane on two pixels: a group of four owns 2x4 pixels of
+// the subtile (LiDAR grids: a group of two, 2x2 rays) and walks only the splats
+// whose box reaches them, so the groups advance through different splats at
+// once; a chunk of 32 splats takes as many steps as its fullest group.  At
+// 128x128 a splat blends 5.6 of a subtile's 64 pixels: 443 steps of two splats
+// for the whole subtile, 303 with 4x4 groups, 256 with 2x4, 241 with 2x2; a
+// shared-memory load is split by quarter-warps, so two addresses in each cost
+// nothing.  Compositing 512 views of 128x128 takes 6.37 ms with 4x4 groups,
+// 6.33 with 4x2, 6.19 with 2x4 and 6.45 with 2x2 (more ballots per chunk, bank
+// conflicts); 32 scans of 64 x 1024 rays 2.35, 2.13, 2.19 and 2.05.  (MODE 3:
+// all lanes walk the same splats; groups with boxes of their own were slower on
+// 128 envs, 8.1 instead of 7.5 ms, as the per-ray boxes cull whole steps).
 template <int MODE>
 __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k_composite_warp(CompParams P) {
     constexpr bool LID = MODE == 1 || MODE == 3;
     constexpr bool GROUPS = MODE != 3;
-    constexpr int GW_ = 2, GH = LID ? 2 : 4, GL = GW_ * GH / 2;  // a group's pixels and lanes
+    constexpr int GPX = 2, GPY = LID ? 2 : 4, GL = GPX * GPY / 2;  // a group's pixels and lanes
     constexpr bool CNT = MODE != 0;
     constexpr int CAP = LID ? 512 : 256;   // ranks per window, and per group of bitmap words
     constexpr int GW = CAP / 32;           // words per group
@@ -764,8 +770,8 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
         wx1 = __reduce_max_sync(kAll, max(L.in0 ? L.cx0 : -big, L.in1 ? L.cx1 : -big));
         wy1 = __reduce_max_sync(kAll, max(L.in0 ? L.cy0 : -big, L.in1 ? L.cy1 : -big));
     } else {
-        const int gx0 = wx0 + GW_ * (grp % (8 / GW_)), gy0 = wy0 + GH * (grp / (8 / GW_));
-        lane_pixels<MODE, GH / 2>(P, w.el, W, H, gx0 + lg % GW_, gy0 + lg / GW_, L);
+        const int gx0 = wx0 + GPX * (grp % (8 / GPX)), gy0 = wy0 + GPY * (grp / (8 / GPX));
+        lane_pixels<MODE, GPY / 2>(P, w.el, W, H, gx0 + lg % GPX, gy0 + lg / GPX, L);
     }
     bool done0 = !L.in0, done1 = !L.in1;
     // the lane's two pixels: .x = (px, py0), .y = (px, py1)
@@ -838,16 +844,16 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
             }
             uint32_t m32;
             if constexpr (GROUPS) {  // per group: the splats whose box reaches it
-                bool cx[8 / GW_], cy[8 / GH];
+                bool cx[8 / GPX], cy[8 / GPY];
 #pragma unroll
-                for (int i = 0; i < 8 / GW_; ++i)
-                    cx[i] = ov && bx0 <= wx0 + GW_ * i + GW_ - 1 && bx1 >= wx0 + GW_ * i;
+                for (int i = 0; i < 8 / GPX; ++i)
+                    cx[i] = ov && bx0 <= wx0 + GPX * i + GPX - 1 && bx1 >= wx0 + GPX * i;
 #pragma unroll
-                for (int i = 0; i < 8 / GH; ++i) cy[i] = by0 <= wy0 + GH * i + GH - 1 && by1 >= wy0 + GH * i;
+                for (int i = 0; i < 8 / GPY; ++i) cy[i] = by0 <= wy0 + GPY * i + GPY - 1 && by1 >= wy0 + GPY * i;
                 m32 = 0u;
 #pragma unroll
                 for (int g = 0; g < 32 / GL; ++g) {
-                    const uint32_t b = __ballot_sync(kAll, cx[g % (8 / GW_)] && cy[g / (8 / GW_)]);
+                    const uint32_t b = __ballot_sync(kAll, cx[g % (8 / GPX)] && cy[g / (8 / GPX)]);
                     if (grp == g) m32 = b;
                 }
                 const uint32_t dm = __ballot_sync(kAll, done0 && done1);
