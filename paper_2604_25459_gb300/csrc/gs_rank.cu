@@ -24,32 +24,66 @@ constexpr int kSampleLooks = 8;     // slots looked at per thread of k_rank_samp
 constexpr int kSortThreads = 256;
 constexpr int kSortCap = 2048;      // keys of a window sorted in shared memory
 constexpr int kSubBins = 1024;      // depth ranges of a window's counting sort
-constexpr int kInsert = 32;         // longest range sorted by counting
+constexpr int kInsert = 128;        // longest range sorted by counting
 
-// Ascending bitonic sort of a[0, m), m a power of two, by the whole block.
-__device__ __forceinline__ void bitonic_sort(unsigned long long* a, int m) {
-    for (int size = 2; size <= m; size <<= 1)
+// Ascending bitonic sort of NT * K keys by a block of NT threads, thread t
+// holding elements K t .. K t + K - 1: exchanges stay in a thread or go by
+// shuffles below 32 K keys, through smp (NT * K keys) above.
+template <int NT, int K>
+__device__ __forceinline__ void block_bitonic(unsigned long long (&v)[K], unsigned long long* smp) {
+    const int tid = threadIdx.x;
+    for (int size = 2; size <= NT * K; size <<= 1)
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            __syncthreads();
-            for (int p = threadIdx.x; p < m / 2; p += blockDim.x) {
-                const int i = 2 * p - (p & (stride - 1)), j = i + stride;
-                const unsigned long long x = a[i], y = a[j];
-                if ((x > y) == ((i & size) == 0)) {
-                    a[i] = y;
-                    a[j] = x;
+            if (stride >= K) {
+                unsigned long long o[K];
+                if (stride >= 32 * K) {
+                    __syncthreads();
+#pragma unroll
+                    for (int k = 0; k < K; ++k) smp[k * NT + tid] = v[k];
+                    __syncthreads();
+#pragma unroll
+                    for (int k = 0; k < K; ++k) o[k] = smp[k * NT + (tid ^ (stride / K))];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < K; ++k) o[k] = __shfl_xor_sync(0xffffffffu, v[k], stride / K);
                 }
+                const bool low = (tid & (stride / K)) == 0;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const bool up = ((K * tid + k) & size) == 0;
+                    v[k] = (v[k] < o[k]) == (up == low) ? v[k] : o[k];
+                }
+            } else {
+#pragma unroll
+                for (int d = K / 2; d > 0; d >>= 1)
+                    if (stride == d) {
+#pragma unroll
+                        for (int k = 0; k < K; ++k) {
+                            const int j = k ^ d;
+                            if (j > k) {
+                                const bool up = ((K * tid + k) & size) == 0;
+                                const unsigned long long x = v[k], y = v[j];
+                                if ((x > y) == up) {
+                                    v[k] = y;
+                                    v[j] = x;
+                                }
+                            }
+                        }
+                    }
             }
         }
-    __syncthreads();
 }
 
 }  // namespace
 
 // One CTA of 1024 threads per env; K sampled keys per thread.  Bound by
-// latency: a strided gather, then a bitonic sort whose exchanges stay in
-// registers below 32 K keys, in shared memory above (15 of its stages).  The
-// stride is odd, so it does not resonate with the 32-slot visibility words or
-// the links' cluster sizes.
+// latency: a strided gather, a sort of the sample, then a search per depth cell.
+// The whole sample is used however few ranges there are: with two samples per
+// range, 8 views of 16,384 splats (32 ranges) had windows of over kSortCap keys
+// and k_rank_sort took 28 us instead of 10.  bins is a power of two, so a
+// splitter's place is a shift (640,000 slots, one env: 28 us with a 64-bit
+// division, 21 with the shift).  The stride is odd, so it does not resonate with
+// the 32-slot visibility words or the links' cluster sizes.
 template <int K>
 __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
     constexpr int M = 1024 * K;
@@ -58,7 +92,7 @@ __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
     const int el = blockIdx.x, tid = threadIdx.x;
     const EnvInfo E = P.envs[el];
     const uint32_t n = E.n_local;
-    const int want = min(2 * P.bins, M);
+    const int want = M;
     uint32_t step = (n + 1024 * kSampleLooks - 1) / (1024 * kSampleLooks);
     if (step > 1) step |= 1u;
     uint32_t seen = 0;  // bit k: slot (tid + 1024 k) step is visible
@@ -88,49 +122,15 @@ __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
     unsigned long long v[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = smp[K * tid + k];
-    for (int size = 2; size <= M; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride >= K) {
-                unsigned long long o[K];
-                if (stride >= 32 * K) {
-                    __syncthreads();
-#pragma unroll
-                    for (int k = 0; k < K; ++k) smp[k * 1024 + tid] = v[k];
-                    __syncthreads();
-#pragma unroll
-                    for (int k = 0; k < K; ++k) o[k] = smp[k * 1024 + (tid ^ (stride / K))];
-                } else {
-#pragma unroll
-                    for (int k = 0; k < K; ++k) o[k] = __shfl_xor_sync(0xffffffffu, v[k], stride / K);
-                }
-                const bool low = (tid & (stride / K)) == 0;
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const bool up = ((K * tid + k) & size) == 0;
-                    v[k] = (v[k] < o[k]) == (up == low) ? v[k] : o[k];
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const int j = k ^ stride;
-                    if (j > k) {
-                        const bool up = ((K * tid + k) & size) == 0;
-                        const unsigned long long a = v[k], b = v[j];
-                        if ((a > b) == up) {
-                            v[k] = b;
-                            v[j] = a;
-                        }
-                    }
-                }
-            }
-        }
+    block_bitonic<1024, K>(v, smp);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < K; ++k) smp[K * tid + k] = v[k];
     __syncthreads();
     unsigned long long* out = P.split + (size_t)el * P.bins;
+    const int lb = __ffs(P.bins) - 1;  // bins are a power of two
     auto splitter = [&](int k) -> unsigned long long {
-        return kept ? smp[min(kept - 1, (int)(((long long)(k + 1) * kept) / P.bins))] : ~0ull;
+        return kept ? smp[min(kept - 1, (int)((uint32_t)((k + 1) * kept) >> lb))] : ~0ull;
     };
     for (int k = tid; k < P.bins - 1; k += 1024) out[k] = splitter(k);
     // the lookup: equal depth cells from the smallest sample
@@ -191,8 +191,9 @@ __global__ void __launch_bounds__(256) k_rank_place(RankParams P) {
 // Sorts an env's windows of whole ranges (positions [win[v], win[v+1])) and
 // writes order and rank.  A window of at most kSortCap keys is sorted in
 // shared memory: a counting sort by kSubBins ranges of its depth bits, a key's
-// place in its range being the number of smaller keys in it, or a bitonic sort of the whole keys when a range
-// holds more than kInsert.  A larger window (a sample that missed a crowd) is
+// place in its range being the number of smaller keys in it (up to kInsert; a
+// face seen head-on crowds hundreds of keys into few ranges), or a bitonic sort
+// when a range holds more.  A larger window (a sample that missed a crowd) is
 // cut into pieces of at most kSortCap keys by radix selection over its keys.
 __global__ void __launch_bounds__(kSortThreads, 4) k_rank_sort(RankParams P) {
     constexpr int NT = kSortThreads;
@@ -257,13 +258,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_rank_sort(RankParams P) {
             crowded |= loc[j] > (uint32_t)kInsert;
         }
         if (__syncthreads_or(crowded)) {
-            int p = 1;
-            while (p < m) p <<= 1;
+            block_bitonic<NT, PT>(k, tmp);  // the keys in any order, ~0 beyond the last
 #pragma unroll
             for (int u = 0; u < PT; ++u)
-                if (tid + u * NT < p) tmp[tid + u * NT] = k[u];
-            bitonic_sort(tmp, p);
-            for (int i = tid; i < m; i += NT) put(first + (uint32_t)i, tmp[i]);
+                if (PT * tid + u < m) put(first + (uint32_t)(PT * tid + u), k[u]);
             __syncthreads();
             return;
         }
