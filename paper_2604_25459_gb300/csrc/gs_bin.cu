@@ -271,9 +271,10 @@ __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const ui
     }
 }
 
-// env_base[e] = sum_{e' < e} env_total[e'], env_base[We] = total
+// env_base[e] = sum_{e' < e} env_total[e'], env_base[We] = total; host_base
+// (pinned host memory, or null) gets the same.
 __global__ void __launch_bounds__(1024) k_scan_base(const unsigned long long* env_total, unsigned long long* env_base,
-                                                    int We) {
+                                                    unsigned long long* host_base, int We) {
     __shared__ unsigned long long wt[32];
     unsigned long long carry = 0;
     for (int base = 0; base < We; base += blockDim.x) {
@@ -281,29 +282,35 @@ __global__ void __launch_bounds__(1024) k_scan_base(const unsigned long long* en
         const unsigned long long v = e < We ? env_total[e] : 0ull;
         unsigned long long tot;
         const unsigned long long ex = block_exclusive_scan<unsigned long long>(v, wt, tot);
-        if (e < We) env_base[e] = carry + ex;
+        if (e < We) {
+            env_base[e] = carry + ex;
+            if (host_base) host_base[e] = carry + ex;
+        }
         carry += tot;
     }
-    if (threadIdx.x == 0) env_base[We] = carry;
+    if (threadIdx.x == 0) {
+        env_base[We] = carry;
+        if (host_base) host_base[We] = carry;
+    }
 }
 
 static_assert(kRankBins <= 2048, "two depth ranges per thread of the scan");
 
 cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
-                              unsigned long long* env_total, unsigned long long* env_base, int We,
-                              const RankParams& R, cudaStream_t st) {
+                              unsigned long long* env_total, unsigned long long* env_base,
+                              unsigned long long* host_base, int We, const RankParams& R, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
     k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, 1, R);
-    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, We);
+    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, host_base, We);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
-                        unsigned long long* env_total, unsigned long long* env_base, int We, int per,
-                        cudaStream_t st) {
+                        unsigned long long* env_total, unsigned long long* env_base,
+                        unsigned long long* host_base, int We, int per, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
     k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, per, RankParams{});
-    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, We);
+    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, host_base, We);
     return cudaGetLastError();
 }
 

@@ -93,6 +93,7 @@ struct gs_scene_s {
     gsb::DevBuf stage_rgb[2], stage_depth[2], stage_alpha[2], poses;
     unsigned long long* pinned = nullptr;
     size_t pinned_n = 0;
+    cudaEvent_t ev_totals = nullptr;  // recorded once pinned holds a wave's totals
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_done[2] = {nullptr, nullptr};
     cudaEvent_t ev_copied[2] = {nullptr, nullptr};
