@@ -467,7 +467,11 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     CK(sc.off.ensure(wt.tiles * 4), "alloc offsets");
     CK(sc.env_total.ensure((size_t)We * 8), "alloc totals");
     CK(sc.env_base.ensure(((size_t)We + 1) * 8), "alloc bases");
-    CK(sc.bins.ensure(rank_tables(R, We, nullptr)), "alloc depth ranges");
+    const int scatter_wpb = scatter_words(wt.max_words, We, wt.max_T);
+    const size_t table_bytes = rank_tables(R, We, nullptr);
+    size_t off_bytes = tile_off_bytes(R, scatter_wpb, We, wt.max_T, io.lidars != nullptr);
+    if (off_bytes > (size_t)s->budget / 64) off_bytes = 0;
+    CK(sc.bins.ensure(table_bytes + off_bytes), "alloc depth ranges");
     rank_tables(R, We, sc.bins.as<unsigned char>());
     CK(sc.zkeys.ensure(wt.recs * 8), "alloc depth keys");
     CK(sc.ranks.ensure(wt.recs * 8), "alloc ranks");
@@ -533,7 +537,11 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     B.e_begin = 0;
     B.tile_w = tw;
     B.tile_h = th;
-    B.words_per_block = scatter_words(wt.max_words, We, wt.max_T);
+    B.words_per_block = scatter_wpb;
+    if (off_bytes) {
+        B.tile_off = reinterpret_cast<uint32_t*>(sc.bins.as<unsigned char>() + table_bytes);
+        B.tile_pitch = (unsigned)wt.max_T;
+    }
     B.counts = counts;
     B.off_local = sc.off.as<uint32_t>();
     B.env_base = sc.env_base.as<unsigned long long>();

@@ -199,6 +199,10 @@ struct BinParams {
     uint32_t* status;
     int wrap;  // LiDAR: a box with x0 > x1 covers columns [x0, cols) and [0, x1]
     int key_shift;           // see CompParams
+    // nullable: per env, block and tile (tile_pitch of them) the block's place in
+    // the tile's bucket, where it has keys there; written by the count
+    uint32_t* tile_off;
+    unsigned int tile_pitch;
 };
 
 struct CompParams {
@@ -351,6 +355,12 @@ constexpr int kDiffTiles = 256;
 // L2 (256 envs: 8.5 us per env with 256, 7.15 with 64, 8.6 with 32); on small
 // grids the per-block tables weigh more (512 envs at 128x128: 2.3 us with 256,
 // 2.7 with 64).
+// Bytes of the places that the count notes for the scatter (BinParams::tile_off);
+// 0 where their blocks differ, and on grids counted by difference arrays.
+inline size_t tile_off_bytes(const RankParams& R, int words_per_block, int We, int max_T, bool wrap) {
+    if (words_per_block != R.words_per_block || (!wrap && max_T >= kDiffTiles)) return 0;
+    return (size_t)We * R.blocks * max_T * 4;
+}
 inline int scatter_words(long long max_words, int n_envs, int max_T) {
     int w = max_T >= kDiffTiles ? 64 : kWordsPerBlock;
     while (w > 16 && (max_words + w - 1) / w * n_envs < 62 * 152) w /= 2;

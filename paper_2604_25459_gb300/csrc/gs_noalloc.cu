@@ -258,6 +258,13 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.tile_w = tw;
         B.tile_h = th;
         B.words_per_block = scatter_words(max_words, Wn, max_T);
+        const size_t off_bytes = tile_off_bytes(R, B.words_per_block, Wn, max_T, false);
+        if (off_bytes && up256((size_t)(tab - base)) + off_bytes <= kNoAllocBytes) {
+            tab = base + up256((size_t)(tab - base));
+            B.tile_off = reinterpret_cast<uint32_t*>(tab);
+            B.tile_pitch = (unsigned)max_T;
+            tab += off_bytes;
+        }
         B.rank = R.rank;
         const bool warp = warp_form(tw, th, (long long)px);
         if (warp) B.key_shift = subtile_bits(tw, th, (unsigned long long)max_words * 32);
