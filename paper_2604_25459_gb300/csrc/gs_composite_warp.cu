@@ -1200,12 +1200,16 @@ static cudaError_t launch_warps(const CompParams& P, cudaStream_t st, int* ctas)
     // 1615 / 855 / 800 / 804, 48 (3.4) 1987 / 1462 / 1153 / 1145, 128 (9) 2488 /
     // 2282 / 2369 / 2583, 256 (18) 3922 / 3842 / 4461 / 5229, 512 (36) 6249 /
     // 7251 / 8503 / -; spinning LiDAR 1 env (0.3) 1011 / 1008 / 517 / 486, 32
-    // (11) 3984 / 3682 / 2853 / 3863, 128 (43) 8291 / 8697 / - / -.  Where every
-    // item has a CTA, all go to teams (a 128x96 view of 16k splats: 57 -> 39).
+    // (11) 3984 / 3682 / 2853 / 3863, 128 (43) 8291 / 8697 / - / -.  Where items
+    // are few per resident CTA, all go to teams (whole calls, us): one 128x96 view
+    // of 16,384 splats (0.2 items per CTA) 57 -> 39, 8 of them (1.7) 145 -> 122,
+    // 16 (3.4) 195 -> 173, but 2 views of 333x251 in the room (2.9) 351 -> 362 and
+    // 4 rosettes (1.7) 1403 -> 1465.
+    constexpr bool LID = MODE == 1 || MODE == 3;
     Q.team_classes = 0;
     if (P.items && P.team_work) {
         const double per_warp = (double)items / ((double)kWarps * full);
-        if (items <= (unsigned long long)full) Q.team_classes = kItemClasses;
+        if (items * 2 <= (LID ? 2ull : 5ull) * full) Q.team_classes = kItemClasses;
         else if (per_warp <= 6.0) Q.team_classes = 3;
         else if (MODE == 1 || MODE == 3) Q.team_classes = per_warp <= 12.0 ? 2 : 0;
         else if (per_warp <= 20.0) Q.team_classes = 1;
