@@ -483,7 +483,6 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     if (debug) CK(sc.dbg_hxy.ensure(wt.recs * 8), "alloc debug");
     uint32_t* const status = io.status ? io.status : s->status;
 
-    CK(cudaMemsetAsync(sc.counts.p, 0, n_zero * 4, st), "memset counters");  // ahead of the kernels' chain
     // A1: link composition
     PhaseTimer t1(s, st, GS_PHASE_LINK, timers);
     CK(launch_link_table(io.poses, wt.cams, wt.envs, We, wt.xf_items, sc.xf.as<LinkXf>(), status, st),
@@ -519,6 +518,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     t2.done(1);
     ++*launches;
     // A3: counts + scan, around the records' depth ranking
+    CK(cudaMemsetAsync(sc.counts.p, 0, n_zero * 4, st), "memset counters");
     R.envs = wt.envs;
     R.mask = P.mask;
     R.r3 = P.r3;

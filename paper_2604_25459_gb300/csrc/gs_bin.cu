@@ -131,7 +131,6 @@ __global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
     extern __shared__ __align__(16) unsigned char csm[];
     __shared__ uint16_t lst[32 * kWordsPerBlock];
     __shared__ uint32_t wtot[32];
-    chain_start();
     unsigned long long* split = reinterpret_cast<unsigned long long*>(csm);
     uint16_t* cell = reinterpret_cast<uint16_t*>(split + R.bins);
     uint32_t* zhist = reinterpret_cast<uint32_t*>(cell + R.cells);
@@ -195,7 +194,8 @@ cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, in
     auto launch = [&](auto fn) -> cudaError_t {
         const cudaError_t e = opt_in_smem((const void*)fn, smem);
         if (e != cudaSuccess) return e;
-        return launch_chained(fn, dim3((unsigned)R.blocks, (unsigned)n_envs), 256, smem, st, P, R);
+        fn<<<dim3((unsigned)R.blocks, (unsigned)n_envs), 256, smem, st>>>(P, R);
+        return cudaGetLastError();
     };
     if (P.wrap) return launch(k_count<true, false>);
     return diff ? launch(k_count<false, true>) : launch(k_count<false, false>);
@@ -237,7 +237,6 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* warp_tot, T& block_tot
 __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                                                    unsigned long long* env_total, int per, RankParams R) {
     __shared__ uint32_t wt[32];
-    chain_start();
     const int el = blockIdx.x;
     const int T = envs[el].T * per;
     const uint32_t* c = counts + (size_t)envs[el].tile_base * per;
@@ -280,7 +279,6 @@ __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const ui
 __global__ void __launch_bounds__(1024) k_scan_base(const unsigned long long* env_total, unsigned long long* env_base,
                                                     unsigned long long* host_base, int We) {
     __shared__ unsigned long long wt[32];
-    chain_start();
     unsigned long long carry = 0;
     for (int base = 0; base < We; base += blockDim.x) {
         const int e = base + threadIdx.x;
@@ -305,20 +303,18 @@ cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint3
                               unsigned long long* env_total, unsigned long long* env_base,
                               unsigned long long* host_base, int We, const RankParams& R, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
-    const cudaError_t e =
-        launch_chained(k_scan_env, dim3((unsigned)We), 1024, 0, st, envs, counts, off_local, env_total, 1, R);
-    if (e != cudaSuccess) return e;
-    return launch_chained(k_scan_base, dim3(1), 1024, 0, st, env_total, env_base, host_base, We);
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, 1, R);
+    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, host_base, We);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                         unsigned long long* env_total, unsigned long long* env_base,
                         unsigned long long* host_base, int We, int per, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
-    const cudaError_t e =
-        launch_chained(k_scan_env, dim3((unsigned)We), 1024, 0, st, envs, counts, off_local, env_total, per, RankParams{});
-    if (e != cudaSuccess) return e;
-    return launch_chained(k_scan_base, dim3(1), 1024, 0, st, env_total, env_base, host_base, We);
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, per, RankParams{});
+    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, host_base, We);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- item order
@@ -331,7 +327,6 @@ __global__ void __launch_bounds__(256) k_item_order(const EnvInfo* envs, int e_b
                                                     const uint32_t* item_cnt, const uint32_t* item_off,
                                                     const unsigned long long* item_base, uint32_t* items,
                                                     uint32_t pitch, uint32_t* class_cnt) {
-    chain_start();
     const int el = e_begin + blockIdx.y, t = blockIdx.x * 256 + threadIdx.x;
     const int T = envs[el].T;
     if (blockIdx.x * 256 >= (unsigned)T) return;
@@ -371,8 +366,9 @@ cudaError_t launch_item_order(const EnvInfo* envs, int e_begin, int n_envs, int 
                               const unsigned long long* item_base, uint32_t* items, uint32_t pitch,
                               uint32_t* class_cnt, cudaStream_t st) {
     if (n_envs == 0 || max_T == 0) return cudaSuccess;
-    return launch_chained(k_item_order, dim3((unsigned)((max_T + 255) / 256), (unsigned)n_envs), 256, 0, st, envs,
-                          e_begin, counts, item_cnt, item_off, item_base, items, pitch, class_cnt);
+    k_item_order<<<dim3((unsigned)((max_T + 255) / 256), (unsigned)n_envs), 256, 0, st>>>(
+        envs, e_begin, counts, item_cnt, item_off, item_base, items, pitch, class_cnt);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- scatter
@@ -412,7 +408,6 @@ __global__ void __launch_bounds__(256, 6) k_scatter(BinParams P) {  // <= 42 reg
     __shared__ uint16_t far[DIFF ? kLongList : 1];
     __shared__ uint32_t wtot[32];
     __shared__ uint32_t n_far;
-    chain_start();
     const int el = P.e_begin + blockIdx.y;
     const EnvInfo E = P.envs[el];
     const int64_t words = (E.n_local + 31) / 32;
@@ -501,8 +496,9 @@ cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int ma
     auto launch = [&](auto fn) -> cudaError_t {
         const cudaError_t e = opt_in_smem((const void*)fn, smem);
         if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)((max_words + P.words_per_block - 1) / P.words_per_block), (unsigned)n_envs);
-        return launch_chained(fn, grid, 256, smem, st, P);
+        fn<<<dim3((unsigned)((max_words + P.words_per_block - 1) / P.words_per_block), (unsigned)n_envs), 256, smem,
+             st>>>(P);
+        return cudaGetLastError();
     };
     if (P.wrap) return mask ? launch(k_scatter<true, true, false>) : launch(k_scatter<true, false, false>);
     if (diff) return mask ? launch(k_scatter<false, true, true>) : launch(k_scatter<false, false, true>);

@@ -7,36 +7,6 @@
 
 namespace gsb {
 
-// The kernels of a render form a chain on their stream, each reading what the
-// ones before it wrote.  Launched with launch_chained, a kernel is set up while
-// the one before it drains; every CTA first calls chain_start, which waits until
-// the kernel before this one has completed and its writes are visible.  As no
-// kernel of a chain completes before the one ahead of it, waiting for one is
-// waiting for all.  Kernels and copies launched in the ordinary way wait for
-// whole kernels as always.  A render has eleven short kernels at small sizes, and
-// what separates them costs as much as some of them take: one 128x96 view of
-// 16,384 splats 106 -> 87 us, 8 of them without allocation 186 -> 165, one
-// 640x480 view of 600,000 261 -> 244, 16 of 333x251 1078 -> 1049.  No kernel
-// lets the next come up before its own CTAs have finished: early CTAs wait in
-// place of working ones (512 views of 128x128 11.9 -> 12.2 ms, two streams of
-// requests 7.9 -> 11.7 ms).
-__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
-                           const A&... args) {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c{};
-    c.gridDim = grid;
-    c.blockDim = dim3(block);
-    c.dynamicSmemBytes = smem;
-    c.stream = st;
-    c.attrs = &at;
-    c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, kernel, P(args)...);
-}
-
 // Resident CTAs of a kernel on the current device, looked up once per device.
 struct PerDevice {
     int n[64] = {0};

@@ -193,7 +193,6 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
     static_assert(sizeof(recs) >= CAP * 4, "the sort scratch shares the records' memory");
     uint32_t* tmp = reinterpret_cast<uint32_t*>(recs);
     __shared__ unsigned int s_item;
-    chain_start();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     auto& rec = recs[warp];
     bool c32_dirty = true;  // the short-bucket sort's counters (bm) need clearing before use
@@ -534,7 +533,8 @@ static cudaError_t launch_tiles(const CompParams& P, cudaStream_t st, int* ctas)
     if (e != cudaSuccess) return e;
     const unsigned claims = (P.item_end - P.item_begin + P.chunk - 1) / P.chunk;
     *ctas = (int)std::min((unsigned)full, claims);
-    return launch_chained(k_composite<TW, TH, SC, CNT>, dim3((unsigned)*ctas), NT, 0, st, P);
+    k_composite<TW, TH, SC, CNT><<<*ctas, NT, 0, st>>>(P);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_composite(const CompParams& P, cudaStream_t st, int* ctas) {

@@ -705,7 +705,6 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
     auto& rec = sm.rec;
     auto& sD = sm.sD;
     auto& sR = sm.sR;
-    chain_start();
     const int lane = threadIdx.x & 31;
     const int lx = __ffs(P.tile_w) - 4, ly = __ffs(P.tile_h) - 4;  // log2 of the tile's subtile columns, rows
     const int lsub = MODE == 3 ? 0 : lx + ly;
@@ -1217,7 +1216,8 @@ static cudaError_t launch_warps(const CompParams& P, cudaStream_t st, int* ctas)
     // few claims: fewer warps per CTA, so that they spread over the SMs
     const int warps = Q.team_classes ? kWarps : (int)std::min((claims + full - 1) / full, (unsigned long long)kWarps);
     *ctas = (int)std::min((unsigned long long)full, Q.team_classes ? claims : (claims + warps - 1) / warps);
-    return launch_chained(k_composite_warp<MODE>, dim3((unsigned)*ctas), 32u * warps, 0, st, Q);
+    k_composite_warp<MODE><<<*ctas, 32 * warps, 0, st>>>(Q);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_composite_warp(const CompParams& P, cudaStream_t st, int* ctas) {

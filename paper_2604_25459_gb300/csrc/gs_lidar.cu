@@ -28,7 +28,7 @@
 // columns [x0, cols) and [0, x1], which the binning kernels and the
 // compositor's LiDAR forms read as two ranges (a box over every column
 // between them would put the Gaussian in every tile of its rows).
-#include "gs_block.cuh"
+#include "gs_internal.cuh"
 
 namespace gsb {
 
@@ -61,7 +61,6 @@ __device__ __forceinline__ uint32_t ray_quad(uint32_t cell) {
 }  // namespace
 
 __global__ void __launch_bounds__(256) k_project_lidar(ProjParams P) {
-    chain_start();
     const ProjBlock blk = P.blocks[blockIdx.x];
     const int t = threadIdx.x;
     const bool act = t < blk.n;
@@ -245,7 +244,8 @@ __global__ void __launch_bounds__(256) k_project_lidar(ProjParams P) {
 
 cudaError_t launch_project_lidar(const ProjParams& P, int n_blocks, cudaStream_t st) {
     if (n_blocks == 0) return cudaSuccess;
-    return launch_chained(k_project_lidar, dim3((unsigned)n_blocks), 256, 0, st, P);
+    k_project_lidar<<<n_blocks, 256, 0, st>>>(P);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- arbitrary rays

@@ -195,6 +195,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
               "copy block table");
         NA_CK(cudaMemcpyAsync(d_cams, cams + e0, sizeof(gs_camera) * (size_t)Wn, cudaMemcpyHostToDevice, st),
               "copy cams");
+        NA_CK(launch_link_table(link_poses, d_cams, d_envs, Wn, sen.xf_base, xf, v.status, st), "link table");
         ProjParams P{};
         P.n_gauss = v.D.n;
         P.p0 = v.D.p0;
@@ -213,6 +214,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         P.mask = reinterpret_cast<uint32_t*>(base + y.mask);
         P.dbg_hxy = nullptr;
         P.bg_index = v.bg_index;
+        NA_CK(launch_project(v.D, P, nb, st), "projection");
         // The part of the array behind the fixed tables: its first half holds the
         // intersection ranks (and, before they exist, the depth keys), its second
         // half the depth ranking.  A wave is accepted when 8 bytes per
@@ -250,6 +252,8 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         uint32_t* cursor = reinterpret_cast<uint32_t*>(base + y.cursor);
         auto* env_total = reinterpret_cast<unsigned long long*>(base + y.env_total);
         auto* env_base = reinterpret_cast<unsigned long long*>(base + y.env_base);
+        NA_CK(cudaMemsetAsync(counts, 0, (size_t)sen.tile_base * 4, st), "clear counts");
+        NA_CK(cudaMemsetAsync(R.bin_cnt, 0, n_bins * 4, st), "clear depth-range counts");
         BinParams B{};
         B.envs = d_envs;
         B.mask = P.mask;
@@ -273,12 +277,6 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.env_base = env_base;
         B.cursor = cursor;
         B.status = v.status;
-        // counters are cleared ahead of the kernels' chain
-        unsigned int* const work = reinterpret_cast<unsigned int*>(base + y.work);
-        NA_CK(cudaMemsetAsync(base + y.counts, 0, y.pairs - y.counts, st), "clear counters");  // to the work counters
-        NA_CK(cudaMemsetAsync(R.bin_cnt, 0, n_bins * 4, st), "clear depth-range counts");
-        NA_CK(launch_link_table(link_poses, d_cams, d_envs, Wn, sen.xf_base, xf, v.status, st), "link table");
-        NA_CK(launch_project(v.D, P, nb, st), "projection");
         NA_CK(launch_rank_sample(R, Wn, st), "depth sample");
         NA_CK(launch_count(B, R, Wn, max_T, (ntx + 1) * (nty + 1), st), "count");
         NA_CK(launch_scan_ranks(d_envs, counts, off, env_total, env_base, nullptr, Wn, R, st), "scan");
@@ -293,6 +291,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
                          "no-allocation scratch too small: %lld intersection keys need %lld bytes, %lld are free "
                          "(use gs_render_batch)",
                          (long long)eb[Wn], (long long)need, (long long)(kNoAllocBytes - y.pairs));
+        NA_CK(cudaMemsetAsync(cursor, 0, (size_t)sen.tile_base * 4, st), "clear cursors");
         B.pair_base = 0;
         B.pair_cap = (kNoAllocBytes - y.pairs) / 8;
         B.pairs = reinterpret_cast<uint32_t*>(base + y.pairs);
@@ -305,7 +304,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         C.item_end = sen.tile_base;
         C.chunk = 1;
         C.n_bg = (unsigned)v.D.n_bg;
-        C.work = work;
+        C.work = reinterpret_cast<unsigned int*>(base + y.work);
         C.r0 = P.r0;
         C.r1 = P.r1;
         C.r2 = P.r2;
@@ -329,6 +328,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         // the work counters, and behind the ranking's tables the warp form's item
         // order, where it fits
         C.team_work = C.work + 1;
+        NA_CK(cudaMemsetAsync(C.work, 0, 8 + 4 * kItemClasses, st), "clear work counters");
         uint32_t* const items = reinterpret_cast<uint32_t*>(base + up256((size_t)(tab - base)));
         if (warp && up256((size_t)(tab - base)) + (size_t)sen.tile_base * kItemClasses * 4 <= kNoAllocBytes) {
             NA_CK(launch_item_order(d_envs, 0, Wn, max_T, counts, nullptr, nullptr, nullptr, items, sen.tile_base,

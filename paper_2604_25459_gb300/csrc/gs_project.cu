@@ -5,7 +5,7 @@
 // forward pass that the batch renderer of Sec. III-C "Throughput Scaling"
 // builds on (step A2: projection of every (env, Gaussian) to a 2D conic with
 // view-dependent SH colour).
-#include "gs_block.cuh"
+#include "gs_internal.cuh"
 
 namespace gsb {
 
@@ -142,7 +142,6 @@ cudaError_t launch_prep(const float* mean, const float* quat, const void* log_sc
 
 __global__ void k_link_table(const float* poses, const gs_camera* cams, const EnvInfo* envs, int We, int n_items,
                              LinkXf* out, uint32_t* status) {
-    chain_start();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n_items) return;
     int lo = 0, hi = We - 1;  // env: last e with envs[e].xf_base <= idx
@@ -187,8 +186,8 @@ __global__ void k_link_table(const float* poses, const gs_camera* cams, const En
 cudaError_t launch_link_table(const float* poses, const gs_camera* cams, const EnvInfo* envs, int We, int n_items,
                               LinkXf* out, uint32_t* status, cudaStream_t st) {
     if (n_items == 0 || We == 0) return cudaSuccess;
-    return launch_chained(k_link_table, dim3((unsigned)(n_items + 127) / 128), 128, 0, st, poses, cams, envs, We,
-                          n_items, out, status);
+    k_link_table<<<(n_items + 127) / 128, 128, 0, st>>>(poses, cams, envs, We, n_items, out, status);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ A2: projection
@@ -385,7 +384,6 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
     // re-reading 192 bytes per visible pair through L1 and L2 is what bounded
     // the kernel.
     extern __shared__ uint4 s_sh[];  // [NP][256]
-    chain_start();
     const ProjBlock blk = P.blocks[blockIdx.x];
     const int t = threadIdx.x;
     const bool act = t < blk.n;
@@ -575,7 +573,8 @@ static cudaError_t launch_project_dt(const ProjParams& P, int n_blocks, cudaStre
     const cudaError_t e =
         cudaFuncSetAttribute((const void*)k_project<D, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_project<D, DT>, dim3((unsigned)n_blocks), 256, smem, st, P);
+    k_project<D, DT><<<n_blocks, 256, smem, st>>>(P);
+    return cudaGetLastError();
 }
 
 template <int D>

@@ -89,7 +89,6 @@ __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
     constexpr int M = 1024 * K;
     __shared__ unsigned long long smp[M];
     __shared__ uint32_t red[32];
-    chain_start();
     const int el = blockIdx.x, tid = threadIdx.x;
     const EnvInfo E = P.envs[el];
     const uint32_t n = E.n_local;
@@ -156,7 +155,6 @@ __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
 // the count, whose blocks this kernel shares.  Streams the records once.
 __global__ void __launch_bounds__(256) k_rank_place(RankParams P) {
     __shared__ uint32_t first[kRankBins];
-    chain_start();
     const int el = blockIdx.y, lane = threadIdx.x & 31;
     const EnvInfo E = P.envs[el];
     const uint32_t words = (E.n_local + 31) / 32;
@@ -206,7 +204,6 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_rank_sort(RankParams P) {
     __shared__ unsigned long long sel_lo, sel_hi;
     __shared__ uint32_t sel_n;
     __shared__ int sel_state;
-    chain_start();
     const int tid = threadIdx.x, el = blockIdx.y;
     const EnvInfo E = P.envs[el];
     const uint32_t nv = P.nvis[el];
@@ -373,17 +370,21 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_rank_sort(RankParams P) {
 
 cudaError_t launch_rank_sample(const RankParams& R, int n_envs, cudaStream_t st) {
     if (n_envs == 0) return cudaSuccess;
-    auto* fn = R.bins <= 512 ? k_rank_sample<1> : R.bins <= 1024 ? k_rank_sample<2> : k_rank_sample<4>;
-    return launch_chained(fn, dim3((unsigned)n_envs), 1024, 0, st, R);
+    if (R.bins <= 512) k_rank_sample<1><<<n_envs, 1024, 0, st>>>(R);
+    else if (R.bins <= 1024) k_rank_sample<2><<<n_envs, 1024, 0, st>>>(R);
+    else k_rank_sample<4><<<n_envs, 1024, 0, st>>>(R);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_rank(const RankParams& R, int n_envs, int max_words, cudaStream_t st) {
     if (n_envs == 0 || max_words == 0) return cudaSuccess;
-    const cudaError_t e = launch_chained(k_rank_place, dim3((unsigned)R.blocks, (unsigned)n_envs), 256, 0, st, R);
+    k_rank_place<<<dim3((unsigned)R.blocks, (unsigned)n_envs), 256, 0, st>>>(R);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // a CTA per window while an env's windows are few; the others loop
     const unsigned wins = (unsigned)std::min((long long)(max_words * 32ll + kRankStride - 1) / kRankStride, 160ll);
-    return launch_chained(k_rank_sort, dim3(wins, (unsigned)n_envs), kSortThreads, 0, st, R);
+    k_rank_sort<<<dim3(wins, (unsigned)n_envs), kSortThreads, 0, st>>>(R);
+    return cudaGetLastError();
 }
 
 }  // namespace gsb
