@@ -1740,7 +1740,7 @@ gs_status gs_debug_copy_records(gs_scene s, int env, uint8_t* visible, float* u,
     const int64_t n_local = E.n_local, nbp = bg_slots(s->D.n_bg);
     const int64_t lg0 = s->D.n_bg + s->link_offsets[E.link_begin];
     std::vector<uint32_t> mask((n_local + 31) / 32);
-    std::vector<float4> a(n_local), b(n_local), c(n_local);
+    std::vector<float4> a(n_local), b(n_local), c(n_local), attr(s->D.n);
     std::vector<float2> h(n_local);
     CK(cudaMemcpy(mask.data(), s->sc.mask.as<uint32_t>() + E.mask_base, mask.size() * 4, cudaMemcpyDeviceToHost),
        "copy");
@@ -1750,6 +1750,8 @@ gs_status gs_debug_copy_records(gs_scene s, int env, uint8_t* visible, float* u,
     CK(cudaMemcpy2D(b.data(), 16, rec + 1, pitch, 16, n_local, cudaMemcpyDeviceToHost), "copy");
     CK(cudaMemcpy2D(c.data(), 16, rec + 2, pitch, 16, n_local, cudaMemcpyDeviceToHost), "copy");
     CK(cudaMemcpy(h.data(), s->sc.dbg_hxy.as<float2>() + E.rec_base, n_local * 8, cudaMemcpyDeviceToHost), "copy");
+    // records hold log2(opacity): the attributes hold the opacity itself
+    CK(cudaMemcpy(attr.data(), s->D.p0, attr.size() * 16, cudaMemcpyDeviceToHost), "copy");
     if (visible) memset(visible, 0, (size_t)s->D.n);
     for (int64_t j = 0; j < n_local; ++j) {
         if (j >= s->D.n_bg && j < nbp) continue;  // padding slots
@@ -1759,7 +1761,7 @@ gs_status gs_debug_copy_records(gs_scene s, int env, uint8_t* visible, float* u,
         if (!vis) continue;
         if (u) u[g] = a[j].x;
         if (v) v[g] = a[j].y;
-        if (opacity) opacity[g] = a[j].z;
+        if (opacity) opacity[g] = attr[j < nbp ? j : lg0 + (j - nbp)].w;
         if (z) z[g] = a[j].w;
         if (conic) {  // records hold L with L^T L = conic * 0.5 log2(e) (upper triangular)
             const double k2 = 0.72134752044448170;

@@ -286,13 +286,12 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                     // kept as it is: it overstates the ellipse least).
                     bool ov = false, bright = false;
                     if (slot < n_local) {
-                        float4 A = sA[lane], B = sB[lane];
+                        const float4 A = sA[lane];
+                        float4 B = sB[lane];
                         const uint32_t rx = __float_as_uint(B.w), ry = __float_as_uint(sC[lane].w);
                         const int bx0 = (int)(rx & 0xffffu), bx1 = (int)(rx >> 16);
                         const int by0 = (int)(ry & 0xffffu), by1 = (int)(ry >> 16);
                         ov = bx0 <= wx1 && bx1 >= wx0 && by0 <= wy1 && by1 >= wy0;
-                        A.z = log2f(A.z);  // folded into the exponent of alpha
-                        sA[lane].z = A.z;
                         bright = ov && A.z > -0.029146346f;  // log2(0.98)
                         if (ov && bx1 - bx0 + by1 - by0 >= 24) {
                             // alpha >= 1/255 iff q <= w = log2(255 o); the cull's 1e-3
@@ -308,7 +307,6 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                     // with q >= 0), so a chunk without brighter splats walks a copy of the
                     // loop without the cap.
                     const bool clamp_chunk = __any_sync(0xffffffffu, bright);
-                    __syncwarp();  // the staged log2(o)
                     // One step blends two splats (TWO): their four alpha evaluations are
                     // independent, the blends run in depth order; an odd last splat has a
                     // step of its own.  No per-pixel box test: a pixel outside a splat's

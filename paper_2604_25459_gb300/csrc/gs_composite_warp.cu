@@ -525,7 +525,7 @@ __device__ __forceinline__ void team_item(const CompParams& P, TeamSmem<MODE == 
                     sm.st[2][tid] = q2;
                     sm.sD[tid] = third_row(q1, q2, __uint_as_float(__ldg(&P.r3[bk.recbase + g].w)));
                 } else {
-                    sm.st[0][tid] = make_float4(q0.x, q0.y, log2f(q0.z), q0.w);
+                    sm.st[0][tid] = q0;
                     sm.st[2][tid] = make_float4(q2.x, q2.y, q2.z, q0.w);
                 }
                 sm.st[1][tid] = q1;
@@ -823,9 +823,6 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
                     sD[lane] = third_row(q1, sC[lane], __uint_as_float(__ldg(&P.r3[bk.recbase + slot].w)));
                     unwrap_box(tx, bx0, bx1);
                     sR[lane] = make_int4(bx0, bx1 - bx0, by0, by1 - by0);
-                } else {
-                    const float o = sA[lane].z;
-                    sA[lane].z = log2f(o);  // folded into the exponent of alpha
                 }
                 ov = bx0 <= wx1 && bx1 >= wx0 && by0 <= wy1 && by1 >= wy0;
             }

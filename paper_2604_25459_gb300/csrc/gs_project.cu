@@ -398,6 +398,11 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
         a2 = __ldg(P.p2 + g);
         a3 = __ldg(P.p3 + g);
     }
+    // The record carries log2(opacity), which the compositor folds into the
+    // exponent of alpha: once per Gaussian here instead of once per staged splat
+    // there (256 views of 640x480: 14.83 -> 14.55 ms a call; 512 of 128x128: 11.63 ->
+    // 11.48).
+    const float log2o = log2f(a0.w);
     const int li = __float_as_int(a3.w) - blk.lb;  // frame offset within the env's link table
     const float qstar = a3.y;
     const bool live = act && qstar >= 0.0f;
@@ -542,7 +547,7 @@ __global__ void __launch_bounds__(256, 3) k_project(ProjParams P) {
                         const uint32_t ry = (uint32_t)j0 | ((uint32_t)j1 << 16);
                         const size_t ri = (size_t)s_rb[ei] + local;
                         float4* sr = s_rec[t >> 5] + 3 * lane;
-                        sr[0] = make_float4(u, v, a0.w, mz);
+                        sr[0] = make_float4(u, v, log2o, mz);
                         sr[1] = make_float4(l00, l01, l11, __uint_as_float(rx));
                         sr[2] = make_float4(r, gg, b, __uint_as_float(ry));
                         P.r3[ri] = make_uint4(rx, ry, __float_as_uint(mz), key_index);
