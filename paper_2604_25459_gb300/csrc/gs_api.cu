@@ -479,6 +479,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     uint32_t* const counts = R.bin_cnt + n_bins;
     uint32_t* const cursor = counts + wt.tiles;
     uint32_t* const work = cursor + wt.tiles;
+    uint32_t* const ticket = work + kWorkWords - 1;  // the scans'
     const bool debug = s->debug && cap == 0;
     if (debug) CK(sc.dbg_hxy.ensure(wt.recs * 8), "alloc debug");
     uint32_t* const status = io.status ? io.status : s->status;
@@ -575,10 +576,10 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     unsigned long long* const h_items = h_keys ? h_keys + We + 1 : nullptr;
     PhaseTimer t4(s, st, GS_PHASE_SCAN, timers);
     CK(launch_scan_ranks(wt.envs, counts, sc.off.as<uint32_t>(), sc.env_total.as<unsigned long long>(),
-                         sc.env_base.as<unsigned long long>(), h_keys, We, R, st),
+                         sc.env_base.as<unsigned long long>(), h_keys, ticket, We, R, st),
        "scan");
-    t4.done(2);
-    *launches += 4;
+    t4.done(1);
+    *launches += 3;
     // arbitrary rays: cells, rays grouped by tile, compositor items (eager only)
     if (io.ray_dirs) {
         if (cap != 0) return fail(GS_ERR_UNSUPPORTED, "arbitrary-ray scans are not planned");
@@ -596,18 +597,18 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
                             s->ray_cnt.as<uint32_t>(), status, st),
            "ray cells");
         CK(launch_scan(wt.envs, s->ray_cnt.as<uint32_t>(), s->ray_off.as<uint32_t>(),
-                       s->ray_tot.as<unsigned long long>(), s->ray_base.as<unsigned long long>(), nullptr, We,
-                       kRayGroups, st),
+                       s->ray_tot.as<unsigned long long>(), s->ray_base.as<unsigned long long>(), nullptr,
+                       ticket, We, kRayGroups, st),
            "ray scan");
         CK(launch_ray_scatter(wt.envs, We, io.n_rays, s->ray_cell.as<uint32_t>(), s->ray_off.as<uint32_t>(),
                               s->ray_cur.as<uint32_t>(), s->ray_list.as<uint32_t>(), s->ray_cnt.as<uint32_t>(),
                               s->item_cnt.as<uint32_t>(), (unsigned)wt.tiles, st),
            "ray lists");
         CK(launch_scan(wt.envs, s->item_cnt.as<uint32_t>(), s->item_off.as<uint32_t>(),
-                       s->item_tot.as<unsigned long long>(), s->item_base.as<unsigned long long>(), h_items, We, 1, st),
+                       s->item_tot.as<unsigned long long>(), s->item_base.as<unsigned long long>(), h_items, ticket, We, 1, st),
            "item scan");
-        tr.done(7);
-        *launches += 7;
+        tr.done(5);
+        *launches += 5;
     }
     if (cap == 0) CK(cudaEventRecord(s->ev_totals, st), "record totals");
     PhaseTimer t4r(s, st, GS_PHASE_SCAN, timers);

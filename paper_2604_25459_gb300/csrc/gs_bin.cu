@@ -230,13 +230,43 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* warp_tot, T& block_tot
     return before + x - v;
 }
 
-// per env: off_local[t] = sum_{t' < t} counts[t'], env_total = sum.  With R
+// Bases of the envs, by one CTA: env_base[e] = sum_{e' < e} env_total[e'],
+// env_base[We] = total; host_base (pinned host memory, or null) gets the same.
+struct EnvBases {
+    unsigned long long *total, *base, *host;
+    unsigned int* ticket;  // CTAs done; 0 before and after the launch
+};
+__device__ __forceinline__ void scan_bases(const EnvBases& B, int We) {
+    __shared__ unsigned long long wt[32];
+    unsigned long long carry = 0;
+    for (int first = 0; first < We; first += blockDim.x) {
+        const int e = first + threadIdx.x;
+        const unsigned long long v = e < We ? __ldcg(B.total + e) : 0ull;
+        unsigned long long tot;
+        const unsigned long long ex = block_exclusive_scan<unsigned long long>(v, wt, tot);
+        if (e < We) {
+            B.base[e] = carry + ex;
+            if (B.host) B.host[e] = carry + ex;
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) {
+        B.base[We] = carry;
+        if (B.host) B.host[We] = carry;
+        *B.ticket = 0u;
+    }
+}
+
+// per env: off_local[t] = sum_{t' < t} counts[t'], total = sum.  With R
 // (bins > 0), also the offsets of the env's depth ranges, the number of ranked
 // records, and the window table: win[v] is the first range start >= v
-// kRankStride, so a window is at most kRankStride plus its last range.
+// kRankStride, so a window is at most kRankStride plus its last range.  The CTA
+// that finishes last scans the envs' totals (a kernel of its own for that cost a
+// launch: one 128x96 view 104 -> 102 us, 8 without allocation 162 -> 158).
 __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
-                                                   unsigned long long* env_total, int per, RankParams R) {
+                                                   EnvBases B, int per, RankParams R) {
     __shared__ uint32_t wt[32];
+    __shared__ bool last;
     const int el = blockIdx.x;
     const int T = envs[el].T * per;
     const uint32_t* c = counts + (size_t)envs[el].tile_base * per;
@@ -250,7 +280,14 @@ __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const ui
         if (t < T) o[t] = carry + ex;
         carry += tot;
     }
-    if (threadIdx.x == 0) env_total[el] = carry;
+    if (threadIdx.x == 0) {
+        B.total[el] = carry;
+        __threadfence();
+        last = atomicAdd(B.ticket, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (last) scan_bases(B, (int)gridDim.x);
     if (R.bins == 0) return;
     // two neighbouring ranges per thread
     const int b = 2 * threadIdx.x;
@@ -274,46 +311,22 @@ __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const ui
     }
 }
 
-// env_base[e] = sum_{e' < e} env_total[e'], env_base[We] = total; host_base
-// (pinned host memory, or null) gets the same.
-__global__ void __launch_bounds__(1024) k_scan_base(const unsigned long long* env_total, unsigned long long* env_base,
-                                                    unsigned long long* host_base, int We) {
-    __shared__ unsigned long long wt[32];
-    unsigned long long carry = 0;
-    for (int base = 0; base < We; base += blockDim.x) {
-        const int e = base + threadIdx.x;
-        const unsigned long long v = e < We ? env_total[e] : 0ull;
-        unsigned long long tot;
-        const unsigned long long ex = block_exclusive_scan<unsigned long long>(v, wt, tot);
-        if (e < We) {
-            env_base[e] = carry + ex;
-            if (host_base) host_base[e] = carry + ex;
-        }
-        carry += tot;
-    }
-    if (threadIdx.x == 0) {
-        env_base[We] = carry;
-        if (host_base) host_base[We] = carry;
-    }
-}
-
 static_assert(kRankBins <= 2048, "two depth ranges per thread of the scan");
 
 cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                               unsigned long long* env_total, unsigned long long* env_base,
-                              unsigned long long* host_base, int We, const RankParams& R, cudaStream_t st) {
+                              unsigned long long* host_base, unsigned int* ticket, int We, const RankParams& R,
+                              cudaStream_t st) {
     if (We == 0) return cudaSuccess;
-    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, 1, R);
-    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, host_base, We);
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, EnvBases{env_total, env_base, host_base, ticket}, 1, R);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                         unsigned long long* env_total, unsigned long long* env_base,
-                        unsigned long long* host_base, int We, int per, cudaStream_t st) {
+                        unsigned long long* host_base, unsigned int* ticket, int We, int per, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
-    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, env_total, per, RankParams{});
-    k_scan_base<<<1, 1024, 0, st>>>(env_total, env_base, host_base, We);
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, EnvBases{env_total, env_base, host_base, ticket}, per, RankParams{});
     return cudaGetLastError();
 }
 

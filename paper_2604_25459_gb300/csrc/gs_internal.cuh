@@ -294,14 +294,16 @@ cudaError_t launch_ray_scatter(const EnvInfo* envs, int We, int n_rays, const ui
 cudaError_t launch_count(const BinParams& P, const RankParams& R, int n_envs, int max_T, int max_hist,
                          cudaStream_t st);
 // per: counters per tile (counts and off_local hold per T from per tile_base).
-// host_base: pinned host memory that gets a copy of env_base, or null.
+// host_base: pinned host memory that gets a copy of env_base, or null; ticket: a
+// word that holds 0, and does so again afterwards.
 cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                         unsigned long long* env_total, unsigned long long* env_base,
-                        unsigned long long* host_base, int We, int per, cudaStream_t st);
+                        unsigned long long* host_base, unsigned int* ticket, int We, int per, cudaStream_t st);
 // As launch_scan, with the scans of the depth ranges and their window tables.
 cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                               unsigned long long* env_total, unsigned long long* env_base,
-                              unsigned long long* host_base, int We, const RankParams& R, cudaStream_t st);
+                              unsigned long long* host_base, unsigned int* ticket, int We, const RankParams& R,
+                              cudaStream_t st);
 cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int max_T, int max_hist, cudaStream_t st);
 // Lists a launch's items by the length of their buckets, longest class first
 // (CompParams::items); class_cnt is zeroed by the caller.  Rays: item_cnt and

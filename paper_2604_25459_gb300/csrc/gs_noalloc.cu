@@ -252,7 +252,9 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         uint32_t* cursor = reinterpret_cast<uint32_t*>(base + y.cursor);
         auto* env_total = reinterpret_cast<unsigned long long*>(base + y.env_total);
         auto* env_base = reinterpret_cast<unsigned long long*>(base + y.env_base);
-        NA_CK(cudaMemsetAsync(counts, 0, (size_t)sen.tile_base * 4, st), "clear counts");
+        // counts to work counters: one region
+        NA_CK(cudaMemsetAsync(base + y.counts, 0, y.pairs - y.counts, st), "clear counters");
+        unsigned int* const work = reinterpret_cast<unsigned int*>(base + y.work);
         NA_CK(cudaMemsetAsync(R.bin_cnt, 0, n_bins * 4, st), "clear depth-range counts");
         BinParams B{};
         B.envs = d_envs;
@@ -279,7 +281,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.status = v.status;
         NA_CK(launch_rank_sample(R, Wn, st), "depth sample");
         NA_CK(launch_count(B, R, Wn, max_T, (ntx + 1) * (nty + 1), st), "count");
-        NA_CK(launch_scan_ranks(d_envs, counts, off, env_total, env_base, nullptr, Wn, R, st), "scan");
+        NA_CK(launch_scan_ranks(d_envs, counts, off, env_total, env_base, nullptr, work + kWorkWords - 1, Wn, R, st), "scan");
         NA_CK(launch_rank(R, Wn, max_words, st), "depth ranks");
         unsigned long long eb[kMaxWave + 1];
         NA_CK(cudaMemcpyAsync(eb, env_base, sizeof(unsigned long long) * (Wn + 1), cudaMemcpyDeviceToHost, st),
@@ -291,7 +293,6 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
                          "no-allocation scratch too small: %lld intersection keys need %lld bytes, %lld are free "
                          "(use gs_render_batch)",
                          (long long)eb[Wn], (long long)need, (long long)(kNoAllocBytes - y.pairs));
-        NA_CK(cudaMemsetAsync(cursor, 0, (size_t)sen.tile_base * 4, st), "clear cursors");
         B.pair_base = 0;
         B.pair_cap = (kNoAllocBytes - y.pairs) / 8;
         B.pairs = reinterpret_cast<uint32_t*>(base + y.pairs);
@@ -304,7 +305,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         C.item_end = sen.tile_base;
         C.chunk = 1;
         C.n_bg = (unsigned)v.D.n_bg;
-        C.work = reinterpret_cast<unsigned int*>(base + y.work);
+        C.work = work;
         C.r0 = P.r0;
         C.r1 = P.r1;
         C.r2 = P.r2;
@@ -328,7 +329,6 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         // the work counters, and behind the ranking's tables the warp form's item
         // order, where it fits
         C.team_work = C.work + 1;
-        NA_CK(cudaMemsetAsync(C.work, 0, 8 + 4 * kItemClasses, st), "clear work counters");
         uint32_t* const items = reinterpret_cast<uint32_t*>(base + up256((size_t)(tab - base)));
         if (warp && up256((size_t)(tab - base)) + (size_t)sen.tile_base * kItemClasses * 4 <= kNoAllocBytes) {
             NA_CK(launch_item_order(d_envs, 0, Wn, max_T, counts, nullptr, nullptr, nullptr, items, sen.tile_base,
