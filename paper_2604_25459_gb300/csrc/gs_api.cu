@@ -451,7 +451,9 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     int n_warp = io.lidars ? We : 0;
     if (!io.lidars && !io.score && quad != 0) {
         auto small = [&](int e) {
-            return warp_form(tw, th, quad < 0 ? (long long)wt.host_envs[e].W * wt.host_envs[e].H : 0);
+            if (quad >= 0) return warp_form(tw, th, 0, kQuadMinSlots, We);
+            return warp_form(tw, th, (long long)wt.host_envs[e].W * wt.host_envs[e].H, wt.max_words * 32ll,
+                             We);
         };
         while (n_warp < We && small(n_warp)) ++n_warp;
         for (int e = n_warp; e < We; ++e)
@@ -613,8 +615,9 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     if (cap == 0) CK(cudaEventRecord(s->ev_totals, st), "record totals");
     PhaseTimer t4r(s, st, GS_PHASE_SCAN, timers);
     CK(launch_rank(R, We, wt.max_words, st), "depth ranks");
-    t4r.done(2);
-    *launches += 2;
+    const int rank_launches = R.bins ? 2 : 0;
+    t4r.done(rank_launches);
+    *launches += rank_launches;
 
     // sub-waves of envs whose keys fit (eager), or the whole wave (planned)
     std::vector<unsigned long long> ebv;
@@ -1497,8 +1500,8 @@ gs_status gs_plan_launch(gs_plan p, const float* link_poses, float* rgb, float* 
             // largest images are beyond its range, for the envs within it (claim
             // size 1, as both forms claim best).
             const gs_camera &first = p->envs.front().cam, &most = p->envs.back().cam;
-            const bool mixed = warp_form(16, 16, (long long)first.width * first.height) &&
-                               !warp_form(16, 16, (long long)most.width * most.height);
+            const bool mixed = warp_form(16, 16, (long long)first.width * first.height, kQuadMinSlots, 1) &&
+                               !warp_form(16, 16, (long long)most.width * most.height, kQuadMinSlots, 1);
             const int shapes[5][2] = {{16, 16}, {32, 8}, {16, 8}, {8, 8}, {32, 16}};
             for (auto& sh : shapes)
                 for (int ch : {1, 4}) {

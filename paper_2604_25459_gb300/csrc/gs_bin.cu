@@ -150,15 +150,17 @@ __global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
     const uint4* gc = reinterpret_cast<const uint4*>(R.cell + (size_t)el * R.cells);
     for (int c = threadIdx.x; c < R.cells / 8; c += blockDim.x) reinterpret_cast<uint4*>(cell)[c] = gc[c];
     const int nvis = block_visible(P.mask + E.mask_base, w0, w1, lst, wtot);
-    const uint32_t z0 = (uint32_t)split[R.bins - 1];
-    const int zshift = (int)(split[R.bins - 1] >> 32);
+    const uint32_t z0 = R.bins ? (uint32_t)split[R.bins - 1] : 0u;
+    const int zshift = R.bins ? (int)(split[R.bins - 1] >> 32) : 0;
     const uint4* r3 = P.r3 + E.rec_base;
     const int sx = __ffs(P.tile_w) - 1, sy = __ffs(P.tile_h) - 1;
     for (int i = threadIdx.x; i < nvis; i += blockDim.x) {
         const uint32_t j = (uint32_t)(w0 * 32) + lst[i];
         const uint4 q = r3[j];
-        const uint32_t b = (uint32_t)rank_bin(split, cell, R.cells, R.bins, z0, zshift, rank_key(R, q, j));
-        R.rank[E.rec_base + j] = b << 13 | atomicAdd(&zhist[b], 1u);
+        if (R.bins) {
+            const uint32_t b = (uint32_t)rank_bin(split, cell, R.cells, R.bins, z0, zshift, rank_key(R, q, j));
+            R.rank[E.rec_base + j] = b << 13 | atomicAdd(&zhist[b], 1u);
+        }
         add_box<WRAP, DIFF>(q.x, q.y, sx, sy, ntx, hist);
     }
     if constexpr (DIFF) block_sum2d(hist, ntx, nty);

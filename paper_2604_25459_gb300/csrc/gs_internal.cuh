@@ -156,7 +156,8 @@ struct RankParams {
     const EnvInfo* envs;
     const uint32_t* mask;
     const uint4* r3;
-    int bins;                     // key ranges per env: a power of two, <= kRankBins
+    long long max_slots;          // of the largest env
+    int bins;                     // key ranges per env: a power of two, <= kRankBins; 0: envs are ranked whole
     int cells;                    // depth cells of the range lookup: a power of two
     int win_pitch;                // window table entries per env
     int words_per_block;          // of the count and of the placement (the same blocks)
@@ -327,6 +328,9 @@ constexpr int kRankBins = 2048;      // depth ranges per env, at most
 constexpr int kRankStride = 768;     // ranks per window of the depth sort
 // Depth ranges of an env of n record slots: one per 512 slots for cameras
 // (which see a quarter of a room), one per 256 for LiDARs (which see all of it).
+// Envs of at most this many slots are ranked whole (up to 4096 was slower: 64
+// envs of 3000 splats at 64x48 151 us a call, by sampling 143).
+constexpr int kSmallRank = 2048;
 inline int rank_bins(long long n, bool lidar) {
     const int most = lidar ? kRankBins : kRankBins / 2;
     int b = 32;
@@ -338,7 +342,8 @@ inline int rank_bins(long long n, bool lidar) {
 // than two per range (a block keeps an offset per range).
 inline RankParams rank_sizes(long long max_words, int We, bool lidar) {
     RankParams R{};
-    R.bins = rank_bins(max_words * 32, lidar);
+    R.max_slots = max_words * 32;
+    R.bins = R.max_slots <= kSmallRank ? 0 : rank_bins(R.max_slots, lidar);
     R.cells = R.bins < 1024 ? 4 * R.bins : 4096;
     R.win_pitch = (int)(max_words * 32 / kRankStride) + 2;
     int w = kWordsPerBlock;
@@ -394,8 +399,15 @@ constexpr int kCompCap = 768;
 // 837 / 776, 64 2290 / 2152; 480x360: 160 / 174, 419 / 352, 835 / 833, 2617 /
 // 2658; 640x480: 155 / 200, 379 / 475, 1007 / 1097, 3399 / 3859.
 constexpr int kQuadMaxPixels = 140000;
-inline bool warp_form(int tile_w, int tile_h, long long most_pixels) {
-    return ((tile_w == 16 && tile_h == 16) || (tile_w == 8 && tile_h == 8)) && most_pixels <= kQuadMaxPixels;
+// A few envs of few slots have short buckets, which the CTA form sorts at once,
+// without an item order.  Calls, warp / CTA form (us): 24 envs of 1500 splats at
+// 64x48 106 / 94, of 4000 at 128x96 132 / 123, of 6000 at 40x30 158 / 236; 64 of
+// 3000 at 64x48 142 / 132, 200 of 2000 160 / 172.
+constexpr long long kQuadMinSlots = 4097;
+constexpr int kQuadMinEnvs = 128;
+inline bool warp_form(int tile_w, int tile_h, long long most_pixels, long long most_slots, int n_envs) {
+    return ((tile_w == 16 && tile_h == 16) || (tile_w == 8 && tile_h == 8)) && most_pixels <= kQuadMaxPixels &&
+           (most_slots >= kQuadMinSlots || n_envs > kQuadMinEnvs);
 }
 // Bits of the subtile mask below the ranks of the warp form's keys: one per 8x8
 // subtile while they and the ranks of n_slots records fit 32 bits, else none.

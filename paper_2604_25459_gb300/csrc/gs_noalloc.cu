@@ -255,7 +255,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         // counts to work counters: one region
         NA_CK(cudaMemsetAsync(base + y.counts, 0, y.pairs - y.counts, st), "clear counters");
         unsigned int* const work = reinterpret_cast<unsigned int*>(base + y.work);
-        NA_CK(cudaMemsetAsync(R.bin_cnt, 0, n_bins * 4, st), "clear depth-range counts");
+        if (n_bins) NA_CK(cudaMemsetAsync(R.bin_cnt, 0, n_bins * 4, st), "clear depth-range counts");
         BinParams B{};
         B.envs = d_envs;
         B.mask = P.mask;
@@ -272,7 +272,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
             tab += off_bytes;
         }
         B.rank = R.rank;
-        const bool warp = warp_form(tw, th, (long long)px);
+        const bool warp = warp_form(tw, th, (long long)px, max_words * 32ll, Wn);
         if (warp) B.key_shift = subtile_bits(tw, th, (unsigned long long)max_words * 32);
         B.counts = counts;
         B.off_local = off;

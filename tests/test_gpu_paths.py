@@ -54,6 +54,15 @@ def test_ranking_of_crowded_depths(n, depths):
     assert vis > 0 or n == 1
 
 
+@pytest.mark.parametrize("n", [0, 32, 1024, 1025, 2048, 2049])
+def test_ranking_of_small_scenes(n):
+    """Scenes ranked whole by one block, up to 2048 slots, and the first above."""
+    w = synth.make_c0(n=max(n, 1))
+    if n == 0:  # nothing visible
+        w = dataclasses.replace(w, background=dataclasses.replace(w.background, mean=w.background.mean - [0, 0, 9]))
+    assert (_check_lists(w, (16, 16), 128, 96) > 0) == (n > 0)
+
+
 @pytest.mark.parametrize("width,height,tile", [(255, 240, (16, 16)), (257, 241, (16, 16)), (641, 479, (16, 16)),
                                                (129, 121, (8, 8)), (333, 251, (32, 8)), (520, 33, (16, 8))])
 def test_binning_of_long_spans(width, height, tile):
@@ -148,6 +157,7 @@ def test_lidar_boxes_hold_near_and_steep_gaussians(rows, cols):
 
 
 @pytest.mark.parametrize("n,width,height,E", [(300, 40, 24, 1), (16_384, 128, 96, 3), (17_001, 129, 97, 2),
+                                              (1500, 64, 48, 24), (700, 40, 24, 130),
                                               (30_000, 400, 360, 1)])
 def test_noalloc_is_the_batched_render(n, width, height, E):
     import torch
