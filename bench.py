@@ -39,9 +39,9 @@ UNIT = "env-frames/s"
 # (dram__bytes_read.sum + dram__bytes_write.sum over a 32-env launch, divided
 # by 32), valid only for the compositor sources it was taken on (the hash
 # below; sources that differ from the captured ones in comments only keep it).
-COMPOSITE_TRAFFIC_PER_ENV = (0.680517e9 + 0.523335e9) / 32
+COMPOSITE_TRAFFIC_PER_ENV = (0.424962e9 + 0.145890e9) / 32
 COMPOSITE_TRAFFIC_SOURCES = ("paper_2604_25459_gb300/csrc/gs_composite.cu",)
-COMPOSITE_TRAFFIC_SHA = "05cb60c8cec62bb9"
+COMPOSITE_TRAFFIC_SHA = "9260d64e036eaff7"
 
 
 def _sources_sha(paths) -> str:

@@ -17,7 +17,7 @@
 //       multiple of 32), then the env's link Gaussians in storage order; slot
 //       (el, j) is slot s = envs[el].rec_base + j, valid where bit j%32 of
 //       mask[envs[el].mask_base + j/32] is set; its first three 16-byte words
-//       r0, r1, r2 lie side by side at float4 index kRecStride s of one array
+//       r0 = (u, v, log2 o, z), r1, r2 lie side by side at float4 index kRecStride s of one array
 //       (the compositor gathers all three: two 32-byte sectors instead of
 //       three half-used ones), its fourth word r3 at index s of another (the
 //       binning reads only r3, coalesced across a warp).

@@ -12,9 +12,9 @@
 // Since q(x) >= |x - mu|^2 / max_k e^{2 s_k} = |x - mu|^2 / max_k |f_k|^2, every
 // point with alpha >= 1/255 (q <= q*) lies within r = sqrt(q*) max_k |f_k| of
 // mu: the rays that can reach it lie within the cone of half-angle
-// asin(r / |mu|).  The cone bounds the elevations; the azimuths are the exact
-// range of the ellipsoid's shadow on the sensor's xy-plane where that is
-// tighter (see below).
+// asin(r / |mu|).  Azimuths are the exact range of the ellipsoid's shadow on the
+// sensor's xy-plane, elevations that of its shadow on the vertical plane through
+// its centre, where they are tighter than the cone (see below).
 //
 // Arbitrary rays (non-repetitive scan patterns) reuse the grid as a binning
 // structure: each ray falls in one cell of its sensor's (azimuth, beam) grid,
