@@ -464,28 +464,30 @@ __global__ void __launch_bounds__(256, 6) k_scatter(BinParams P) {  // <= 42 reg
         if (pos < P.pair_cap) P.pairs[pos] = v;
         else dropped = true;
     };
-    // uniform trip count: the block drains its list of long spans together
+    // Uniform trip count: the block drains its list of long spans together.  The
+    // list's length for that decision is counted at the barrier and kept by every
+    // thread; n_far only hands out places.  (Read after the barrier, n_far may
+    // already hold places taken in the next round by warps that are ahead, and
+    // warps that disagree on draining part at the barriers below.)
+    uint32_t nf = 0;
     for (int i0 = 0; i0 < nvis; i0 += blockDim.x) {
         const int i = i0 + threadIdx.x;
+        bool longer = false;
         if (i < nvis) {
             const uint4 q = r3[lst[i]];
-            bool walk = true;
             if constexpr (DIFF) {
                 int tx0, tx1, ty0, ty1;
                 tile_span(q.x, q.y, sx, sy, tx0, tx1, ty0, ty1);
-                if ((tx1 - tx0 + 1) * (ty1 - ty0 + 1) > kLongSpan) {
-                    far[atomicAdd(&n_far, 1u)] = (uint16_t)i;  // at most blockDim.x more per round
-                    walk = false;
-                }
+                longer = (tx1 - tx0 + 1) * (ty1 - ty0 + 1) > kLongSpan;
+                if (longer) far[atomicAdd(&n_far, 1u)] = (uint16_t)i;  // at most blockDim.x more per round
             }
-            if (walk) {
+            if (!longer) {
                 const uint32_t key = rank[lst[i]];
                 for_span<WRAP>(q.x, q.y, sx, sy, ntx, [&](int, int tx, int ty) { put(q, key, tx, ty); });
             }
         }
         if constexpr (DIFF) {
-            __syncthreads();
-            const uint32_t nf = n_far;
+            nf += (uint32_t)__syncthreads_count(longer);
             if (nf + blockDim.x > (uint32_t)kLongList || (i0 + (int)blockDim.x >= nvis && nf)) {
                 for (uint32_t k = threadIdx.x >> 5; k < nf; k += blockDim.x >> 5) {
                     const uint4 q = r3[lst[far[k]]];
@@ -498,6 +500,7 @@ __global__ void __launch_bounds__(256, 6) k_scatter(BinParams P) {  // <= 42 reg
                 __syncthreads();
                 if (threadIdx.x == 0) n_far = 0u;
                 __syncthreads();
+                nf = 0u;
             }
         }
     }

@@ -1,0 +1,53 @@
+"""Edges of the renderer's binning, ranking and host paths that ordinary scenes
+do not reach."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from gpu_helpers import ensure_built, gpu_render
+from oracle import oracle
+from paper_2604_25459_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    ensure_built()
+
+
+def _check_lists(scene, w, e, tile, W, H):
+    """Counts and depth-ordered lists of env e of the last debug render, from the GPU's own records."""
+    rec = scene.debug_records(e, w.background.n + w.links.n)
+    vis = np.nonzero(rec["visible"])[0]
+    counts, lists = scene.debug_tiles(e, (-(-W // tile[0])) * (-(-H // tile[1])))
+    oc, ol = oracle.bin_records(rec["u"][vis], rec["v"][vis], rec["hx"][vis], rec["hy"][vis],
+                                rec["z"][vis].view(np.uint32), vis.astype(np.uint32), W, H, *tile)
+    np.testing.assert_array_equal(counts.astype(np.int64), oc)
+    np.testing.assert_array_equal(lists, ol)
+    return rec, vis
+
+
+@pytest.mark.parametrize("tile,n_envs,words", [((16, 16), 192, 64), ((32, 8), 192, 64), ((16, 16), 1, 16)])
+def test_blocks_full_of_long_spans(tile, n_envs, words):
+    """A robot whose Gaussians cover a third of the image and more, in blocks of the
+    scatter of `words` visibility words (2048 slots in large batches, 512 for one
+    view): a block lists more spans of over 64 tiles than its list holds, so it
+    drains the list several times before its last round.  Keys with subtile
+    masks (square tiles) and without."""
+    W = H = 256
+    w = synth.make_c1(n_envs=n_envs, width=W, height=H, f=200.0, n_bg=100_000, per_link=300)
+    links = dataclasses.replace(w.links, log_scale=(w.links.log_scale + np.float32(2.0)).astype(np.float32))
+    w = dataclasses.replace(w, links=links)
+    out = gpu_render(w, tile=tile, debug=True, keep_scene=True)
+    most = 0
+    for e in {0, n_envs // 2, n_envs - 1}:
+        rec, vis = _check_lists(out["scene"], w, e, tile, W, H)
+        r = rec["range"][vis].astype(np.int64)
+        tiles = (r[:, 1] // tile[0] - r[:, 0] // tile[0] + 1) * (r[:, 3] // tile[1] - r[:, 2] // tile[1] + 1)
+        far = vis[(tiles > 64) & (vis >= w.background.n)]  # links keep their storage order
+        block = (far - w.background.n + (w.background.n + 31) // 32 * 32) // (32 * words)
+        most = max(most, int(np.bincount(block).max()))
+    out["scene"].close()
+    assert most > (1024 if words == 64 else 384)
