@@ -243,7 +243,6 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
     const uint32_t* Lk = P.pairs + start;
     const size_t recbase = (size_t)__ldg(&Ep->rec_base);
     const uint32_t* order = P.order + recbase;  // record slot of each rank
-    const uint32_t n_rank = __ldg(P.nvis + el);
     // contribution pass: record slot -> global Gaussian index
     const long long g_link0 = SC ? __ldg(&Ep->g_link0) : 0ll;
     auto score_index = [&](uint32_t j) -> long long {
@@ -420,7 +419,8 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                 hi = max(hi, k);
             }
             block_minmax_u32<NT>(lo, hi, red);
-            whole = rank_sort<NT, SB>(keys, tmp, bm, red, (int)n, lo, hi, c32_dirty);
+            // (a rank beyond the env's, in a corrupted bucket: the bitmaps leave it out)
+            whole = hi < __ldg(P.nvis + el) && rank_sort<NT, SB>(keys, tmp, bm, red, (int)n, lo, hi, c32_dirty);
             if (!whole) continue;  // crowded ranks: through bitmaps
             wn = n;
         } else {
@@ -430,6 +430,7 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                 __syncthreads();  // bm is rewritten for the next ranks
             }
             if (!loaded) {
+                const uint32_t n_rank = __ldg(P.nvis + el);  // read here: a register less through the blend loop
                 if (r0 >= n_rank) {  // ranks beyond the env's: a corrupted bucket
                     if (tid == 0) atomicOr(P.status, kStOverflow);
                     break;
@@ -442,6 +443,17 @@ __global__ void __launch_bounds__(TW* TH / 2, (TW * TH >= 512 ? 4 : (TW * TH >= 
                     if (d < (uint32_t)(BMW * 32)) atomicOr(&bm[d >> 5], 1u << (d & 31u));
                 });
                 __syncthreads();
+                if (n_rank - r0 < (uint32_t)(BMW * 32)) {  // the env's last ranks: a bit beyond is a corrupted bucket's
+                    bool stray = false;
+                    for (uint32_t i = ((n_rank - r0) >> 5) + tid; i < (uint32_t)BMW; i += NT) {
+                        const uint32_t first = r0 + 32u * i, m = bm[i];
+                        const uint32_t keep = n_rank > first ? (1u << (n_rank - first)) - 1u : 0u;
+                        stray |= (m & ~keep) != 0u;
+                        bm[i] = m & keep;
+                    }
+                    if (stray) atomicOr(P.status, kStOverflow);
+                    __syncthreads();
+                }
                 // ranks set before each group: thread t counts groups GPT t ..
                 constexpr int GPT = NG < NT ? 1 : NG / NT;
                 uint32_t c[GPT], sum = 0;

@@ -341,7 +341,7 @@ __device__ __forceinline__ bool in_box(const int4& R, int x, int y) {
 struct Bucket {
     const uint32_t* keys;
     uint32_t n;
-    uint32_t n_rank;        // ranks of the env
+    uint32_t n_rank;        // ranks of the env; keys beyond them (a corrupted bucket's) are left out
     const uint32_t* order;  // record slot of each rank
     size_t recbase;
     uint32_t n_local;
@@ -557,7 +557,7 @@ __device__ __forceinline__ void team_item(const CompParams& P, TeamSmem<MODE == 
         for (int i = tid; i < kTeamWords / 4; i += NT) reinterpret_cast<uint4*>(sm.bm)[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         const uint32_t k0 = r0 << kshift;
-        const unsigned long long span = (unsigned long long)(kTeamWords * 32) << kshift;
+        const unsigned long long span = (unsigned long long)min((uint32_t)(kTeamWords * 32), bk.n_rank - r0) << kshift;
         auto set = [&](uint32_t k, bool valid) {
             const uint32_t d = k - k0;
             if (valid && d < span && ((k & submask) | any_sub) != 0u)
@@ -1008,7 +1008,7 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
     uint32_t r0 = 0;       // next ranks of the bitmap
     bool loaded = false;   // a bitmap is set up
     if (bk.n <= kShort) {
-        whole = bk.n ? gather(0u, kAll) : 0u;
+        whole = bk.n ? gather(0u, bk.n_rank) : 0u;
         if (whole <= (uint32_t)CAP) how = kWhole;
     }
     if (how == kBitmap) {
@@ -1068,7 +1068,7 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
             const uint32_t a = (uint32_t)g0 << hs;
             g0 = lo;
             if (wn == 0) continue;
-            gather(a, ((uint32_t)lo << hs) - a);
+            gather(a, min((uint32_t)lo << hs, bk.n_rank) - a);
         } else {
             if (loaded && g0 >= NG) {
                 loaded = false;
@@ -1079,7 +1079,7 @@ __global__ void __launch_bounds__(32 * kWarps, MODE == 1 || MODE == 3 ? 5 : 6) k
                 for (int i = lane; i < kWords / 4; i += 32)
                     reinterpret_cast<uint4*>(bm)[i] = make_uint4(0u, 0u, 0u, 0u);
                 __syncwarp();
-                const uint32_t k0 = r0 << kshift, span = (uint32_t)(kWords * 32) << kshift;
+                const uint32_t k0 = r0 << kshift, span = min((uint32_t)(kWords * 32), bk.n_rank - r0) << kshift;
                 warp_keys(bk.keys, bk.n, [&](uint32_t k, bool valid) {
                     const uint32_t d = k - k0;
                     if (valid && d < span && taken(k)) atomicOr(&bm[d >> (5 + kshift)], 1u << ((d >> kshift) & 31u));

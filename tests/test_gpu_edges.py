@@ -1,12 +1,16 @@
 """Edges of the renderer's binning, ranking and host paths that ordinary scenes
 do not reach."""
+import ctypes
 import dataclasses
+import os
+import subprocess
 
 import numpy as np
 import pytest
 
 from gpu_helpers import ensure_built, gpu_render
 from oracle import oracle
+from paper_2604_25459_gb300 import build as cuda_build
 from paper_2604_25459_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -51,3 +55,37 @@ def test_blocks_full_of_long_spans(tile, n_envs, words):
         most = max(most, int(np.bincount(block).max()))
     out["scene"].close()
     assert most > (1024 if words == 64 else 384)
+
+
+@pytest.fixture(scope="module")
+def corrupt_bucket(tmp_path_factory):
+    """tests/corrupt_bucket.cu, linked with the library."""
+    so = str(tmp_path_factory.mktemp("native") / "corrupt_bucket.so")
+    here = os.path.dirname(os.path.abspath(__file__))
+    libdir = os.path.dirname(cuda_build.LIB)
+    subprocess.run([cuda_build.nvcc(), *cuda_build.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC",
+                    "--expt-relaxed-constexpr", "-I", cuda_build.INCLUDE, "-I", cuda_build.CSRC, "-shared", "-cudart",
+                    "static", "-o", so, os.path.join(here, "corrupt_bucket.cu"), "-L", libdir, "-l:libgsbatch.so",
+                    "-Xlinker", "-rpath", "-Xlinker", libdir], check=True)
+    lib = ctypes.CDLL(so)
+    lib.corrupt_bucket.restype = ctypes.c_int
+
+    def run(form, n, bad):
+        alpha, status = np.full((16, 16), -1.0, np.float32), ctypes.c_uint32(0)
+        assert lib.corrupt_bucket(form, n, bad, alpha.ctypes.data_as(ctypes.c_void_p), ctypes.byref(status)) == 0
+        return alpha, status.value
+
+    return run
+
+
+@pytest.mark.parametrize("form", [0, 1, 2])
+@pytest.mark.parametrize("n", [40, 600, 1490])
+def test_rank_beyond_the_ranked_records_is_left_out(corrupt_bucket, form, n):
+    """A key that names no ranked record (a corrupted bucket): its place in the
+    order is not read and the other splats are blended; the CTA form, which
+    accounts for every key of a bucket, also sets the status word."""
+    alpha, status = corrupt_bucket(form, n, 0)
+    assert status == 0 and np.all(np.abs(alpha - (1.0 - (1.0 - 0.0045) ** n)) < 5e-3)
+    again, status = corrupt_bucket(form, n, 1)
+    assert status == (4 if form == 0 else 0)
+    np.testing.assert_array_equal(again, alpha)
