@@ -643,7 +643,8 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         if (cap == 0) {
             ebd = ea + 1;
             if (eb[ebd] - eb[ea] > cap_keys)
-                return fail(GS_ERR_OOM, "environment %d has %llu intersections, beyond the scratch budget", ea,
+                return fail(GS_ERR_OOM, "environment %d has %llu intersections, beyond the scratch budget",
+                            wt.host_envs[ea].env,
                             (unsigned long long)(eb[ebd] - eb[ea]));
             while (ebd < We && eb[ebd + 1] - eb[ea] <= cap_keys) ++ebd;
             npairs = eb[ebd] - eb[ea];
@@ -767,7 +768,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
 
 enum class Out { Device, Host };
 
-gs_status render_specs(gs_scene s, const std::vector<EnvSpec>& specs, const float* poses_dev, const Outputs& o,
+gs_status render_specs(gs_scene s, std::vector<EnvSpec>& specs, const float* poses_dev, const Outputs& o,
                        cudaStream_t st, Out mode, int64_t pix_per_env_host) {
     float* const rgb = o.rgb;
     float* const depth = o.depth;
@@ -783,20 +784,31 @@ gs_status render_specs(gs_scene s, const std::vector<EnvSpec>& specs, const floa
     if (mode == Out::Host) extra = (size_t)pix_per_env_host * (o.rgb_px() + o.depth_px() + (alpha ? 4 : 0)) * 2;
     std::vector<std::pair<int, int>> waves;
     ST(plan_waves(s, specs, tw, th, s->debug != 0, s->max_wave, extra, &waves));
+    // Low resolutions first within a wave (see gs_plan_create): their images then
+    // take the compositor's warp form.  Outputs are placed by pixel_offset and the
+    // debug copies look an env up by the caller's index, so the order is not
+    // visible.  Debug renders keep the caller's order, by which their lists of the
+    // last sub-wave are taken.
+    if (!s->debug)
+        for (auto& w : waves) {
+            auto smaller = [](const EnvSpec& a, const EnvSpec& b) {
+                return (int64_t)a.cam->width * a.cam->height < (int64_t)b.cam->width * b.cam->height;
+            };
+            const auto b = specs.begin() + w.first, e = specs.begin() + w.second;
+            if (!std::is_sorted(b, e, smaller)) std::stable_sort(b, e, smaller);
+        }
     int64_t launches = 0;
     if (mode == Out::Device) {
         for (auto& w : waves) {
             WaveTables wt{};
             ST(upload_tables(s, specs, w.first, w.second, tw, th, 0, s->sc.envs, s->sc.blocks, s->sc.cams, st, false,
                              &wt));
-            s->last_envs.assign(wt.host_envs, wt.host_envs + wt.We + 1);
             WaveIO io{poses_dev, rgb, depth, alpha, 0};
             io.rgb8 = o.rgb8;
             io.depth16 = o.depth16;
             io.appear = o.appear ? o.appear + w.first : nullptr;
             ST(run_wave(s, s->sc, wt, io, tw, th, 1, 0, st, true, &launches, nullptr));
-            s->last_e0 = w.first;
-            s->last_We = wt.We;
+            s->last_envs.assign(wt.host_envs, wt.host_envs + wt.We);
             s->stats.waves++;
         }
     } else {
@@ -822,7 +834,6 @@ gs_status render_specs(gs_scene s, const std::vector<EnvSpec>& specs, const floa
             WaveTables wt{};
             ST(upload_tables(s, specs, w.first, w.second, tw, th, rebase, s->sc.envs, s->sc.blocks, s->sc.cams, st,
                              false, &wt));
-            s->last_envs.assign(wt.host_envs, wt.host_envs + wt.We + 1);
             WaveIO io{poses_dev, s->stage_rgb[k].as<float>(), s->stage_depth[k].as<float>(),
                       alpha ? s->stage_alpha[k].as<float>() : nullptr, rebase};
             if (o.obs()) {
@@ -833,8 +844,7 @@ gs_status render_specs(gs_scene s, const std::vector<EnvSpec>& specs, const floa
                 io.appear = o.appear ? o.appear + w.first : nullptr;
             }
             ST(run_wave(s, s->sc, wt, io, tw, th, 1, 0, st, true, &launches, nullptr));
-            s->last_e0 = w.first;
-            s->last_We = We;
+            s->last_envs.assign(wt.host_envs, wt.host_envs + wt.We);
             CK(cudaEventRecord(s->ev_done[k], st), "record");
             CK(cudaStreamWaitEvent(s->copy_stream, s->ev_done[k], 0), "wait render");
             if (o.obs()) {
@@ -967,7 +977,7 @@ gs_status render_uniform(gs_scene s, int E, const float* link_poses, const gs_ca
         return clear_outputs(rgb, depth, alpha, (size_t)E * px, st, host_mode);
     }
     std::vector<EnvSpec> specs((size_t)E);
-    for (int e = 0; e < E; ++e) specs[e] = EnvSpec{cams + e, 0, L, (long long)e * L, (long long)e * px};
+    for (int e = 0; e < E; ++e) specs[e] = EnvSpec{cams + e, 0, L, (long long)e * L, (long long)e * px, e};
     const float* poses_dev = link_poses;
     if (host_mode && L > 0) {
         CK(s->poses.ensure((size_t)E * L * 28), "alloc poses");
@@ -996,7 +1006,8 @@ gs_status specs_from_envs(gs_scene s, int n, const gs_env* envs, std::vector<Env
     specs->resize((size_t)n);
     for (int e = 0; e < n; ++e) {
         const gs_env& v = envs[e];
-        (*specs)[e] = EnvSpec{&v.cam, v.link_begin, v.link_end, (long long)v.pose_offset, (long long)v.pixel_offset};
+        (*specs)[e] =
+            EnvSpec{&v.cam, v.link_begin, v.link_end, (long long)v.pose_offset, (long long)v.pixel_offset, e};
     }
     (void)s;
     return GS_OK;
@@ -1293,7 +1304,7 @@ gs_status lidar_scan(gs_scene s, int n_envs, const float* link_poses, const gs_l
     }
     const int tw = 16, th = 16;
     std::vector<EnvSpec> specs((size_t)n_envs);
-    for (int e = 0; e < n_envs; ++e) specs[e] = EnvSpec{&cams[e], 0, L, (long long)e * L, (long long)e * (long long)px};
+    for (int e = 0; e < n_envs; ++e) specs[e] = EnvSpec{&cams[e], 0, L, (long long)e * L, (long long)e * (long long)px, e};
     ST(check_specs(s, specs, tw, th));
     std::vector<std::pair<int, int>> waves;
     ST(plan_waves(s, specs, tw, th, false, s->max_wave, 0, &waves));
@@ -1346,7 +1357,7 @@ gs_status gs_scene_contribution(gs_scene s, int n_envs, const float* link_poses,
     CK(cudaSetDevice(s->device), "set device");
     const int tw = 16, th = 16;  // the contribution pass bins and composites on 16x16 tiles
     std::vector<EnvSpec> specs((size_t)n_envs);
-    for (int e = 0; e < n_envs; ++e) specs[e] = EnvSpec{cams + e, 0, L, (long long)e * L, 0};
+    for (int e = 0; e < n_envs; ++e) specs[e] = EnvSpec{cams + e, 0, L, (long long)e * L, 0, e};
     ST(check_specs(s, specs, tw, th));
     std::vector<std::pair<int, int>> waves;
     ST(plan_waves(s, specs, tw, th, false, s->max_wave, 0, &waves));
@@ -1392,14 +1403,6 @@ gs_status gs_render_batch_v(gs_scene s, int n_envs, const gs_env* envs, const fl
     if (any_links && !link_poses) return fail(GS_ERR_INVALID, "null link_poses");
     std::vector<EnvSpec> specs;
     ST(specs_from_envs(s, n_envs, envs, &specs));
-    ST(check_specs(s, specs, s->tile_w, s->tile_h));
-    // Low resolutions first (see gs_plan_create): their images then take the
-    // compositor's warp form.  Outputs are placed by pixel_offset, so the order
-    // is not visible; debug renders keep the caller's, by which the copies index.
-    if (!s->debug)
-        std::stable_sort(specs.begin(), specs.end(), [](const EnvSpec& a, const EnvSpec& b) {
-            return (int64_t)a.cam->width * a.cam->height < (int64_t)b.cam->width * b.cam->height;
-        });
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     CK(cudaSetDevice(s->device), "set device");
     if (s->D.n == 0) {
@@ -1732,15 +1735,22 @@ gs_status gs_scene_get_stats(gs_scene s, gs_stats* out) {
     return GS_OK;
 }
 
+// The place in the last rendered wave of the caller's env, or -1.
+static int last_place(gs_scene s, int env) {
+    for (size_t el = 0; el < s->last_envs.size(); ++el)
+        if (s->last_envs[el].env == env) return (int)el;
+    return -1;
+}
+
 gs_status gs_debug_copy_records(gs_scene s, int env, uint8_t* visible, float* u, float* v, float* hx, float* hy,
                                 float* z, float* opacity, float* conic, float* rgb, int32_t* range) {
     if (!s) return fail(GS_ERR_INVALID, "null scene");
-    if (s->last_e0 < 0 || env < s->last_e0 || env >= s->last_e0 + s->last_We)
-        return fail(GS_ERR_INVALID, "env %d is not in the last wave rendered", env);
+    const int el = last_place(s, env);
+    if (el < 0) return fail(GS_ERR_INVALID, "env %d is not in the last wave rendered", env);
     if (!s->debug || !s->sc.dbg_hxy.p) return fail(GS_ERR_INVALID, "debug was not enabled for the last render");
     CK(cudaSetDevice(s->device), "set device");
     CK(cudaDeviceSynchronize(), "sync");
-    const EnvInfo& E = s->last_envs[env - s->last_e0];
+    const EnvInfo& E = s->last_envs[el];
     const int64_t n_local = E.n_local, nbp = bg_slots(s->D.n_bg);
     const int64_t lg0 = s->D.n_bg + s->link_offsets[E.link_begin];
     std::vector<uint32_t> mask((n_local + 31) / 32);
@@ -1798,9 +1808,8 @@ gs_status gs_debug_copy_records(gs_scene s, int env, uint8_t* visible, float* u,
 gs_status gs_debug_copy_tiles(gs_scene s, int env, uint32_t* counts, int64_t n_counts, uint32_t* lists,
                               int64_t n_lists) {
     if (!s || !counts) return fail(GS_ERR_INVALID, "null argument");
-    if (s->last_e0 < 0 || env < s->last_e0 || env >= s->last_e0 + s->last_We)
-        return fail(GS_ERR_INVALID, "env %d is not in the last wave rendered", env);
-    const int el = env - s->last_e0;
+    const int el = last_place(s, env);
+    if (el < 0) return fail(GS_ERR_INVALID, "env %d is not in the last wave rendered", env);
     const EnvInfo& E = s->last_envs[el];
     if (n_counts < E.T) return fail(GS_ERR_INVALID, "counts holds %lld < %d tiles", (long long)n_counts, E.T);
     CK(cudaSetDevice(s->device), "set device");

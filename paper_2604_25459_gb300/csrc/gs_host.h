@@ -99,7 +99,7 @@ struct gs_scene_s {
     cudaEvent_t ev_copied[2] = {nullptr, nullptr};
     // host tables of the last wave (debug hooks)
     std::vector<gsb::EnvInfo> last_envs;
-    int last_e0 = -1, last_We = 0, last_ea = 0, last_eb = 0, last_shift = 0;
+    int last_ea = 0, last_eb = 0, last_shift = 0;
     const uint32_t* last_counts = nullptr;  // device: tile counts of the last wave
     unsigned long long last_pair_base = 0;
     gs_stats stats{};

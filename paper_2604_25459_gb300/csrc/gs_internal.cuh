@@ -108,7 +108,7 @@ struct EnvInfo {
     int xf_base;                   // first link-table entry
     int link_begin, n_links;       // links of the scene rendered in this env
     int W, H, ntx, T;              // image and tile grid
-    int pad;
+    int env;                       // index of the environment in the caller's batch
     long long g_link0;             // storage (= caller's) index of the env's first link Gaussian (slot bg_slots)
     float lim[4];                  // camera guard band: 1.3 cx/fx, 1.3 (W-cx)/fx, 1.3 cy/fy, 1.3 (H-cy)/fy
 };
@@ -435,6 +435,7 @@ struct EnvSpec {        // one env as requested by the caller
     int link_begin, link_end;
     long long pose_offset;    // pose index of link_begin
     long long pixel_offset;   // first pixel of the image
+    int env = 0;              // its index in the caller's batch
 };
 int64_t bg_slots(int64_t n_bg);  // background slots padded to 32
 // Fills envs (n+1 entries; the last holds the totals in rec_base, mask_base,

@@ -166,7 +166,7 @@ gs_status server_launch(gs_server sv, gs_server_s::Slot& sl) {
         const auto& ev = sv->envs[rq.env];
         const int nl = ev.link_end - ev.link_begin;
         if (nl > 0) memcpy(sl.h_poses + i * (size_t)L * 7, rq.poses.data(), sizeof(float) * nl * 7);
-        specs[i] = EnvSpec{&ev.cam, ev.link_begin, ev.link_end, (long long)i * L, (long long)ev.pix_off};
+        specs[i] = EnvSpec{&ev.cam, ev.link_begin, ev.link_end, (long long)i * L, (long long)ev.pix_off, rq.env};
         const double k = keys_estimate(sv, ev);
         if (k < 0) known = false;
         est += k;

@@ -92,7 +92,7 @@ void build_wave_tables(const DevGaussians& D, const int64_t* link_offsets, const
         ei.H = H;
         ei.ntx = ntx;
         ei.T = ntx * nty;
-        ei.pad = 0;
+        ei.env = sp.env;
         ei.g_link0 = D.n_bg + (link_offsets ? link_offsets[sp.link_begin] : 0);
         // guard-band limits of the EWA Jacobian (IEEE float division, as on the device)
         const gs_camera& c = *sp.cam;

@@ -11,7 +11,7 @@ import pytest
 from gpu_helpers import ensure_built, gpu_render
 from oracle import oracle
 from paper_2604_25459_gb300 import build as cuda_build
-from paper_2604_25459_gb300 import synth
+from paper_2604_25459_gb300 import gsbatch, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +89,34 @@ def test_rank_beyond_the_ranked_records_is_left_out(corrupt_bucket, form, n):
     again, status = corrupt_bucket(form, n, 1)
     assert status == (4 if form == 0 else 0)
     np.testing.assert_array_equal(again, alpha)
+
+
+@pytest.mark.parametrize("wave", [0, 2])
+def test_tile_counts_of_mixed_resolutions_are_the_named_envs(wave):
+    """render_v orders a wave by resolution inside; the counts it leaves are
+    looked up by the caller's index, and an env outside the last wave is refused."""
+    import torch
+
+    sizes = [(320, 240), (64, 48), (130, 94), (96, 200), (33, 21)]
+    ws = [synth.make_c1(n_envs=1, width=a, height=b, f=0.8 * a, n_bg=20_000, per_link=200) for a, b in sizes]
+    envs = gsbatch.make_envs(np.concatenate([w.cams for w in ws]),
+                             link_ranges=np.tile([0, ws[0].n_links], (len(ws), 1)),
+                             pose_offsets=np.zeros(len(ws)))
+    scene = gsbatch.scene_from_workload(ws[0])
+    poses = torch.from_numpy(ws[0].link_poses).cuda()
+    tiles = [(-(-a // 16)) * (-(-b // 16)) for a, b in sizes]
+    alone = []
+    for w, t in zip(ws, tiles):
+        scene.render(poses, w.cams)
+        alone.append(scene.debug_tiles(0, t, with_lists=False)[0])
+    scene.set_wave(wave)
+    npx = sum(a * b for a, b in sizes)
+    scene.render_v(envs, poses, torch.empty(npx * 3, device="cuda"), torch.empty(npx, device="cuda"))
+    last = range(len(sizes)) if wave == 0 else range(4, 5)
+    for e in range(len(sizes)):
+        if e in last:
+            np.testing.assert_array_equal(scene.debug_tiles(e, tiles[e], with_lists=False)[0], alone[e])
+        else:
+            with pytest.raises(gsbatch.GsError):
+                scene.debug_tiles(e, tiles[e], with_lists=False)
+    scene.close()
