@@ -752,11 +752,11 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         }
         t6.done(kernels);
         *launches += kernels;
-        if (cap == 0) {
+        if (&sc == &s->sc) {  // for the debug copies, which read the scene's own scratch
             s->last_ea = ea;
             s->last_eb = ebd;
             s->last_shift = B.key_shift;
-            s->last_counts = counts;
+            s->last_counts = n_bins;
             s->last_pair_base = base;
         }
         ea = ebd;
@@ -1814,7 +1814,8 @@ gs_status gs_debug_copy_tiles(gs_scene s, int env, uint32_t* counts, int64_t n_c
     if (n_counts < E.T) return fail(GS_ERR_INVALID, "counts holds %lld < %d tiles", (long long)n_counts, E.T);
     CK(cudaSetDevice(s->device), "set device");
     CK(cudaDeviceSynchronize(), "sync");
-    CK(cudaMemcpy(counts, s->last_counts + E.tile_base, (size_t)E.T * 4, cudaMemcpyDeviceToHost),
+    CK(cudaMemcpy(counts, s->sc.counts.as<uint32_t>() + s->last_counts + E.tile_base, (size_t)E.T * 4,
+                  cudaMemcpyDeviceToHost),
        "copy counts");
     if (!lists) return GS_OK;
     if (!s->debug || !s->sc.dbg_hxy.p) return fail(GS_ERR_INVALID, "debug was not enabled for the last render");

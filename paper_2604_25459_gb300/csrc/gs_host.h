@@ -100,7 +100,7 @@ struct gs_scene_s {
     // host tables of the last wave (debug hooks)
     std::vector<gsb::EnvInfo> last_envs;
     int last_ea = 0, last_eb = 0, last_shift = 0;
-    const uint32_t* last_counts = nullptr;  // device: tile counts of the last wave
+    size_t last_counts = 0;  // first tile count of the last wave in sc.counts
     unsigned long long last_pair_base = 0;
     gs_stats stats{};
     // profiling (per-phase CUDA events on the render stream) and counters

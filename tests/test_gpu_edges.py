@@ -120,3 +120,26 @@ def test_tile_counts_of_mixed_resolutions_are_the_named_envs(wave):
             with pytest.raises(gsbatch.GsError):
                 scene.debug_tiles(e, tiles[e], with_lists=False)
     scene.close()
+
+
+def test_tile_counts_outlive_a_plan():
+    """A plan measures its batch with eager passes in its own scratch; the
+    scene's counts of its last render stay readable, also when the plan is gone."""
+    import torch
+
+    w = synth.make_c1(n_envs=1, width=130, height=94, f=100.0, n_bg=20_000, per_link=200)
+    other = synth.make_c1(n_envs=3, width=200, height=120, f=160.0, n_bg=20_000, per_link=200)
+    scene = gsbatch.scene_from_workload(w)
+    scene.render(torch.from_numpy(w.link_poses).cuda(), w.cams)
+    before = scene.debug_tiles(0, 54, with_lists=False)[0]
+    envs = gsbatch.make_envs(other.cams, link_ranges=np.tile([0, w.n_links], (3, 1)),
+                             pose_offsets=np.arange(3) * w.n_links)
+    npx = 3 * 200 * 120
+    plan = scene.plan(envs)
+    plan.launch(torch.from_numpy(other.link_poses).cuda(), torch.empty(npx * 3, device="cuda"),
+                torch.empty(npx, device="cuda"))
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(scene.debug_tiles(0, 54, with_lists=False)[0], before)
+    plan.close()
+    np.testing.assert_array_equal(scene.debug_tiles(0, 54, with_lists=False)[0], before)
+    scene.close()
