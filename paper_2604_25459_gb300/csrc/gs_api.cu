@@ -63,6 +63,7 @@ struct gs_plan_s {
         int n_blocks = 0, xf_items = 0, max_words = 0, max_T = 0, max_hist = 0;
         unsigned long long recs = 0, words = 0, tiles = 0;
         unsigned long long cap = 0;  // intersection-key capacity
+        int n_warp = 0;              // envs in the compositor's warp form
     };
     std::vector<Wave> waves;
     bool tuned = false;
@@ -437,6 +438,22 @@ gs_status upload_tables(gs_scene s, const std::vector<EnvSpec>& specs, int e0, i
     return GS_OK;
 }
 
+// Envs [0, n) of a wave of images go to the compositor's warp form, the others
+// to the CTA form: all of them by the largest image, or, in a wave of mixed
+// resolutions in ascending order, each by its own.  Returns n.
+int warp_envs(const WaveTables& wt, int tw, int th, int quad) {
+    if (quad == 0) return 0;
+    auto small = [&](int e) {
+        if (quad > 0) return warp_form(tw, th, 0, kQuadMinSlots, wt.We);
+        return warp_form(tw, th, (long long)wt.host_envs[e].W * wt.host_envs[e].H, wt.max_words * 32ll, wt.We);
+    };
+    int n = 0;
+    while (n < wt.We && small(n)) ++n;
+    for (int e = n; e < wt.We; ++e)
+        if (small(e)) return 0;  // unordered: by the largest image
+    return n;
+}
+
 // Launch one wave.  Eager (cap == 0): reads the wave's intersection totals back
 // (host sync), grows the key buffer and splits the wave into sub-waves that
 // fit the budget.  Planned (cap > 0): no host sync; keys beyond cap are dropped
@@ -445,20 +462,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
                    unsigned long long cap, cudaStream_t st, bool timers, int64_t* launches,
                    unsigned long long* total_out, int quad) {
     const int We = wt.We;
-    // Envs [0, n_warp) go to the compositor's warp form, the others to the CTA
-    // form: all of them by the largest image, or, in a batch of mixed
-    // resolutions in ascending order, each by its own.
-    int n_warp = io.lidars ? We : 0;
-    if (!io.lidars && !io.score && quad != 0) {
-        auto small = [&](int e) {
-            if (quad >= 0) return warp_form(tw, th, 0, kQuadMinSlots, We);
-            return warp_form(tw, th, (long long)wt.host_envs[e].W * wt.host_envs[e].H, wt.max_words * 32ll,
-                             We);
-        };
-        while (n_warp < We && small(n_warp)) ++n_warp;
-        for (int e = n_warp; e < We; ++e)
-            if (small(e)) n_warp = 0;  // unordered: by the largest image
-    }
+    const int n_warp = io.lidars ? We : io.score ? 0 : warp_envs(wt, tw, th, quad);
     CK(sc.xf.ensure(sizeof(LinkXf) * (size_t)std::max(wt.xf_items, 1)), "alloc link table");
     CK(sc.r012.ensure(wt.recs * 16 * kRecStride), "alloc records");
     CK(sc.r3.ensure(wt.recs * 16), "alloc records");
@@ -1051,6 +1055,7 @@ gs_status plan_tables(gs_plan p, const std::vector<EnvSpec>& specs) {
         w.recs = wt.recs;
         w.words = wt.words;
         w.tiles = wt.tiles;
+        w.n_warp = warp_envs(wt, p->tile_w, p->tile_h, p->quad);
         w.cap = i < caps.size() ? caps[i] : 0;
     }
     return GS_OK;
@@ -1597,13 +1602,15 @@ gs_status gs_plan_get_info(gs_plan p, gs_plan_info* out) {
     i.tile_w = p->tile_w;
     i.tile_h = p->tile_h;
     i.chunk = p->chunk;
-    i.quad = p->quad != 0;
     i.waves = (int)p->waves.size();
     i.graph = p->exec != nullptr;
     i.tuned_candidates = p->tuned_candidates;
     i.tuned_ms = p->tuned_ms;
     i.regrows = p->regrows;
-    for (auto& w : p->waves) i.key_capacity += (int64_t)w.cap;
+    for (auto& w : p->waves) {
+        i.key_capacity += (int64_t)w.cap;
+        if (w.n_warp > 0) i.quad = 1;
+    }
     i.scratch_bytes = p->sc.bytes();
     *out = i;
     return GS_OK;

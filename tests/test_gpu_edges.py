@@ -143,3 +143,23 @@ def test_tile_counts_outlive_a_plan():
     plan.close()
     np.testing.assert_array_equal(scene.debug_tiles(0, 54, with_lists=False)[0], before)
     scene.close()
+
+
+@pytest.mark.parametrize("width,height,tile,quad", [(200, 120, (16, 16), 1), (640, 480, (16, 16), 0),
+                                                    (200, 120, (32, 8), 0)])
+def test_plan_info_names_the_form_that_runs(width, height, tile, quad):
+    """An untuned plan takes the warp form by resolution, on square tiles."""
+    import torch
+
+    w = synth.make_c1(n_envs=2, width=width, height=height, f=0.8 * width, n_bg=20_000, per_link=200)
+    scene = gsbatch.scene_from_workload(w)
+    scene.set_tile(*tile)
+    envs = gsbatch.make_envs(w.cams, link_ranges=np.tile([0, w.n_links], (2, 1)), pose_offsets=np.arange(2) * w.n_links)
+    plan = scene.plan(envs, autotune=False)
+    npx = 2 * width * height
+    plan.launch(torch.from_numpy(w.link_poses).cuda(), torch.empty(npx * 3, device="cuda"),
+                torch.empty(npx, device="cuda"))
+    torch.cuda.synchronize()
+    assert plan.info()["quad"] == quad
+    plan.close()
+    scene.close()
