@@ -291,22 +291,44 @@ gs_status check_specs(gs_scene s, const std::vector<EnvSpec>& specs, int tw, int
     return GS_OK;
 }
 
-// Fixed scratch bytes of one env (records, visibility, tile counters, link table).
+// Scratch bytes of one env: 80 per record slot (48 + 16 of record, 8 of depth
+// key, 4 each of order and rank), visibility, tile counters, link table.
 size_t env_bytes(gs_scene s, const EnvSpec& sp, int tw, int th, bool debug) {
     const int64_t nlg = s->link_offsets[sp.link_end] - s->link_offsets[sp.link_begin];
     const int64_t n_local = bg_slots(s->D.n_bg) + nlg;
     const int64_t T = (int64_t)((sp.cam->width + tw - 1) / tw) * ((sp.cam->height + th - 1) / th);
-    size_t b = (size_t)n_local * 64 + (size_t)((n_local + 31) / 32) * 4 + (size_t)T * 12 + 16 +
+    size_t b = (size_t)n_local * 80 + (size_t)((n_local + 31) / 32) * 4 + (size_t)T * 12 + 16 +
                (size_t)(1 + sp.link_end - sp.link_begin) * sizeof(LinkXf) + sizeof(gs_camera) + sizeof(EnvInfo) + 64;
     if (debug) b += (size_t)n_local * 8;
     return b;
 }
 
-// Split envs into waves whose fixed scratch fits 60 % of the budget.
+// Record slots and tiles of one env, by the largest of which a wave's tables are sized.
+EnvSize env_size(gs_scene s, const EnvSpec& sp, int tw, int th) {
+    const int64_t n_local = bg_slots(s->D.n_bg) + s->link_offsets[sp.link_end] - s->link_offsets[sp.link_begin];
+    return EnvSize{(n_local + 31) / 32, ((sp.cam->width + tw - 1) / tw) * ((sp.cam->height + th - 1) / th)};
+}
+
+// Scratch bytes of the tables of a wave of We envs of at most this size: the
+// depth ranking's, the places that the count notes, the item order.
+size_t wave_table_bytes(const EnvSize& z, int We, bool lidar, size_t budget) {
+    RankParams R = rank_sizes(z.words, We, lidar);
+    size_t b = rank_tables(R, We, nullptr) + (size_t)We * R.bins * 4;
+    const size_t off = tile_off_bytes(R, scatter_words(z.words, We, z.T), We, z.T, lidar);
+    if (off <= off_limit(budget)) b += off;
+    const size_t items = (size_t)We * z.T * kItemClasses * 4;
+    if (items <= item_limit(budget)) b += items;
+    return b;
+}
+
+// Split envs into waves whose records and tables fit 80 % of the budget; the
+// rest is for intersection keys (see run_wave).  extra_per_env: staging or ray
+// tables of the caller.
 gs_status plan_waves(gs_scene s, const std::vector<EnvSpec>& specs, int tw, int th, bool debug, int max_wave,
-                     size_t extra_per_env, std::vector<std::pair<int, int>>* waves) {
+                     size_t extra_per_env, std::vector<std::pair<int, int>>* waves, bool lidar = false) {
     waves->clear();
-    const double cap = (double)s->budget * 0.6;
+    const double cap = (double)s->budget * 0.8;
+    const size_t budget = (size_t)s->budget;
     const int E = (int)specs.size();
     // uniform batches: balanced waves of equal size
     bool uniform = true;
@@ -315,12 +337,15 @@ gs_status plan_waves(gs_scene s, const std::vector<EnvSpec>& specs, int tw, int 
                   specs[e].link_begin == specs[0].link_begin && specs[e].link_end == specs[0].link_end;
     if (uniform && E > 0) {
         const double per = (double)(env_bytes(s, specs[0], tw, th, debug) + extra_per_env);
+        const EnvSize z = env_size(s, specs[0], tw, th);
         int64_t wmax = (int64_t)(cap / per);
-        if (wmax < 1)
-            return fail(GS_ERR_OOM, "one environment needs %.0f bytes of scratch; budget is %lld", per,
-                        (long long)s->budget);
         if (max_wave > 0 && wmax > max_wave) wmax = max_wave;
         if (wmax > E) wmax = E;
+        // the tables are at most 2.3 bytes per slot and the share of the rules' limits: a few steps
+        while (wmax > 0 && (double)wmax * per + (double)wave_table_bytes(z, (int)wmax, lidar, budget) > cap) --wmax;
+        if (wmax < 1)
+            return fail(GS_ERR_OOM, "one environment needs %.0f bytes of scratch; budget is %lld",
+                        per + (double)wave_table_bytes(z, 1, lidar, budget), (long long)s->budget);
         const int64_t nw = (E + wmax - 1) / wmax;
         const int We = (int)((E + nw - 1) / nw);
         for (int e0 = 0; e0 < E; e0 += We) waves->push_back({e0, std::min(E, e0 + We)});
@@ -328,16 +353,22 @@ gs_status plan_waves(gs_scene s, const std::vector<EnvSpec>& specs, int tw, int 
     }
     int e0 = 0;
     double acc = 0;
+    EnvSize most;
     for (int e = 0; e < E; ++e) {
         const double b = (double)(env_bytes(s, specs[e], tw, th, debug) + extra_per_env);
-        if (b > cap) return fail(GS_ERR_OOM, "env %d needs %.0f bytes of scratch; budget is %lld", e, b,
-                                 (long long)s->budget);
-        if (e > e0 && (acc + b > cap || (max_wave > 0 && e - e0 >= max_wave))) {
+        const EnvSize z = env_size(s, specs[e], tw, th);
+        const double alone = b + (double)wave_table_bytes(z, 1, lidar, budget);
+        if (alone > cap) return fail(GS_ERR_OOM, "env %d needs %.0f bytes of scratch; budget is %lld", e, alone,
+                                     (long long)s->budget);
+        if (e > e0 && (acc + b + (double)wave_table_bytes(most.with(z), e - e0 + 1, lidar, budget) > cap ||
+                       (max_wave > 0 && e - e0 >= max_wave))) {
             waves->push_back({e0, e});
             e0 = e;
             acc = 0;
+            most = EnvSize{};
         }
         acc += b;
+        most = most.with(z);
     }
     if (E > e0) waves->push_back({e0, E});
     return GS_OK;
@@ -476,7 +507,8 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     const int scatter_wpb = scatter_words(wt.max_words, We, wt.max_T);
     const size_t table_bytes = rank_tables(R, We, nullptr);
     size_t off_bytes = tile_off_bytes(R, scatter_wpb, We, wt.max_T, io.lidars != nullptr);
-    if (off_bytes > (size_t)s->budget / 64) off_bytes = 0;
+    const size_t budget = io.budget ? io.budget : (size_t)s->budget;
+    if (off_bytes > off_limit(budget)) off_bytes = 0;
     CK(sc.bins.ensure(table_bytes + off_bytes), "alloc depth ranges");
     rank_tables(R, We, sc.bins.as<unsigned char>());
     CK(sc.zkeys.ensure(wt.recs * 8), "alloc depth keys");
@@ -624,7 +656,6 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     *launches += rank_launches;
 
     // sub-waves of envs whose keys fit (eager), or the whole wave (planned)
-    std::vector<unsigned long long> ebv;
     const unsigned long long* eb = nullptr;
     unsigned long long cap_keys = cap;
     if (cap == 0) {
@@ -632,12 +663,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         eb = h_keys;
         if (total_out) *total_out = eb[We];
         s->stats.intersections += (int64_t)eb[We];
-        double cap_d = (double)s->budget * 0.4;
-        const size_t key_bytes = debug ? 16 : 8;
-        cap_keys = (unsigned long long)(cap_d / key_bytes);
-    } else {
-        ebv.assign(2, 0);
-        ebv[1] = cap;
+        cap_keys = (unsigned long long)((double)s->budget * 0.2 / 4);  // 4 bytes a key
     }
     int ea = 0;
     while (ea < We) {
@@ -730,7 +756,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
             if (!io.ray_dirs) Q.item_end = wt.host_envs[es].tile_base;
             Q.e_end = es;
             const unsigned long long n_items = Q.item_end - Q.item_begin;  // long buckets first
-            if (n_items * kItemClasses * 4 <= (unsigned long long)s->budget / 64) {
+            if (n_items * kItemClasses * 4 <= item_limit(budget)) {
                 CK(sc.items.ensure((size_t)n_items * kItemClasses * 4), "alloc item order");
                 CK(launch_item_order(wt.envs, ea, es - ea, wt.max_T, counts,
                                      io.ray_dirs ? s->item_cnt.as<uint32_t>() : nullptr,
@@ -1312,7 +1338,10 @@ gs_status lidar_scan(gs_scene s, int n_envs, const float* link_poses, const gs_l
     for (int e = 0; e < n_envs; ++e) specs[e] = EnvSpec{&cams[e], 0, L, (long long)e * L, (long long)e * (long long)px, e};
     ST(check_specs(s, specs, tw, th));
     std::vector<std::pair<int, int>> waves;
-    ST(plan_waves(s, specs, tw, th, false, s->max_wave, 0, &waves));
+    // rays: cell and list entry each; counters, cursors and offsets per tile and quadrant, items per tile
+    const size_t tiles = (size_t)((cols + tw - 1) / tw) * ((rows + th - 1) / th);
+    const size_t extra = ray_dirs ? (size_t)n_rays * 8 + tiles * (12 * kRayGroups + 8) + 32 : 0;
+    ST(plan_waves(s, specs, tw, th, false, s->max_wave, extra, &waves, true));
     int64_t launches = 0;
     for (auto& w : waves) {
         const int We = w.second - w.first;

@@ -150,6 +150,7 @@ struct WaveIO {
     const gs_lidar* lidars = nullptr;  // LiDAR scan: device table of the wave's sensors
     const float* ray_dirs = nullptr;   // with lidars: arbitrary rays [wave env][n_rays][3] (sensor frame)
     int n_rays = 0;
+    size_t budget = 0;  // scratch budget that the optional tables are held against (0: the scene's)
 };
 
 struct WaveTables {       // device copies of one wave's tables
@@ -164,8 +165,19 @@ struct WaveTables {       // device copies of one wave's tables
 // Validates one camera (env index e for the message).
 gs_status check_cam(const gs_camera& c, int e);
 
-// Fixed scratch bytes of one env (records, visibility, tile counters, link table).
+// Scratch of a wave: env_bytes of each env, wave_table_bytes for all of them,
+// and 4 bytes per intersection key.
 size_t env_bytes(gs_scene s, const EnvSpec& sp, int tw, int th, bool debug);
+struct EnvSize {
+    long long words = 0;  // visibility words: a bit per record slot
+    int T = 0;            // tiles
+    EnvSize with(const EnvSize& o) const { return EnvSize{words > o.words ? words : o.words, T > o.T ? T : o.T}; }
+};
+EnvSize env_size(gs_scene s, const EnvSpec& sp, int tw, int th);
+size_t wave_table_bytes(const EnvSize& z, int We, bool lidar, size_t budget);
+// Largest optional tables: the places noted by the count, the item order.
+inline size_t off_limit(size_t budget) { return budget / 64; }
+inline size_t item_limit(size_t budget) { return budget / 128; }
 
 // Builds the tables of specs[e0, e1) and uploads them into the given device
 // buffers on st (synchronously when sync_copy).

@@ -89,6 +89,8 @@ struct gs_server_s {
 
 namespace {
 
+constexpr unsigned long long kSpareKeys = 65536;  // in every batch's key capacity
+
 void CUDART_CB server_slot_done(void* p) {
     auto* sl = static_cast<gs_server_s::Slot*>(p);
     sl->t_done = std::chrono::duration<double>(std::chrono::steady_clock::now() - sl->t0).count();
@@ -102,13 +104,15 @@ double keys_estimate(gs_server sv, const gs_server_s::EnvRec& ev) {
     return it != sv->keys_ema.end() ? it->second : -1.0;
 }
 
+// Scratch of a request beside its batch's tables: its records and its keys,
+// 4 bytes each, with the headroom of a batch's key capacity.
 double request_bytes(gs_server sv, const gs_server_s::EnvRec& ev) {
     gs_scene s = sv->scenes[ev.scene]->s;
     EnvSpec sp{&ev.cam, ev.link_begin, ev.link_end, 0, 0};
     const int tw = sv->cfg.tile_w, th = sv->cfg.tile_h;
     double keys = keys_estimate(sv, ev);
     if (keys < 0) keys = (double)(sv->scenes[ev.scene]->s->D.n);  // first of its kind: about one key per Gaussian
-    return (double)env_bytes(s, sp, tw, th, false) + keys * 8.0 * 1.3;
+    return (double)env_bytes(s, sp, tw, th, false) + keys * 4.0 * 1.3;
 }
 
 // Launch one batch (requests of one scene, in sl.batch) on its slot.  Called
@@ -185,8 +189,9 @@ gs_status server_launch(gs_server sv, gs_server_s::Slot& sl) {
     unsigned long long keys = 0;
     // capacity: 25% over the averages, plus room for one env at the most seen
     // of its kind (what a batch of a few envs needs)
-    const unsigned long long cap = eager ? 0ull : (unsigned long long)(est * 1.25 + spread) + 65536ull;
+    const unsigned long long cap = eager ? 0ull : (unsigned long long)(est * 1.25 + spread) + kSpareKeys;
     WaveIO io{sl.poses.as<float>(), sr.rgb.as<float>(), sr.depth.as<float>(), nullptr, 0, sl.dstat.as<uint32_t>()};
+    io.budget = (size_t)(sv->cfg.budget_bytes / sv->cfg.max_inflight);
     ST(run_wave(s, sl.sc, wt, io, sv->cfg.tile_w, sv->cfg.tile_h, 1, cap, sl.st, false, &launches, &keys));
     CK(cudaMemcpyAsync(sl.h_meta, sl.dstat.p, 4, cudaMemcpyDeviceToHost, sl.st), "read status");
     CK(cudaMemcpyAsync(sl.h_meta + 1, sl.sc.env_base.p, (n + 1) * 8, cudaMemcpyDeviceToHost, sl.st), "read keys");
@@ -262,7 +267,8 @@ void server_loop(gs_server sv) {
                 if (slp->busy || sv->pending.empty()) continue;
                 int scene = -1;
                 std::vector<int64_t> batch;
-                double bytes = 0;
+                double bytes = 0, rows = 0;  // the batch's scratch, and the requests' part of it
+                EnvSize most;
                 std::deque<int64_t> keep;
                 std::vector<char> taken(sv->envs.size(), 0);
                 while (!sv->pending.empty()) {
@@ -271,21 +277,29 @@ void server_loop(gs_server sv) {
                     auto& rq = sv->reqs[id];
                     auto& ev = sv->envs[rq.env];
                     const bool fits_scene = scene < 0 || ev.scene == scene;
-                    const double b = request_bytes(sv, ev);
+                    const EnvSpec sp{&ev.cam, ev.link_begin, ev.link_end, 0, 0};
+                    const EnvSize z =
+                        most.with(env_size(sv->scenes[ev.scene]->s, sp, sv->cfg.tile_w, sv->cfg.tile_h));
+                    const double r = request_bytes(sv, ev);
+                    const double with = rows + r + kSpareKeys * 4.0 +
+                                        (double)wave_table_bytes(z, (int)batch.size() + 1, false,
+                                                                 (size_t)(sv->cfg.budget_bytes / sv->cfg.max_inflight));
                     // a batch holds at most budget / slots (a slot's scratch keeps its
                     // high-water mark, so the slots together stay within the budget);
                     // the batches in flight together at most the budget; a request
                     // larger than that runs alone when nothing else is in flight
                     const double budget = (double)sv->cfg.budget_bytes;
                     const bool fits_budget =
-                        batch.empty() ? (sv->inflight_bytes + b <= budget || inflight == 0)
-                                      : (bytes + b <= budget / sv->cfg.max_inflight &&
-                                         sv->inflight_bytes + bytes + b <= budget);
+                        batch.empty() ? (sv->inflight_bytes + with <= budget || inflight == 0)
+                                      : (with <= budget / sv->cfg.max_inflight &&
+                                         sv->inflight_bytes + with <= budget);
                     if (!ev.busy && !taken[rq.env] && fits_scene && fits_budget &&
                         (int)batch.size() < sv->cfg.max_batch_envs) {
                         scene = ev.scene;
                         batch.push_back(id);
-                        bytes += b;
+                        bytes = with;
+                        rows += r;
+                        most = z;
                         taken[rq.env] = 1;
                     } else {
                         keep.push_back(id);

@@ -12,6 +12,7 @@ from gpu_helpers import ensure_built, gpu_render
 from oracle import oracle
 from paper_2604_25459_gb300 import build as cuda_build
 from paper_2604_25459_gb300 import gsbatch, synth
+from test_gpu_lidar import _sensors
 
 pytestmark = pytest.mark.gpu
 
@@ -163,3 +164,73 @@ def test_plan_info_names_the_form_that_runs(width, height, tile, quad):
     assert plan.info()["quad"] == quad
     plan.close()
     scene.close()
+
+
+@pytest.mark.parametrize("kind,width,height,mib", [("render", 64, 48, 24), ("render", 320, 240, 40), ("lidar", 128, 32, 24),
+                                                   ("rays", 64, 64, 24)])
+def test_scratch_stays_within_the_budget(kind, width, height, mib):
+    """Several waves of 24 envs of 22,000 slots under a small budget: the scratch
+    that the scene then holds, every table of it, is within the budget."""
+    import torch
+
+    n = 24
+    w = synth.make_c1(n_envs=n, width=width, height=height, f=0.8 * width, n_bg=20_000, per_link=100)
+    scene = gsbatch.scene_from_workload(w)
+    scene.set_budget(mib << 20)
+    poses = torch.from_numpy(w.link_poses).cuda()
+    if kind == "render":
+        scene.render(poses, w.cams)
+    else:
+        sens = _sensors(n, rows=height, cols=width)
+        if kind == "lidar":
+            scene.render_lidar(poses, sens)
+        else:
+            scene.render_rays(poses, sens, torch.from_numpy(synth.rosette_rays(n, 500)).cuda())
+    torch.cuda.synchronize()
+    st = scene.stats()
+    assert st["waves"] > 1
+    assert st["scratch_bytes"] <= mib << 20
+    scene.close()
+
+
+@pytest.mark.parametrize("n,width,height", [(20_000, 64, 48), (15_000, 1000, 30), (70_000, 33, 21)])
+def test_one_environment_fits_the_budget_it_always_fitted(n, width, height):
+    """64 bytes a slot and 12 a tile within 60 % of the budget: what one env
+    needed before records were ranked is still enough for it."""
+    import torch
+
+    w = synth.make_c0(n=n, width=width, height=height, f=0.8 * width)
+    slots, tiles = (n + 31) // 32 * 32, (-(-width // 16)) * (-(-height // 16))
+    scene = gsbatch.scene_from_workload(w)
+    scene.set_budget(int((slots * 64 + slots // 32 * 4 + tiles * 12 + 600) / 0.6))
+    scene.render(None, w.cams)
+    torch.cuda.synchronize()
+    scene.close()
+
+
+def test_server_scratch_stays_within_its_budget():
+    """Requests of low resolution, whose scratch is records and ranking and few
+    keys: the device memory that a slot takes is within what admission allowed it,
+    up to the rounding of 17 buffers to 2 MiB."""
+    import torch
+
+    E, budget = 96, 2 << 30
+    w = synth.make_c1(n_envs=E, width=64, height=48, f=50.0, n_bg=600_000, per_link=200)
+    scene = gsbatch.scene_from_workload(w)
+    for rounds, limit in ((1, 256 << 20), (3, budget)):  # the first server loads the kernels
+        sv = gsbatch.Server(budget_bytes=limit, max_inflight=1, max_batch_envs=E)
+        sid = sv.add_scene(scene)
+        ids = [sv.add_env(sid, w.cams[e:e + 1], 0, w.n_links) for e in range(E)]
+        sv.start()
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        for _ in range(rounds):
+            for e in ids:
+                sv.submit(e, w.link_poses[e])
+            sv.drain(300.0)
+        used = free - torch.cuda.mem_get_info()[0]
+        most = sv.stats()["max_batch"]
+        sv.close()
+    scene.close()
+    assert 8 <= most < E
+    assert used <= budget + (17 * 2 << 20)
