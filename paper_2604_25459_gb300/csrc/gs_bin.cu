@@ -181,9 +181,19 @@ __global__ void __launch_bounds__(256) k_count(BinParams P, RankParams R) {
     }
 }
 
+// The kernels' largest dynamic shared memory: the ranges and depth cells of a
+// LiDAR scan's ranking and the histogram of the largest grid that the entry
+// points take (kMaxTiles tiles of at least 8 pixels in images of at most 16384:
+// 2048 x 8).  The attribute belongs to the function, not to the launch, so every
+// launch sets this one value: with its own size, a launch failed when another
+// thread set a smaller one in between.
+constexpr int kMaxTiles = 16384;
+constexpr size_t kMaxBinSmem = kRankBins * 12 + 4096 * 2 + (size_t)(kMaxTiles + 2048 + 8 + 1) * 4;
+
 static cudaError_t opt_in_smem(const void* fn, size_t smem) {
     if (smem <= 30 * 1024) return cudaSuccess;  // plus at most 17.2 KB of static shared memory
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > kMaxBinSmem) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBinSmem);
 }
 
 static_assert(kWordsPerBlock <= 256, "binning blocks: one visibility word per thread of 256, places below 2^13");

@@ -234,3 +234,47 @@ def test_server_scratch_stays_within_its_budget():
     scene.close()
     assert 8 <= most < E
     assert used <= budget + (17 * 2 << 20)
+
+
+def test_threads_may_render_grids_of_different_sizes():
+    """Scenes of their own on threads and streams of their own, on grids whose
+    histograms need shared memory beyond the default, of three sizes: no launch
+    may depend on what another thread's last one needed."""
+    import threading
+
+    import torch
+
+    errors = []
+
+    def work(width, height, tile, seed):
+        try:
+            w = synth.make_c0(seed=seed, n=300, width=width, height=height, f=0.8 * width)
+            scene = gsbatch.scene_from_workload(w)
+            scene.set_tile(*tile)
+            stream = torch.cuda.Stream()
+            out = [torch.empty((1, height, width) + s, device="cuda") for s in ((3,), (), ())]
+            torch.cuda.synchronize()
+            for _ in range(400):
+                scene.render(None, w.cams, *out, stream=stream)
+            stream.synchronize()
+            scene.close()
+        except Exception as e:
+            errors.append(e)
+
+    jobs = [(1920, 1080, (16, 16), 0), (2560, 1440, (16, 16), 1), (1024, 1024, (8, 8), 2)]
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
+
+
+@pytest.mark.parametrize("width,height,tile", [(16384, 64, (8, 8)), (64, 16384, (8, 8)), (2048, 2048, (16, 16))])
+def test_largest_grids(width, height, tile):
+    """16384 tiles, the most an image may have, square and in the longest rows."""
+    w = synth.make_c0(n=3000, width=width, height=height, f=60.0)
+    out = gpu_render(w, tile=tile, debug=True, keep_scene=True)
+    _, vis = _check_lists(out["scene"], w, 0, tile, width, height)
+    out["scene"].close()
+    assert len(vis) > 1000
