@@ -12,7 +12,7 @@ from gpu_helpers import ensure_built, gpu_render
 from oracle import oracle
 from paper_2604_25459_gb300 import build as cuda_build
 from paper_2604_25459_gb300 import gsbatch, synth
-from test_gpu_lidar import _sensors
+from test_gpu_lidar import _check_scan, _oracle_rays, _ray_sensors, _sensors
 
 pytestmark = pytest.mark.gpu
 
@@ -278,3 +278,87 @@ def test_largest_grids(width, height, tile):
     _, vis = _check_lists(out["scene"], w, 0, tile, width, height)
     out["scene"].close()
     assert len(vis) > 1000
+
+
+@pytest.mark.parametrize("depths", ["spread", "equal", "half_equal"])
+def test_ranking_of_a_window_that_the_sample_missed(depths):
+    """Of 20,000 slots the ranking samples every third; with all of those culled
+    (too faint) it has no splitters, so 13,333 records share one depth range: a
+    window far above what one block sorts, cut by radix selection."""
+    w = synth.make_c0(n=20_000)
+    g = w.background
+    mean = g.mean.copy()
+    if depths == "equal":
+        mean[:, 2] = 0.0
+    elif depths == "half_equal":
+        mean[::2, 2] = 0.25
+    g = dataclasses.replace(g, mean=mean)
+    scene = gsbatch.scene_from_workload(dataclasses.replace(w, background=g))
+    order = scene.storage_order()  # by the means alone
+    scene.close()
+    opacity = np.maximum(g.opacity, np.float32(0.1))
+    opacity[order[::3]] = 0.001
+    w = dataclasses.replace(w, background=dataclasses.replace(g, opacity=opacity))
+    out = gpu_render(w, debug=True, keep_scene=True)
+    assert np.array_equal(out["scene"].storage_order(), order)
+    _, vis = _check_lists(out["scene"], w, 0, (16, 16), 128, 96)
+    out["scene"].close()
+    assert len(vis) > 10_000 and not np.isin(vis, order[::3]).any()
+
+
+def _shell(n, half_az, half_el, seed):
+    """n faint Gaussians of 2 cm, 2 to 6 m around the origin, within +-half_az and +-half_el."""
+    rng = np.random.default_rng([seed, 91])
+    w = synth.make_c0(seed=seed, n=n)
+    az, el, r = rng.uniform(-half_az, half_az, n), rng.uniform(-half_el, half_el, n), rng.uniform(2.0, 6.0, n)
+    mean = np.stack([r * np.cos(el) * np.cos(az), r * np.cos(el) * np.sin(az), r * np.sin(el)], 1)
+    return dataclasses.replace(w, background=dataclasses.replace(
+        w.background, mean=mean.astype(np.float32), log_scale=np.full((n, 3), np.log(0.02), np.float32),
+        opacity=rng.uniform(0.02, 0.2, n).astype(np.float32)))
+
+
+def _at(sens, n, pos_seed=7):
+    s = np.repeat(sens[:1], n)
+    s["t_ws"] = -np.random.default_rng(pos_seed).uniform(-0.05, 0.05, (n, 3))
+    return s
+
+
+def test_scans_of_many_gaussians_in_short_buckets():
+    """300,000 ranked Gaussians and buckets of some 2,000 keys: with 24 sensors a
+    warp orders a bucket by runs of a histogram over the ranks; alone, a scan's
+    buckets go to teams and their bitmaps.  The same bits either way."""
+    import torch
+
+    w = _shell(300_000, np.pi, 0.5, 1)
+    scene = gsbatch.scene_from_workload(w)
+    sens = _at(_sensors(1, rows=64, cols=1024), 24)
+    rng, hit = scene.render_lidar(None, sens)
+    torch.cuda.synchronize()
+    scene.sync_status()
+    assert 0.2 < float(hit.mean()) < 0.95
+    for e in (0, 23):
+        r1, h1 = scene.render_lidar(None, sens[e:e + 1])
+        assert torch.equal(hit[e], h1[0]) and torch.equal(rng[e], r1[0])
+    scene.close()
+
+
+def test_rays_through_many_gaussians_in_short_buckets():
+    """The same for rays, 72 sensors and one, and a part of them against the oracle."""
+    import torch
+
+    n_env, n_rays = 72, 16_000
+    w = _shell(150_000, 0.65, 0.65, 2)
+    w = dataclasses.replace(w, link_poses=np.zeros((n_env, 0, 7), np.float32))
+    scene = gsbatch.scene_from_workload(w)
+    sens = _at(_ray_sensors(1, rows=256, cols=256), n_env)
+    dirs = synth.rosette_rays(n_env, n_rays, seed=5)
+    rng, hit = scene.render_rays(None, sens, torch.from_numpy(dirs).cuda())
+    torch.cuda.synchronize()
+    scene.sync_status()
+    for e in (0, n_env - 1):
+        r1, h1 = scene.render_rays(None, sens[e:e + 1], torch.from_numpy(dirs[e:e + 1].copy()).cuda())
+        assert torch.equal(hit[e], h1[0]) and torch.equal(rng[e], r1[0])
+    scene.close()
+    some = np.arange(0, n_rays, 160)
+    _check_scan(rng[0, some].cpu().numpy(), hit[0, some].cpu().numpy(),
+                _oracle_rays(w, 0, sens[0], dirs[0][some].copy()), "rays of the shell")
