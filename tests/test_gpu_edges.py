@@ -58,22 +58,27 @@ def test_blocks_full_of_long_spans(tile, n_envs, words):
     assert most > (1024 if words == 64 else 384)
 
 
-@pytest.fixture(scope="module")
-def corrupt_bucket(tmp_path_factory):
-    """tests/corrupt_bucket.cu, linked with the library."""
-    so = str(tmp_path_factory.mktemp("native") / "corrupt_bucket.so")
+def _native(name, folder):
+    """tests/<name>.cu, linked with the library; its function <name>."""
+    so = str(folder / f"{name}.so")
     here = os.path.dirname(os.path.abspath(__file__))
     libdir = os.path.dirname(cuda_build.LIB)
     subprocess.run([cuda_build.nvcc(), *cuda_build.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC",
                     "--expt-relaxed-constexpr", "-I", cuda_build.INCLUDE, "-I", cuda_build.CSRC, "-shared", "-cudart",
-                    "static", "-o", so, os.path.join(here, "corrupt_bucket.cu"), "-L", libdir, "-l:libgsbatch.so",
+                    "static", "-o", so, os.path.join(here, f"{name}.cu"), "-L", libdir, "-l:libgsbatch.so",
                     "-Xlinker", "-rpath", "-Xlinker", libdir], check=True)
-    lib = ctypes.CDLL(so)
-    lib.corrupt_bucket.restype = ctypes.c_int
+    f = getattr(ctypes.CDLL(so), name)
+    f.restype = ctypes.c_int
+    return f
+
+
+@pytest.fixture(scope="module")
+def corrupt_bucket(tmp_path_factory):
+    native = _native("corrupt_bucket", tmp_path_factory.mktemp("native"))
 
     def run(form, n, bad):
         alpha, status = np.full((16, 16), -1.0, np.float32), ctypes.c_uint32(0)
-        assert lib.corrupt_bucket(form, n, bad, alpha.ctypes.data_as(ctypes.c_void_p), ctypes.byref(status)) == 0
+        assert native(form, n, bad, alpha.ctypes.data_as(ctypes.c_void_p), ctypes.byref(status)) == 0
         return alpha, status.value
 
     return run
@@ -362,3 +367,23 @@ def test_rays_through_many_gaussians_in_short_buckets():
     some = np.arange(0, n_rays, 160)
     _check_scan(rng[0, some].cpu().numpy(), hit[0, some].cpu().numpy(),
                 _oracle_rays(w, 0, sens[0], dirs[0][some].copy()), "rays of the shell")
+
+
+@pytest.fixture(scope="module")
+def rank_ranges(tmp_path_factory):
+    return _native("rank_ranges", tmp_path_factory.mktemp("native"))
+
+
+@pytest.mark.parametrize("n", [3000, 8192, 20_000, 120_000, 300_000])
+@pytest.mark.parametrize("seen", [1.0, 0.5])
+def test_depth_ranges_are_balanced(rank_ranges, n, seen):
+    """The sample is kept from all over the storage order, whatever share of it is
+    seen: no range of an env whose depths follow the order holds more than three
+    times the average (a range spans two to thirty samples, evenly spaced but for what is not seen)."""
+    rng = np.random.default_rng([n, int(10 * seen)])
+    bits = rng.random(n) < seen if seen < 1.0 else np.ones(n, bool)
+    mask = np.packbits(np.pad(bits, (0, -n % 32)), bitorder="little").view(np.uint32)
+    per = np.zeros(4096, np.uint32)
+    bins = rank_ranges(n, mask.ctypes.data_as(ctypes.c_void_p), per.ctypes.data_as(ctypes.c_void_p), len(per))
+    assert bins > 0 and per[:bins].sum() == bits.sum()
+    assert per[:bins].max() <= 3.0 * bits.sum() / bins
