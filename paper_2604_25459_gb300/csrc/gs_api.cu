@@ -493,7 +493,6 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
                    unsigned long long cap, cudaStream_t st, bool timers, int64_t* launches,
                    unsigned long long* total_out, int quad) {
     const int We = wt.We;
-    const int n_warp = io.lidars ? We : io.score ? 0 : warp_envs(wt, tw, th, quad);
     CK(sc.xf.ensure(sizeof(LinkXf) * (size_t)std::max(wt.xf_items, 1)), "alloc link table");
     CK(sc.r012.ensure(wt.recs * 16 * kRecStride), "alloc records");
     CK(sc.r3.ensure(wt.recs * 16), "alloc records");
@@ -588,7 +587,6 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     B.rank = R.rank;
     B.status = status;
     B.wrap = io.lidars ? 1 : 0;         // LiDAR boxes may wrap across azimuth 0
-    if (n_warp > 0) B.key_shift = subtile_bits(tw, th, (unsigned long long)wt.max_words * 32);
     PhaseTimer t3(s, st, GS_PHASE_COUNT, timers);
     CK(launch_rank_sample(R, We, st), "depth sample");
     CK(launch_count(B, R, We, wt.max_T, wt.max_hist, st), "count");
@@ -612,9 +610,13 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     }
     unsigned long long* const h_keys = cap == 0 ? s->pinned : nullptr;
     unsigned long long* const h_items = h_keys ? h_keys + We + 1 : nullptr;
+    // the longest bucket too, where the form depends on it (warp_pays)
+    const int n_small = io.lidars || io.score ? 0 : warp_envs(wt, tw, th, quad);
+    const bool longest = h_keys && quad == -2 && n_small > 0 && wt.tiles >= kEvenTiles;
+    unsigned long long most = 0;
     PhaseTimer t4(s, st, GS_PHASE_SCAN, timers);
     CK(launch_scan_ranks(wt.envs, counts, sc.off.as<uint32_t>(), sc.env_total.as<unsigned long long>(),
-                         sc.env_base.as<unsigned long long>(), h_keys, ticket, We, R, st),
+                         sc.env_base.as<unsigned long long>(), h_keys, longest, ticket, We, R, st),
        "scan");
     t4.done(1);
     *launches += 3;
@@ -660,11 +662,21 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
     unsigned long long cap_keys = cap;
     if (cap == 0) {
         CK(cudaEventSynchronize(s->ev_totals), "sync totals");
+        for (int e = 0; e < We && longest; ++e) {
+            most = std::max(most, h_keys[e] >> kTotalBits);
+            h_keys[e] &= (1ull << kTotalBits) - 1ull;
+        }
         eb = h_keys;
         if (total_out) *total_out = eb[We];
         s->stats.intersections += (int64_t)eb[We];
         cap_keys = (unsigned long long)((double)s->budget * 0.2 / 4);  // 4 bytes a key
     }
+    int n_warp = io.lidars ? We : n_small;
+    if (quad == -2 && eb && n_small > 0) {  // all of them or none, by their buckets
+        const unsigned long long tiles = wt.host_envs[n_small].tile_base;
+        if (!warp_pays(tiles, eb[n_small], most)) n_warp = 0;
+    }
+    if (n_warp > 0) B.key_shift = subtile_bits(tw, th, (unsigned long long)wt.max_words * 32);
     int ea = 0;
     while (ea < We) {
         int ebd = We;

@@ -243,22 +243,24 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* warp_tot, T& block_tot
 }
 
 // Bases of the envs, by one CTA: env_base[e] = sum_{e' < e} env_total[e'],
-// env_base[We] = total; host_base (pinned host memory, or null) gets the same.
+// env_base[We] = total; host_base (pinned host memory, or null) gets the same,
+// with the env's longest bucket where that is asked for.
 struct EnvBases {
     unsigned long long *total, *base, *host;
     unsigned int* ticket;  // CTAs done; 0 before and after the launch
+    bool longest;          // total and host carry the longest bucket above kTotalBits bits
 };
 __device__ __forceinline__ void scan_bases(const EnvBases& B, int We) {
     __shared__ unsigned long long wt[32];
     unsigned long long carry = 0;
     for (int first = 0; first < We; first += blockDim.x) {
         const int e = first + threadIdx.x;
-        const unsigned long long v = e < We ? __ldcg(B.total + e) : 0ull;
+        const unsigned long long t = e < We ? __ldcg(B.total + e) : 0ull, v = t & ((1ull << kTotalBits) - 1ull);
         unsigned long long tot;
         const unsigned long long ex = block_exclusive_scan<unsigned long long>(v, wt, tot);
         if (e < We) {
             B.base[e] = carry + ex;
-            if (B.host) B.host[e] = carry + ex;
+            if (B.host) B.host[e] = (carry + ex) | (t - v);
         }
         carry += tot;
     }
@@ -279,7 +281,10 @@ __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const ui
                                                    EnvBases B, int per, RankParams R) {
     __shared__ uint32_t wt[32];
     __shared__ bool last;
+    __shared__ uint32_t longest;
     const int el = blockIdx.x;
+    if (threadIdx.x == 0) longest = 0u;  // the scan's barriers come before its use
+    uint32_t most = 0;
     const int T = envs[el].T * per;
     const uint32_t* c = counts + (size_t)envs[el].tile_base * per;
     uint32_t* o = off_local + (size_t)envs[el].tile_base * per;
@@ -287,13 +292,19 @@ __global__ void __launch_bounds__(1024) k_scan_env(const EnvInfo* envs, const ui
     for (int base = 0; base < T; base += blockDim.x) {
         const int t = base + threadIdx.x;
         const uint32_t v = t < T ? c[t] : 0u;
+        most = max(most, v);
         uint32_t tot;
         const uint32_t ex = block_exclusive_scan<uint32_t>(v, wt, tot);
         if (t < T) o[t] = carry + ex;
         carry += tot;
     }
+    if (B.longest) {
+        most = __reduce_max_sync(0xffffffffu, most);
+        if (most && (threadIdx.x & 31) == 0) atomicMax(&longest, most);
+        __syncthreads();
+    }
     if (threadIdx.x == 0) {
-        B.total[el] = carry;
+        B.total[el] = carry | (unsigned long long)min(longest, kTotalMost) << kTotalBits;
         __threadfence();
         last = atomicAdd(B.ticket, 1u) == gridDim.x - 1;
         __threadfence();
@@ -327,10 +338,10 @@ static_assert(kRankBins <= 2048, "two depth ranges per thread of the scan");
 
 cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                               unsigned long long* env_total, unsigned long long* env_base,
-                              unsigned long long* host_base, unsigned int* ticket, int We, const RankParams& R,
-                              cudaStream_t st) {
+                              unsigned long long* host_base, bool longest, unsigned int* ticket, int We,
+                              const RankParams& R, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
-    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, EnvBases{env_total, env_base, host_base, ticket}, 1, R);
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, EnvBases{env_total, env_base, host_base, ticket, longest}, 1, R);
     return cudaGetLastError();
 }
 
@@ -338,7 +349,8 @@ cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* o
                         unsigned long long* env_total, unsigned long long* env_base,
                         unsigned long long* host_base, unsigned int* ticket, int We, int per, cudaStream_t st) {
     if (We == 0) return cudaSuccess;
-    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, EnvBases{env_total, env_base, host_base, ticket}, per, RankParams{});
+    k_scan_env<<<We, 1024, 0, st>>>(envs, counts, off_local, EnvBases{env_total, env_base, host_base, ticket, false}, per,
+                                    RankParams{});
     return cudaGetLastError();
 }
 

@@ -190,9 +190,10 @@ gs_status upload_tables(gs_scene s, const std::vector<EnvSpec>& specs, int e0, i
 // cap > 0: planned (no host sync; keys beyond cap dropped and flagged).
 // quad: the compositor's warp form on 16x16 or 8x8 camera tiles: 1 for every
 // env, 0 for none, -1 for the envs of at most kQuadMaxPixels when the envs are
-// in ascending order of their pixels, else for all when no image has more.
+// in ascending order of their pixels, else for all when no image has more; -2 the
+// same, in an eager wave only where their buckets make it pay (warp_pays).
 gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& io, int tw, int th, int chunk,
                    unsigned long long cap, cudaStream_t st, bool timers, int64_t* launches,
-                   unsigned long long* total_out, int quad = -1);
+                   unsigned long long* total_out, int quad = -2);
 
 }  // namespace gsb

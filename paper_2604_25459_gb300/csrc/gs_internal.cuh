@@ -301,10 +301,14 @@ cudaError_t launch_scan(const EnvInfo* envs, const uint32_t* counts, uint32_t* o
                         unsigned long long* env_total, unsigned long long* env_base,
                         unsigned long long* host_base, unsigned int* ticket, int We, int per, cudaStream_t st);
 // As launch_scan, with the scans of the depth ranges and their window tables.
+// longest: host_base gets the keys of each env's longest bucket (at most
+// kTotalMost) above its low kTotalBits bits.
+constexpr int kTotalBits = 40;
+constexpr uint32_t kTotalMost = (1u << (64 - kTotalBits)) - 1u;
 cudaError_t launch_scan_ranks(const EnvInfo* envs, const uint32_t* counts, uint32_t* off_local,
                               unsigned long long* env_total, unsigned long long* env_base,
-                              unsigned long long* host_base, unsigned int* ticket, int We, const RankParams& R,
-                              cudaStream_t st);
+                              unsigned long long* host_base, bool longest, unsigned int* ticket, int We,
+                              const RankParams& R, cudaStream_t st);
 cudaError_t launch_scatter(const BinParams& P, int n_envs, int max_words, int max_T, int max_hist, cudaStream_t st);
 // Lists a launch's items by the length of their buckets, longest class first
 // (CompParams::items); class_cnt is zeroed by the caller.  Rays: item_cnt and
@@ -408,6 +412,23 @@ constexpr int kQuadMinEnvs = 128;
 inline bool warp_form(int tile_w, int tile_h, long long most_pixels, long long most_slots, int n_envs) {
     return ((tile_w == 16 && tile_h == 16) || (tile_w == 8 && tile_h == 8)) && most_pixels <= kQuadMaxPixels &&
            (most_slots >= kQuadMinSlots || n_envs > kQuadMinEnvs);
+}
+// Whether the warp form pays for images of `tiles` tiles with `keys` keys, the
+// longest bucket `most` (of the envs that warp_form admits).  On buckets that are
+// short on average, four warps that share a window beat four that each order
+// their own, unless long buckets among them would leave a CTA behind alone, or
+// the tiles are so few that latency counts.  Scatter + compositing, CTA form / warp
+// form (us).  The room, where a tenth of the tiles holds most keys: 333x251, 32
+// views of 9,000 slots (78 keys per tile) 180 / 227, of 30,000 (200) 315 / 289, of
+// 600,000 (2233) 1112 / 1119; 128x96, 64 views of 600,000 (6396) 4591 / 1521.  An
+// even cube: 300x250, 8 views of 120,000 (1209 per tile, 2432 tiles) 165 / 313; 128x96
+// of 30,000 (1095): 64 views (3072 tiles) 347 / 427, 4 views (192) 119 / 77; of
+// 120,000 (4361): 64 views 571 / 462.
+constexpr unsigned long long kEvenTiles = 400;
+inline bool warp_pays(unsigned long long tiles, unsigned long long keys, unsigned long long most) {
+    if (keys < 100 * tiles) return false;
+    const bool even = most * tiles < 4 * keys;
+    return !even || tiles < kEvenTiles || keys >= 3200 * tiles;
 }
 // Bits of the subtile mask below the ranks of the warp form's keys: one per 8x8
 // subtile while they and the ranks of n_slots records fit 32 bits, else none.

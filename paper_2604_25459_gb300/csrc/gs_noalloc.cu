@@ -281,7 +281,8 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         B.status = v.status;
         NA_CK(launch_rank_sample(R, Wn, st), "depth sample");
         NA_CK(launch_count(B, R, Wn, max_T, (ntx + 1) * (nty + 1), st), "count");
-        NA_CK(launch_scan_ranks(d_envs, counts, off, env_total, env_base, nullptr, work + kWorkWords - 1, Wn, R, st), "scan");
+        NA_CK(launch_scan_ranks(d_envs, counts, off, env_total, env_base, nullptr, false, work + kWorkWords - 1, Wn, R, st),
+              "scan");
         NA_CK(launch_rank(R, Wn, max_words, st), "depth ranks");
         unsigned long long eb[kMaxWave + 1];
         NA_CK(cudaMemcpyAsync(eb, env_base, sizeof(unsigned long long) * (Wn + 1), cudaMemcpyDeviceToHost, st),

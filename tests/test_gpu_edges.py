@@ -387,3 +387,26 @@ def test_depth_ranges_are_balanced(rank_ranges, n, seen):
     bins = rank_ranges(n, mask.ctypes.data_as(ctypes.c_void_p), per.ctypes.data_as(ctypes.c_void_p), len(per))
     assert bins > 0 and per[:bins].sum() == bits.sum()
     assert per[:bins].max() <= 3.0 * bits.sum() / bins
+
+
+@pytest.mark.parametrize("scene,n,width,height,envs", [("cube", 30_000, 300, 250, 8), ("cube", 30_000, 64, 48, 3),
+                                                       ("cube", 120_000, 40, 30, 2), ("room", 5_000, 200, 150, 4),
+                                                       ("room", 60_000, 200, 150, 4)])
+def test_images_do_not_depend_on_the_buckets_form(scene, n, width, height, envs):
+    """Even and uneven scenes with short and long buckets, few and many tiles: the
+    buckets decide between the compositor's forms, and the images are those of
+    32x16 tiles, which know one form only."""
+    import torch
+
+    if scene == "cube":
+        w = synth.make_c0(n=n)
+        cams, poses = np.repeat(synth.make_c0(n=1, width=width, height=height, f=0.86 * width).cams, envs), None
+    else:
+        w = synth.make_c1(n_envs=envs, width=width, height=height, f=0.8 * width, n_bg=n, per_link=n // 100)
+        cams, poses = w.cams, torch.from_numpy(w.link_poses).cuda()
+    s = gsbatch.scene_from_workload(w)
+    out = [t.clone() for t in s.render(poses, cams)]
+    s.set_tile(32, 16)
+    for a, b in zip(out, s.render(poses, cams)):
+        assert torch.equal(a, b)
+    s.close()
