@@ -410,3 +410,23 @@ def test_images_do_not_depend_on_the_buckets_form(scene, n, width, height, envs)
     for a, b in zip(out, s.render(poses, cams)):
         assert torch.equal(a, b)
     s.close()
+
+
+@pytest.mark.parametrize("n", [31, 1000, 1024, 1025, 2000, 2048])
+@pytest.mark.parametrize("depths", ["equal", "crowd", "far"])
+def test_ranking_of_small_scenes_of_crowded_depths(n, depths):
+    """Scenes ranked by one block whose depths fill one counting range or a few:
+    all equal, a crowd among spread ones, and one splat far behind the others."""
+    w = synth.make_c0(n=n)
+    mean = w.background.mean.copy()
+    if depths == "equal":
+        mean[:, 2] = 0.0
+    elif depths == "crowd":
+        mean[: n // 20 + 33, 2] = 0.25
+    else:
+        mean[0] = [0.0, 0.0, 4000.0]
+    w = dataclasses.replace(w, background=dataclasses.replace(w.background, mean=mean))
+    out = gpu_render(w, debug=True, keep_scene=True)
+    _, vis = _check_lists(out["scene"], w, 0, (16, 16), 128, 96)
+    out["scene"].close()
+    assert len(vis) > n // 2
