@@ -475,8 +475,8 @@ gs_status upload_tables(gs_scene s, const std::vector<EnvSpec>& specs, int e0, i
 int warp_envs(const WaveTables& wt, int tw, int th, int quad) {
     if (quad == 0) return 0;
     auto small = [&](int e) {
-        if (quad > 0) return warp_form(tw, th, 0, kQuadMinSlots, wt.We);
-        return warp_form(tw, th, (long long)wt.host_envs[e].W * wt.host_envs[e].H, wt.max_words * 32ll, wt.We);
+        if (quad > 0) return warp_form(tw, th, 0, kQuadMinSlots);
+        return warp_form(tw, th, (long long)wt.host_envs[e].W * wt.host_envs[e].H, wt.max_words * 32ll);
     };
     int n = 0;
     while (n < wt.We && small(n)) ++n;
@@ -1549,8 +1549,8 @@ gs_status gs_plan_launch(gs_plan p, const float* link_poses, float* rgb, float* 
             // largest images are beyond its range, for the envs within it (claim
             // size 1, as both forms claim best).
             const gs_camera &first = p->envs.front().cam, &most = p->envs.back().cam;
-            const bool mixed = warp_form(16, 16, (long long)first.width * first.height, kQuadMinSlots, 1) &&
-                               !warp_form(16, 16, (long long)most.width * most.height, kQuadMinSlots, 1);
+            const bool mixed = warp_form(16, 16, (long long)first.width * first.height, kQuadMinSlots) &&
+                               !warp_form(16, 16, (long long)most.width * most.height, kQuadMinSlots);
             const int shapes[5][2] = {{16, 16}, {32, 8}, {16, 8}, {8, 8}, {32, 16}};
             for (auto& sh : shapes)
                 for (int ch : {1, 4}) {

@@ -403,15 +403,15 @@ constexpr int kCompCap = 768;
 // 837 / 776, 64 2290 / 2152; 480x360: 160 / 174, 419 / 352, 835 / 833, 2617 /
 // 2658; 640x480: 155 / 200, 379 / 475, 1007 / 1097, 3399 / 3859.
 constexpr int kQuadMaxPixels = 140000;
-// A few envs of few slots have short buckets, which the CTA form sorts at once,
-// without an item order.  Calls, warp / CTA form (us): 24 envs of 1500 splats at
-// 64x48 106 / 94, of 4000 at 128x96 132 / 123, of 6000 at 40x30 158 / 236; 64 of
-// 3000 at 64x48 142 / 132, 200 of 2000 160 / 172.
+// Envs of few slots have short buckets, which the CTA form sorts at once, without
+// an item order.  Calls, warp / CTA form (us): 24 envs of 1500 splats at 64x48 106
+// / 94, of 4000 at 128x96 132 / 123, of 6000 at 40x30 158 / 236; 64 of 3000 at 64x48
+// 142 / 132; 200 of 1100 in the room at 32x24 130 / 118, of 2200 at 64x48 167 / 156,
+// 200 even cubes of 2000 at 64x48 165 / 176.
 constexpr long long kQuadMinSlots = 4097;
-constexpr int kQuadMinEnvs = 128;
-inline bool warp_form(int tile_w, int tile_h, long long most_pixels, long long most_slots, int n_envs) {
+inline bool warp_form(int tile_w, int tile_h, long long most_pixels, long long most_slots) {
     return ((tile_w == 16 && tile_h == 16) || (tile_w == 8 && tile_h == 8)) && most_pixels <= kQuadMaxPixels &&
-           (most_slots >= kQuadMinSlots || n_envs > kQuadMinEnvs);
+           most_slots >= kQuadMinSlots;
 }
 // Whether the warp form pays for images of `tiles` tiles with `keys` keys, the
 // longest bucket `most` (of the envs that warp_form admits).  On buckets that are

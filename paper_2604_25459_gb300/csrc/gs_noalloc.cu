@@ -272,7 +272,7 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
             tab += off_bytes;
         }
         B.rank = R.rank;
-        const bool warp = warp_form(tw, th, (long long)px, max_words * 32ll, Wn);
+        const bool warp = warp_form(tw, th, (long long)px, max_words * 32ll);
         if (warp) B.key_shift = subtile_bits(tw, th, (unsigned long long)max_words * 32);
         B.counts = counts;
         B.off_local = off;
