@@ -730,8 +730,6 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         C.chunk = chunk;
         C.work = work;
         C.r0 = P.r0;
-        C.r1 = P.r1;
-        C.r2 = P.r2;
         C.nvis = R.nvis;
         C.order = R.order;
         C.counts = counts;
@@ -753,7 +751,6 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         C.score = io.score;
         C.nbp = (unsigned)bg_slots(s->D.n_bg);
         C.bg_index = s->bg_order.empty() ? nullptr : s->bg_index.as<int>();
-        C.n_bg = (unsigned)s->D.n_bg;
         C.lidars = io.lidars;
         C.r3 = P.r3;
         C.status = status;

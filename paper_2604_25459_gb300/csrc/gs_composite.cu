@@ -11,9 +11,9 @@
 // depth-ordered windows of at most kCompCap ranks, so ordering stops at the
 // window where every pixel has terminated.  A short bucket is one window,
 // sorted in shared memory by a counting sort.  A long one is ordered by setting
-// a bit per rank in a bitmap of the next kGroups x 512 ranks and reading the
-// bits back in order: ranks are unique, so the bitmap is the sorted list, at
-// one shared-memory OR per key.  A window's ranks are mapped to record
+// a bit per rank in a bitmap of the next 65,536 ranks (128 groups of 512; fewer
+// on tiles below 16x16) and reading the bits back in order: ranks are unique, so
+// the bitmap is the sorted list, at one shared-memory OR per key.  A window's ranks are mapped to record
 // slots; each warp then walks the window on its own, 32 splats at a time:
 // a lane stages one of them (its record copied while the 32 before are
 // blended) and tests it against the warp's subtile (box, then the exact
@@ -25,9 +25,9 @@
 // slots used, now 72 %): 256 views of 640x480 11.0 -> 10.7 ms.  What bounds
 // it is instruction issue: 72 steps of 2 splats x 64 pixels per subtile, 75
 // instructions each.  Besides the image form the kernel has an observation
-// form (8-bit colour after per-env appearance, half depth), a contribution
-// form (per-Gaussian blending weights, for pruning) and a LiDAR form (rays of
-// an (azimuth, beam) grid, Gaussians evaluated in ray space).
+// form (8-bit colour after per-env appearance, half depth) and a contribution
+// form (per-Gaussian blending weights, for pruning); images of low resolution
+// and LiDAR scans are composited by gs_composite_warp.cu.
 #include "gs_blend.cuh"
 #include "gs_block.cuh"
 #include <type_traits>

@@ -219,9 +219,7 @@ struct CompParams {
     unsigned int item_pitch;
     unsigned int* team_work;  // nullable: the teams' work counter (zeroed before the launch)
     int team_classes;         // set by the launch: the first classes go to teams of four warps
-    const float4* r0;
-    const float4* r1;
-    const float4* r2;
+    const float4* r0;                // records, r0, r1 and r2 side by side (kRecStride)
     const uint32_t* nvis;            // per env of the wave: ranked records
     const uint32_t* order;           // record slot of rank r at rec_base + r
     const uint32_t* counts;
@@ -246,7 +244,6 @@ struct CompParams {
     float* score;         // nullable: contribution pass (no images): score[g] += sum of alpha T
     unsigned int nbp;     // background slots (slot j < nbp is the background Gaussian stored at j)
     const int* bg_index;  // nullable: caller's index of the background Gaussian in slot j (contribution pass, debug)
-    unsigned int n_bg;
     const gs_lidar* lidars;  // nullable: LiDAR scan (range in depth, hit in alpha), per env of the wave
     const uint4* r3;         // LiDAR scan: records' fourth word (|g2|)
     uint32_t* status;
@@ -360,18 +357,18 @@ inline RankParams rank_sizes(long long max_words, int We, bool lidar) {
 // (average spans at 128x128, 64 tiles, are 2.1 tiles; at 320x240, 300: 4.5; at
 // 640x480: 11).
 constexpr int kDiffTiles = 256;
-// Visibility words per scatter block: many blocks per SM, as one block may hold
-// a link that fills the image (at 640x480, 32 envs: 30 us per env with 256
-// words, 13 with 32), and on large grids 64, whose writes stay in reach of the
-// L2 (256 envs: 8.5 us per env with 256, 7.15 with 64, 8.6 with 32); on small
-// grids the per-block tables weigh more (512 envs at 128x128: 2.3 us with 256,
-// 2.7 with 64).
 // Bytes of the places that the count notes for the scatter (BinParams::tile_off);
 // 0 where their blocks differ, and on grids counted by difference arrays.
 inline size_t tile_off_bytes(const RankParams& R, int words_per_block, int We, int max_T, bool wrap) {
     if (words_per_block != R.words_per_block || (!wrap && max_T >= kDiffTiles)) return 0;
     return (size_t)We * R.blocks * max_T * 4;
 }
+// Visibility words per scatter block: many blocks per SM, as one block may hold
+// a link that fills the image (at 640x480, 32 envs: 30 us per env with 256
+// words, 13 with 32), and on large grids 64, whose writes stay in reach of the
+// L2 (256 envs: 8.5 us per env with 256, 7.15 with 64, 8.6 with 32); on small
+// grids the per-block tables weigh more (512 envs at 128x128: 2.3 us with 256,
+// 2.7 with 64).
 inline int scatter_words(long long max_words, int n_envs, int max_T) {
     int w = max_T >= kDiffTiles ? 64 : kWordsPerBlock;
     while (w > 16 && (max_words + w - 1) / w * n_envs < 62 * 152) w /= 2;

@@ -305,11 +305,8 @@ extern "C" gs_status gs_render_batch_noalloc(gs_scene s, int n_envs, const float
         C.item_begin = 0;
         C.item_end = sen.tile_base;
         C.chunk = 1;
-        C.n_bg = (unsigned)v.D.n_bg;
         C.work = work;
         C.r0 = P.r0;
-        C.r1 = P.r1;
-        C.r2 = P.r2;
         C.nvis = R.nvis;
         C.order = R.order;
         C.counts = counts;
