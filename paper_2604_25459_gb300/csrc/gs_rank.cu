@@ -20,7 +20,7 @@ namespace gsb {
 
 namespace {
 
-constexpr int kSampleLooks = 8;     // slots looked at per thread of k_rank_sample
+constexpr int kSampleLooks = 8;     // slots looked at per thread of k_rank_sample: a byte of bits
 constexpr int kSortThreads = 256;
 constexpr int kSortCap = 2048;      // keys of a window sorted in shared memory
 constexpr int kSubBins = 1024;      // depth ranges of a window's counting sort
@@ -83,29 +83,37 @@ __device__ __forceinline__ void block_bitonic(unsigned long long (&v)[K], unsign
 // and k_rank_sort took 28 us instead of 10.  bins is a power of two, so a
 // splitter's place is a shift (640,000 slots, one env: 28 us with a 64-bit
 // division, 21 with the shift).  The stride is odd, so it does not resonate with
-// the 32-slot visibility words or the links' cluster sizes.  A thread looks at
-// neighbouring places, so that the samples are numbered in storage order and every
-// n-th of them is kept from all over it: numbered by threads with 1024 places
-// between a thread's looks, views that see every slot kept each thread's first
-// look, the first eighth of the (Morton) order, and one range got up to half of
-// the records (8 views of 120,000 splats: ranking after the scan 175 us, now 29).
+// the 32-slot visibility words or the links' cluster sizes.  A thread numbers eight
+// neighbouring looks, so that the visible ones are numbered in storage order and
+// every n-th, which is kept, comes from all over it: numbered by threads with 1024
+// looks between a thread's, views that see every slot kept each thread's first, the
+// first eighth of the (Morton) order, and one range got up to half of the records
+// (8 views of 120,000 splats: ranking after the scan 175 us, now 29).  The looks
+// themselves are taken across the block, and the kept ones listed before one thread
+// loads each: with both by the numbering thread the kernel took 11.3 us instead of
+// 10.3 for 3,000 slots and 22.5 instead of 20.5 for 600,000.
 template <int K>
 __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
     constexpr int M = 1024 * K;
     __shared__ unsigned long long smp[M];
     __shared__ uint32_t red[32];
+    __shared__ uint32_t words[32 * kSampleLooks];
+    __shared__ uint16_t where[M];  // the kept looks
     const int el = blockIdx.x, tid = threadIdx.x;
     const EnvInfo E = P.envs[el];
     const uint32_t n = E.n_local;
     const int want = M;
     uint32_t step = (n + 1024 * kSampleLooks - 1) / (1024 * kSampleLooks);
     if (step > 1) step |= 1u;
-    uint32_t seen = 0;  // bit k: slot (kSampleLooks tid + k) step is visible
 #pragma unroll
-    for (int k = 0; k < kSampleLooks; ++k) {
-        const unsigned long long j = (unsigned long long)(kSampleLooks * tid + k) * step;
-        if (j < n && ((__ldg(P.mask + E.mask_base + (j >> 5)) >> (j & 31u)) & 1u)) seen |= 1u << k;
+    for (int k = 0; k < kSampleLooks; ++k) {  // bit i of the words: look i, slot i step, is visible
+        const unsigned long long j = (unsigned long long)(tid + 1024 * k) * step;
+        const uint32_t m =
+            __ballot_sync(0xffffffffu, j < n && ((__ldg(P.mask + E.mask_base + (j >> 5)) >> (j & 31u)) & 1u));
+        if ((tid & 31) == 0) words[32 * k + (tid >> 5)] = m;
     }
+    __syncthreads();
+    const uint32_t seen = reinterpret_cast<const uint8_t*>(words)[tid];  // looks kSampleLooks tid + k
     uint32_t total = 0;
     uint32_t at = block_excl_scan_total<1024>((uint32_t)__popc(seen), red, total);
     const uint32_t every = (total + (uint32_t)want - 1) / (uint32_t)want;
@@ -116,12 +124,16 @@ __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
 #pragma unroll
     for (int k = 0; k < kSampleLooks; ++k) {
         if (!((seen >> k) & 1u)) continue;
-        if (at % every == 0) {
-            const unsigned long long j = (unsigned long long)(kSampleLooks * tid + k) * step;
-            smp[at / every] = rank_key(P, P.r3[E.rec_base + j], (uint32_t)j);
-        }
+        if (at % every == 0) where[at / every] = (uint16_t)(kSampleLooks * tid + k);
         ++at;
     }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (tid + 1024 * k < kept) {
+            const uint32_t j = (uint32_t)where[tid + 1024 * k] * step;  // < n
+            smp[tid + 1024 * k] = rank_key(P, P.r3[E.rec_base + j], j);
+        }
     __syncthreads();
     // thread t holds elements K t .. K t + K - 1
     unsigned long long v[K];
