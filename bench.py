@@ -38,10 +38,12 @@ UNIT = "env-frames/s"
 # DRAM traffic of the compositor per env of a launch, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum over a 32-env launch, divided
 # by 32), valid only for the compositor sources it was taken on (the hash
-# below; sources that differ from the captured ones in comments only keep it).
-COMPOSITE_TRAFFIC_PER_ENV = (0.424962e9 + 0.145890e9) / 32
-COMPOSITE_TRAFFIC_SOURCES = ("paper_2604_25459_gb300/csrc/gs_composite.cu",)
-COMPOSITE_TRAFFIC_SHA = "9260d64e036eaff7"
+# below, over the kernel and every header of the library that it includes;
+# sources that differ from the captured ones in comments only keep it).
+COMPOSITE_TRAFFIC_PER_ENV = (0.422816e9 + 0.144039e9) / 32
+COMPOSITE_TRAFFIC_SOURCES = tuple("paper_2604_25459_gb300/csrc/" + f for f in (
+    "gs_composite.cu", "gs_blend.cuh", "gs_block.cuh", "gs_internal.cuh"))
+COMPOSITE_TRAFFIC_SHA = "497a7a9d5669a19e"
 
 
 def _sources_sha(paths) -> str:
