@@ -276,17 +276,17 @@ gs_status check_cam(const gs_camera& c, int e) {
 gs_status check_specs(gs_scene s, const std::vector<EnvSpec>& specs, int tw, int th) {
     for (size_t e = 0; e < specs.size(); ++e) {
         const EnvSpec& sp = specs[e];
-        ST(check_cam(*sp.cam, (int)e));
+        ST(check_cam(*sp.cam, sp.env));
         const int ntx = (sp.cam->width + tw - 1) / tw, nty = (sp.cam->height + th - 1) / th;
         if (ntx * nty > 16384)
-            return fail(GS_ERR_UNSUPPORTED, "env %d: %d tiles exceed the 16384 supported (use larger tiles)", (int)e,
+            return fail(GS_ERR_UNSUPPORTED, "env %d: %d tiles exceed the 16384 supported (use larger tiles)", sp.env,
                         ntx * nty);
         if (sp.link_begin < 0 || sp.link_end < sp.link_begin || sp.link_end > s->D.n_links)
-            return fail(GS_ERR_INVALID, "env %d: link range [%d, %d) outside [0, %d]", (int)e, sp.link_begin,
+            return fail(GS_ERR_INVALID, "env %d: link range [%d, %d) outside [0, %d]", sp.env, sp.link_begin,
                         sp.link_end, s->D.n_links);
         if (sp.link_end > sp.link_begin && sp.pose_offset < 0)
-            return fail(GS_ERR_INVALID, "env %d: negative pose_offset", (int)e);
-        if (sp.pixel_offset < 0) return fail(GS_ERR_INVALID, "env %d: negative pixel_offset", (int)e);
+            return fail(GS_ERR_INVALID, "env %d: negative pose_offset", sp.env);
+        if (sp.pixel_offset < 0) return fail(GS_ERR_INVALID, "env %d: negative pixel_offset", sp.env);
     }
     return GS_OK;
 }
@@ -358,7 +358,7 @@ gs_status plan_waves(gs_scene s, const std::vector<EnvSpec>& specs, int tw, int 
         const double b = (double)(env_bytes(s, specs[e], tw, th, debug) + extra_per_env);
         const EnvSize z = env_size(s, specs[e], tw, th);
         const double alone = b + (double)wave_table_bytes(z, 1, lidar, budget);
-        if (alone > cap) return fail(GS_ERR_OOM, "env %d needs %.0f bytes of scratch; budget is %lld", e, alone,
+        if (alone > cap) return fail(GS_ERR_OOM, "env %d needs %.0f bytes of scratch; budget is %lld", specs[e].env, alone,
                                      (long long)s->budget);
         if (e > e0 && (acc + b + (double)wave_table_bytes(most.with(z), e - e0 + 1, lidar, budget) > cap ||
                        (max_wave > 0 && e - e0 >= max_wave))) {
@@ -807,7 +807,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
 
 enum class Out { Device, Host };
 
-gs_status render_specs(gs_scene s, std::vector<EnvSpec>& specs, const float* poses_dev, const Outputs& o,
+gs_status render_specs(gs_scene s, const std::vector<EnvSpec>& specs, const float* poses_dev, const Outputs& o,
                        cudaStream_t st, Out mode, int64_t pix_per_env_host) {
     float* const rgb = o.rgb;
     float* const depth = o.depth;
@@ -823,19 +823,6 @@ gs_status render_specs(gs_scene s, std::vector<EnvSpec>& specs, const float* pos
     if (mode == Out::Host) extra = (size_t)pix_per_env_host * (o.rgb_px() + o.depth_px() + (alpha ? 4 : 0)) * 2;
     std::vector<std::pair<int, int>> waves;
     ST(plan_waves(s, specs, tw, th, s->debug != 0, s->max_wave, extra, &waves));
-    // Low resolutions first within a wave (see gs_plan_create): their images then
-    // take the compositor's warp form.  Outputs are placed by pixel_offset and the
-    // debug copies look an env up by the caller's index, so the order is not
-    // visible.  Debug renders keep the caller's order, by which their lists of the
-    // last sub-wave are taken.
-    if (!s->debug)
-        for (auto& w : waves) {
-            auto smaller = [](const EnvSpec& a, const EnvSpec& b) {
-                return (int64_t)a.cam->width * a.cam->height < (int64_t)b.cam->width * b.cam->height;
-            };
-            const auto b = specs.begin() + w.first, e = specs.begin() + w.second;
-            if (!std::is_sorted(b, e, smaller)) std::stable_sort(b, e, smaller);
-        }
     int64_t launches = 0;
     if (mode == Out::Device) {
         for (auto& w : waves) {
@@ -1446,6 +1433,18 @@ gs_status gs_render_batch_v(gs_scene s, int n_envs, const gs_env* envs, const fl
     if (any_links && !link_poses) return fail(GS_ERR_INVALID, "null link_poses");
     std::vector<EnvSpec> specs;
     ST(specs_from_envs(s, n_envs, envs, &specs));
+    ST(check_specs(s, specs, s->tile_w, s->tile_h));
+    // Low resolutions first (see gs_plan_create): their images then take the
+    // compositor's warp form.  Over the whole batch, so that a wave holds images of
+    // one kind: in order inside each wave of the caller's split only, 4096 envs of
+    // mixed resolutions in eight scenes took 215 ms instead of 178.  Outputs are
+    // placed by pixel_offset and the debug copies look an env up by the caller's
+    // index, so the order is not visible; debug renders keep the caller's, by which
+    // their lists of the last sub-wave are taken.
+    if (!s->debug)
+        std::stable_sort(specs.begin(), specs.end(), [](const EnvSpec& a, const EnvSpec& b) {
+            return (int64_t)a.cam->width * a.cam->height < (int64_t)b.cam->width * b.cam->height;
+        });
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     CK(cudaSetDevice(s->device), "set device");
     if (s->D.n == 0) {
