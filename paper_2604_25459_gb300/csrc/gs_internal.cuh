@@ -329,9 +329,11 @@ constexpr int kRankBins = 2048;      // depth ranges per env, at most
 constexpr int kRankStride = 768;     // ranks per window of the depth sort
 // Depth ranges of an env of n record slots: one per 512 slots for cameras
 // (which see a quarter of a room), one per 256 for LiDARs (which see all of it).
-// Envs of at most this many slots are ranked whole (up to 4096 was slower: 64
-// envs of 3000 splats at 64x48 151 us a call, by sampling 143).
-constexpr int kSmallRank = 2048;
+// Envs of at most this many slots are ranked whole, by one CTA each, as many keys
+// as its shared memory sorts.  Calls by sampling / whole (us): 8 views of 128x96 of
+// 3000 splats without allocation 98 / 79, 24 of 4000 120 / 105; 64 of 64x48 of 3000
+// 135 / 128, 200 201 / 185; one of 300x250 of 4000 75 / 69.
+constexpr int kSmallRank = 4096;
 inline int rank_bins(long long n, bool lidar) {
     const int most = lidar ? kRankBins : kRankBins / 2;
     int b = 32;

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(1024) k_rank_sample(RankParams P) {
 // The kernel on 200 views of 32x24, 1100 slots each: 25 us with the bitonic sort
 // for all, now 9.  Calls without allocation (us; before records were ranked / by
 // sampling / by the bitonic sort / now): one 64x48 view of 900 splats 73 / 94 / 71 /
-// 71, 24 views of 1500 90 / 119 / 92 / 84.
+// 71, 24 views of 1500 90 / 119 / 92 / 84.  K = 4 takes 16 us for 200 views.
 constexpr int kSmallBins = 2048;
 constexpr int kSmallInsert = 32;
 template <int K>
@@ -465,13 +465,14 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_rank_sort(RankParams P) {
     }
 }
 
-static_assert(kSmallRank <= 2 * 1024 && kSmallBins == 2 * 1024, "small envs fit one CTA's keys and counters");
+static_assert(kSmallRank <= 4 * 1024 && kSmallBins == 2 * 1024, "small envs fit one CTA's keys and counters");
 
 cudaError_t launch_rank_sample(const RankParams& R, int n_envs, cudaStream_t st) {
     if (n_envs == 0) return cudaSuccess;
     if (R.bins == 0) {
         if (R.max_slots <= 1024) k_rank_small<1><<<n_envs, 1024, 0, st>>>(R);
-        else k_rank_small<2><<<n_envs, 1024, 0, st>>>(R);
+        else if (R.max_slots <= 2048) k_rank_small<2><<<n_envs, 1024, 0, st>>>(R);
+        else k_rank_small<4><<<n_envs, 1024, 0, st>>>(R);
         return cudaGetLastError();
     }
     if (R.bins <= 512) k_rank_sample<1><<<n_envs, 1024, 0, st>>>(R);

@@ -374,7 +374,7 @@ def rank_ranges(tmp_path_factory):
     return _native("rank_ranges", tmp_path_factory.mktemp("native"))
 
 
-@pytest.mark.parametrize("n", [3000, 8192, 20_000, 120_000, 300_000])
+@pytest.mark.parametrize("n", [5000, 8192, 20_000, 120_000, 300_000])
 @pytest.mark.parametrize("seen", [1.0, 0.5])
 def test_depth_ranges_are_balanced(rank_ranges, n, seen):
     """The sample is kept from all over the storage order, whatever share of it is
@@ -412,11 +412,12 @@ def test_images_do_not_depend_on_the_buckets_form(scene, n, width, height, envs)
     s.close()
 
 
-@pytest.mark.parametrize("n", [31, 1000, 1024, 1025, 2000, 2048])
+@pytest.mark.parametrize("n", [31, 1000, 1024, 1025, 2000, 2048, 2049, 3000, 4096, 4097])
 @pytest.mark.parametrize("depths", ["equal", "crowd", "far"])
 def test_ranking_of_small_scenes_of_crowded_depths(n, depths):
-    """Scenes ranked by one block whose depths fill one counting range or a few:
-    all equal, a crowd among spread ones, and one splat far behind the others."""
+    """Scenes ranked by one block (up to 4096 slots, and the first above) whose depths
+    fill one counting range or a few: all equal, a crowd among spread ones, and one
+    splat far behind the others."""
     w = synth.make_c0(n=n)
     mean = w.background.mean.copy()
     if depths == "equal":
