@@ -672,8 +672,10 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         cap_keys = (unsigned long long)((double)s->budget * 0.2 / 4);  // 4 bytes a key
     }
     int n_warp = io.lidars ? We : n_small;
+    bool even = false;
     if (quad == -2 && eb && n_small > 0) {  // all of them or none, by their buckets
         const unsigned long long tiles = wt.host_envs[n_small].tile_base;
+        even = even_buckets(tiles, eb[n_small], most);
         if (!warp_pays(tiles, eb[n_small], most)) n_warp = 0;
     }
     if (n_warp > 0) B.key_shift = subtile_bits(tw, th, (unsigned long long)wt.max_words * 32);
@@ -762,6 +764,7 @@ gs_status run_wave(gs_scene s, Scratch& sc, const WaveTables& wt, const WaveIO& 
         if (es > ea) {
             CompParams Q = C;
             Q.quad = 1;
+            Q.even = even;
             if (!io.ray_dirs) Q.item_end = wt.host_envs[es].tile_base;
             Q.e_end = es;
             const unsigned long long n_items = Q.item_end - Q.item_begin;  // long buckets first

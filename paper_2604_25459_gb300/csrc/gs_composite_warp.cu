@@ -1200,12 +1200,16 @@ static cudaError_t launch_warps(const CompParams& P, cudaStream_t st, int* ctas)
     // are few per resident CTA, all go to teams (whole calls, us): one 128x96 view
     // of 16,384 splats (0.2 items per CTA) 57 -> 39, 8 of them (1.7) 145 -> 122,
     // 16 (3.4) 195 -> 173, but 2 views of 333x251 in the room (2.9) 351 -> 362 and
-    // 4 rosettes (1.7) 1403 -> 1465.
+    // 4 rosettes (1.7) 1403 -> 1465.  Even scenes have no long buckets to wait for: whole
+    // calls with teams for three classes / without (us), 64 views of 128x96 of an even
+    // cube of 120,000 (3.4 items per warp) 1145 / 912, 24 of them (1.3) 508 / 484, 200 of
+    // 64x48 (2.6) 2057 / 1803.
     constexpr bool LID = MODE == 1 || MODE == 3;
     Q.team_classes = 0;
     if (P.items && P.team_work) {
         const double per_warp = (double)items / ((double)kWarps * full);
         if (items * 2 <= (LID ? 2ull : 5ull) * full) Q.team_classes = kItemClasses;
+        else if (P.even && per_warp > 1.0) Q.team_classes = 0;
         else if (per_warp <= 6.0) Q.team_classes = 3;
         else if (MODE == 1 || MODE == 3) Q.team_classes = per_warp <= 12.0 ? 2 : 0;
         else if (per_warp <= 20.0) Q.team_classes = 1;

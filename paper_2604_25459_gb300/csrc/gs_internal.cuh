@@ -231,6 +231,7 @@ struct CompParams {
     unsigned long long* neval;       // nullable: composited (pixel, Gaussian) pair counter
     int tile_w, tile_h;
     int quad;       // camera images: the warp form (k_composite_warp)
+    int even;       // no bucket of four times the average: no tail of long ones for teams
     // Keys of waves with envs in the warp form carry, below the rank, one bit
     // per 8x8 subtile of the tile that the record's box reaches (row-major): key
     // = rank << key_shift | mask.  key_shift = 0: no mask (plain ranks).
@@ -424,10 +425,11 @@ inline bool warp_form(int tile_w, int tile_h, long long most_pixels, long long m
 // of 30,000 (1095): 64 views (3072 tiles) 347 / 427, 4 views (192) 119 / 77; of
 // 120,000 (4361): 64 views 571 / 462.
 constexpr unsigned long long kEvenTiles = 400;
+inline bool even_buckets(unsigned long long tiles, unsigned long long keys, unsigned long long most) {
+    return tiles >= kEvenTiles && most * tiles < 4 * keys;
+}
 inline bool warp_pays(unsigned long long tiles, unsigned long long keys, unsigned long long most) {
-    if (keys < 100 * tiles) return false;
-    const bool even = most * tiles < 4 * keys;
-    return !even || tiles < kEvenTiles || keys >= 3200 * tiles;
+    return keys >= 100 * tiles && (!even_buckets(tiles, keys, most) || keys >= 3200 * tiles);
 }
 // Bits of the subtile mask below the ranks of the warp form's keys: one per 8x8
 // subtile while they and the ranks of n_slots records fit 32 bits, else none.

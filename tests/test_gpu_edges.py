@@ -391,7 +391,7 @@ def test_depth_ranges_are_balanced(rank_ranges, n, seen):
 
 @pytest.mark.parametrize("scene,n,width,height,envs", [("cube", 30_000, 300, 250, 8), ("cube", 30_000, 64, 48, 3),
                                                        ("cube", 120_000, 40, 30, 2), ("room", 5_000, 200, 150, 4),
-                                                       ("room", 60_000, 200, 150, 4)])
+                                                       ("room", 60_000, 200, 150, 4), ("cube", 60_000, 64, 48, 110)])
 def test_images_do_not_depend_on_the_buckets_form(scene, n, width, height, envs):
     """Even and uneven scenes with short and long buckets, few and many tiles: the
     buckets decide between the compositor's forms, and the images are those of
